@@ -89,9 +89,8 @@ int tiles_of(int w, int h) { return ((w + kTile - 1) / kTile) * ((h + kTile - 1)
 size_t shared_bytes(int64_t n, int64_t code_rows_k) {
   const size_t un = (size_t)n;
   size_t b = align_up(sizeof(WsHeader));
-  b += 2 * align_up(sizeof(float) * 3 * un);              // spatially ordered means, scales
-  b += align_up(sizeof(float) * 4 * un);                  // quats
-  b += 4 * align_up(sizeof(float) * un);                  // opacity, tau, orig, cell
+  b += align_up(sizeof(SceneRec) * un);                   // spatially ordered scene records
+  b += 2 * align_up(sizeof(float) * un);                  // orig, cell
   b += align_up(reorder_scratch_bytes());
   b += 2 * align_up((size_t)code_rows_k * 4);             // filtered codes (s > K)
   return b;
@@ -124,11 +123,7 @@ size_t carve_scene_part(void* base, int64_t n, int64_t code_rows_k, UpliftWs* w,
   const size_t un = (size_t)n;
   auto take = [&](size_t sz) { char* q = p + off; off += align_up(sz); return (void*)q; };
   w->hdr = (WsHeader*)take(sizeof(WsHeader));
-  w->sp.means = (float*)take(sizeof(float) * 3 * un);
-  w->sp.scales = (float*)take(sizeof(float) * 3 * un);
-  w->sp.quats = (float*)take(sizeof(float) * 4 * un);
-  w->sp.opacity = (float*)take(sizeof(float) * un);
-  w->sp.tau = (float*)take(sizeof(float) * un);
+  w->sp.rec = (SceneRec*)take(sizeof(SceneRec) * un);
   w->sp.orig = (int32_t*)take(sizeof(int32_t) * un);
   w->cell = (uint32_t*)take(sizeof(uint32_t) * un);
   w->cells_scratch = (uint32_t*)take(reorder_scratch_bytes());
@@ -564,18 +559,13 @@ int uplift_call(const UpliftCall& c, void* workspace, size_t ws_bytes, int warp_
   const UpliftWs& ws = wsl[0];
   const int64_t n = scene->n;
   cudaError_t e;
-  if ((e = cudaMemsetAsync(ws.hdr, 0, sizeof(WsHeader), st)) != cudaSuccess) return cuda_fail(e, "memset");
+  if ((e = launch_begin(wsl, chunked ? 0 : lanes, max_tiles, st)) != cudaSuccess) return cuda_fail(e, "begin");
   const bool compensated = (accum_mode & SCOUP_ACCUM_COMPENSATED) != 0;
   float* comp = compensated ? accum + (size_t)n * (size_t)Crow : nullptr;
   if (n > 0 && !(accum_mode & SCOUP_ACCUM_CONTINUE) &&
       (e = cudaMemsetAsync(accum, 0, sizeof(float) * (size_t)n * (size_t)Crow * (compensated ? 2 : 1), st)) !=
           cudaSuccess)
     return cuda_fail(e, "memset accum");
-  for (int l = 0; l < (chunked ? 0 : lanes); ++l)
-    if ((e = cudaMemsetAsync(wsl[l].tile_glob, 0, sizeof(uint32_t) * ((size_t)max_tiles + 1), st)) != cudaSuccess ||
-        (e = cudaMemsetAsync(wsl[l].tile_count, 0, sizeof(uint32_t) * ((size_t)max_tiles + 1), st)) != cudaSuccess ||
-        (e = cudaMemsetAsync(wsl[l].dhist, 0, sizeof(uint32_t) * kDepthBuckets, st)) != cudaSuccess)
-      return cuda_fail(e, "memset");
   const SlabPlan plan = uplift_slab_plan();
   const int32_t* ci = code_idx;
   const float* cv = code_val;
@@ -851,8 +841,8 @@ int scoup_uplift_plan(const scoup_scene* scene, const scoup_camera* cams, int32_
   int32_t* ci = nullptr;
   float* cv = nullptr;
   UpliftWs ws = carve(workspace, ws_bytes, scene->n, max_tiles, 0, &ci, &cv);
-  cudaError_t e = cudaMemsetAsync(ws.hdr, 0, sizeof(WsHeader), st);
-  if (e != cudaSuccess) return cuda_fail(e, "memset");
+  cudaError_t e = launch_begin(&ws, 0, max_tiles, st);
+  if (e != cudaSuccess) return cuda_fail(e, "begin");
   if ((e = launch_reorder(*scene, ws, st)) != cudaSuccess) return cuda_fail(e, "reorder");
   int64_t best = 0;
   for (int v = 0; v < V; ++v) {
@@ -966,10 +956,7 @@ int scoup_render(const scoup_scene* scene, const int32_t* topk_idx, const float*
   const int64_t n = scene->n;
   const CamArgs ca = cam_args(*cam);
   cudaError_t e;
-  if ((e = cudaMemsetAsync(ws.hdr, 0, sizeof(WsHeader), st)) != cudaSuccess) return cuda_fail(e, "memset");
-  if ((e = cudaMemsetAsync(ws.tile_glob, 0, sizeof(uint32_t) * ((size_t)max_tiles + 1), st)) != cudaSuccess ||
-      (e = cudaMemsetAsync(ws.tile_count, 0, sizeof(uint32_t) * ((size_t)max_tiles + 1), st)) != cudaSuccess)
-    return cuda_fail(e, "memset");
+  if ((e = launch_begin(&ws, 1, max_tiles, st)) != cudaSuccess) return cuda_fail(e, "begin");
   {
     PhaseScope ps(SCOUP_PHASE_TAU, st);
     if ((e = launch_reorder(*scene, ws, st)) != cudaSuccess) return cuda_fail(e, "reorder");
@@ -1018,10 +1005,7 @@ int scoup_render_backward(const scoup_scene* scene, const int32_t* topk_idx, con
   const int64_t n = scene->n;
   const CamArgs ca = cam_args(*cam);
   cudaError_t e;
-  if ((e = cudaMemsetAsync(ws.hdr, 0, sizeof(WsHeader), st)) != cudaSuccess) return cuda_fail(e, "memset");
-  if ((e = cudaMemsetAsync(ws.tile_glob, 0, sizeof(uint32_t) * ((size_t)max_tiles + 1), st)) != cudaSuccess ||
-      (e = cudaMemsetAsync(ws.tile_count, 0, sizeof(uint32_t) * ((size_t)max_tiles + 1), st)) != cudaSuccess)
-    return cuda_fail(e, "memset");
+  if ((e = launch_begin(&ws, 1, max_tiles, st)) != cudaSuccess) return cuda_fail(e, "begin");
   {
     PhaseScope ps(SCOUP_PHASE_TAU, st);
     if ((e = launch_reorder(*scene, ws, st)) != cudaSuccess) return cuda_fail(e, "reorder");

@@ -307,7 +307,7 @@ int drain_enqueue(DrainLayout* d, const std::vector<scoup_batch_item>& items, in
     const scoup_batch_item& it = items[b];
     const UpliftWs& sw = d->scene[b];
     const int64_t n = it.scene.n;
-    if ((e = cudaMemsetAsync(sw.hdr, 0, sizeof(WsHeader), st)) != cudaSuccess) return fail_cuda(e, "header");
+    if ((e = launch_begin(&sw, 0, 0, st)) != cudaSuccess) return fail_cuda(e, "header");
     if (n == 0) continue;
     if (!(accum_mode & SCOUP_ACCUM_CONTINUE) &&
         (e = cudaMemsetAsync(it.accum, 0, sizeof(float) * (size_t)n * (size_t)C * (compensated ? 2 : 1), st)) !=

@@ -88,9 +88,7 @@ __device__ void slab_bounds(const SlabArgs& sa, WsHeader* __restrict__ hdr, int 
 // Thread p projects Gaussian p of the spatially ordered copy; the record is
 // stored at its original index, depth and rectangle in spatial order.
 __global__ void __launch_bounds__(256) preprocess_kernel(
-    const float* __restrict__ means, const float* __restrict__ scales,
-    const float* __restrict__ quats, const float* __restrict__ opacity,
-    const float* __restrict__ tau, const int32_t* __restrict__ orig, int64_t n, CamArgs cam,
+    const SceneRec* __restrict__ rec, const int32_t* __restrict__ orig, int64_t n, CamArgs cam,
     ProjRec* __restrict__ proj,
     uint32_t* __restrict__ depth_bits, ushort4* __restrict__ rects, WsHeader* __restrict__ hdr,
     int slot, SlabArgs sa) {
@@ -114,10 +112,9 @@ __global__ void __launch_bounds__(256) preprocess_kernel(
     ushort4 rect = make_ushort4(0, 0, 0, 0);
     // every input of the Gaussian is loaded up front, so that all its loads
     // are in flight together (one memory round trip instead of two)
-    const float m0 = means[3 * i], m1 = means[3 * i + 1], m2 = means[3 * i + 2];
-    const float4 q = *reinterpret_cast<const float4*>(quats + 4 * i);
-    const float s0 = scales[3 * i], s1 = scales[3 * i + 1], s2 = scales[3 * i + 2];
-    const float op_i = opacity[i], tau_i = tau[i];
+    const float4 mo = rec[i].mean_op, q = rec[i].quat, stau = rec[i].scale_tau;
+    const float m0 = mo.x, m1 = mo.y, m2 = mo.z, s0 = stau.x, s1 = stau.y, s2 = stau.z;
+    const float op_i = mo.w, tau_i = stau.w;
     const int32_t orig_i = orig[i];
     const float* W = cam.vm;
     float t0 = W[0] * m0 + W[1] * m1 + W[2] * m2 + W[3];
@@ -277,9 +274,8 @@ cudaError_t launch_preprocess(const scoup_scene& sc, const CamArgs& cam, const U
   sa.pix_state = ws.pix_state;
   sa.tile_done = ws.tile_done;
   sa.ntiles = cam.gx * cam.gy;
-  preprocess_kernel<<<blocks, 256, 0, st>>>(ws.sp.means, ws.sp.scales, ws.sp.quats, ws.sp.opacity,
-                                            ws.sp.tau, ws.sp.orig, sc.n, cam, ws.proj, ws.depth, ws.rect,
-                                            ws.hdr, slot, sa);
+  preprocess_kernel<<<blocks, 256, 0, st>>>(ws.sp.rec, ws.sp.orig, sc.n, cam, ws.proj, ws.depth, ws.rect, ws.hdr,
+                                            slot, sa);
   g_launches += 1;
   return cudaGetLastError();
 }

@@ -202,13 +202,15 @@ struct TileJob {
   int scene;
 };
 
-// Scene copy in spatial (Morton) order; orig[p] is the caller's index.
+// Scene copy in spatial (Morton) order: one 48-byte record per Gaussian;
+// orig[p] is the caller's index.
+struct __align__(16) SceneRec {
+  float4 mean_op;    // mean, opacity
+  float4 quat;       // w, x, y, z as given
+  float4 scale_tau;  // scales, alpha-threshold exponent tau
+};
 struct SceneP {
-  float* means;    // [n,3]
-  float* scales;   // [n,3]
-  float* quats;    // [n,4], 16-byte aligned
-  float* opacity;  // [n]
-  float* tau;      // [n] alpha-threshold exponent
+  SceneRec* rec;   // [n]
   int32_t* orig;   // [n]
 };
 
@@ -216,7 +218,7 @@ struct SceneP {
 struct UpliftWs {
   WsHeader* hdr;
   SceneP sp;
-  uint32_t* cell;           // [n] Morton cell of each Gaussian
+  uint32_t* cell;           // [n] Morton cell of each Gaussian and its rank in the cell (reorder)
   uint32_t* cells_scratch;  // counting-sort scratch (reorder_scratch_bytes())
   ProjRec* proj;            // [n] by original index
   uint32_t* depth;          // [n] float bits of camera depth, spatial order
@@ -290,6 +292,9 @@ void header_stats(const struct WsHeader& h, scoup_stats* stats);
 
 // Launchers (each defined in its own translation unit).
 size_t reorder_scratch_bytes();
+// First launch of a call: sets up the header parts[0].hdr, the reorder's cell
+// counts and the binning counters of up to two view parts.
+cudaError_t launch_begin(const UpliftWs* parts, int nparts, int max_tiles, cudaStream_t st);
 cudaError_t launch_reorder(const scoup_scene& sc, const UpliftWs& ws, cudaStream_t st);
 // With slabs (plan and plan->nslabs > 1) the projection also clears the
 // per-pixel slab state and builds the depth histogram from which its last CTA
