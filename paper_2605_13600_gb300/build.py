@@ -1,9 +1,9 @@
 """Build libscoup.so (sm_103a) in-tree with nvcc; no CMake.
 
 Each .cu under csrc/ is compiled to an object in parallel and the objects are
-linked into ``paper_2605_13600_gb300/libscoup.so``.  ``preprocess.cu`` is
-compiled with ``--fmad=false`` so its binary32 projection is evaluated with
-every operation rounded, in source order.
+linked into ``paper_2605_13600_gb300/libscoup.so``.  ``preprocess.cu``
+and ``reorder.cu`` are compiled with ``--fmad=false`` so the binary32 projection
+is evaluated with every operation rounded, in source order.
 """
 from __future__ import annotations
 
@@ -22,7 +22,7 @@ LIB = os.path.join(HERE, "libscoup.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 COMMON = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
           "-Xptxas", "-warn-spills"]
-PER_FILE = {"preprocess.cu": ["--fmad=false"]}
+PER_FILE = {"preprocess.cu": ["--fmad=false"], "reorder.cu": ["--fmad=false"]}
 
 
 def _nvcc() -> str:

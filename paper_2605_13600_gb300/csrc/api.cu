@@ -96,16 +96,25 @@ size_t shared_bytes(int64_t n, int64_t code_rows_k) {
   return b;
 }
 
+// Regions of a view part whose use the sizes of the view decide (carve_view_part):
+// run_bytes: the binning groups' reserved-run offsets (16 KB per group of
+// bin_group(n) Gaussians, at least 512), and behind them, with the larger
+// groups from 64k Gaussians on, the kept bits and the depth cut's arrays;
+// aux: the part's header and the kept bits of a smaller scene.
+constexpr size_t kAuxBytes = 8192;
+constexpr size_t kRunBytes = 16384;
+size_t run_bytes(int64_t n) { return kRunBytes * (size_t)((n + 511) / 512); }
+
 size_t lane_bytes(int64_t n, int max_tiles) {
   const size_t un = (size_t)n;
   size_t b = align_up(sizeof(ProjRec) * un);              // proj
   b += align_up(sizeof(uint32_t) * un);                   // depth
   b += align_up(sizeof(ushort4) * un);                    // rect
   b += 4 * align_up(sizeof(uint32_t) * ((size_t)max_tiles + 1));
-  b += align_up(binning_run_base_bytes(n));               // binning: reserved-run offsets
-  b += align_up(sizeof(float) * kTilePixels * (size_t)max_tiles);  // per-pixel state between slabs
-  b += align_up((size_t)max_tiles);                       // tile done flags
-  b += align_up(sizeof(uint32_t) * kDepthBuckets);        // depth histogram
+  b += align_up(run_bytes(n));                            // binning runs, kept bits, depth cut
+  b += align_up(sizeof(float) * kTilePixels * (size_t)max_tiles);  // pixels of open tiles / depth-cut histogram
+  b += align_up((size_t)max_tiles);
+  b += kAuxBytes;
   return b;
 }
 
@@ -143,20 +152,73 @@ size_t carve_view_part(void* base, int64_t n, int max_tiles, UpliftWs* w) {
   w->rect = (ushort4*)take(sizeof(ushort4) * un);
   w->tile_count = (uint32_t*)take(sizeof(uint32_t) * ((size_t)max_tiles + 1));
   w->tile_glob = (uint32_t*)take(sizeof(uint32_t) * ((size_t)max_tiles + 1));
-  w->run_base = (uint32_t*)take(binning_run_base_bytes(n));
+  char* runs = (char*)take(run_bytes(n));
   w->tile_start = (uint32_t*)take(sizeof(uint32_t) * ((size_t)max_tiles + 1));
   w->tile_fill = (uint32_t*)take(sizeof(uint32_t) * ((size_t)max_tiles + 1));
   w->pix_state = (float*)take(sizeof(float) * kTilePixels * (size_t)max_tiles);
-  w->tile_done = (uint8_t*)take((size_t)max_tiles);
-  w->dhist = (uint32_t*)take(sizeof(uint32_t) * kDepthBuckets);
+  take((size_t)max_tiles);
+  char* aux = (char*)take(kAuxBytes);
+  w->vhdr = (WsHeader*)aux;
+  w->run_base = (uint32_t*)runs;
+  w->keep = (uint32_t*)(aux + sizeof(WsHeader));
+  w->zcut = w->open_bits = w->open_list = nullptr;
+  const int64_t group = bin_group(n);
+  if (group > 512) {
+    size_t at = kRunBytes * (size_t)((n + group - 1) / group);
+    w->keep = (uint32_t*)(runs + at);
+    at += align_up(sizeof(uint32_t) * (size_t)((n + 31) / 32));
+    const size_t per_tile = align_up(sizeof(uint32_t) * (size_t)max_tiles);
+    if (at + 3 * per_tile <= run_bytes(n)) {
+      w->zcut = (uint32_t*)(runs + at);
+      w->open_list = (uint32_t*)(runs + at + per_tile);
+      w->open_bits = (uint32_t*)(runs + at + 2 * per_tile);
+    }
+  }
   return off;
+}
+
+// From 64k Gaussians on the shorter lists pay for the cut's four small launches
+// (figures at launch_depth_cut); a cut belongs to a block's list.
+bool use_depth_cut(int64_t n, const CamArgs& cam, const UpliftWs& ws) {
+  return ws.zcut && n > 63488 && list_shift(n, cam.gx, cam.gy) == 1;
+}
+
+ViewJob view_job(const scoup_scene& sc, const CamArgs& cam, const UpliftWs& ws, WsHeader* hdr, bool cut) {
+  ViewJob v;
+  v.cam = cam;
+  v.means = sc.means;
+  v.scales = sc.scales;
+  v.opacity = sc.opacity;
+  v.rec = ws.sp.rec;
+  v.orig = ws.sp.orig;
+  v.proj = ws.proj;
+  v.depth = ws.depth;
+  v.rect = ws.rect;
+  v.keep = ws.keep;
+  v.tile_count = ws.tile_count;
+  v.tile_glob = ws.tile_glob;
+  v.run_base = ws.run_base;
+  v.tile_start = ws.tile_start;
+  v.tile_fill = ws.tile_fill;
+  v.keys = ws.keys;
+  v.capacity = ws.dup_capacity;
+  v.hdr = hdr;
+  v.hist = cut ? (uint32_t*)ws.pix_state : nullptr;
+  v.zcut = ws.zcut;
+  v.open_bits = cut ? ws.open_bits : nullptr;
+  v.open_list = ws.open_list;
+  v.pix_state = ws.pix_state;
+  v.n = (int)sc.n;
+  v.group = bin_group(sc.n);
+  v.shift = list_shift(sc.n, cam.gx, cam.gy);
+  return v;
 }
 
 namespace {
 
-// Carves `lanes` view pipelines out of the workspace; out[l] share the header
+// Carves `lanes` view parts out of the workspace; out[l] share the scene header
 // and the scene copy.
-void carve_lanes(void* ws, size_t bytes, int64_t n, int max_tiles, int64_t code_rows_k, int lanes,
+void carve_parts(void* ws, size_t bytes, int64_t n, int max_tiles, int64_t code_rows_k, int lanes,
                  int32_t** codes_i, float** codes_v, UpliftWs* out) {
   UpliftWs w;
   char* p = (char*)ws;
@@ -175,7 +237,7 @@ void carve_lanes(void* ws, size_t bytes, int64_t n, int max_tiles, int64_t code_
 UpliftWs carve(void* ws, size_t bytes, int64_t n, int max_tiles, int64_t code_rows_k,
                int32_t** codes_i, float** codes_v) {
   UpliftWs w;
-  carve_lanes(ws, bytes, n, max_tiles, code_rows_k, 1, codes_i, codes_v, &w);
+  carve_parts(ws, bytes, n, max_tiles, code_rows_k, 1, codes_i, codes_v, &w);
   return w;
 }
 
@@ -195,8 +257,8 @@ int num_sms() {
 
 namespace {
 
-// The library's second stream for the odd views of an uplift (one per host
-// thread and device, created on first use).
+// The library's second stream for an uplift's odd chunks of views (one per
+// host thread and device, created on first use).
 cudaStream_t view_lane_stream() {
   thread_local cudaStream_t streams[64] = {};
   int dev = 0;
@@ -218,40 +280,14 @@ cudaStream_t map_copy_stream() {
   return streams[dev];
 }
 
-// The library's streams of the chunked form beyond the caller's and the view
-// lane stream: [0] the second chunk lane, [1], [2] the lanes' second
-// projection streams (one set per host thread and device).
-cudaStream_t chunk_stream(int i) {
-  thread_local cudaStream_t streams[64][3] = {};
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (dev < 0 || dev >= 64 || i < 0 || i >= 3) return nullptr;
-  if (!streams[dev][i] && cudaStreamCreateWithFlags(&streams[dev][i], cudaStreamNonBlocking) != cudaSuccess)
-    streams[dev][i] = nullptr;
-  return streams[dev][i];
-}
-
 // Chunked form of one scene: kChunkLanes lanes of kChunkViews views per
 // chunk, i.e. kChunkLanes x kChunkViews view parts in the workspace.
 constexpr int kChunkLanes = 2, kChunkViews = 8;
 
 // Bytes of the chunked layout with `dup` keys per view part.
 size_t chunked_bytes(int64_t n, int max_tiles, int64_t code_rows_k, int64_t dup) {
-  const size_t part = align_up(sizeof(WsHeader)) + lane_bytes(n, max_tiles) +
-                      align_up(sizeof(unsigned long long) * (size_t)dup);
-  return shared_bytes(n, code_rows_k) + (size_t)(kChunkLanes * kChunkViews) * part +
-         align_up(sizeof(unsigned) * kChunkLanes);
-}
-
-// Depth slabs of the uplift.  Splitting a view into front-to-back slabs bins
-// far fewer (Gaussian, tile) pairs (3 slabs at the 5% and 20% depth quantiles
-// list 13% of the pairs of a 1M-Gaussian 988x731 view), but every slab pays a
-// fixed cost of about 25 us per binning kernel plus a second per-tile setup,
-// which measured more than the pairs it saves: one slab is the default.
-SlabPlan uplift_slab_plan() {
-  SlabPlan p;
-  p.nslabs = 1;
-  return p;
+  const size_t part = lane_bytes(n, max_tiles) + align_up(sizeof(unsigned long long) * (size_t)dup);
+  return shared_bytes(n, code_rows_k) + (size_t)(kChunkLanes * kChunkViews) * part;
 }
 
 CamArgs cam_args(const scoup_camera& c) {
@@ -329,131 +365,85 @@ int finish_with_stats(const WsHeader* dev_hdr, scoup_stats* stats, cudaStream_t 
 namespace scoup {
 int set_error(int code, const char* msg) { return fail(code, "%s", msg); }
 
-// The views of one scene in chunks (SCOUP_UPLIFT_CHUNKED): view v goes to
-// chunk v / kChunkViews on lane chunk % kChunkLanes; each chunk is projected
-// and binned into the lane's view parts, composited by one drain launch and
-// merged into the scene header sw.hdr.  The scene part (header, Morton-ordered
-// copy) is set up; the view parts follow it in the workspace.  With host
-// region maps (c.maps_on_host) view part q reads its map from ring slot q:
-// a lane's copies for a chunk wait for the lane's previous drain (the last
-// reader of its slots) and the chunk's drain waits for the copies; projection
-// and binning do not read the maps and run meanwhile.
-static int uplift_views_chunked(const UpliftCall& c, const int32_t* region_maps, int32_t R_total, const UpliftWs& sw,
-                                void* workspace, size_t ws_bytes, int max_tiles, int64_t code_rows_k,
-                                const int32_t* ci, const float* cv, int s_eff, float* comp, int warp_w,
-                                cudaStream_t st) {
-  const int64_t n = c.scene->n;
-  const int V = c.V;
-  constexpr int kParts = kChunkLanes * kChunkViews;
-  // the layout: scene part, kParts x (header, view part, keys), lane counters
-  const size_t fixed = chunked_bytes(n, max_tiles, code_rows_k, 0);
-  if (ws_bytes < fixed + (size_t)kParts * 256)
-    return fail(SCOUP_ERR_OOM, "workspace too small for the chunked form: %zu < %zu bytes before tile lists", ws_bytes,
-                fixed + (size_t)kParts * 256);
-  const size_t keys_each = (ws_bytes - fixed) / kParts / 256 * 256;
-  char* p = (char*)workspace;
-  size_t off = shared_bytes(n, code_rows_k);
-  UpliftWs parts[kParts];
-  DrainViewInit init[kParts];
-  for (int q = 0; q < kParts; ++q) {
-    UpliftWs& w = parts[q];
-    w = sw;
-    w.hdr = (WsHeader*)(p + off);
-    off += align_up(sizeof(WsHeader));
-    off += carve_view_part(p + off, n, max_tiles, &w);
-    w.keys = (unsigned long long*)(p + off);
-    w.dup_capacity = (int64_t)(keys_each / sizeof(unsigned long long));
-    off += keys_each;
-    init[q] = DrainViewInit{w.hdr, w.tile_count, w.tile_glob, w.dhist};
-  }
-  unsigned* counters = (unsigned*)(p + off);
+// The views of one scene, in chunks of `chunk` views on `lanes` streams: chunk
+// k runs on lane k % lanes, in that lane's view parts; its views are projected
+// and binned together, composited by one drain launch (and a second one for
+// the tiles open behind their depth cut) and merged into the scene header
+// sw.hdr.  Lane 0 is `st`, lane 1 a library stream forked from and joined back
+// into it (graph capture follows the events).  With host region maps
+// (c.maps_on_host) the staging ring's `slots` slots are taken in turn by sets
+// of `chunk`: the copies for a set wait for the drain that last read it, and
+// the chunk's drain waits for the copies; projection and binning do not read
+// the maps and run meanwhile.
+static int uplift_views(const UpliftCall& c, const scoup_level* lv, int L, const UpliftWs& sw, const UpliftWs* parts,
+                        int lanes, int chunk, int slots, int max_tiles, float* comp, int warp_w, cudaStream_t st) {
+  const int V = c.V, nchunks = (V + chunk - 1) / chunk, sets = c.maps_on_host ? slots / chunk : 1;
+  constexpr int kMaxSets = 4;
   cudaError_t e;
-  if ((e = launch_view_init(init, kParts, max_tiles, st)) != cudaSuccess) return cuda_fail(e, "view parts");
-  // streams: lane 0 is `st`, lane 1 a library stream; each lane has a second projection stream
-  const cudaStream_t lane_st[kChunkLanes] = {st, chunk_stream(0)};
-  const cudaStream_t aux_st[kChunkLanes] = {chunk_stream(1), chunk_stream(2)};
-  if (!lane_st[1] || !aux_st[0] || !aux_st[1]) return fail(SCOUP_ERR_CUDA, "could not create the chunk streams");
-  cudaEvent_t ev[2 + 2 * kChunkLanes] = {};
-  for (cudaEvent_t& x : ev)
-    if ((e = cudaEventCreateWithFlags(&x, cudaEventDisableTiming)) != cudaSuccess) {
-      for (cudaEvent_t y : ev)
-        if (y) cudaEventDestroy(y);
-      return cuda_fail(e, "chunk events");
-    }
-  const cudaEvent_t fork = ev[0], join = ev[1];
-  // host maps: copy stream forked from `st`; ready[l] = lane l's chunk maps are staged,
-  // used[l] = lane l's last drain has been enqueued after them
-  cudaStream_t cps = nullptr;
-  cudaEvent_t mev[2 + 2 * kChunkLanes] = {};
+  DrainViewInit init[kChunkLanes * kChunkViews];
+  const int nparts = std::min(lanes, nchunks) * chunk;
+  for (int q = 0; q < nparts; ++q) init[q] = DrainViewInit{parts[q].vhdr, parts[q].tile_count, parts[q].tile_glob};
+  if ((e = launch_view_init(init, nparts, max_tiles, st)) != cudaSuccess) return cuda_fail(e, "view parts");
+  const bool two = lanes > 1 && nchunks > 1;
+  const cudaStream_t lane_st[2] = {st, two ? view_lane_stream() : nullptr};
+  if (two && !lane_st[1]) return fail(SCOUP_ERR_CUDA, "could not create the second view stream");
+  // events: [0] fork, [1] join of the second lane; [2] fork, [3] join of the copy stream;
+  // then per set of ring slots [4 + s] its maps are staged, [4 + kMaxSets + s] its last drain is enqueued
+  cudaEvent_t ev[4 + 2 * kMaxSets] = {};
   auto destroy_events = [&]() {
-    for (cudaEvent_t y : ev) cudaEventDestroy(y);
-    for (cudaEvent_t y : mev)
-      if (y) cudaEventDestroy(y);
+    for (cudaEvent_t x : ev)
+      if (x) cudaEventDestroy(x);
   };
+  cudaStream_t cps = nullptr;
+  bool ok = true;
+  auto make = [&](int k) { ok = ok && cudaEventCreateWithFlags(&ev[k], cudaEventDisableTiming) == cudaSuccess; };
+  if (two) {
+    make(0);
+    make(1);
+    ok = ok && cudaEventRecord(ev[0], st) == cudaSuccess && cudaStreamWaitEvent(lane_st[1], ev[0], 0) == cudaSuccess;
+  }
   if (c.maps_on_host) {
     cps = map_copy_stream();
-    bool ok = cps != nullptr;
-    for (cudaEvent_t& x : mev) ok = ok && cudaEventCreateWithFlags(&x, cudaEventDisableTiming) == cudaSuccess;
-    ok = ok && cudaEventRecord(mev[0], st) == cudaSuccess && cudaStreamWaitEvent(cps, mev[0], 0) == cudaSuccess;
-    if (!ok) {
-      destroy_events();
-      return fail(SCOUP_ERR_CUDA, "map copy stream");
-    }
+    ok = ok && cps != nullptr && sets >= 1 && sets <= kMaxSets;
+    for (int k = 2; k < 4 + 2 * kMaxSets && ok; ++k) make(k);
+    ok = ok && cudaEventRecord(ev[2], st) == cudaSuccess && cudaStreamWaitEvent(cps, ev[2], 0) == cudaSuccess;
+  }
+  if (!ok) {
+    destroy_events();
+    return fail(SCOUP_ERR_CUDA, "view streams");
   }
   int rc = SCOUP_OK;
-  const int nchunks = (V + kChunkViews - 1) / kChunkViews;
-  const bool lane1 = nchunks > 1;
-  if (lane1 && ((e = cudaEventRecord(fork, st)) != cudaSuccess ||
-                (e = cudaStreamWaitEvent(lane_st[1], fork, 0)) != cudaSuccess))
-    rc = cuda_fail(e, "chunk lanes");
   TileJob jobs[kChunkViews];
-  uint32_t tile0[kChunkViews];
-  UpliftWs views[kChunkViews];
-  const scoup_scene* scenes[kChunkViews];
+  ViewJob views[kChunkViews];
   for (int ch = 0; ch < nchunks && rc == SCOUP_OK; ++ch) {
-    const int lane = ch % kChunkLanes;
-    const int v0 = ch * kChunkViews, nv = std::min(kChunkViews, V - v0);
-    uint32_t items = 0;
+    const int lane = ch % lanes, set = ch % sets;
+    const int v0 = ch * chunk, nv = std::min(chunk, V - v0);
     for (int k = 0; k < nv; ++k) {
       const int v = v0 + k;
-      const UpliftWs& w = parts[lane * kChunkViews + k];
-      TileJob& J = jobs[k];
-      J = TileJob();
-      J.cam = cam_args(c.cams[v]);
-      J.lc = LevelCodes();
-      J.lc.L = 1;
-      J.lc.s_tot = s_eff;
-      J.lc.rmap[0] = c.maps_on_host ? c.map_stage + (size_t)(lane * kChunkViews + k) * c.map_stage_cap
-                                    : region_maps + c.map_offsets[v];
-      J.lc.ci[0] = ci;
-      J.lc.cv[0] = cv;
-      J.lc.s[0] = s_eff;
-      J.lc.R[0] = R_total;
-      J.proj = w.proj;
-      J.keys = w.keys;
-      J.tile_start = w.tile_start;
-      J.accum = c.accum;
-      J.comp = comp;
-      J.hdr = w.hdr;
-      J.scene_hdr = sw.hdr;
-      J.slot = (ch / kChunkLanes) & 1;
-      J.C = c.C;
-      J.tiles = J.cam.gx * J.cam.gy;
-      J.scene = 0;
-      tile0[k] = items;
-      items += (uint32_t)J.tiles;
-      views[k] = w;
-      scenes[k] = c.scene;
+      const UpliftWs& w = parts[lane * chunk + k];
+      const CamArgs cam = cam_args(c.cams[v]);
+      views[k] = view_job(*c.scene, cam, w, w.vhdr, use_depth_cut(c.scene->n, cam, w));
+      LevelCodes lc = LevelCodes();
+      lc.L = L;
+      for (int l = 0; l < L; ++l) {
+        lc.rmap[l] = c.maps_on_host ? c.map_stage + (size_t)(set * chunk + k) * c.map_stage_cap
+                                    : lv[l].region_maps + c.map_offsets[v];
+        lc.ci[l] = lv[l].code_idx;
+        lc.cv[l] = lv[l].code_val;
+        lc.s[l] = lv[l].s;
+        lc.R[l] = lv[l].R_total;
+        lc.s_tot += lv[l].s;
+      }
+      jobs[k] = tile_job(views[k], lc, c.accum, comp, sw.hdr, c.C, L * c.C, 0);
     }
-    ChunkStreams cs{lane_st[lane], aux_st[lane], ev[2 + 2 * lane], ev[3 + 2 * lane]};
+    ChunkStreams cs{lane_st[lane]};
     if (c.maps_on_host) {
-      // stage the chunk's maps into the lane's slots once the lane's previous drain has run
-      cudaEvent_t ready = mev[2 + 2 * lane], used = mev[3 + 2 * lane];
-      if (ch >= kChunkLanes && (e = cudaStreamWaitEvent(cps, used, 0)) != cudaSuccess) rc = cuda_fail(e, "map copy");
+      cudaEvent_t ready = ev[4 + set], used = ev[4 + kMaxSets + set];
+      if (ch >= sets && (e = cudaStreamWaitEvent(cps, used, 0)) != cudaSuccess) rc = cuda_fail(e, "map copy");
       for (int k = 0; k < nv && rc == SCOUP_OK; ++k) {
         const int v = v0 + k;
         const size_t bytes = sizeof(int32_t) * (size_t)c.cams[v].width * (size_t)c.cams[v].height;
-        if ((e = cudaMemcpyAsync((void*)jobs[k].lc.rmap[0], region_maps + c.map_offsets[v], bytes,
+        if ((e = cudaMemcpyAsync((void*)jobs[k].lc.rmap[0], lv[0].region_maps + c.map_offsets[v], bytes,
                                  cudaMemcpyHostToDevice, cps)) != cudaSuccess)
           rc = cuda_fail(e, "region map copy");
       }
@@ -462,22 +452,22 @@ static int uplift_views_chunked(const UpliftCall& c, const int32_t* region_maps,
       cs.before_drain = ready;
       cs.after_drain = used;
     }
-    rc = run_chunk(jobs, tile0, nv, views, scenes, counters + lane, comp != nullptr, warp_w, cs);
+    rc = run_chunk(views, jobs, nv, sw.hdr->drain_ctr[lane], comp != nullptr, warp_w, cs);
   }
+  // join even on an error, so that a capture in progress stays well formed
   if (c.maps_on_host &&
-      ((e = cudaEventRecord(mev[1], cps)) != cudaSuccess || (e = cudaStreamWaitEvent(st, mev[1], 0)) != cudaSuccess) &&
+      ((e = cudaEventRecord(ev[3], cps)) != cudaSuccess || (e = cudaStreamWaitEvent(st, ev[3], 0)) != cudaSuccess) &&
       rc == SCOUP_OK)
     rc = cuda_fail(e, "map copy stream");
-  // join even on an error, so that a capture in progress stays well formed
-  if (lane1 && ((e = cudaEventRecord(join, lane_st[1])) != cudaSuccess ||
-                (e = cudaStreamWaitEvent(st, join, 0)) != cudaSuccess) && rc == SCOUP_OK)
-    rc = cuda_fail(e, "chunk lanes");
+  if (two && ((e = cudaEventRecord(ev[1], lane_st[1])) != cudaSuccess ||
+              (e = cudaStreamWaitEvent(st, ev[1], 0)) != cudaSuccess) && rc == SCOUP_OK)
+    rc = cuda_fail(e, "view streams");
   destroy_events();
   return rc;
 }
 
 int uplift_call(const UpliftCall& c, void* workspace, size_t ws_bytes, int warp_w, const WsHeader** hdr_out,
-                cudaStream_t st, int view_lanes) {
+                cudaStream_t st, int view_lanes, int lane_views) {
   const scoup_scene* scene = c.scene;
   const scoup_camera* cams = c.cams;
   const int32_t V = c.V, C = c.C, K = c.K, accum_mode = c.accum_mode;
@@ -549,165 +539,43 @@ int uplift_call(const UpliftCall& c, void* workspace, size_t ws_bytes, int warp_
     return fail(SCOUP_ERR_OOM, "workspace too small for the chunked form: %zu < %zu bytes before tile lists", ws_bytes,
                 chunked_bytes(scene->n, max_tiles, code_rows_k, 0) + (size_t)kChunkLanes * kChunkViews * 256);
 
-  // two view pipelines (even / odd views on two streams) when the workspace holds them
-  const int lanes =
-      (!chunked && view_lanes >= 2 && V >= 2 && ws_bytes >= uplift_fixed_bytes(scene->n, max_tiles, code_rows_k, 2) + 64) ? 2 : 1;
+  // the view parts: the chunked form's, the caller's lanes x views, or one or
+  // two of single views (two pipelines when the workspace holds them)
+  int lanes = chunked ? kChunkLanes : view_lanes, chunk = chunked ? kChunkViews : lane_views;
+  if (!chunked && lane_views == 1)
+    lanes = (view_lanes >= 2 && V >= 2 && ws_bytes >= uplift_fixed_bytes(scene->n, max_tiles, code_rows_k, 2) + 64) ? 2 : 1;
+  if (lanes > kChunkLanes || chunk > kChunkViews || ws_bytes < uplift_fixed_bytes(scene->n, max_tiles, code_rows_k, lanes * chunk))
+    return fail(SCOUP_ERR_OOM, "workspace too small for %d view parts", lanes * chunk);
   int32_t* fci = nullptr;
   float* fcv = nullptr;
-  UpliftWs wsl[2];
-  carve_lanes(workspace, ws_bytes, scene->n, max_tiles, code_rows_k, lanes, &fci, &fcv, wsl);
-  const UpliftWs& ws = wsl[0];
+  UpliftWs parts[kChunkLanes * kChunkViews];
+  carve_parts(workspace, ws_bytes, scene->n, max_tiles, code_rows_k, lanes * chunk, &fci, &fcv, parts);
+  const UpliftWs& ws = parts[0];
   const int64_t n = scene->n;
   cudaError_t e;
-  if ((e = launch_begin(wsl, chunked ? 0 : lanes, max_tiles, st)) != cudaSuccess) return cuda_fail(e, "begin");
+  if ((e = launch_begin(ws, false, max_tiles, st)) != cudaSuccess) return cuda_fail(e, "begin");
   const bool compensated = (accum_mode & SCOUP_ACCUM_COMPENSATED) != 0;
   float* comp = compensated ? accum + (size_t)n * (size_t)Crow : nullptr;
   if (n > 0 && !(accum_mode & SCOUP_ACCUM_CONTINUE) &&
       (e = cudaMemsetAsync(accum, 0, sizeof(float) * (size_t)n * (size_t)Crow * (compensated ? 2 : 1), st)) !=
           cudaSuccess)
     return cuda_fail(e, "memset accum");
-  const SlabPlan plan = uplift_slab_plan();
-  const int32_t* ci = code_idx;
-  const float* cv = code_val;
-  int s_eff = s;
   if (L == 1 && s > K && R_total > 0) {
     PhaseScope ps(SCOUP_PHASE_CODE_TOPK, st);
     if ((e = launch_code_topk(code_idx, code_val, R_total, s, K, fci, fcv, st)) != cudaSuccess)
       return cuda_fail(e, "code top-k");
-    ci = fci;
-    cv = fcv;
-    s_eff = K;
+    lv[0].code_idx = fci;
+    lv[0].code_val = fcv;
+    lv[0].s = K;
   }
-  if (n > 0 && V > 0 && chunked) {
+  if (n > 0 && V > 0) {
     {
       PhaseScope ps(SCOUP_PHASE_TAU, st);
       if ((e = launch_reorder(*scene, ws, st)) != cudaSuccess) return cuda_fail(e, "reorder");
     }
-    const int rcc = uplift_views_chunked(c, region_maps, R_total, ws, workspace, ws_bytes, max_tiles, code_rows_k, ci,
-                                         cv, s_eff, comp, warp_w, st);
-    if (rcc != SCOUP_OK) return rcc;
-  }
-  if (n > 0 && V > 0 && !chunked) {
-    {
-      PhaseScope ps(SCOUP_PHASE_TAU, st);
-      if ((e = launch_reorder(*scene, ws, st)) != cudaSuccess) return cuda_fail(e, "reorder");
-    }
-    // view v runs in pipeline v % lanes; the second pipeline forks from and
-    // joins back into `st` through events (graph capture follows them)
-    cudaStream_t sts[2] = {st, st};
-    cudaEvent_t fork = nullptr, join = nullptr;
-    if (lanes == 2) {
-      sts[1] = view_lane_stream();
-      if (!sts[1]) return fail(SCOUP_ERR_CUDA, "could not create the second view stream");
-      if ((e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming)) != cudaSuccess ||
-          (e = cudaEventCreateWithFlags(&join, cudaEventDisableTiming)) != cudaSuccess ||
-          (e = cudaEventRecord(fork, st)) != cudaSuccess || (e = cudaStreamWaitEvent(sts[1], fork, 0)) != cudaSuccess) {
-        if (fork) cudaEventDestroy(fork);
-        if (join) cudaEventDestroy(join);
-        return cuda_fail(e, "view streams");
-      }
-    }
-    // host maps: copy stream forked from `st`; ready[q] = slot q holds its
-    // view's map, used[q] = the tile kernel that read slot q has finished
-    cudaStream_t cs = nullptr;
-    cudaEvent_t cfork = nullptr, cjoin = nullptr, ready[kMapStageSlots] = {}, used[kMapStageSlots] = {};
-    auto destroy_copy_events = [&]() {
-      for (cudaEvent_t* ev : {&cfork, &cjoin}) if (*ev) cudaEventDestroy(*ev);
-      for (int q = 0; q < kMapStageSlots; ++q) {
-        if (ready[q]) cudaEventDestroy(ready[q]);
-        if (used[q]) cudaEventDestroy(used[q]);
-      }
-    };
-    if (c.maps_on_host) {
-      cs = map_copy_stream();
-      bool ok = cs != nullptr;
-      ok = ok && cudaEventCreateWithFlags(&cfork, cudaEventDisableTiming) == cudaSuccess &&
-           cudaEventCreateWithFlags(&cjoin, cudaEventDisableTiming) == cudaSuccess;
-      for (int q = 0; q < kMapStageSlots && ok; ++q)
-        ok = cudaEventCreateWithFlags(&ready[q], cudaEventDisableTiming) == cudaSuccess &&
-             cudaEventCreateWithFlags(&used[q], cudaEventDisableTiming) == cudaSuccess;
-      ok = ok && cudaEventRecord(cfork, st) == cudaSuccess && cudaStreamWaitEvent(cs, cfork, 0) == cudaSuccess;
-      if (!ok) {
-        destroy_copy_events();
-        if (lanes == 2) { cudaEventDestroy(fork); cudaEventDestroy(join); }
-        return fail(SCOUP_ERR_CUDA, "map copy stream");
-      }
-    }
-    int rc_views = SCOUP_OK;
-    for (int v = 0; v < V && rc_views == SCOUP_OK; ++v) {
-      const int lane = v % lanes, slot = 2 * lane + ((v / lanes) & 1);
-      const cudaStream_t vs = sts[lane];
-      const UpliftWs& wv = wsl[lane];
-      const CamArgs ca = cam_args(cams[v]);
-      {
-        PhaseScope ps(SCOUP_PHASE_PREPROCESS, vs);
-        if ((e = launch_preprocess(*scene, ca, wv, slot, vs, &plan)) != cudaSuccess) { rc_views = cuda_fail(e, "preprocess"); break; }
-      }
-      const int q = v % kMapStageSlots;
-      if (c.maps_on_host) {
-        // the copy waits for the tile kernel that last read slot q (view v - kMapStageSlots)
-        const size_t bytes = sizeof(int32_t) * (size_t)cams[v].width * (size_t)cams[v].height;
-        if ((v >= kMapStageSlots && (e = cudaStreamWaitEvent(cs, used[q], 0)) != cudaSuccess) ||
-            (e = cudaMemcpyAsync(c.map_stage + (size_t)q * c.map_stage_cap, region_maps + map_offsets[v], bytes,
-                                 cudaMemcpyHostToDevice, cs)) != cudaSuccess ||
-            (e = cudaEventRecord(ready[q], cs)) != cudaSuccess) {
-          rc_views = cuda_fail(e, "region map copy");
-          break;
-        }
-      }
-      {
-        LevelCodes lc;
-        lc.L = L;
-        lc.s_tot = L == 1 ? s_eff : s_tot;
-        for (int l = 0; l < kMaxLevels; ++l) {
-          const bool on = l < L;
-          lc.rmap[l] = on ? (c.maps_on_host ? c.map_stage + (size_t)q * c.map_stage_cap
-                                            : lv[l].region_maps + map_offsets[v])
-                          : nullptr;
-          lc.ci[l] = on ? (L == 1 ? ci : lv[l].code_idx) : nullptr;
-          lc.cv[l] = on ? (L == 1 ? cv : lv[l].code_val) : nullptr;
-          lc.s[l] = on ? (L == 1 ? s_eff : lv[l].s) : 0;
-          lc.R[l] = on ? lv[l].R_total : 0;
-        }
-        // slabs front to back: bin slab s (into the tiles still open), then composite it
-        for (int sl = 0; sl < plan.nslabs && rc_views == SCOUP_OK; ++sl) {
-          {
-            PhaseScope ps(SCOUP_PHASE_BINNING, vs);
-            if ((e = launch_binning(ca, n, wv, slot, vs, plan.nslabs > 1 ? sl : -1, sl == plan.nslabs - 1)) !=
-                cudaSuccess)
-              rc_views = cuda_fail(e, "binning");
-          }
-          if (rc_views != SCOUP_OK) break;
-          // the first tile pass is the first reader of a staged region map
-          if (sl == 0 && c.maps_on_host && (e = cudaStreamWaitEvent(vs, ready[q], 0)) != cudaSuccess) {
-            rc_views = cuda_fail(e, "region map copy");
-            break;
-          }
-          PhaseScope ps(SCOUP_PHASE_UPLIFT_TILES, vs);
-          if ((e = launch_uplift_tiles(ca, wv, slot, lc, C, Crow, accum, comp, warp_w, vs, sl, plan.nslabs)) !=
-              cudaSuccess)
-            rc_views = cuda_fail(e, "uplift tiles");
-        }
-        if (rc_views != SCOUP_OK) break;
-      }
-      if (c.maps_on_host && (e = cudaEventRecord(used[q], vs)) != cudaSuccess) {
-        rc_views = cuda_fail(e, "region map copy");
-        break;
-      }
-    }
-    if (c.maps_on_host) {
-      if ((e = cudaEventRecord(cjoin, cs)) != cudaSuccess || (e = cudaStreamWaitEvent(st, cjoin, 0)) != cudaSuccess)
-        if (rc_views == SCOUP_OK) rc_views = cuda_fail(e, "map copy stream");
-      destroy_copy_events();
-    }
-    if (lanes == 2) {
-      // join even on an error, so that a capture in progress stays well formed
-      if ((e = cudaEventRecord(join, sts[1])) != cudaSuccess || (e = cudaStreamWaitEvent(st, join, 0)) != cudaSuccess)
-        if (rc_views == SCOUP_OK) rc_views = cuda_fail(e, "view streams");
-      cudaEventDestroy(fork);
-      cudaEventDestroy(join);
-    }
-    if (rc_views != SCOUP_OK) return rc_views;
+    const int slots = chunked ? kChunkLanes * kChunkViews : kMapStageSlots;
+    const int rcv = uplift_views(c, lv, L, ws, parts, lanes, chunk, slots, max_tiles, comp, warp_w, st);
+    if (rcv != SCOUP_OK) return rcv;
   }
   if (topk_idx && n > 0) {
     PhaseScope ps(SCOUP_PHASE_TOPK, st);
@@ -722,58 +590,80 @@ int uplift_call(const UpliftCall& c, void* workspace, size_t ws_bytes, int warp_
 }
 
 size_t uplift_required_bytes(int64_t n, const scoup_camera* cams, int32_t V, int32_t s, int32_t K, int32_t R_total,
-                             int64_t dup_capacity) {
+                             int64_t dup_capacity, int parts) {
   int max_tiles = 1;
   for (int v = 0; v < V; ++v) {
     const int t = tiles_of(cams[v].width, cams[v].height);
     if (t > max_tiles) max_tiles = t;
   }
   const int64_t code_rows_k = s > K ? (int64_t)R_total * K : 0;
-  return uplift_fixed_bytes(n, max_tiles, code_rows_k) + sizeof(unsigned long long) * (size_t)dup_capacity;
+  return uplift_fixed_bytes(n, max_tiles, code_rows_k, parts) +
+         (size_t)parts * sizeof(unsigned long long) * (size_t)dup_capacity;
 }
 
-int run_chunk(const TileJob* jobs, const uint32_t* tile0, int njobs, const UpliftWs* views,
-              const scoup_scene* const* scenes, unsigned* counter, bool compensated, int warp_w,
+TileJob tile_job(const ViewJob& v, const LevelCodes& lc, float* accum, float* comp, WsHeader* scene_hdr, int C, int Crow,
+                 int scene) {
+  TileJob J = TileJob();
+  J.cam = v.cam;
+  J.lc = lc;
+  J.proj = v.proj;
+  J.keys = v.keys;
+  J.tile_start = v.tile_start;
+  J.zcut = v.hist ? v.zcut : nullptr;
+  J.open_bits = v.open_bits;
+  J.open_list = v.open_list;
+  J.pix_state = v.pix_state;
+  J.accum = accum;
+  J.comp = comp;
+  J.hdr = v.hdr;
+  J.scene_hdr = scene_hdr;
+  J.C = C;
+  J.Crow = Crow;
+  J.shift = v.shift;
+  J.tiles = v.cam.gx * v.cam.gy;
+  J.scene = scene;
+  return J;
+}
+
+int run_chunk(const ViewJob* views, const TileJob* jobs, int nv, uint32_t* ctr, bool compensated, int warp_w,
               const ChunkStreams& cs) {
-  auto fail_cuda = [](cudaError_t e, const char* where) { return cuda_fail(e, where); };
-  if (njobs <= 0) return SCOUP_OK;
-  if (njobs > kMaxDrainJobs) return set_error(SCOUP_ERR_INVALID_ARG, "more views in a chunk than one drain takes");
+  if (nv <= 0) return SCOUP_OK;
+  if (nv > kMaxDrainJobs) return set_error(SCOUP_ERR_INVALID_ARG, "more views in a chunk than one drain takes");
   cudaError_t e;
-  int rc = SCOUP_OK;
-  // the second stream starts after the lane's previous drain (the view parts are reused)
-  const bool split = njobs > 1 && cs.as != nullptr;
-  if (split && ((e = cudaEventRecord(cs.fork, cs.ls)) != cudaSuccess ||
-                (e = cudaStreamWaitEvent(cs.as, cs.fork, 0)) != cudaSuccess))
-    return fail_cuda(e, "fork");
-  for (int j = 0; j < njobs && rc == SCOUP_OK; ++j) {
-    const cudaStream_t vs = (split && (j & 1)) ? cs.as : cs.ls;
-    const TileJob& J = jobs[j];
-    {
-      PhaseScope ps(SCOUP_PHASE_PREPROCESS, vs);
-      if ((e = launch_preprocess(*scenes[j], J.cam, views[j], J.slot, vs)) != cudaSuccess) {
-        rc = fail_cuda(e, "preprocess");
-        break;
-      }
-    }
-    PhaseScope ps(SCOUP_PHASE_BINNING, vs);
-    if ((e = launch_binning(J.cam, scenes[j]->n, views[j], J.slot, vs)) != cudaSuccess) rc = fail_cuda(e, "binning");
+  bool cut = false;
+  for (int j = 0; j < nv; ++j) cut = cut || views[j].hist;
+  {
+    PhaseScope ps(SCOUP_PHASE_PREPROCESS, cs.ls);
+    if ((e = launch_depth_cut(views, nv, cs.ls)) != cudaSuccess || (e = launch_project(views, nv, cs.ls)) != cudaSuccess)
+      return cuda_fail(e, "projection");
   }
-  // join even on an error, so that a capture in progress stays well formed
-  if (split && ((e = cudaEventRecord(cs.join, cs.as)) != cudaSuccess ||
-                (e = cudaStreamWaitEvent(cs.ls, cs.join, 0)) != cudaSuccess) && rc == SCOUP_OK)
-    rc = fail_cuda(e, "join");
-  if (rc != SCOUP_OK) return rc;
+  {
+    PhaseScope ps(SCOUP_PHASE_BINNING, cs.ls);
+    if ((e = launch_binning(views, nv, false, ctr, cs.ls)) != cudaSuccess) return cuda_fail(e, "binning");
+  }
+  // the first drain is the first reader of a staged region map
   if (cs.before_drain && (e = cudaStreamWaitEvent(cs.ls, cs.before_drain, 0)) != cudaSuccess)
-    return fail_cuda(e, "region map copy");
-  if ((e = cudaMemsetAsync(counter, 0, sizeof(unsigned), cs.ls)) != cudaSuccess) return fail_cuda(e, "counter");
+    return cuda_fail(e, "region map copy");
   {
     PhaseScope ps(SCOUP_PHASE_UPLIFT_TILES, cs.ls);
-    if ((e = launch_uplift_drain(jobs, tile0, njobs, counter, compensated, warp_w, cs.ls)) != cudaSuccess)
-      return fail_cuda(e, "drain");
+    if ((e = launch_uplift_drain(jobs, nv, false, ctr, compensated, warp_w, cs.ls)) != cudaSuccess)
+      return cuda_fail(e, "drain");
   }
-  if ((e = launch_view_merge(jobs, njobs, cs.ls)) != cudaSuccess) return fail_cuda(e, "merge");
+  if (cut) {
+    // the tiles still open behind their cut (all of these leave at once when there is none)
+    {
+      PhaseScope ps(SCOUP_PHASE_BINNING, cs.ls);
+      if ((e = launch_recover(views, nv, false, cs.ls)) != cudaSuccess ||
+          (e = launch_binning(views, nv, true, ctr + 1, cs.ls)) != cudaSuccess)
+        return cuda_fail(e, "second binning");
+    }
+    PhaseScope ps(SCOUP_PHASE_UPLIFT_TILES, cs.ls);
+    if ((e = launch_uplift_drain(jobs, nv, true, ctr + 1, compensated, warp_w, cs.ls)) != cudaSuccess)
+      return cuda_fail(e, "second drain");
+  }
+  if ((e = launch_view_merge(jobs, nv, cs.ls)) != cudaSuccess) return cuda_fail(e, "merge");
   if (cs.after_drain && (e = cudaEventRecord(cs.after_drain, cs.ls)) != cudaSuccess)
-    return fail_cuda(e, "region map copy");
+    return cuda_fail(e, "region map copy");
   return SCOUP_OK;
 }
 
@@ -841,7 +731,7 @@ int scoup_uplift_plan(const scoup_scene* scene, const scoup_camera* cams, int32_
   int32_t* ci = nullptr;
   float* cv = nullptr;
   UpliftWs ws = carve(workspace, ws_bytes, scene->n, max_tiles, 0, &ci, &cv);
-  cudaError_t e = launch_begin(&ws, 0, max_tiles, st);
+  cudaError_t e = launch_begin(ws, false, max_tiles, st);
   if (e != cudaSuccess) return cuda_fail(e, "begin");
   if ((e = launch_reorder(*scene, ws, st)) != cudaSuccess) return cuda_fail(e, "reorder");
   int64_t best = 0;
@@ -849,7 +739,8 @@ int scoup_uplift_plan(const scoup_scene* scene, const scoup_camera* cams, int32_
     const CamArgs ca = cam_args(cams[v]);
     if ((e = cudaMemsetAsync(&ws.hdr->duplicates, 0, sizeof(unsigned long long), st)) != cudaSuccess)
       return cuda_fail(e, "memset");
-    if ((e = launch_preprocess(*scene, ca, ws, v & 1, st)) != cudaSuccess) return cuda_fail(e, "preprocess");
+    const ViewJob vj = view_job(*scene, ca, ws, ws.hdr, false);
+    if (scene->n > 0 && (e = launch_project(&vj, 1, st)) != cudaSuccess) return cuda_fail(e, "projection");
     unsigned long long d = 0;
     if ((e = cudaMemcpyAsync(&d, &ws.hdr->duplicates, sizeof(d), cudaMemcpyDeviceToHost, st)) != cudaSuccess)
       return cuda_fail(e, "read");
@@ -931,6 +822,33 @@ int scoup_uplift_levels(const scoup_scene* scene, const scoup_camera* cams, int3
   return SCOUP_OK;
 }
 
+// The tile lists of a render's view, from the caller's scene.
+static int bin_view(const scoup_scene& scene, const ViewJob& view, const UpliftWs& ws, cudaStream_t st) {
+  cudaError_t e;
+  {
+    PhaseScope ps(SCOUP_PHASE_TAU, st);
+    if ((e = launch_reorder(scene, ws, st)) != cudaSuccess) return cuda_fail(e, "reorder");
+  }
+  if (view.n > 0) {
+    PhaseScope ps(SCOUP_PHASE_PREPROCESS, st);
+    if ((e = launch_depth_cut(&view, 1, st)) != cudaSuccess || (e = launch_project(&view, 1, st)) != cudaSuccess)
+      return cuda_fail(e, "projection");
+  }
+  PhaseScope ps(SCOUP_PHASE_BINNING, st);
+  if ((e = launch_binning(&view, 1, false, nullptr, st)) != cudaSuccess) return cuda_fail(e, "binning");
+  return SCOUP_OK;
+}
+
+// The whole lists of the tiles that the first pass recorded as open.
+static int rebin_view(const ViewJob& view, cudaStream_t st) {
+  PhaseScope ps(SCOUP_PHASE_BINNING, st);
+  cudaError_t e;
+  if ((e = launch_recover(&view, 1, true, st)) != cudaSuccess ||
+      (e = launch_binning(&view, 1, true, nullptr, st)) != cudaSuccess)
+    return cuda_fail(e, "second binning");
+  return SCOUP_OK;
+}
+
 int scoup_render(const scoup_scene* scene, const int32_t* topk_idx, const float* topk_val, int32_t K,
                  int32_t C, const scoup_camera* cam, void* out_codes, int32_t out_dtype, float* out_T,
                  int32_t* out_last, void* workspace, size_t ws_bytes, scoup_stats* stats, void* stream) {
@@ -956,22 +874,13 @@ int scoup_render(const scoup_scene* scene, const int32_t* topk_idx, const float*
   const int64_t n = scene->n;
   const CamArgs ca = cam_args(*cam);
   cudaError_t e;
-  if ((e = launch_begin(&ws, 1, max_tiles, st)) != cudaSuccess) return cuda_fail(e, "begin");
-  {
-    PhaseScope ps(SCOUP_PHASE_TAU, st);
-    if ((e = launch_reorder(*scene, ws, st)) != cudaSuccess) return cuda_fail(e, "reorder");
-  }
-  if (n > 0) {
-    PhaseScope ps(SCOUP_PHASE_PREPROCESS, st);
-    if ((e = launch_preprocess(*scene, ca, ws, 0, st)) != cudaSuccess) return cuda_fail(e, "preprocess");
-  }
-  {
-    PhaseScope ps(SCOUP_PHASE_BINNING, st);
-    if ((e = launch_binning(ca, n, ws, 0, st)) != cudaSuccess) return cuda_fail(e, "binning");
-  }
-  {
+  if ((e = launch_begin(ws, true, max_tiles, st)) != cudaSuccess) return cuda_fail(e, "begin");
+  const ViewJob view = view_job(*scene, ca, ws, ws.hdr, use_depth_cut(n, ca, ws));
+  if ((rc = bin_view(*scene, view, ws, st)) != SCOUP_OK) return rc;
+  for (int pass = 0; pass < (view.hist ? 2 : 1); ++pass) {
+    if (pass > 0 && (rc = rebin_view(view, st)) != SCOUP_OK) return rc;
     PhaseScope ps(SCOUP_PHASE_RENDER, st);
-    if ((e = launch_render_tiles(ca, ws, 0, topk_idx, topk_val, K, C, out_codes, out_dtype, out_T, out_last, st)) !=
+    if ((e = launch_render_tiles(view, pass > 0, topk_idx, topk_val, K, C, out_codes, out_dtype, out_T, out_last, st)) !=
         cudaSuccess)
       return cuda_fail(e, "render tiles");
   }
@@ -1005,22 +914,13 @@ int scoup_render_backward(const scoup_scene* scene, const int32_t* topk_idx, con
   const int64_t n = scene->n;
   const CamArgs ca = cam_args(*cam);
   cudaError_t e;
-  if ((e = launch_begin(&ws, 1, max_tiles, st)) != cudaSuccess) return cuda_fail(e, "begin");
-  {
-    PhaseScope ps(SCOUP_PHASE_TAU, st);
-    if ((e = launch_reorder(*scene, ws, st)) != cudaSuccess) return cuda_fail(e, "reorder");
-  }
-  if (n > 0) {
-    PhaseScope ps(SCOUP_PHASE_PREPROCESS, st);
-    if ((e = launch_preprocess(*scene, ca, ws, 0, st)) != cudaSuccess) return cuda_fail(e, "preprocess");
-  }
-  {
-    PhaseScope ps(SCOUP_PHASE_BINNING, st);
-    if ((e = launch_binning(ca, n, ws, 0, st)) != cudaSuccess) return cuda_fail(e, "binning");
-  }
-  {
+  if ((e = launch_begin(ws, true, max_tiles, st)) != cudaSuccess) return cuda_fail(e, "begin");
+  const ViewJob view = view_job(*scene, ca, ws, ws.hdr, use_depth_cut(n, ca, ws));
+  if ((rc = bin_view(*scene, view, ws, st)) != SCOUP_OK) return rc;
+  for (int pass = 0; pass < (view.hist ? 2 : 1); ++pass) {
+    if (pass > 0 && (rc = rebin_view(view, st)) != SCOUP_OK) return rc;
     PhaseScope ps(SCOUP_PHASE_RENDER_BWD, st);
-    if ((e = launch_render_bwd(ca, ws, 0, topk_idx, topk_val, K, C, dL_dcodes, d_topk_val, d_opacity, st)) !=
+    if ((e = launch_render_bwd(view, pass > 0, topk_idx, topk_val, K, C, dL_dcodes, d_topk_val, d_opacity, st)) !=
         cudaSuccess)
       return cuda_fail(e, "render backward");
   }

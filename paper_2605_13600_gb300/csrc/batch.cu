@@ -51,6 +51,10 @@ namespace scoup {
 namespace {
 
 constexpr int kMaxLanes = 8;
+// Views that a lane composites together (its workspace holds as many view
+// parts): the tiles of one view of a mid-sized scene are two or three waves of
+// the chip.
+constexpr int kLaneViews = 4;
 
 int err(int code, const char* msg) { return set_error(code, msg); }
 
@@ -167,7 +171,7 @@ int enqueue_batch(scoup_plan* p, int lanes, int warp_w, int sample, bool copy_st
       const UpliftCall c{&it.scene, cams, V, it.region_maps, offs, it.R_total, it.code_idx, it.code_val, it.s,
                          p->C, p->K, it.accum, p->accum_mode, it.topk_idx, it.topk_val};
       const WsHeader* hdr = nullptr;
-      const int rc = uplift_call(c, p->lane_ws[l], p->lane_bytes, warp_w, &hdr, ls);
+      const int rc = uplift_call(c, p->lane_ws[l], p->lane_bytes, warp_w, &hdr, ls, 1, kLaneViews);
       if (rc != SCOUP_OK) return rc;
       if (copy_stats &&
           (e = cudaMemcpyAsync(p->stats_dev + b, hdr, sizeof(WsHeader), cudaMemcpyDeviceToDevice, ls)) !=
@@ -274,7 +278,7 @@ int scoup_plan_create(const scoup_batch_item* items, int32_t B, int32_t C, int32
   for (int b = 0; b < B; ++b) {
     const scoup_batch_item& it = p->items[b];
     p->lane_bytes = std::max(p->lane_bytes, uplift_required_bytes(it.scene.n, it.cams, it.V, it.s, K, it.R_total,
-                                                                  p->max_dups[b] + 1));
+                                                                  p->max_dups[b] + 1, kLaneViews));
   }
   if ((e = cudaEventCreateWithFlags(&p->fork_ev, cudaEventDisableTiming)) != cudaSuccess ||
       (e = cudaStreamCreateWithFlags(&p->cap_st, cudaStreamNonBlocking)) != cudaSuccess ||

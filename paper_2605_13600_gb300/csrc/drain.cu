@@ -38,19 +38,18 @@ struct InitArgs {
   int max_tiles;
 };
 
-// Resets view parts before their first use: headers (counters, status, the
-// depth range of every slot) and the binning counters.
+// Resets view parts before their first use: headers (counters, status, depth
+// range) and the binning counters.
 __global__ void view_init_kernel(const __grid_constant__ InitArgs a) {
   const DrainViewInit& v = a.part[blockIdx.y];
   const int stride = gridDim.x * blockDim.x;
   const int t0 = blockIdx.x * blockDim.x + threadIdx.x;
   if (t0 == 0) {
     WsHeader h = {};
-    for (int q = 0; q < 4; ++q) { h.drange[q][0] = 0xffffffffu; h.drange[q][1] = 0u; }
+    h.drange[0] = 0xffffffffu;
     *v.hdr = h;
   }
   for (int t = t0; t <= a.max_tiles; t += stride) { v.tile_count[t] = 0u; v.tile_glob[t] = 0u; }
-  for (int t = t0; t < kDepthBuckets; t += stride) v.dhist[t] = 0u;
 }
 
 struct MergeArgs {
@@ -80,6 +79,9 @@ __global__ void view_merge_kernel(const __grid_constant__ MergeArgs a) {
   v->flushes = v->atomics = v->listed = v->split_windows = 0ull;
   v->max_dups_view = 0;
   v->status = 0;
+  v->drange[0] = 0xffffffffu;
+  v->drange[1] = 0u;
+  v->open_tiles = 0u;
 }
 
 }  // namespace
@@ -115,24 +117,7 @@ cudaError_t launch_view_merge(const TileJob* jobs, int njobs, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-namespace {
-
-void release_aux(DrainLayout* d) {
-  for (cudaStream_t s : d->aux) {
-    cudaStreamSynchronize(s);
-    cudaStreamDestroy(s);
-  }
-  for (cudaEvent_t e : d->aux_fork) cudaEventDestroy(e);
-  for (cudaEvent_t e : d->aux_join) cudaEventDestroy(e);
-  d->aux.clear();
-  d->aux_fork.clear();
-  d->aux_join.clear();
-}
-
-}  // namespace
-
 void drain_release(DrainLayout* d) {
-  release_aux(d);
   if (d->mem) cudaFree(d->mem);
   *d = DrainLayout();
 }
@@ -184,28 +169,9 @@ int drain_prepare(DrainLayout* d, const std::vector<scoup_batch_item>& items, co
   const int nparts = lanes * chunk;
   const size_t part_bytes = align_up(uplift_view_part_bytes(n_max, max_tiles));
   const size_t keys_bytes = align_up(sizeof(unsigned long long) * (size_t)dups_max);
-  const size_t hdr_bytes = align_up(sizeof(WsHeader));
-  const size_t need = scene_bytes + (size_t)nparts * (hdr_bytes + part_bytes + keys_bytes) +
-                      align_up(sizeof(unsigned) * (size_t)lanes);
+  const size_t need = scene_bytes + (size_t)nparts * (part_bytes + keys_bytes) +
+                      align_up(2 * sizeof(uint32_t) * (size_t)lanes);
   cudaError_t e;
-  if ((int)d->aux.size() != lanes) {
-    release_aux(d);
-    for (int l = 0; l < lanes; ++l) {
-      cudaStream_t s = nullptr;
-      cudaEvent_t f = nullptr, j = nullptr;
-      if ((e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking)) != cudaSuccess ||
-          (e = cudaEventCreateWithFlags(&f, cudaEventDisableTiming)) != cudaSuccess ||
-          (e = cudaEventCreateWithFlags(&j, cudaEventDisableTiming)) != cudaSuccess) {
-        if (s) cudaStreamDestroy(s);
-        if (f) cudaEventDestroy(f);
-        release_aux(d);
-        return set_error(SCOUP_ERR_CUDA, "chunked batch: streams");
-      }
-      d->aux.push_back(s);
-      d->aux_fork.push_back(f);
-      d->aux_join.push_back(j);
-    }
-  }
   if (need > d->bytes) {
     if ((e = cudaDeviceSynchronize()) != cudaSuccess)  // a run still in flight may use the old memory
       return set_error(SCOUP_ERR_CUDA, cudaGetErrorString(e));
@@ -234,53 +200,38 @@ int drain_prepare(DrainLayout* d, const std::vector<scoup_batch_item>& items, co
   d->init.assign(nparts, DrainViewInit());
   for (int q = 0; q < nparts; ++q) {
     UpliftWs& w = d->view[q];
-    w.hdr = (WsHeader*)(p + off);
-    off += hdr_bytes;
-    off += carve_view_part(p + off, n_max, max_tiles, &w);
+    off += align_up(carve_view_part(p + off, n_max, max_tiles, &w));
     w.keys = (unsigned long long*)(p + off);
     w.dup_capacity = dups_max;
     off += keys_bytes;
-    d->init[q] = DrainViewInit{w.hdr, w.tile_count, w.tile_glob, w.dhist};
+    d->init[q] = DrainViewInit{w.vhdr, w.tile_count, w.tile_glob};
   }
-  d->counters_dev = (unsigned*)(p + off);
+  d->counters_dev = (uint32_t*)(p + off);
   // the schedule
+  d->views.assign(njobs, ViewJob());
   d->jobs.assign(njobs, TileJob());
-  d->job_view_part.assign(njobs, 0);
   d->chunk_begin.assign(nchunks + 1, njobs);
-  d->tile0.assign(std::max(njobs, 1), 0u);
   for (int c = 0; c < nchunks; ++c) {
     d->chunk_begin[c] = c * chunk;
-    uint32_t items_c = 0;
     for (int j = c * chunk; j < std::min(njobs, (c + 1) * chunk); ++j) {
       const int b = order[j].first, v = order[j].second;
       const scoup_batch_item& it = items[b];
-      const int q = (c % lanes) * chunk + (j - c * chunk);
-      const UpliftWs& w = d->view[q];
-      TileJob& J = d->jobs[j];
-      J.cam = camera_args(it.cams[v]);
-      const bool cut = d->fci[b] != nullptr;
-      J.lc = LevelCodes();
-      J.lc.L = 1;
-      J.lc.s_tot = cut ? K : it.s;
-      J.lc.rmap[0] = it.region_maps + it.map_offsets[v];
-      J.lc.ci[0] = cut ? d->fci[b] : it.code_idx;
-      J.lc.cv[0] = cut ? d->fcv[b] : it.code_val;
-      J.lc.s[0] = J.lc.s_tot;
-      J.lc.R[0] = it.R_total;
-      J.proj = w.proj;
-      J.keys = w.keys;
-      J.tile_start = w.tile_start;
-      J.accum = it.accum;
-      J.comp = compensated ? it.accum + (size_t)it.scene.n * (size_t)C : nullptr;
-      J.hdr = w.hdr;
-      J.scene_hdr = d->scene[b].hdr;
-      J.slot = (c / lanes) & 1;
-      J.C = C;
-      J.tiles = J.cam.gx * J.cam.gy;
-      J.scene = b;
-      d->job_view_part[j] = q;
-      d->tile0[j] = items_c;
-      items_c += (uint32_t)J.tiles;
+      // a view part laid out for the largest scene, with scene b's copy
+      UpliftWs w = d->view[(c % lanes) * chunk + (j - c * chunk)];
+      w.sp = d->scene[b].sp;
+      const CamArgs cam = camera_args(it.cams[v]);
+      d->views[j] = view_job(it.scene, cam, w, w.vhdr, use_depth_cut(it.scene.n, cam, w));
+      d->views[j].group = bin_group(n_max);  // the part's run offsets are laid out for this group size
+      const bool filtered = d->fci[b] != nullptr;
+      LevelCodes lc = LevelCodes();
+      lc.L = 1;
+      lc.s_tot = lc.s[0] = filtered ? K : it.s;
+      lc.rmap[0] = it.region_maps + it.map_offsets[v];
+      lc.ci[0] = filtered ? d->fci[b] : it.code_idx;
+      lc.cv[0] = filtered ? d->fcv[b] : it.code_val;
+      lc.R[0] = it.R_total;
+      float* comp = compensated ? it.accum + (size_t)it.scene.n * (size_t)C : nullptr;
+      d->jobs[j] = tile_job(d->views[j], lc, it.accum, comp, d->scene[b].hdr, C, C, b);
     }
   }
   d->chunk = chunk;
@@ -307,7 +258,7 @@ int drain_enqueue(DrainLayout* d, const std::vector<scoup_batch_item>& items, in
     const scoup_batch_item& it = items[b];
     const UpliftWs& sw = d->scene[b];
     const int64_t n = it.scene.n;
-    if ((e = launch_begin(&sw, 0, 0, st)) != cudaSuccess) return fail_cuda(e, "header");
+    if ((e = launch_begin(sw, false, 0, st)) != cudaSuccess) return fail_cuda(e, "header");
     if (n == 0) continue;
     if (!(accum_mode & SCOUP_ACCUM_CONTINUE) &&
         (e = cudaMemsetAsync(it.accum, 0, sizeof(float) * (size_t)n * (size_t)C * (compensated ? 2 : 1), st)) !=
@@ -327,25 +278,10 @@ int drain_enqueue(DrainLayout* d, const std::vector<scoup_batch_item>& items, in
   for (int l = 0; l < used; ++l)
     if ((e = cudaStreamWaitEvent(lane_st[l], fork_ev, 0)) != cudaSuccess) return fail_cuda(e, "fork wait");
   int rc = SCOUP_OK;
-  std::vector<UpliftWs> vw;
-  std::vector<const scoup_scene*> vs;
   for (int c = 0; c < nchunks && rc == SCOUP_OK; ++c) {
-    const int lane = c % d->lanes;
-    const int j0 = d->chunk_begin[c], j1 = d->chunk_begin[c + 1];
-    vw.clear();
-    vs.clear();
-    for (int j = j0; j < j1; ++j) {
-      const TileJob& J = d->jobs[j];
-      UpliftWs w = d->view[d->job_view_part[j]];
-      w.sp = d->scene[J.scene].sp;
-      w.cell = d->scene[J.scene].cell;
-      w.cells_scratch = d->scene[J.scene].cells_scratch;
-      vw.push_back(w);
-      vs.push_back(&items[J.scene].scene);
-    }
-    const ChunkStreams cs{lane_st[lane], d->aux[lane], d->aux_fork[lane], d->aux_join[lane]};
-    rc = run_chunk(d->jobs.data() + j0, d->tile0.data() + j0, j1 - j0, vw.data(), vs.data(), d->counters_dev + lane,
-                   compensated, warp_w, cs);
+    const int lane = c % d->lanes, j0 = d->chunk_begin[c], j1 = d->chunk_begin[c + 1];
+    rc = run_chunk(d->views.data() + j0, d->jobs.data() + j0, j1 - j0, d->counters_dev + 2 * lane, compensated, warp_w,
+                   ChunkStreams{lane_st[lane]});
   }
   // join even on an error, so that a capture in progress stays well formed
   for (int l = 0; l < used; ++l)

@@ -149,19 +149,23 @@ __device__ __forceinline__ void write_row(void* __restrict__ out, int64_t pix, b
 // (measured 9.1 -> 5.5 ms per 1920x1080 view against 2 CTAs per SM; 5 spills more)
 template <bool kStaged>
 __global__ void __launch_bounds__(kRThreads, 4) render_tile_kernel(
-    CamArgs cam, const ProjRec* __restrict__ proj, const unsigned long long* __restrict__ keys,
-    const uint32_t* __restrict__ tile_start, int slot, const int32_t* __restrict__ topk_idx,
+    const __grid_constant__ ViewJob view, int second, const int32_t* __restrict__ topk_idx,
     const float* __restrict__ topk_val, int K, int C, void* __restrict__ out, int out_bf16, float* __restrict__ out_T,
-    int32_t* __restrict__ out_last, WsHeader* __restrict__ hdr) {
+    int32_t* __restrict__ out_last) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   RenderSmem& sm = *reinterpret_cast<RenderSmem*>(smem_raw);
-  const int tile = blockIdx.x;
+  const CamArgs& cam = view.cam;
+  WsHeader* __restrict__ const hdr = view.hdr;
+  const ProjRec* __restrict__ const proj = view.proj;
+  if (second && blockIdx.x >= hdr->open_tiles) return;
+  const int tile = second ? (int)view.open_list[blockIdx.x] : (int)blockIdx.x;
+  const TileList list = tile_list(view.keys, view.tile_start, second || !view.hist ? nullptr : view.zcut, view.shift,
+                                  cam.gx, tile);
+  const uint32_t cut = list.cut;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int tx = tile % cam.gx, ty = tile / cam.gx;
-  const uint32_t begin = tile_start[tile];
-  const int n = (int)(tile_start[tile + 1] - begin);
+  const int n = list.n;
   if (hdr->status & kStatCapacity) return;
-  const unsigned long long* tkeys = keys + begin;
   float* acc = warp_acc(sm, warp, C);
   const StagedCodes sc = staged_codes(sm, C, K);
 
@@ -172,15 +176,15 @@ __global__ void __launch_bounds__(kRThreads, 4) render_tile_kernel(
     sm.done[p] = !(px < cam.width && py < cam.height);
   }
   if (tid < 2) sm.cnt[tid] = 0ull;
-  const OrderBuckets bk = order_buckets<ROrder>(hdr, slot);
-  order_init(sm.ord, tkeys, n, bk);  // ends with a barrier
+  const OrderBuckets bk = order_buckets<ROrder>(hdr, cut);
+  order_init(sm.ord, list, bk);  // ends with a barrier
   unsigned n_eval = 0, n_contrib = 0;
 
   OrderState st;
   int wbase = 0;
   bool first_window = true;
   while (true) {
-    const int m = n > 0 ? order_next_window(sm.ord, tkeys, n, bk, st, hdr) : 0;
+    const int m = n > 0 ? order_next_window(sm.ord, list, bk, st, hdr) : 0;
     if (m < 0) break;
     if (m == 0 && !first_window) break;
     for (int j = tid; j < m; j += kRThreads) {
@@ -242,7 +246,12 @@ __global__ void __launch_bounds__(kRThreads, 4) render_tile_kernel(
     for (int p = tid; p < kTilePixels; p += kRThreads) open |= !sm.done[p];
     if (!__syncthreads_or(open)) break;
   }
-  if (lane == 0) {
+  // a tile still open at its depth cut is recorded and rendered again, from its whole list
+  int left = 0;
+  for (int p = tid; p < kTilePixels; p += kRThreads) left |= !sm.done[p];
+  const bool again = cut != kNoCut && __syncthreads_or(left);
+  if (again && tid == 0) record_open(hdr, view.open_bits, view.open_list, cam.gx, tile);
+  if (lane == 0 && !again) {
     atomicAdd(&sm.cnt[0], (unsigned long long)n_eval);
     atomicAdd(&sm.cnt[1], (unsigned long long)n_contrib);
   }
@@ -272,25 +281,18 @@ size_t render_smem_bytes(int C, int K) {
          (render_stages(K) ? staged_bytes(K) : 0);
 }
 
-cudaError_t launch_render_tiles(const CamArgs& cam, const UpliftWs& ws, int slot, const int32_t* topk_idx,
+cudaError_t launch_render_tiles(const ViewJob& v, bool second, const int32_t* topk_idx,
                                 const float* topk_val, int K, int C, void* out, int out_bf16, float* out_T,
                                 int32_t* out_last, cudaStream_t st) {
   if (render_uses_mma(C, K))
-    return launch_render_mma(cam, ws, slot, topk_idx, topk_val, K, C, out, out_bf16, out_T, out_last, st);
-  const int ntiles = cam.gx * cam.gy;
+    return launch_render_mma(v, second, topk_idx, topk_val, K, C, out, out_bf16, out_T, out_last, st);
+  const int ntiles = v.cam.gx * v.cam.gy;
   if (ntiles <= 0) return cudaSuccess;
   const size_t smem = render_smem_bytes(C, K);
-  const bool staged = render_stages(K);
-  cudaError_t err = cudaFuncSetAttribute(staged ? render_tile_kernel<true> : render_tile_kernel<false>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  auto kern = render_stages(K) ? render_tile_kernel<true> : render_tile_kernel<false>;
+  cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
-  if (staged)
-    render_tile_kernel<true><<<ntiles, kRThreads, smem, st>>>(cam, ws.proj, ws.keys, ws.tile_start, slot, topk_idx,
-                                                              topk_val, K, C, out, out_bf16, out_T, out_last, ws.hdr);
-  else
-    render_tile_kernel<false><<<ntiles, kRThreads, smem, st>>>(cam, ws.proj, ws.keys, ws.tile_start, slot,
-                                                               topk_idx, topk_val, K, C, out, out_bf16, out_T, out_last,
-                                                               ws.hdr);
+  kern<<<ntiles, kRThreads, smem, st>>>(v, second ? 1 : 0, topk_idx, topk_val, K, C, out, out_bf16, out_T, out_last);
   g_launches += 1;
   return cudaGetLastError();
 }

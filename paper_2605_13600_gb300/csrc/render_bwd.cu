@@ -149,24 +149,28 @@ __device__ __forceinline__ bool walk_bwd(BwdSmem& sm, const BwdDyn& dy, const fl
 // sums, measured 4.9 -> 2.1 ms per 800x600 view (2 or 3 CTAs per SM: 2.4 ms)
 template <bool kStaged>
 __global__ void __launch_bounds__(kBThreads, 4) render_bwd_kernel(
-    CamArgs cam, const ProjRec* __restrict__ proj, const unsigned long long* __restrict__ keys,
-    const uint32_t* __restrict__ tile_start, int slot, const int32_t* __restrict__ topk_idx,
+    const __grid_constant__ ViewJob view, int second, const int32_t* __restrict__ topk_idx,
     const float* __restrict__ topk_val, int K, int C, const float* __restrict__ dL_dcodes,
-    float* __restrict__ d_val, float* __restrict__ d_opacity, WsHeader* __restrict__ hdr) {
+    float* __restrict__ d_val, float* __restrict__ d_opacity) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   BwdSmem& sm = *reinterpret_cast<BwdSmem*>(smem_raw);
-  const int tile = blockIdx.x;
+  const CamArgs& cam = view.cam;
+  WsHeader* __restrict__ const hdr = view.hdr;
+  const ProjRec* __restrict__ const proj = view.proj;
+  if (second && blockIdx.x >= hdr->open_tiles) return;
+  const int tile = second ? (int)view.open_list[blockIdx.x] : (int)blockIdx.x;
+  const TileList list = tile_list(view.keys, view.tile_start, second || !view.hist ? nullptr : view.zcut, view.shift,
+                                  cam.gx, tile);
+  const uint32_t cut = list.cut;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int tx = tile % cam.gx, ty = tile / cam.gx;
-  const uint32_t begin = tile_start[tile];
-  const int n = (int)(tile_start[tile + 1] - begin);
-  if (n == 0) return;
+  const int n = list.n;
+  if (n == 0 && cut == kNoCut) return;
   if (hdr->status & kStatCapacity) return;
-  const unsigned long long* tkeys = keys + begin;
   const BwdDyn dy = bwd_dyn(sm, C, K);
   float* grow = dy.g + warp * C;
-  const OrderBuckets bk = order_buckets<BOrder>(hdr, slot);
-  order_init(sm.ord, tkeys, n, bk);
+  const OrderBuckets bk = order_buckets<BOrder>(hdr, cut);
+  order_init(sm.ord, list, bk);
 
   for (int pass = 1; pass <= 2; ++pass) {
     for (int p = tid; p < kTilePixels; p += kBThreads) {
@@ -179,7 +183,7 @@ __global__ void __launch_bounds__(kBThreads, 4) render_bwd_kernel(
     __syncthreads();
     OrderState st;
     while (true) {
-      const int m = order_next_window(sm.ord, tkeys, n, bk, st, hdr);
+      const int m = order_next_window(sm.ord, list, bk, st, hdr);
       if (m <= 0) break;
       for (int j = tid; j < m; j += kBThreads) {
         const ProjRec pr = proj[(int)(sm.ord.win[j] & 0xffffffffull)];
@@ -243,6 +247,16 @@ __global__ void __launch_bounds__(kBThreads, 4) render_bwd_kernel(
       if (!__syncthreads_or(open)) break;
     }
     __syncthreads();
+    if (pass == 1 && cut != kNoCut) {
+      // a tile still open at its depth cut is recorded and walked again, from
+      // its whole list: no gradient of it has been added yet
+      int left = 0;
+      for (int p = tid; p < kTilePixels; p += kBThreads) left |= !sm.done[p];
+      if (__syncthreads_or(left)) {
+        if (tid == 0) record_open(hdr, view.open_bits, view.open_list, cam.gx, tile);
+        return;
+      }
+    }
   }
 }
 
@@ -255,23 +269,16 @@ size_t render_bwd_smem_bytes(int C, int K) {
          (bwd_stages(K) ? (size_t)K * BOrder::kWin * (sizeof(float) + sizeof(short)) : 0);
 }
 
-cudaError_t launch_render_bwd(const CamArgs& cam, const UpliftWs& ws, int slot, const int32_t* topk_idx,
+cudaError_t launch_render_bwd(const ViewJob& v, bool second, const int32_t* topk_idx,
                               const float* topk_val, int K, int C, const float* dL_dcodes, float* d_val,
                               float* d_opacity, cudaStream_t st) {
-  const int ntiles = cam.gx * cam.gy;
+  const int ntiles = v.cam.gx * v.cam.gy;
   if (ntiles <= 0) return cudaSuccess;
   const size_t smem = render_bwd_smem_bytes(C, K);
-  const bool staged = bwd_stages(K);
-  cudaError_t err = cudaFuncSetAttribute(staged ? render_bwd_kernel<true> : render_bwd_kernel<false>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  auto kern = bwd_stages(K) ? render_bwd_kernel<true> : render_bwd_kernel<false>;
+  cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
-  if (staged)
-    render_bwd_kernel<true><<<ntiles, kBThreads, smem, st>>>(cam, ws.proj, ws.keys, ws.tile_start, slot, topk_idx,
-                                                             topk_val, K, C, dL_dcodes, d_val, d_opacity, ws.hdr);
-  else
-    render_bwd_kernel<false><<<ntiles, kBThreads, smem, st>>>(cam, ws.proj, ws.keys, ws.tile_start, slot,
-                                                              topk_idx, topk_val, K, C, dL_dcodes, d_val,
-                                                              d_opacity, ws.hdr);
+  kern<<<ntiles, kBThreads, smem, st>>>(v, second ? 1 : 0, topk_idx, topk_val, K, C, dL_dcodes, d_val, d_opacity);
   g_launches += 1;
   return cudaGetLastError();
 }

@@ -227,21 +227,26 @@ __device__ __forceinline__ bool walkers_or(bool p) {
 
 // One CTA per tile; one CTA per SM (the accumulator takes the SM's 512 TMEM
 // columns at C = 256, and the shared memory keeps a second CTA out).
+// second: the tiles recorded as open, each from the start of its whole list.
 __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
-    CamArgs cam, const ProjRec* __restrict__ proj, const unsigned long long* __restrict__ keys,
-    const uint32_t* __restrict__ tile_start, int slot, const int32_t* __restrict__ topk_idx,
+    const __grid_constant__ ViewJob view, int second, const int32_t* __restrict__ topk_idx,
     const float* __restrict__ topk_val, int K, int C, void* __restrict__ out, int out_bf16,
-    float* __restrict__ out_T, int32_t* __restrict__ out_last, WsHeader* __restrict__ hdr) {
+    float* __restrict__ out_T, int32_t* __restrict__ out_last) {
   extern __shared__ __align__(128) unsigned char msm_raw[];
   unsigned char* base = msm_raw + ((128u - (ptx::smem_u32(msm_raw) & 127u)) & 127u);
   RenderMmaSmem& sm = *reinterpret_cast<RenderMmaSmem*>(base);
+  const CamArgs& cam = view.cam;
+  WsHeader* __restrict__ const hdr = view.hdr;
+  const ProjRec* __restrict__ const proj = view.proj;
   if (hdr->status & kStatCapacity) return;  // set by the binning before this launch: uniform
-  const int tile = blockIdx.x;
+  if (second && blockIdx.x >= hdr->open_tiles) return;
+  const int tile = second ? (int)view.open_list[blockIdx.x] : (int)blockIdx.x;
+  const TileList list = tile_list(view.keys, view.tile_start, second || !view.hist ? nullptr : view.zcut, view.shift,
+                                  cam.gx, tile);
+  const uint32_t cut = list.cut;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int tx = tile % cam.gx, ty = tile / cam.gx;
-  const uint32_t begin = tile_start[tile];
-  const int n = (int)(tile_start[tile + 1] - begin);
-  const unsigned long long* tkeys = keys + begin;
+  const int n = list.n;
   const int Np = (C + 15) & ~15;  // MMA N: C rounded up to a multiple of 16
   const uint32_t cols = mma_tmem_cols(Np), half_cols = cols / 2;
 
@@ -311,8 +316,8 @@ __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
   float T = 1.0f;
   int last = 0;
   bool done = !inside;
-  const OrderBuckets bk = order_buckets<MOrder>(hdr, slot);
-  order_init<MOrder, 16>(sm.ord, tkeys, n, bk);
+  const OrderBuckets bk = order_buckets<MOrder>(hdr, cut);
+  order_init<MOrder, 16>(sm.ord, list, bk);
 
   unsigned n_eval = 0, n_contrib = 0;
   unsigned acc_init = 0u;  // bit h: pixel half h has received an MMA
@@ -324,7 +329,7 @@ __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
   int chunk = 0, wbase = 0;
   OrderState ost;
   while (!all_done && !aborted) {
-    const int m = n > 0 ? order_next_window<MOrder, 16>(sm.ord, tkeys, n, bk, ost, hdr) : 0;
+    const int m = n > 0 ? order_next_window<MOrder, 16>(sm.ord, list, bk, ost, hdr) : 0;
     if (m <= 0) break;  // list exhausted, or an inconsistency (status already set)
     // records of the window; the positions up to the next chunk boundary get
     // a record no pixel accepts (tau = +inf)
@@ -460,7 +465,11 @@ __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
     fin_ok = ptx::mbar_wait_bounded(&sm.fin, 0u, kWaitIters) && fin_ok;
     if (!fin_ok) atomicOr(&hdr->status, kStatTimeout);
   }
-  const bool bad = walkers_or(!fin_ok) || aborted;
+  // a tile still open at its depth cut is recorded and rendered again, from
+  // its whole list: nothing of it is written or counted now
+  const bool again = cut != kNoCut && !all_done && !aborted;
+  if (again && tid == 0) record_open(hdr, view.open_bits, view.open_list, cam.gx, tile);
+  const bool bad = walkers_or(!fin_ok) || aborted || again;
   ptx::tc_fence_after();
 
   // epilogue: each thread reads its own pixel's row (TMEM lane)
@@ -523,13 +532,13 @@ __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
       if (inside && !bad) store_cols(out, pix, C, c0, out_bf16 != 0, v);
     }
   }
-  if (inside) {
+  if (inside && !again) {
     if (out_T) out_T[pix] = T;
     if (out_last) out_last[pix] = last;
   }
   const unsigned we = __reduce_add_sync(0xffffffffu, n_eval);
   const unsigned wc = __reduce_add_sync(0xffffffffu, n_contrib);
-  if (lane == 0) {
+  if (lane == 0 && !again) {
     atomicAdd(&sm.cnt[0], (unsigned long long)we);
     atomicAdd(&sm.cnt[1], (unsigned long long)wc);
   }
@@ -549,16 +558,16 @@ bool render_mma_supported(int C, int K) { return C >= 1 && C <= kMaxN && K >= 1 
 
 size_t render_mma_smem_bytes() { return sizeof(RenderMmaSmem) + 128; }
 
-cudaError_t launch_render_mma(const CamArgs& cam, const UpliftWs& ws, int slot, const int32_t* topk_idx,
+cudaError_t launch_render_mma(const ViewJob& v, bool second, const int32_t* topk_idx,
                               const float* topk_val, int K, int C, void* out, int out_bf16, float* out_T,
                               int32_t* out_last, cudaStream_t st) {
-  const int ntiles = cam.gx * cam.gy;
+  const int ntiles = v.cam.gx * v.cam.gy;
   if (ntiles <= 0) return cudaSuccess;
   const size_t smem = render_mma_smem_bytes();
   cudaError_t err = cudaFuncSetAttribute(render_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
-  render_mma_kernel<<<ntiles, kCtaThreads, smem, st>>>(cam, ws.proj, ws.keys, ws.tile_start, slot, topk_idx, topk_val,
-                                                      K, C, out, out_bf16, out_T, out_last, ws.hdr);
+  render_mma_kernel<<<ntiles, kCtaThreads, smem, st>>>(v, second ? 1 : 0, topk_idx, topk_val, K, C, out, out_bf16, out_T,
+                                                      out_last);
   g_launches += 1;
   return cudaGetLastError();
 }

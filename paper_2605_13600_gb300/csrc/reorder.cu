@@ -7,8 +7,12 @@
 // consecutive Gaussians covers a compact set of tiles and writes long
 // contiguous runs of keys.  The original index travels with every Gaussian:
 // keys, records and accumulator rows stay addressed by it, so no result
-// depends on this order.  The per-Gaussian alpha-threshold exponent tau is
-// computed here as well.
+// depends on this order.  What of the projection does not depend on the view
+// -- the 3D covariance Sigma3 and the alpha-threshold exponent tau -- is
+// computed here once per call instead of once per view.
+//
+// This translation unit is compiled with --fmad=false like preprocess.cu:
+// Sigma3 is part of the binary32 projection, each operation rounded in order.
 #include <math.h>
 #include <stddef.h>
 
@@ -188,31 +192,51 @@ __global__ void __launch_bounds__(256) gather_kernel(const float* __restrict__ m
     const float o = opacity[i];
     SceneRec r;
     r.mean_op = make_float4(means[3 * i], means[3 * i + 1], means[3 * i + 2], o);
-    r.quat = *reinterpret_cast<const float4*>(quats + 4 * i);
-    r.scale_tau = make_float4(scales[3 * i], scales[3 * i + 1], scales[3 * i + 2], alpha_threshold(o));
+    const float4 q = *reinterpret_cast<const float4*>(quats + 4 * i);
+    const float s0 = scales[3 * i], s1 = scales[3 * i + 1], s2 = scales[3 * i + 2];
+    // Sigma3 = (R S)(R S)^T from the normalised quaternion and scales
+    const float qn = q.x * q.x + q.y * q.y + q.z * q.z + q.w * q.w;
+    const float inv = 1.0f / sqrtf(qn);
+    const float w = q.x * inv, x = q.y * inv, y = q.z * inv, z = q.w * inv;
+    const float R00 = 1.0f - 2.0f * (y * y + z * z);
+    const float R01 = 2.0f * (x * y - w * z);
+    const float R02 = 2.0f * (x * z + w * y);
+    const float R10 = 2.0f * (x * y + w * z);
+    const float R11 = 1.0f - 2.0f * (x * x + z * z);
+    const float R12 = 2.0f * (y * z - w * x);
+    const float R20 = 2.0f * (x * z - w * y);
+    const float R21 = 2.0f * (y * z + w * x);
+    const float R22 = 1.0f - 2.0f * (x * x + y * y);
+    const float M00 = R00 * s0, M01 = R01 * s1, M02 = R02 * s2;
+    const float M10 = R10 * s0, M11 = R11 * s1, M12 = R12 * s2;
+    const float M20 = R20 * s0, M21 = R21 * s1, M22 = R22 * s2;
+    r.cov_a = make_float4(M00 * M00 + M01 * M01 + M02 * M02, M00 * M10 + M01 * M11 + M02 * M12,
+                          M00 * M20 + M01 * M21 + M02 * M22, M10 * M10 + M11 * M11 + M12 * M12);
+    r.cov_b = make_float4(M10 * M20 + M11 * M21 + M12 * M22, M20 * M20 + M21 * M21 + M22 * M22, alpha_threshold(o),
+                          __int_as_float((int32_t)i));
     sp.rec[p] = r;
     sp.orig[p] = (int32_t)i;
   }
 }
 
 // Everything a call starts from, in one launch: the header (zero but for the
-// empty depth ranges and bounding box), the cell counts, and the binning
-// counters of its view parts.
+// empty depth range and bounding box), the cell counts, and the binning
+// counters of a render's view.
 struct BeginArgs {
   WsHeader* hdr;
   uint32_t* cnt;
-  uint32_t* zero[4];  // arrays of max_tiles + 1 words (null: none)
+  uint32_t* zero[2];  // arrays of max_tiles + 1 words (null: none)
   int max_tiles;
 };
 
 __global__ void __launch_bounds__(256) begin_kernel(const __grid_constant__ BeginArgs a) {
   const int t0 = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
-  static_assert(offsetof(WsHeader, drange) == 8 && offsetof(WsHeader, bbox) == 40, "words below");
+  static_assert(offsetof(WsHeader, drange) == 8 && offsetof(WsHeader, bbox) == 16, "words below");
   if (t0 < (int)(sizeof(WsHeader) / 4))
-    reinterpret_cast<uint32_t*>(a.hdr)[t0] = (t0 >= 2 && t0 < 16 && !(t0 & 1)) ? 0xffffffffu : 0u;
+    reinterpret_cast<uint32_t*>(a.hdr)[t0] = (t0 >= 2 && t0 < 10 && !(t0 & 1)) ? 0xffffffffu : 0u;
   for (int t = t0; t < kCells; t += stride) a.cnt[t] = 0u;
 #pragma unroll
-  for (int q = 0; q < 4; ++q)
+  for (int q = 0; q < 2; ++q)
     if (a.zero[q])
       for (int t = t0; t <= a.max_tiles; t += stride) a.zero[q][t] = 0u;
 }
@@ -227,14 +251,14 @@ int grid_for(int64_t n, int per_sm) {
 
 size_t reorder_scratch_bytes() { return sizeof(uint32_t) * (size_t)(3 * kCells); }
 
-cudaError_t launch_begin(const UpliftWs* parts, int nparts, int max_tiles, cudaStream_t st) {
+cudaError_t launch_begin(const UpliftWs& ws, bool view, int max_tiles, cudaStream_t st) {
   BeginArgs a = {};
-  a.hdr = parts[0].hdr;
-  a.cnt = parts[0].cells_scratch;
+  a.hdr = ws.hdr;
+  a.cnt = ws.cells_scratch;
   a.max_tiles = max_tiles;
-  for (int l = 0; l < nparts && l < 2; ++l) {
-    a.zero[2 * l] = parts[l].tile_count;
-    a.zero[2 * l + 1] = parts[l].tile_glob;
+  if (view) {
+    a.zero[0] = ws.tile_count;
+    a.zero[1] = ws.tile_glob;
   }
   begin_kernel<<<32, 256, 0, st>>>(a);
   g_launches += 1;

@@ -26,23 +26,14 @@ constexpr int kStatCapacity = 1;
 constexpr int kStatDeviceCheck = 2;
 constexpr int kStatTimeout = 4;
 
-// Depth slabs.  The visible Gaussians of a view are split by depth into up to
-// kMaxSlabs slabs (front to back) at quantiles of their depth; every key of
-// slab s is smaller than every key of slab s + 1, so compositing the slabs in
-// turn, each in exact (depth, index) order, is compositing the whole list in
-// that order.  Slab s > 0 is binned only into tiles with a pixel that is still
-// open, which skips the Gaussians hidden behind saturated tiles.
-constexpr int kMaxSlabs = 6;
-constexpr int kDepthBuckets = 2048;        // depth histogram: float bits >> 16, from 0.2 up
-constexpr uint32_t kDepthBucketBase = 0x3E4Cu;  // (bits of 0.2f) >> 16
-
-// Workspace header: status word, per-view depth range (double-buffered by
-// view parity in each of the two view pipelines), scene bounding box,
-// counters and the slab bounds of each slot, 256 bytes.
+// Workspace header: status word, depth range of the view's visible Gaussians,
+// scene bounding box and counters, 256 bytes.  A scene has one (its status and
+// the counters of the whole call); every view part of an uplift has its own,
+// whose counters are merged into the scene's after each chunk of views.
 struct WsHeader {
   int32_t status;
   int32_t max_dups_view;
-  uint32_t drange[4][2];  // [2 lane + (view & 1)] = {min, max} float bits of visible depths
+  uint32_t drange[2];     // {min, max} float bits of visible depths
   uint32_t bbox[3][2];    // order-preserving bits of the means' bounding box
   unsigned long long visible;
   unsigned long long duplicates;
@@ -51,19 +42,12 @@ struct WsHeader {
   unsigned long long flushes;
   unsigned long long atomics;
   unsigned long long listed;
-  uint32_t slab_lo[4][kMaxSlabs];  // [slot][s]: smallest depth bits of slab s (slab 0 starts at 0)
-  uint32_t pp_blocks[4];           // projection CTAs finished in this slot's view (last one sets slab_lo)
   unsigned long long split_windows;  // windows cut out of a depth bucket holding more than a window
-  unsigned long long reserved[2];
+  uint32_t open_tiles;               // tiles still open behind the depth cut (length of open_list)
+  uint32_t drain_ctr[2][2];          // scene header: item counters of each chunk lane's two drains
+  uint32_t reserved[33];
 };
 static_assert(sizeof(WsHeader) == 256, "header size");
-
-// Slab schedule of one uplift: nslabs slabs whose bounds sit at the given
-// quantiles of the visible Gaussians' depths (nslabs - 1 of them, ascending).
-struct SlabPlan {
-  int nslabs;
-  float q[kMaxSlabs - 1];
-};
 
 // Projected Gaussian of one view, 32 bytes:
 //   a = (mx, my, qa, qb), b = (qc, opacity, tau, log2(opacity))
@@ -184,35 +168,102 @@ struct CamArgs {
   int gx, gy;  // tile grid
 };
 
-// One view of a batched chunk, as the drain kernel takes it: the arguments
-// of the per-view tile kernel (single level, one slab) and the view's tiles.
+// One view of a chunk, as the drain kernel takes it.
 struct TileJob {
   CamArgs cam;
   LevelCodes lc;
   const ProjRec* proj;
   const unsigned long long* keys;
   const uint32_t* tile_start;
+  const uint32_t* zcut;        // depth cut per tile block, or null (DepthCut below)
+  uint32_t* open_bits;
+  uint32_t* open_list;
+  float* pix_state;
   float* accum;
   float* comp;                 // compensation array (compensated form) or null
   WsHeader* hdr;        // the view's own header: depth range, counters, status
   WsHeader* scene_hdr;  // the scene's header, into which the view's counters are merged
-  int slot;                    // depth-range slot of the view in its own header
-  int C;
+  int C, Crow;          // accumulator rows hold Crow = levels x C floats
+  int shift;            // of the view's tile lists (TileList)
   int tiles;
   int scene;
 };
 
-// Scene copy in spatial (Morton) order: one 48-byte record per Gaussian;
-// orig[p] is the caller's index.
+// Scene copy in spatial (Morton) order: one 48-byte record per Gaussian, with
+// what of the projection does not depend on the view; orig[p] is the caller's
+// index.
 struct __align__(16) SceneRec {
-  float4 mean_op;    // mean, opacity
-  float4 quat;       // w, x, y, z as given
-  float4 scale_tau;  // scales, alpha-threshold exponent tau
+  float4 mean_op;  // mean, opacity
+  float4 cov_a;    // Sigma3: S00, S01, S02, S11
+  float4 cov_b;    // S12, S22, alpha-threshold exponent tau, the caller's index (int bits)
 };
 struct SceneP {
   SceneRec* rec;   // [n]
   int32_t* orig;   // [n]
 };
+
+// Depth cut.  A tile's pixels are opaque long before its list ends (of 4500
+// listed Gaussians per tile of a 1M-Gaussian view about 280 are composited),
+// so each block of 2 x 2 tiles gets a depth zcut, estimated from a sample of
+// the scene's optical depth, and a Gaussian is listed only if it lies in
+// front of the cut of some block that its rectangle meets.  A tile's list is
+// then complete up to its cut, and keys behind it are left out.  A tile that
+// is still open at its cut is recorded, with its pixels' state, and a second
+// pass lists what lies behind the cut for the recorded tiles alone.  The
+// estimate decides speed only: every tile sees its whole list, in order.
+constexpr int kCutBins = 512;                // 64 per octave of depth, from 0.2 up
+constexpr uint32_t kCutBase = 0x3E4CCCCDu;   // bits of 0.2f
+constexpr int kCutShift = 17;
+constexpr uint32_t kNoCut = 0xffffffffu;
+__host__ __device__ inline int cut_blocks(int g) { return (g + 1) >> 1; }
+__host__ __device__ inline int open_words(int gx) { return (cut_blocks(gx) + 31) >> 5; }  // per row of blocks
+
+
+// Tile lists.  A list belongs to a block of 2 x 2 tiles: a Gaussian meets
+// several neighbouring tiles, so a view has less than half as many (Gaussian,
+// block) items as (Gaussian, tile) ones to count, place and write, and a tile
+// takes its own out of the block's list in the pass over it that it makes
+// anyway.  Key: depth bits << 32 | index << 4 | the block's tiles that the
+// rectangle meets (bit (ty & 1) * 2 + (tx & 1)).  Views less than 4 tiles wide
+// or high, where blocks save nothing, and scenes of 2^28 Gaussians, whose
+// index leaves no room for the bits, have one list per tile and no bits
+// (shift 0).
+struct TileList {
+  const unsigned long long* keys;
+  int n;             // keys of the list; those of the tile are among them
+  uint32_t bit;      // the tile's bit (0: every key is the tile's)
+  int id_shift;      // of the index in the key's low word
+  uint32_t cut;      // the tile's depth cut
+  __device__ __forceinline__ bool mine(unsigned long long k) const { return ((uint32_t)k & bit) == bit; }
+  // the key without tile bits: depth bits << 32 | index
+  __device__ __forceinline__ unsigned long long plain(unsigned long long k) const {
+    return (k & 0xffffffff00000000ull) | ((uint32_t)k >> id_shift);
+  }
+};
+__host__ __device__ inline int list_shift(int64_t n, int gx, int gy) {
+  return n < (1ll << 28) && gx >= 4 && gy >= 4 ? 1 : 0;
+}
+__host__ __device__ inline int list_dim(int g, int shift) { return (g + shift) >> shift; }
+
+__device__ __forceinline__ TileList tile_list(const unsigned long long* keys, const uint32_t* list_start,
+                                              const uint32_t* zcut, int shift, int gx, int tile) {
+  const int tx = tile % gx, ty = tile / gx;
+  const int b = (ty >> shift) * list_dim(gx, shift) + (tx >> shift);
+  const uint32_t begin = list_start[b];
+  TileList l;
+  l.keys = keys + begin;
+  l.n = (int)(list_start[b + 1] - begin);
+  l.bit = shift ? 1u << ((ty & 1) * 2 + (tx & 1)) : 0u;
+  l.id_shift = shift ? 4 : 0;
+  l.cut = zcut ? zcut[b] : kNoCut;  // a cut goes with shift 1: one per block
+  return l;
+}
+// Records a tile as open (one thread per tile).
+__device__ __forceinline__ void record_open(WsHeader* hdr, uint32_t* open_bits, uint32_t* open_list, int gx, int tile) {
+  const int bx = (tile % gx) >> 1, by = (tile / gx) >> 1;
+  atomicOr(&open_bits[by * open_words(gx) + (bx >> 5)], 1u << (bx & 31));
+  open_list[atomicAdd(&hdr->open_tiles, 1u)] = (uint32_t)tile;
+}
 
 // Workspace carve-up for one uplift call.
 struct UpliftWs {
@@ -220,23 +271,68 @@ struct UpliftWs {
   SceneP sp;
   uint32_t* cell;           // [n] Morton cell of each Gaussian and its rank in the cell (reorder)
   uint32_t* cells_scratch;  // counting-sort scratch (reorder_scratch_bytes())
+  WsHeader* vhdr;           // the view part's own header
   ProjRec* proj;            // [n] by original index
   uint32_t* depth;          // [n] float bits of camera depth, spatial order
   ushort4* rect;            // [n] listed tiles (x_lo, y_lo, x_hi, y_hi), spatial order: the 3DGS
                             //     rectangle cut to the alpha >= 1/255 ellipse's box; empty if culled
-  uint32_t* tile_count;     // [max_tiles + 1] runs reserved per tile (binning)
-  uint32_t* tile_glob;      // [max_tiles + 1] big-rectangle items per tile (binning)
-  uint32_t* run_base;       // [chunks x box tiles] offset of each binning CTA's run in a tile list
-  uint32_t* tile_start;     // [max_tiles + 1]
+  uint32_t* keep;           // [ceil(n / 32)] bit i: Gaussian i (spatial order) is listed in this pass
+  uint32_t* tile_count;     // [max_tiles + 1] runs reserved per list (binning)
+  uint32_t* tile_glob;      // [max_tiles + 1] big-rectangle items per list (binning)
+  uint32_t* run_base;       // [groups x box blocks] offset of each binning CTA's run in a list
+  uint32_t* tile_start;     // [max_tiles + 1] first key of each list (TileList)
   uint32_t* tile_fill;      // [max_tiles]
-  float* pix_state;         // [max_tiles * 256] per pixel between slabs: 0 = untouched (T = 1),
-                            //     > 0 = transmittance T, < 0 = stopped
-  uint8_t* tile_done;       // [max_tiles] 1 once every pixel of the tile has stopped
-  uint32_t* dhist;          // [kDepthBuckets] depth histogram of the view being projected
-  unsigned long long* keys; // [dup_capacity] (depth bits << 32 | gid)
+  float* pix_state;         // [max_tiles * 256] per pixel of an open tile: T, or < 0 = stopped; holds
+                            //     the depth cut's histogram while the view is projected
+  uint32_t* zcut;           // [blocks] depth cut per block of 2 x 2 tiles (null: the part has no room)
+  uint32_t* open_bits;      // [blocks high x open_words(gx)] bit per block with a tile recorded as open
+  uint32_t* open_list;      // [max_tiles] the recorded tiles
+  unsigned long long* keys; // [dup_capacity] (TileList)
   int64_t dup_capacity;
   int max_tiles;
 };
+
+// One view as the projection and binning kernels take it.
+struct ViewJob {
+  CamArgs cam;
+  const float* means;    // the caller's arrays, in the caller's order (depth-cut sample)
+  const float* scales;
+  const float* opacity;
+  const SceneRec* rec;
+  const int32_t* orig;
+  ProjRec* proj;
+  uint32_t* depth;
+  ushort4* rect;
+  uint32_t* keep;
+  uint32_t* tile_count;
+  uint32_t* tile_glob;
+  uint32_t* run_base;
+  uint32_t* tile_start;
+  uint32_t* tile_fill;
+  unsigned long long* keys;
+  long long capacity;
+  WsHeader* hdr;
+  uint32_t* hist;        // depth cut: [blocks][kCutBins] optical mass; null = no cut for this view
+  uint32_t* zcut;
+  uint32_t* open_bits;
+  uint32_t* open_list;
+  float* pix_state;
+  int n;
+  int group;             // Gaussians per binning CTA (bin_group(n))
+  int shift;             // 1: one list per block of 2 x 2 tiles, 0: per tile (TileList)
+};
+constexpr int kMaxDrainJobs = 64;
+template <int N>
+struct ViewArgs {
+  ViewJob v[N];
+};
+static_assert(sizeof(ViewArgs<kMaxDrainJobs>) <= 32000, "kernel parameter space");
+ViewJob view_job(const scoup_scene& sc, const CamArgs& cam, const UpliftWs& ws, WsHeader* hdr, bool cut);
+// Whether views of this size get a depth cut (given room in the view part).
+bool use_depth_cut(int64_t n, const CamArgs& cam, const UpliftWs& ws);
+// Gaussians per binning CTA; larger groups from 64k Gaussians on, of which the
+// depth cut leaves a fraction.
+inline int bin_group(int64_t n) { return n <= 63488 ? 512 : 1024; }
 
 // Records msg as the calling thread's last error and returns code.
 int set_error(int code, const char* msg);
@@ -259,8 +355,8 @@ struct UpliftCall {
   int32_t L = 0;                        // > 0: semantic levels in `levels` replace the
   const scoup_level* levels = nullptr;  // single-level region map and code fields above
   // region_maps in HOST memory (single level): each view's map is copied into
-  // a device ring of kMapStageSlots slots of map_stage_cap entries, on a
-  // library copy stream, just ahead of the view's tile kernel
+  // a device ring of slots of map_stage_cap entries, on a library copy
+  // stream, just ahead of the drain of the view's chunk
   bool maps_on_host = false;
   int32_t* map_stage = nullptr;
   int64_t map_stage_cap = 0;
@@ -271,15 +367,16 @@ constexpr int kMapStageSlots = 4;
 // the tile kernel's warp pixel-block width (8, 16 or 4).  *hdr_out receives
 // the workspace header that holds the call's status and counters.
 // view_lanes = 2 runs even and odd views in two pipelines (a second stream)
-// when the workspace holds both.
+// when the workspace holds both; lane_views > 1 runs them in chunks of that
+// many (the workspace then holds view_lanes x lane_views view parts).
 int uplift_call(const UpliftCall& c, void* workspace, size_t ws_bytes, int warp_w, const struct WsHeader** hdr_out,
-                cudaStream_t st, int view_lanes = 1);
+                cudaStream_t st, int view_lanes = 1, int lane_views = 1);
 size_t uplift_required_bytes(int64_t n, const scoup_camera* cams, int32_t V, int32_t s, int32_t K, int32_t R_total,
-                             int64_t dup_capacity);
+                             int64_t dup_capacity, int parts = 1);
 int uplift_stats(const struct WsHeader* dev_hdr, scoup_stats* stats, cudaStream_t st);
 // Parts of an uplift workspace (api.cu): the scene part (header, Morton-ordered
 // scene copy, codes filtered to K entries) and one view part (records, depth,
-// rectangles, tile counters, slab state); the carve functions lay a part out
+// rectangles, tile counters, state of open tiles); the carve functions lay a part out
 // from a 256-byte aligned base and return its size.
 size_t uplift_scene_part_bytes(int64_t n, int64_t code_rows_k);
 size_t uplift_view_part_bytes(int64_t n, int max_tiles);
@@ -292,47 +389,39 @@ void header_stats(const struct WsHeader& h, scoup_stats* stats);
 
 // Launchers (each defined in its own translation unit).
 size_t reorder_scratch_bytes();
-// First launch of a call: sets up the header parts[0].hdr, the reorder's cell
-// counts and the binning counters of up to two view parts.
-cudaError_t launch_begin(const UpliftWs* parts, int nparts, int max_tiles, cudaStream_t st);
+// First launch of a call: sets up the scene header, the reorder's cell counts
+// and (view: a render, whose view uses the scene's header) the binning counters.
+cudaError_t launch_begin(const UpliftWs& ws, bool view, int max_tiles, cudaStream_t st);
 cudaError_t launch_reorder(const scoup_scene& sc, const UpliftWs& ws, cudaStream_t st);
-// With slabs (plan and plan->nslabs > 1) the projection also clears the
-// per-pixel slab state and builds the depth histogram from which its last CTA
-// sets hdr->slab_lo[slot].
-cudaError_t launch_preprocess(const scoup_scene& sc, const CamArgs& cam, const UpliftWs& ws,
-                              int slot, cudaStream_t st, const SlabPlan* plan = nullptr);
-size_t binning_run_base_bytes(int64_t n);
-// slab < 0: every listed Gaussian into every tile of its rectangle.  slab s >= 0:
-// only Gaussians of slab s (bounds in hdr->slab_lo[slot]; s = last takes no
-// upper bound), and for s > 0 only into tiles not yet marked done.
-cudaError_t launch_binning(const CamArgs& cam, int64_t n, const UpliftWs& ws, int slot,
-                           cudaStream_t st, int slab = -1, bool last_slab = true);
-// Accumulator rows are Crow = L * C floats wide; level l owns columns [l C, (l + 1) C).
-// slab / nslabs: the tiles composite slab `slab` of nslabs, resuming each
-// pixel from ws.pix_state unless slab == 0 and saving it unless it is the last.
-cudaError_t launch_uplift_tiles(const CamArgs& cam, const UpliftWs& ws, int slot, const LevelCodes& lc, int C,
-                                int Crow, float* accum, float* comp, int warp_w, cudaStream_t st,
-                                int slab = 0, int nslabs = 1);
-// Batched chunk: one persistent launch composites every tile of njobs <=
-// kMaxDrainJobs views (HOST jobs[njobs], copied into the launch's parameters).
-// tile0[j] is the index of view j's first tile in the chunk's item space
-// (tile0[0] = 0, each the sum of the tiles before it); CTAs take items from
-// *counter (DEVICE, zero before the launch).
-constexpr int kMaxDrainJobs = 64;
-cudaError_t launch_uplift_drain(const TileJob* jobs, const uint32_t* tile0, int njobs, unsigned* counter,
-                                bool compensated, int warp_w, cudaStream_t st);
+// Chunk of nv <= kMaxDrainJobs views (HOST array, copied into the launches'
+// parameters): depth cut (for the views that have one), projection, tile lists.
+cudaError_t launch_depth_cut(const ViewJob* v, int nv, cudaStream_t st);
+cudaError_t launch_project(const ViewJob* v, int nv, cudaStream_t st);
+// Second pass, for the tiles recorded as open: keeps the Gaussians that reach
+// one of them behind its cut (restart: at any depth), with their records.
+cudaError_t launch_recover(const ViewJob* v, int nv, bool restart, cudaStream_t st);
+// Tile lists of the kept Gaussians; second: only of the open tiles.  The lane's
+// drain counter of the pass (ctr, may be null) is cleared on the way.
+cudaError_t launch_binning(const ViewJob* v, int nv, bool second, uint32_t* ctr, cudaStream_t st);
+// One persistent launch composites every tile of njobs <= kMaxDrainJobs views
+// (HOST jobs[njobs], copied into the launch's parameters); second: their open
+// tiles, resumed from pix_state.  CTAs take items from *ctr (DEVICE, zero
+// before the launch).  All jobs have the same number of levels.
+cudaError_t launch_uplift_drain(const TileJob* jobs, int njobs, bool second, uint32_t* ctr, bool compensated,
+                                int warp_w, cudaStream_t st);
 size_t render_smem_bytes(int C, int K);
 bool render_uses_mma(int C, int K);
 bool render_mma_supported(int C, int K);
 size_t render_mma_smem_bytes();
-cudaError_t launch_render_mma(const CamArgs& cam, const UpliftWs& ws, int slot, const int32_t* topk_idx,
+cudaError_t launch_render_mma(const ViewJob& v, bool second, const int32_t* topk_idx,
                               const float* topk_val, int K, int C, void* out, int out_bf16, float* out_T,
                               int32_t* out_last, cudaStream_t st);
-cudaError_t launch_render_tiles(const CamArgs& cam, const UpliftWs& ws, int slot, const int32_t* topk_idx,
+// second: the open tiles only, from the start of their (then whole) lists.
+cudaError_t launch_render_tiles(const ViewJob& v, bool second, const int32_t* topk_idx,
                                 const float* topk_val, int K, int C, void* out, int out_bf16, float* out_T,
                                 int32_t* out_last, cudaStream_t st);
 size_t render_bwd_smem_bytes(int C, int K);
-cudaError_t launch_render_bwd(const CamArgs& cam, const UpliftWs& ws, int slot, const int32_t* topk_idx,
+cudaError_t launch_render_bwd(const ViewJob& v, bool second, const int32_t* topk_idx,
                               const float* topk_val, int K, int C, const float* dL_dcodes, float* d_val,
                               float* d_opacity, cudaStream_t st);
 constexpr int kOutBF16 = 0, kOutF32 = 1, kOutCos = 2, kOutRel = 3;

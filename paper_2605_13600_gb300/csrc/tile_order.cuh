@@ -1,8 +1,8 @@
 // tile_order.cuh -- front-to-back ordering of one tile's key list, window by
 // window, for a whole CTA (used by the render and render-backward kernels).
 //
-// Keys are (depth bits << 32 | original Gaussian index), unique per tile.  A
-// histogram over kNB buckets (a monotone map of the depth bits onto the
+// Keys are (depth bits << 32 | original Gaussian index), unique per tile, taken
+// out of the block's list (TileList).  A histogram over kNB buckets (a monotone map of the depth bits onto the
 // view's depth range) is built once; each window is a run of whole buckets
 // holding at most kWin keys, gathered by a counting sort by bucket and then
 // ordered exactly by rank inside each bucket.  A bucket with more than kWin
@@ -42,14 +42,19 @@ struct OrderSmem {
   int sel_digit, sel_rank, win_b1;
 };
 
+// Depths [lo, lo + span] over nb buckets, monotone in the key; keys behind the
+// tile's depth cut go to nb, which no window takes.
 struct OrderBuckets {
-  uint32_t dmin;
+  uint32_t lo, span;
   int shift;
   int nb;
-  // monotone in the key and always inside [0, nb)
   __device__ __forceinline__ int operator()(unsigned long long key) const {
-    const uint32_t d = (uint32_t)(key >> 32);
-    return (int)min((d > dmin ? d - dmin : 0u) >> shift, (uint32_t)(nb - 1));
+    const uint32_t d = (uint32_t)(key >> 32) - lo;
+    return d <= span ? (int)(d >> shift) : nb;
+  }
+  // of a key of the block's list: nb also for another tile's
+  __device__ __forceinline__ int operator()(const TileList& l, unsigned long long key) const {
+    return l.mine(key) ? (*this)(key) : nb;
   }
 };
 
@@ -60,13 +65,14 @@ struct OrderState {
   int consumed = 0;
 };
 
+// Buckets over the view's visible depths up to `cut`.
 template <class S>
-__device__ OrderBuckets order_buckets(const WsHeader* hdr, int slot) {
+__device__ OrderBuckets order_buckets(const WsHeader* hdr, uint32_t cut) {
   OrderBuckets bk;
-  const uint32_t dmin = hdr->drange[slot][0], dmax = hdr->drange[slot][1];
-  const uint32_t span = dmax >= dmin ? dmax - dmin : 0u;
-  const int nb = span ? 32 - __clz((int)span) : 0;
-  bk.dmin = dmin;
+  const uint32_t dmin = hdr->drange[0], dmax = min(hdr->drange[1], cut);
+  bk.lo = dmax >= dmin ? dmin : 0u;  // nothing in front of the cut: no key has depth bits 0
+  bk.span = dmax >= dmin ? dmax - dmin : 0u;
+  const int nb = bk.span ? 32 - __clz((int)bk.span) : 0;
   bk.shift = nb > S::kLogNB ? nb - S::kLogNB : 0;
   bk.nb = S::kNB;
   return bk;
@@ -75,8 +81,8 @@ __device__ OrderBuckets order_buckets(const WsHeader* hdr, int slot) {
 // Histogram + exclusive scan into sm.bstart (S::nthreads() threads, a
 // multiple of 32 dividing kNB).
 template <class S, int kLB = kLoadBatch>
-__device__ void order_init(S& sm, const unsigned long long* __restrict__ keys, int n, const OrderBuckets& bk) {
-  const int tid = threadIdx.x, nt = S::nthreads(), lane = tid & 31, warp = tid >> 5;
+__device__ void order_init(S& sm, const TileList& l, const OrderBuckets& bk) {
+  const int n = l.n, tid = threadIdx.x, nt = S::nthreads(), lane = tid & 31, warp = tid >> 5;
   for (int b = tid; b < S::kNB; b += nt) sm.bcur[b] = 0u;
   S::sync();
   // kLB keys per thread are loaded before their atomics, so each
@@ -86,11 +92,13 @@ __device__ void order_init(S& sm, const unsigned long long* __restrict__ keys, i
 #pragma unroll
     for (int u = 0; u < kLB; ++u) {
       const int i = i0 + u * nt;
-      kk[u] = i < n ? keys[i] : 0ull;
+      kk[u] = i < n ? l.keys[i] : 0ull;
     }
 #pragma unroll
-    for (int u = 0; u < kLB; ++u)
-      if (i0 + u * nt < n) atomicAdd(&sm.bcur[bk(kk[u])], 1u);
+    for (int u = 0; u < kLB; ++u) {
+      const int b = bk(l, kk[u]);
+      if (i0 + u * nt < n && b < S::kNB) atomicAdd(&sm.bcur[b], 1u);
+    }
   }
   S::sync();
   const int per = S::kNB / nt;
@@ -116,16 +124,15 @@ __device__ void order_init(S& sm, const unsigned long long* __restrict__ keys, i
 
 // The rank-th smallest (0-based) key in bucket b with (first || key > last).
 template <class S>
-__device__ unsigned long long order_select(S& sm, const unsigned long long* __restrict__ keys, int n,
-                                           const OrderBuckets& bk, int b, unsigned long long last,
-                                           bool first, int rank) {
-  const int tid = threadIdx.x, nt = S::nthreads();
+__device__ unsigned long long order_select(S& sm, const TileList& l, const OrderBuckets& bk, int b,
+                                           unsigned long long last, bool first, int rank) {
+  const int n = l.n, tid = threadIdx.x, nt = S::nthreads();
   if (tid == 0) { sm.red_min = ~0ull; sm.red_max = 0ull; }
   S::sync();
   unsigned long long lmin = ~0ull, lmax = 0ull;
   for (int i = tid; i < n; i += nt) {
-    const unsigned long long k = keys[i];
-    if (bk(k) == b && (first || k > last)) { lmin = min(lmin, k); lmax = max(lmax, k); }
+    const unsigned long long raw = l.keys[i], k = l.plain(raw);
+    if (bk(l, raw) == b && (first || k > last)) { lmin = min(lmin, k); lmax = max(lmax, k); }
   }
   for (int off = 16; off > 0; off >>= 1) {
     lmin = min(lmin, __shfl_xor_sync(0xffffffffu, lmin, off));
@@ -140,8 +147,8 @@ __device__ unsigned long long order_select(S& sm, const unsigned long long* __re
     for (int d = tid; d < 256; d += nt) sm.hist[d] = 0u;
     S::sync();
     for (int i = tid; i < n; i += nt) {
-      const unsigned long long k = keys[i];
-      if (bk(k) == b && (first || k > last)) {
+      const unsigned long long raw = l.keys[i], k = l.plain(raw);
+      if (bk(l, raw) == b && (first || k > last)) {
         const unsigned long long x = k - base;
         if ((x & pmask) == prefix) atomicAdd(&sm.hist[(x >> shift) & 255u], 1u);
       }
@@ -177,9 +184,8 @@ __device__ unsigned long long order_select(S& sm, const unsigned long long* __re
 // the list is exhausted, or -1 on an internal inconsistency (status set).
 // Block-uniform; every thread of the CTA must call it.
 template <class S, int kLB = kLoadBatch>
-__device__ int order_next_window(S& sm, const unsigned long long* __restrict__ keys, int n,
-                                 const OrderBuckets& bk, OrderState& st, WsHeader* hdr) {
-  const int tid = threadIdx.x, nt = S::nthreads();
+__device__ int order_next_window(S& sm, const TileList& l, const OrderBuckets& bk, OrderState& st, WsHeader* hdr) {
+  const int n = l.n, tid = threadIdx.x, nt = S::nthreads();
   constexpr int kWin = S::kWin, kNB = S::kNB;
   // the in-place permutation below reads a whole window before writing it
   if (kWin > 4 * nt) {
@@ -230,14 +236,14 @@ __device__ int order_next_window(S& sm, const unsigned long long* __restrict__ k
 #pragma unroll
       for (int u = 0; u < kLB; ++u) {
         const int i = i0 + u * nt;
-        kk[u] = i < n ? keys[i] : 0ull;
+        kk[u] = i < n ? l.keys[i] : 0ull;
       }
 #pragma unroll
       for (int u = 0; u < kLB; ++u) {
-        const int b = bk(kk[u]);
+        const int b = bk(l, kk[u]);
         if (i0 + u * nt < n && b >= st.b0 && b < b1) {
           const uint32_t pos = atomicAdd(&sm.bcur[b], 1u);
-          if (pos < (uint32_t)kWin) sm.win[pos] = kk[u];
+          if (pos < (uint32_t)kWin) sm.win[pos] = l.plain(kk[u]);
         }
       }
     }
@@ -271,12 +277,12 @@ __device__ int order_next_window(S& sm, const unsigned long long* __restrict__ k
     if (tid == 0) atomicAdd(&hdr->split_windows, 1ull);
     const int left = total_b0 - st.consumed;
     unsigned long long hi_key = ~0ull;
-    if (left > kWin) hi_key = order_select(sm, keys, n, bk, st.b0, st.split_last, st.split_first, kWin - 1);
+    if (left > kWin) hi_key = order_select(sm, l, bk, st.b0, st.split_last, st.split_first, kWin - 1);
     if (tid == 0) sm.cursor = 0u;
     S::sync();
     for (int i = tid; i < n; i += nt) {
-      const unsigned long long k = keys[i];
-      if (bk(k) == st.b0 && (st.split_first || k > st.split_last) && k <= hi_key) {
+      const unsigned long long raw = l.keys[i], k = l.plain(raw);
+      if (bk(l, raw) == st.b0 && (st.split_first || k > st.split_last) && k <= hi_key) {
         const unsigned pos = atomicAdd(&sm.cursor, 1u);
         if (pos < (unsigned)kWin) sm.win[pos] = k;
       }

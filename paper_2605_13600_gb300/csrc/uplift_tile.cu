@@ -46,10 +46,13 @@
 // soon as its 32 pixels are saturated; the block meets again only at the end
 // of the window.
 //
-// Depth slabs.  With several slabs per view the kernel runs once per slab;
-// each pixel's transmittance (or its stop) is carried from one slab to the
-// next in pix_state, and a tile whose pixels have all stopped is marked done:
-// it returns at once in later slabs, and binning lists nothing for it.
+// Depth cut (scoup_internal.cuh).  With a cut, the first pass composites the
+// keys up to the tile's cut; a tile with an open pixel left is recorded
+// (open_bits, open_list) with its pixels' transmittance or stop (pix_state),
+// and the second pass resumes the recorded tiles on the keys behind the cut.
+//
+// Persistent CTAs (152 SMs x 4, 3 compensated) take the (view, tile) items of
+// a chunk of views from one atomic counter; no CTA waits on another.
 #include <math.h>
 #include <string.h>
 
@@ -67,7 +70,11 @@ static_assert(kThreads / 32 == 8, "one 8-bit block mask per record: eight warps 
 constexpr int kWin = 256;
 constexpr int kLogNB = 10;
 constexpr int kNB = 1 << kLogNB;
-constexpr int kMaxSlots = 4;
+// Distinct regions of a tile that get a partial-sum slot; a pixel of a further
+// one adds its weights to the accumulator directly, s atomics per Gaussian.
+// With 4 slots the few tiles with more regions outlasted all others: 500k
+// Gaussians, 800x600, three levels, one view: 465 us with 4, 173 with 8.
+constexpr int kMaxSlots = 8;
 constexpr int kMaxS = 64;  // codes of up to kMaxS entries are staged in shared memory; longer
                            // ones (dense features, Eq. 3) are read from the code table in the flush
 constexpr int kGroup = 8;
@@ -111,32 +118,38 @@ struct TileSmem {
   int sel_digit;
   int sel_rank;
   int win_b1;
+  TileList list;  // read back where it is needed (not held in registers)
+  uint32_t tile;
   unsigned long long cnt[4];
 };
 
+// Depths [lo, hi] over kNB buckets, monotone in the key; keys outside (the
+// other pass's, behind or in front of the cut) go to kNB, which no window takes.
 struct Buckets {
-  uint32_t dmin;
+  uint32_t lo, span;  // span = hi - lo
   int shift;
-  // monotone in the key and always inside [0, kNB)
   __device__ __forceinline__ int operator()(unsigned long long key) const {
-    const uint32_t d = (uint32_t)(key >> 32);
-    return (int)min((d > dmin ? d - dmin : 0u) >> shift, (uint32_t)(kNB - 1));
+    const uint32_t d = (uint32_t)(key >> 32) - lo;
+    return d <= span ? (int)(d >> shift) : kNB;
+  }
+  // of a key of the block's list: kNB also for another tile's
+  __device__ __forceinline__ int operator()(const TileList& l, unsigned long long key) const {
+    return l.mine(key) ? (*this)(key) : kNB;
   }
 };
 
 // Block-wide: the rank-th smallest (0-based) key among those in bucket b
 // with (first || key > last).  Keys are unique; requires rank < their count.
 template <class Smem>
-__device__ unsigned long long select_in_bucket(Smem& sm, const unsigned long long* __restrict__ keys,
-                                               int n, const Buckets& bk, int b, unsigned long long last,
-                                               bool first, int rank) {
-  const int tid = threadIdx.x;
+__device__ __noinline__ unsigned long long select_in_bucket(Smem& sm, const TileList& l, const Buckets& bk, int b,
+                                                            unsigned long long last, bool first, int rank) {
+  const int tid = threadIdx.x, n = l.n;
   if (tid == 0) { sm.red_min = ~0ull; sm.red_max = 0ull; }
   __syncthreads();
   unsigned long long lmin = ~0ull, lmax = 0ull;
   for (int i = tid; i < n; i += kThreads) {
-    const unsigned long long k = keys[i];
-    if (bk(k) == b && (first || k > last)) { lmin = min(lmin, k); lmax = max(lmax, k); }
+    const unsigned long long raw = l.keys[i], k = l.plain(raw);
+    if (bk(l, raw) == b && (first || k > last)) { lmin = min(lmin, k); lmax = max(lmax, k); }
   }
   for (int off = 16; off > 0; off >>= 1) {
     lmin = min(lmin, __shfl_xor_sync(kFull, lmin, off));
@@ -151,8 +164,8 @@ __device__ unsigned long long select_in_bucket(Smem& sm, const unsigned long lon
     sm.hist[tid] = 0u;
     __syncthreads();
     for (int i = tid; i < n; i += kThreads) {
-      const unsigned long long k = keys[i];
-      if (bk(k) == b && (first || k > last)) {
+      const unsigned long long raw = l.keys[i], k = l.plain(raw);
+      if (bk(l, raw) == b && (first || k > last)) {
         const unsigned long long x = k - base;
         if ((x & pmask) == prefix) atomicAdd(&sm.hist[(x >> shift) & 255u], 1u);
       }
@@ -256,41 +269,37 @@ __device__ __forceinline__ void acc_add(float* accum, float* comp, int64_t x, fl
 }
 
 // The whole pass over one tile of one view: ordering, compositing, flush and
-// counters.  Called by the per-view kernel (one CTA per tile) and by the
-// batched drain kernel (a CTA takes tiles of several views in turn); every
-// early return is taken by the whole CTA.
-template <bool kComp, int kBW, int kL>
-__device__ __forceinline__ void tile_pass(
-    TileSmem<kComp, kL>& sm, const int tile, const CamArgs& cam, const ProjRec* __restrict__ proj,
-    const unsigned long long* __restrict__ keys, const uint32_t* __restrict__ tile_start, int slot,
-    const LevelCodes& lc, int C, int Crow, float* __restrict__ accum, float* __restrict__ comp,
-    WsHeader* __restrict__ hdr, float* __restrict__ pix_state, uint8_t* __restrict__ tile_done, int slab,
-    int nslabs) {
-  const bool first_slab = slab == 0, last_slab = slab == nslabs - 1;
+// counters.  A CTA takes tiles of several views in turn; every early return is
+// taken by the whole CTA.
+template <bool kComp, int kBW, int kL, bool kSecond>
+__device__ __forceinline__ void tile_pass(TileSmem<kComp, kL>& sm, const int tile, const TileJob& job) {
   using RK = typename RegionKey<kL>::T;
+  const CamArgs& cam = job.cam;
+  const LevelCodes& lc = job.lc;
+  WsHeader* __restrict__ const hdr = job.hdr;
+  const ProjRec* __restrict__ const proj = job.proj;
+  float* __restrict__ const accum = job.accum;
+  float* __restrict__ const comp = job.comp;
+  const int C = job.C, Crow = job.Crow;
   // code entries per slot (the concatenated level codes with several levels)
   const int s = kL == 1 ? lc.s[0] : lc.s_tot;
   const int32_t* __restrict__ code_idx = lc.ci[0];
   const float* __restrict__ code_val = lc.cv[0];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (pix_state && !first_slab && tile_done[tile]) return;  // every pixel stopped in an earlier slab
-  const uint32_t begin = tile_start[tile];
-  const int n = (int)(tile_start[tile + 1] - begin);
-  if (n == 0) return;  // nothing of this slab here: the pixels' state stays as it is
+  const TileList list = tile_list(job.keys, job.tile_start, job.zcut, job.shift, cam.gx, tile);
+  const int n = list.n;
+  const uint32_t cut = list.cut;
+  if (n == 0 && (kSecond || cut == kNoCut)) return;
   if (hdr->status & kStatCapacity) return;
-  const unsigned long long* tkeys = keys + begin;
 
   Buckets bk;
   {
-    // the buckets span the view's visible depths, cut to this slab's range
-    uint32_t dmin = hdr->drange[slot][0], dmax = hdr->drange[slot][1];
-    if (nslabs > 1) {
-      dmin = max(dmin, hdr->slab_lo[slot][slab]);
-      if (!last_slab && hdr->slab_lo[slot][slab + 1] > 0u) dmax = min(dmax, hdr->slab_lo[slot][slab + 1] - 1u);
-    }
-    const uint32_t span = dmax >= dmin ? dmax - dmin : 0u;
-    const int nb = span ? 32 - __clz((int)span) : 0;
-    bk.dmin = dmin;
+    // the buckets span the view's visible depths on this pass's side of the cut
+    const uint32_t dmin = kSecond ? max(hdr->drange[0], cut + 1u) : hdr->drange[0];
+    const uint32_t dmax = kSecond ? hdr->drange[1] : min(hdr->drange[1], cut);
+    bk.lo = dmax >= dmin ? dmin : 0u;  // no depth on this side: no key has depth bits 0
+    bk.span = dmax >= dmin ? dmax - dmin : 0u;
+    const int nb = bk.span ? 32 - __clz((int)bk.span) : 0;
     bk.shift = nb > kLogNB ? nb - kLogNB : 0;
   }
 
@@ -324,10 +333,6 @@ __device__ __forceinline__ void tile_pass(
     if (leader) sm.warp_regions[warp][__popc(leaders & ((1u << lane) - 1u))] = region;
     if (lane == 0) sm.warp_nreg[warp] = __popc(leaders);
   }
-  for (int k = tid; k < kMaxSlots * kWin; k += kThreads) (&sm.part[0][0])[k] = 0.0f;
-  if constexpr (kComp)
-    for (int k = tid; k < kMaxSlots * kWin; k += kThreads) (&sm.part_c[0][0])[k] = 0.0f;
-  for (int k = tid; k < kMaxSlots * kWin / 4; k += kThreads) reinterpret_cast<uint32_t*>(&sm.nzb[0][0])[k] = 0u;
   if (tid == 0) {
     // power = 0 for any pixel, never >= tau = +inf: no pixel accepts it
     sm.rec_a[kWin] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
@@ -335,8 +340,12 @@ __device__ __forceinline__ void tile_pass(
   }
   for (int b = tid; b < kNB; b += kThreads) sm.bcur[b] = 0u;
   if (tid < 4) sm.cnt[tid] = 0ull;
+  if (tid == 0) { sm.list = list; sm.tile = (uint32_t)tile; }
   __syncthreads();
-  for (int i = tid; i < n; i += kThreads) atomicAdd(&sm.bcur[bk(tkeys[i])], 1u);
+  for (int i = tid; i < n; i += kThreads) {
+    const int b = bk(list, list.keys[i]);
+    if (b < kNB) atomicAdd(&sm.bcur[b], 1u);
+  }
   if (tid == 0) {
     int ns = 0;
     for (int w = 0; w < kThreads / 32; ++w)
@@ -370,6 +379,10 @@ __device__ __forceinline__ void tile_pass(
     if (tid == kThreads - 1) sm.bstart[kNB] = run;
   }
   const int nslots = sm.nslots;
+  for (int k = tid; k < nslots * kWin; k += kThreads) (&sm.part[0][0])[k] = 0.0f;
+  if constexpr (kComp)
+    for (int k = tid; k < nslots * kWin; k += kThreads) (&sm.part_c[0][0])[k] = 0.0f;
+  for (int k = tid; k < nslots * kWin / 4; k += kThreads) reinterpret_cast<uint32_t*>(&sm.nzb[0][0])[k] = 0u;
   for (int k = tid; k < (s <= kMaxS ? nslots * s : 0); k += kThreads) {
     const int q = k / s, a = k - q * s;
     if constexpr (kL == 1) {
@@ -409,10 +422,10 @@ __device__ __forceinline__ void tile_pass(
 
   float T = 1.0f;
   bool done = !inside;
-  if (pix_state && !first_slab) {
-    const float sv = pix_state[(int64_t)tile * kTilePixels + tid];
+  if constexpr (kSecond) {
+    const float sv = job.pix_state[(int64_t)tile * kTilePixels + tid];
     if (sv < 0.0f) done = true;
-    else if (sv > 0.0f) T = sv;
+    else T = sv;
   }
   unsigned n_eval = 0, n_contrib = 0, n_flush = 0, n_atom = 0;  // per thread and tile: fits 32 bits
 
@@ -463,12 +476,13 @@ __device__ __forceinline__ void tile_pass(
       m = (int)(sm.bstart[b1] - base);
       for (int b = b0 + tid; b < b1; b += kThreads) sm.bcur[b] = sm.bstart[b] - base;
       __syncthreads();
-      for (int i = tid; i < n; i += kThreads) {
-        const unsigned long long k = tkeys[i];
-        const int b = bk(k);
+      const TileList& list = sm.list;
+      for (int i = tid; i < list.n; i += kThreads) {
+        const unsigned long long k = list.keys[i];
+        const int b = bk(list, k);
         if (b >= b0 && b < b1) {
           const uint32_t pos = atomicAdd(&sm.bcur[b], 1u);
-          if (pos < (uint32_t)kWin) sm.win[pos] = k;
+          if (pos < (uint32_t)kWin) sm.win[pos] = list.plain(k);
         }
       }
       __syncthreads();
@@ -499,12 +513,13 @@ __device__ __forceinline__ void tile_pass(
       if (tid == 0) atomicAdd(&hdr->split_windows, 1ull);
       const int left = total_b0 - consumed;
       unsigned long long hi_key = ~0ull;
-      if (left > kWin) hi_key = select_in_bucket(sm, tkeys, n, bk, b0, split_last, split_first, kWin - 1);
+      const TileList& list = sm.list;
+      if (left > kWin) hi_key = select_in_bucket(sm, list, bk, b0, split_last, split_first, kWin - 1);
       if (tid == 0) sm.cursor = 0u;
       __syncthreads();
-      for (int i = tid; i < n; i += kThreads) {
-        const unsigned long long k = tkeys[i];
-        if (bk(k) == b0 && (split_first || k > split_last) && k <= hi_key) {
+      for (int i = tid; i < list.n; i += kThreads) {
+        const unsigned long long raw = list.keys[i], k = list.plain(raw);
+        if (bk(list, raw) == b0 && (split_first || k > split_last) && k <= hi_key) {
           const unsigned pos = atomicAdd(&sm.cursor, 1u);
           if (pos < (unsigned)kWin) sm.win[pos] = k;
         }
@@ -717,10 +732,11 @@ __device__ __forceinline__ void tile_pass(
     __syncthreads();
   }
 
-  // ---- state for the next slab ----
-  if (pix_state && !last_slab) {
-    pix_state[(int64_t)tile * kTilePixels + tid] = done ? -1.0f : T;
-    if (__syncthreads_and(done) && tid == 0) tile_done[tile] = 1;
+  // ---- a tile still open at its cut goes to the second pass ----
+  if (!kSecond && sm.list.cut != kNoCut && !__syncthreads_and(done)) {
+    const int t = (int)sm.tile;
+    job.pix_state[(int64_t)t * kTilePixels + tid] = done ? -1.0f : T;
+    if (tid == 0) record_open(job.hdr, job.open_bits, job.open_list, job.cam.gx, t);
   }
 
   // ---- counters ----
@@ -745,155 +761,112 @@ __device__ __forceinline__ void tile_pass(
   }
 }
 
-template <bool kComp, int kBW, int kL>
-__global__ void __launch_bounds__(kThreads, kComp ? 3 : 4) uplift_tile_kernel(
-    const __grid_constant__ CamArgs cam, const ProjRec* __restrict__ proj,
-    const unsigned long long* __restrict__ keys, const uint32_t* __restrict__ tile_start, int slot,
-    const __grid_constant__ LevelCodes lc, int C, int Crow, float* __restrict__ accum, float* __restrict__ comp,
-    WsHeader* __restrict__ hdr, float* __restrict__ pix_state, uint8_t* __restrict__ tile_done, int slab,
-    int nslabs) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  tile_pass<kComp, kBW, kL>(*reinterpret_cast<TileSmem<kComp, kL>*>(smem_raw), blockIdx.x, cam, proj, keys,
-                            tile_start, slot, lc, C, Crow, accum, comp, hdr, pix_state, tile_done, slab, nslabs);
-}
-
-// Batched chunk: a persistent CTA takes (view, tile) items from the chunk's
-// counter until none is left and runs the same per-tile pass on each.  The
-// chunk's views travel in the kernel's parameter space (like the per-view
-// kernel's arguments, read through the constant cache), which keeps them out
-// of the pass's registers.  No CTA waits on another.
+// A persistent CTA takes (view, tile) items from the chunk's counter until
+// none is left and runs the tile pass on each: the views' tiles in the first
+// pass, their open tiles in the second.  The chunk's views travel in the
+// kernel's parameter space (read through the constant cache), which keeps
+// them out of the pass's registers.
+template <int N>
 struct DrainArgs {
-  uint32_t tile0[kMaxDrainJobs];  // first item of each view (ascending, tile0[0] = 0)
+  TileJob jobs[N];
   int njobs;
-  uint32_t total;
-  TileJob jobs[kMaxDrainJobs];
 };
-static_assert(sizeof(DrainArgs) <= 32000, "kernel parameter space");
+static_assert(sizeof(DrainArgs<kMaxDrainJobs>) <= 32000, "kernel parameter space");
 
-template <bool kComp, int kBW>
-__global__ void __launch_bounds__(kThreads, kComp ? 3 : 4) uplift_drain_kernel(const __grid_constant__ DrainArgs a,
-                                                                             unsigned* __restrict__ counter) {
+template <bool kComp, int kBW, int kL, bool kSecond, int N>
+__global__ void __launch_bounds__(kThreads, kComp ? 3 : 4) uplift_drain_kernel(
+    const __grid_constant__ DrainArgs<N> a, unsigned* __restrict__ counter) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  TileSmem<kComp, 1>& sm = *reinterpret_cast<TileSmem<kComp, 1>*>(smem_raw);
-  __shared__ uint32_t s_item;
+  TileSmem<kComp, kL>& sm = *reinterpret_cast<TileSmem<kComp, kL>*>(smem_raw);
+  __shared__ uint32_t s_end[N];  // items up to and including each view's
+  __shared__ uint32_t s_tile;
   __shared__ int s_job;
+  if (threadIdx.x == 0) {
+    uint32_t run = 0u;
+    for (int j = 0; j < a.njobs; ++j) {
+      run += kSecond ? a.jobs[j].hdr->open_tiles : (uint32_t)a.jobs[j].tiles;
+      s_end[j] = run;
+    }
+  }
   for (;;) {
     __syncthreads();  // the previous pass is done with the tile's shared memory
     if (threadIdx.x == 0) {
-      const uint32_t t = atomicAdd(counter, 1u);
-      int lo = 0;
-      if (t < a.total) {
-        int hi = a.njobs - 1;  // last view whose first item is at or before t
-        while (lo < hi) {
-          const int mid = (lo + hi + 1) >> 1;
-          if (a.tile0[mid] <= t) lo = mid; else hi = mid - 1;
+      const uint32_t t = s_end[a.njobs - 1] ? atomicAdd(counter, 1u) : 0u;
+      int j = -1;
+      if (t < s_end[a.njobs - 1]) {
+        int hi = a.njobs - 1;  // first view whose items end after t
+        j = 0;
+        while (j < hi) {
+          const int mid = (j + hi) >> 1;
+          if (s_end[mid] > t) hi = mid; else j = mid + 1;
         }
+        const uint32_t k = t - (j > 0 ? s_end[j - 1] : 0u);
+        s_tile = kSecond ? a.jobs[j].open_list[k] : k;
       }
-      s_item = t;
-      s_job = lo;
+      s_job = j;
     }
     __syncthreads();
-    const uint32_t t = s_item;
-    if (t >= a.total) return;
-    const TileJob& job = a.jobs[s_job];
-    tile_pass<kComp, kBW, 1>(sm, (int)(t - a.tile0[s_job]), job.cam, job.proj, job.keys, job.tile_start, job.slot,
-                             job.lc, job.C, job.C, job.accum, job.comp, job.hdr, nullptr, nullptr, 0, 1);
+    const int j = s_job;
+    if (j < 0) return;
+    tile_pass<kComp, kBW, kL, kSecond>(sm, (int)s_tile, a.jobs[j]);
   }
 }
 
-struct SlabLaunch {
-  float* pix_state;  // null with a single slab
-  uint8_t* tile_done;
-  int slab, nslabs;
-};
-
-template <bool kComp, int kBW, int kL>
-cudaError_t launch_tiles_t(const CamArgs& cam, const UpliftWs& ws, int slot, const LevelCodes& lc, int C, int Crow,
-                           float* accum, float* comp, const SlabLaunch& sl, cudaStream_t st) {
-  const int ntiles = cam.gx * cam.gy;
+template <bool kComp, int kBW, int kL, bool kSecond, int N>
+cudaError_t launch_drain_n(const TileJob* jobs, int njobs, unsigned* counter, cudaStream_t st) {
+  DrainArgs<N> args;
+  memset(&args, 0, sizeof(args));
+  args.njobs = njobs;
+  long long total = 0;
+  for (int j = 0; j < njobs; ++j) {
+    args.jobs[j] = jobs[j];
+    total += jobs[j].tiles;
+  }
+  if (total <= 0) return cudaSuccess;
+  if (total > 0xffffffffLL) return cudaErrorInvalidValue;
   const size_t smem = sizeof(TileSmem<kComp, kL>);
-  cudaError_t err = cudaFuncSetAttribute(uplift_tile_kernel<kComp, kBW, kL>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (err != cudaSuccess) return err;
-  uplift_tile_kernel<kComp, kBW, kL><<<ntiles, kThreads, smem, st>>>(
-      cam, ws.proj, ws.keys, ws.tile_start, slot, lc, C, Crow, accum, comp, ws.hdr, sl.pix_state, sl.tile_done,
-      sl.slab, sl.nslabs);
-  g_launches += 1;
-  return cudaGetLastError();
-}
-
-template <bool kComp>
-cudaError_t launch_tiles_shape(int warp_w, const CamArgs& cam, const UpliftWs& ws, int slot, const LevelCodes& lc,
-                               int C, int Crow, float* accum, float* comp, const SlabLaunch& sl, cudaStream_t st) {
-  if (lc.L > 1) return launch_tiles_t<kComp, 8, 3>(cam, ws, slot, lc, C, Crow, accum, comp, sl, st);
-  switch (warp_w) {
-    case 16: return launch_tiles_t<kComp, 16, 1>(cam, ws, slot, lc, C, Crow, accum, comp, sl, st);
-    case 4: return launch_tiles_t<kComp, 4, 1>(cam, ws, slot, lc, C, Crow, accum, comp, sl, st);
-    default: return launch_tiles_t<kComp, 8, 1>(cam, ws, slot, lc, C, Crow, accum, comp, sl, st);
-  }
-}
-
-template <bool kComp, int kBW>
-cudaError_t launch_drain_t(const DrainArgs& args, unsigned* counter, cudaStream_t st) {
-  const size_t smem = sizeof(TileSmem<kComp, 1>);
-  auto kern = uplift_drain_kernel<kComp, kBW>;
+  auto kern = uplift_drain_kernel<kComp, kBW, kL, kSecond, N>;
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
   // CTAs resident per SM by the launch bounds (the shared memory of four fits);
   // a CTA beyond them would only start later and drain what is left
   const long long resident = (long long)num_sms() * (kComp ? 3 : 4);
-  const int grid = (int)(args.total < (uint32_t)resident ? args.total : (uint32_t)resident);
-  kern<<<grid, kThreads, smem, st>>>(args, counter);
+  kern<<<(int)(total < resident ? total : resident), kThreads, smem, st>>>(args, counter);
   g_launches += 1;
   return cudaGetLastError();
 }
 
-}  // namespace
+template <bool kComp, int kBW, int kL, bool kSecond>
+cudaError_t launch_drain_t(const TileJob* jobs, int njobs, unsigned* counter, cudaStream_t st) {
+  if (njobs <= 8) return launch_drain_n<kComp, kBW, kL, kSecond, 8>(jobs, njobs, counter, st);
+  if constexpr (kL == 1) return launch_drain_n<kComp, kBW, kL, kSecond, kMaxDrainJobs>(jobs, njobs, counter, st);
+  return cudaErrorInvalidValue;  // several levels run at most 8 views at a time
+}
 
-cudaError_t launch_uplift_drain(const TileJob* jobs, const uint32_t* tile0, int njobs, unsigned* counter,
-                                bool compensated, int warp_w, cudaStream_t st) {
-  if (njobs <= 0) return cudaSuccess;
-  if (njobs > kMaxDrainJobs) return cudaErrorInvalidValue;
-  DrainArgs args;
-  memset(&args, 0, sizeof(args));
-  args.njobs = njobs;
-  uint32_t total = 0;
-  for (int j = 0; j < njobs; ++j) {
-    if (tile0[j] != total) return cudaErrorInvalidValue;
-    args.tile0[j] = tile0[j];
-    args.jobs[j] = jobs[j];
-    total += (uint32_t)jobs[j].tiles;
-  }
-  args.total = total;
-  if (total == 0) return cudaSuccess;
-  if (compensated) {
-    switch (warp_w) {
-      case 16: return launch_drain_t<true, 16>(args, counter, st);
-      case 4: return launch_drain_t<true, 4>(args, counter, st);
-      default: return launch_drain_t<true, 8>(args, counter, st);
-    }
-  }
+template <bool kComp, bool kSecond>
+cudaError_t launch_drain_shape(const TileJob* jobs, int njobs, unsigned* counter, int warp_w, cudaStream_t st) {
+  if (jobs[0].lc.L > 1) return launch_drain_t<kComp, 8, 3, kSecond>(jobs, njobs, counter, st);
   switch (warp_w) {
-    case 16: return launch_drain_t<false, 16>(args, counter, st);
-    case 4: return launch_drain_t<false, 4>(args, counter, st);
-    default: return launch_drain_t<false, 8>(args, counter, st);
+    case 16: return launch_drain_t<kComp, 16, 1, kSecond>(jobs, njobs, counter, st);
+    case 4: return launch_drain_t<kComp, 4, 1, kSecond>(jobs, njobs, counter, st);
+    default: return launch_drain_t<kComp, 8, 1, kSecond>(jobs, njobs, counter, st);
   }
 }
 
-cudaError_t launch_uplift_tiles(const CamArgs& cam, const UpliftWs& ws, int slot, const LevelCodes& lc, int C,
-                                int Crow, float* accum, float* comp, int warp_w, cudaStream_t st, int slab,
-                                int nslabs) {
+}  // namespace
+
+cudaError_t launch_uplift_drain(const TileJob* jobs, int njobs, bool second, uint32_t* ctr, bool compensated,
+                                int warp_w, cudaStream_t st) {
   static_assert(sizeof(TileSmem<false, 1>) <= 55 * 1024, "4 CTAs per SM");
   static_assert(sizeof(TileSmem<false, 3>) <= 55 * 1024, "4 CTAs per SM");
   static_assert(sizeof(TileSmem<true, 3>) <= 74 * 1024, "3 CTAs per SM");
-  if (cam.gx * cam.gy <= 0) return cudaSuccess;
-  SlabLaunch sl;
-  sl.pix_state = nslabs > 1 ? ws.pix_state : nullptr;
-  sl.tile_done = ws.tile_done;
-  sl.slab = nslabs > 1 ? slab : 0;
-  sl.nslabs = nslabs > 1 ? nslabs : 1;
-  if (comp) return launch_tiles_shape<true>(warp_w, cam, ws, slot, lc, C, Crow, accum, comp, sl, st);
-  return launch_tiles_shape<false>(warp_w, cam, ws, slot, lc, C, Crow, accum, nullptr, sl, st);
+  if (njobs <= 0) return cudaSuccess;
+  if (njobs > kMaxDrainJobs) return cudaErrorInvalidValue;
+  if (compensated)
+    return second ? launch_drain_shape<true, true>(jobs, njobs, ctr, warp_w, st)
+                  : launch_drain_shape<true, false>(jobs, njobs, ctr, warp_w, st);
+  return second ? launch_drain_shape<false, true>(jobs, njobs, ctr, warp_w, st)
+                : launch_drain_shape<false, false>(jobs, njobs, ctr, warp_w, st);
 }
 
 }  // namespace scoup

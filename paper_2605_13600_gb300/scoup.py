@@ -643,10 +643,17 @@ class Uplift:
     uplift (all views + Top-K) on the current stream.
     """
 
+    # Largest workspace of the chunked form that run() takes by itself (see
+    # __init__): eight views of 300k Gaussians at 640x480 on each of two lanes.
+    CHUNK_BYTES = 1 << 30
+
     def __init__(self, wl, device: str = "cuda", dup_capacity: Optional[int] = None,
                  headroom: float = 1.0, compensated: bool = False, topk: bool = True, chunked: bool = False):
         """chunked=True: run() uses the chunked form (SCOUP_UPLIFT_CHUNKED) and
-        the workspace is sized for it."""
+        the workspace is sized for it.  Otherwise run() still takes that form
+        (same results and counters) where its workspace is at most
+        CHUNK_BYTES and there is more than one view: views of such scenes
+        leave most of the chip idle when composited one at a time."""
         import torch
         dev = torch.device(device)
         sc = wl.scene
@@ -674,7 +681,9 @@ class Uplift:
             del probe
         self.dup_capacity = dup_capacity
         self.chunked = bool(chunked)
-        size = scoup_uplift_chunked_workspace_size if self.chunked else scoup_uplift_workspace_size
+        self._chunk_views = self.chunked or (
+            len(self.cams) > 1 and scoup_uplift_chunked_workspace_size(n, maxw, maxh, dup_capacity) <= self.CHUNK_BYTES)
+        size = scoup_uplift_chunked_workspace_size if self._chunk_views else scoup_uplift_workspace_size
         self.workspace = torch.empty(size(n, maxw, maxh, dup_capacity) + extra, dtype=torch.uint8, device=dev)
         self.maxw, self.maxh, self.extra, self.device = maxw, maxh, extra, dev
         self._host_ws = None
@@ -691,7 +700,7 @@ class Uplift:
         offs = self.map_offsets if views is None else self.map_offsets[list(views)]
         if self.compensated:
             accum_mode |= SCOUP_ACCUM_COMPENSATED
-        if self.chunked:
+        if self._chunk_views:
             accum_mode |= SCOUP_UPLIFT_CHUNKED
         return scoup_uplift(self.scene, cams, self.region_maps, offs, self.R_total, self.code_idx,
                             self.code_val, self.s, self.C, self.K, self.accum, accum_mode,
