@@ -7,7 +7,8 @@
 // L = sum_p |F(p) - F*(p)|^2 over labelled pixels, and dL/dF(p) = 2 (F - F*).
 // A first kernel decodes every region's target once (R x D floats, resident
 // in L2), a second one streams the pixels: one warp per pixel row of D
-// features, lanes over the features.
+// features, lanes over the features (eight at a time where the alignment
+// allows).
 #include <cuda_bf16.h>
 
 #include "scoup_internal.cuh"
@@ -15,24 +16,112 @@
 namespace scoup {
 namespace {
 
-// F*_r[d] = sum_j v_j C[j][d] for every region r (one warp per region).
+// F*_r[d] = sum_j v_j C[j][d] for every region r: one CTA per region and 256
+// features, a thread per feature, the code's entries loaded once into shared
+// memory and eight codebook loads in flight per thread (a warp per region with
+// the entries re-read for every feature took 41 us for 200 regions, 8 entries,
+// D = 512, against 4.6).
+constexpr int kCodeChunk = 64;
 __global__ void __launch_bounds__(256) region_target_kernel(const int32_t* __restrict__ ci,
                                                             const float* __restrict__ cv, int R, int s,
                                                             const float* __restrict__ codebook, int C, int D,
                                                             float* __restrict__ target, int* __restrict__ status) {
+  __shared__ int s_j[kCodeChunk];
+  __shared__ float s_v[kCodeChunk];
+  const int d = blockIdx.x * 256 + threadIdx.x;
+  for (int64_t r = blockIdx.y; r < R; r += gridDim.y) {
+    float acc = 0.0f;
+    for (int e0 = 0; e0 < s; e0 += kCodeChunk) {
+      const int m = min(kCodeChunk, s - e0);
+      __syncthreads();
+      if (threadIdx.x < m) {
+        const int j = ci[r * s + e0 + threadIdx.x];
+        if (j >= C) atomicOr(status, kStatDeviceCheck);
+        s_j[threadIdx.x] = j < C ? j : -1;
+        s_v[threadIdx.x] = cv[r * s + e0 + threadIdx.x];
+      }
+      __syncthreads();
+      if (d < D)
+        for (int e = 0; e < m; e += 8) {
+          float x[8];
+#pragma unroll
+          for (int u = 0; u < 8; ++u)
+            x[u] = e + u < m && s_j[e + u] >= 0 ? codebook[(int64_t)s_j[e + u] * D + d] : 0.0f;
+#pragma unroll
+          for (int u = 0; u < 8; ++u)
+            if (e + u < m && s_j[e + u] >= 0) acc = fmaf(s_v[e + u], x[u], acc);
+        }
+    }
+    if (d < D) target[r * D + d] = acc;
+  }
+}
+
+// Eight consecutive features as one access.
+__device__ __forceinline__ void load8(const __nv_bfloat16* p, float (&x)[8]) {
+  const uint4 w = *reinterpret_cast<const uint4*>(p);
+  const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&w);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const float2 f = __bfloat1622float2(h[k]);
+    x[2 * k] = f.x;
+    x[2 * k + 1] = f.y;
+  }
+}
+__device__ __forceinline__ void load8(const float* p, float (&x)[8]) {
+  const float4 a = reinterpret_cast<const float4*>(p)[0], b = reinterpret_cast<const float4*>(p)[1];
+  x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w;
+  x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
+}
+__device__ __forceinline__ void store8(__nv_bfloat16* p, const float (&x)[8]) {
+  uint4 w;
+  __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&w);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) h[k] = __floats2bfloat162_rn(x[2 * k], x[2 * k + 1]);
+  *reinterpret_cast<uint4*>(p) = w;
+}
+__device__ __forceinline__ void store8(float* p, const float (&x)[8]) {
+  reinterpret_cast<float4*>(p)[0] = make_float4(x[0], x[1], x[2], x[3]);
+  reinterpret_cast<float4*>(p)[1] = make_float4(x[4], x[5], x[6], x[7]);
+}
+
+// Rows of D features, D a multiple of 8 and both matrices 16-byte aligned: a
+// warp takes a row, eight features per lane and step, so that a 512-feature
+// bf16 row is two 16-byte loads and stores per lane.  Bound by HBM: read and
+// write once (480k x 512 bf16, 983 MB: 200 us with a feature per lane and
+// step, 174 now).
+template <typename TIn, typename TOut>
+__global__ void __launch_bounds__(256) l2_grad_vec_kernel(const TIn* __restrict__ F, int64_t P, int D,
+                                                          const int32_t* __restrict__ rmap, int R,
+                                                          const float* __restrict__ target, TOut* __restrict__ dF,
+                                                          double* __restrict__ loss, int* __restrict__ status) {
   const int lane = threadIdx.x & 31;
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t r = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < R; r += warps) {
-    for (int d = lane; d < D; d += 32) {
-      float acc = 0.0f;
-      for (int e = 0; e < s; ++e) {
-        const int j = ci[r * s + e];
-        if (j >= C) { atomicOr(status, kStatDeviceCheck); continue; }
-        if (j >= 0) acc = fmaf(cv[r * s + e], codebook[(int64_t)j * D + d], acc);
-      }
-      target[r * D + d] = acc;
+  double part = 0.0;
+  for (int64_t p = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); p < P; p += warps) {
+    int r = rmap[p];
+    if (r >= R) {
+      if (lane == 0) atomicOr(status, kStatDeviceCheck);
+      r = -1;
     }
+    float sq = 0.0f;
+#pragma unroll 2
+    for (int d = 8 * lane; d < D; d += 256) {
+      float f[8], t[8];
+      load8(F + p * D + d, f);
+      // unlabelled pixels (region -1) have no target: no loss, no gradient
+      if (r >= 0) load8(target + (int64_t)r * D + d, t);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const float diff = r >= 0 ? f[k] - t[k] : 0.0f;
+        sq = fmaf(diff, diff, sq);
+        f[k] = 2.0f * diff;
+      }
+      store8(dF + p * D + d, f);
+    }
+    part += (double)sq;
   }
+  for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
+  if (lane == 0 && loss && part != 0.0) atomicAdd(loss, part);
 }
 
 template <bool kInBF16, bool kOutBF16>
@@ -77,7 +166,8 @@ int blocks_for_warps(int64_t rows) {
 cudaError_t launch_region_targets(const int32_t* ci, const float* cv, int R, int s, const float* codebook, int C,
                                   int D, float* target, int* status, cudaStream_t st) {
   if (R <= 0) return cudaSuccess;
-  region_target_kernel<<<blocks_for_warps(R), 256, 0, st>>>(ci, cv, R, s, codebook, C, D, target, status);
+  region_target_kernel<<<dim3((D + 255) / 256, R < 65535 ? R : 65535), 256, 0, st>>>(ci, cv, R, s, codebook, C, D,
+                                                                                   target, status);
   g_launches += 1;
   return cudaGetLastError();
 }
@@ -86,6 +176,19 @@ cudaError_t launch_l2_grad(const void* F, int F_bf16, int64_t P, int D, const in
                            const float* target, void* dF, int dF_bf16, double* loss, int* status, cudaStream_t st) {
   if (P <= 0) return cudaSuccess;
   const int b = blocks_for_warps(P);
+  if (D % 8 == 0 && (((uintptr_t)F | (uintptr_t)dF) & 15u) == 0) {  // target is the workspace's, aligned
+    auto run = [&](auto* f, auto* d) {
+      l2_grad_vec_kernel<<<b, 256, 0, st>>>(f, P, D, rmap, R, target, d, loss, status);
+    };
+    const __nv_bfloat16* fb = (const __nv_bfloat16*)F;
+    __nv_bfloat16* db = (__nv_bfloat16*)dF;
+    if (F_bf16 && dF_bf16) run(fb, db);
+    else if (F_bf16) run(fb, (float*)dF);
+    else if (dF_bf16) run((const float*)F, db);
+    else run((const float*)F, (float*)dF);
+    g_launches += 1;
+    return cudaGetLastError();
+  }
   if (F_bf16 && dF_bf16) l2_grad_kernel<true, true><<<b, 256, 0, st>>>(F, P, D, rmap, R, target, dF, loss, status);
   else if (F_bf16) l2_grad_kernel<true, false><<<b, 256, 0, st>>>(F, P, D, rmap, R, target, dF, loss, status);
   else if (dF_bf16) l2_grad_kernel<false, true><<<b, 256, 0, st>>>(F, P, D, rmap, R, target, dF, loss, status);
