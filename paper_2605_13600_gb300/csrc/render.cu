@@ -276,7 +276,7 @@ bool render_uses_mma(int C, int K) {
 }
 
 size_t render_smem_bytes(int C, int K) {
-  if (render_uses_mma(C, K)) return render_mma_smem_bytes();
+  if (render_uses_mma(C, K)) return render_mma_smem_bytes(K);
   return sizeof(RenderSmem) + sizeof(float) * (size_t)kRWarps * (size_t)(2 * C + 16) +
          (render_stages(K) ? staged_bytes(K) : 0);
 }

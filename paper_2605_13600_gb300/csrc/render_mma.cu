@@ -27,6 +27,19 @@
 // MMAs of the previous one.  A chunk in which a pixel half has no weight
 // issues no MMA for that half.
 //
+// The bound is the walkers' instruction issue with nine warps to an SM (the
+// pipes are below 40 % busy, DRAM below 10 %), so the work per chunk is kept
+// down: codes are merged and split into their bf16 parts once per window and
+// not per chunk, the warps a Gaussian may reach are a byte staged with it, the
+// walk multiplies the transmittance down without a test per step and masks the
+// weights behind the stop, and W is cleared by undoing the entries that were
+// written (32 KB of zeros per chunk at C = 256 otherwise).  With these, 1M
+// Gaussians at 1080p, C = 256, K = 8 (reorder to similarity in one call) went
+// from 2.87 to 2.83 ms, forward and backward of an 800 x 600 view from 2.04 to
+// 2.02 ms and a 161 x 119 view of 10k Gaussians at C = 64 from 155 to 146 us.
+// Half-tile CTAs, two to an SM, take 1.84 ms where this kernel takes 1.61 ms
+// (1080p): every half orders and stages the tile's list again.
+//
 // Every wait (the MMA warp's on a chunk, the walkers' on a completion) is
 // bounded; a wait that gives up sets the timeout status, the walkers stop,
 // a stop still reaches the MMA warp, and TMEM is freed on every path.  The
@@ -68,13 +81,15 @@ struct alignas(128) ChunkBuf {
   unsigned char w[2][kWBytes];     // [hi, lo]
 };
 
+template <int KT>
 struct RenderMmaSmem {
   ChunkBuf buf[2];
   MOrder ord;
   float4 rec_a[MOrder::kWin];
   float4 rec_b[MOrder::kWin];
-  float code_val[kMaxK * MOrder::kWin];  // entry-major: [k][window position]
-  short code_idx[kMaxK * MOrder::kWin];
+  uint32_t code_val[KT * MOrder::kWin];  // [k][window position]: the value's bf16 parts, hi | lo << 16
+  short code_idx[KT * MOrder::kWin];     // atom; -1: no entry, or added to an earlier entry of the atom
+  uint8_t rows[MOrder::kWin];            // bit w: the Gaussian may reach warp w's 16 x 2 block
   uint64_t mma_done[2];  // per chunk buffer: the MMAs that read it have completed
   uint64_t ready[2];     // per chunk buffer: the walkers have written E and W (and ctl)
   uint64_t fin;
@@ -104,23 +119,18 @@ __device__ __forceinline__ void split_bf16x2(float x, float y, uint32_t& hi, uin
 
 // Walks the thread's pixel over window positions j0 .. j0 + 31 and writes its
 // row of E (hi and lo parts, zero where a Gaussian does not contribute);
-// returns whether any weight of the row is nonzero.
+// returns whether any weight of the row is nonzero.  T below the cutoff: the
+// pixel has stopped, and Tout holds its transmittance.
 // Gaussians that cannot pass the alpha test at any pixel of the warp's 16 x 2
-// block (box_may_hit) are skipped, 8 at a time when none of 8 can.
-__device__ __forceinline__ bool walk_chunk(const RenderMmaSmem& sm, int j0, int m, int wbase, float fpx, float fpy,
-                                           float bx0, float by0, float& T, int& last, bool& done, unsigned& n_eval,
-                                           unsigned& n_contrib, unsigned char* e_hi, unsigned char* e_lo, int row) {
+// block (sm.rows) are skipped, 8 at a time when none of 8 can.
+template <int KT>
+__device__ __forceinline__ bool walk_chunk(const RenderMmaSmem<KT>& sm, int j0, int m, int wbase, float fpx, float fpy,
+                                           float& T, float& Tout, int& last, unsigned& n_eval, unsigned& n_contrib,
+                                           unsigned char* e_hi, unsigned char* e_lo, int row) {
   unsigned rel = 0u;
-  if (!__all_sync(0xffffffffu, done)) {
+  if (!__all_sync(0xffffffffu, T < 1e-4f)) {
     const int jl = j0 + (int)(threadIdx.x & 31);
-    bool r = false;
-    if (jl < m) {
-      ProjRec pr;
-      pr.a = sm.rec_a[jl];
-      pr.b = sm.rec_b[jl];
-      r = box_may_hit(pr, bx0, by0, (float)kTile, 2.0f);
-    }
-    rel = __ballot_sync(0xffffffffu, r);
+    rel = __ballot_sync(0xffffffffu, jl < m && ((sm.rows[jl] >> (threadIdx.x >> 5)) & 1u));
   }
   bool any = false;
 #pragma unroll
@@ -135,7 +145,8 @@ __device__ __forceinline__ bool walk_chunk(const RenderMmaSmem& sm, int j0, int 
     // flight).  Positions past the window hold records that never pass (tau =
     // +inf), and a Gaussian outside the warp's box cannot pass either, so
     // alpha > 0 exactly when the Gaussian passes the alpha test here.
-    float al[8];
+    float al[8], om[8];
+    unsigned pass = 0u;
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
       const int j = j0 + g * 8 + u;
@@ -143,27 +154,39 @@ __device__ __forceinline__ bool walk_chunk(const RenderMmaSmem& sm, int j0, int 
       const float4 b = sm.rec_b[j];
       const float dx = a.x - fpx, dy = a.y - fpy;
       const float power = fmaf(dx, fmaf(a.z, dx, __fmul_rn(a.w, dy)), __fmul_rn(__fmul_rn(b.x, dy), dy));
-      al[u] = (power <= 0.0f && power >= b.z) ? fminf(0.99f, b.y * __expf(power)) : 0.0f;
+      const bool ok = power <= 0.0f && power >= b.z;
+      al[u] = ok ? fminf(0.99f, b.y * __expf(power)) : 0.0f;
+      om[u] = 1.0f - al[u];
+      if (ok) pass |= 1u << u;
     }
-    // serial front to back: transmittance, T-stop, weights
+    // front to back: T only falls, so once a product is below the cutoff all
+    // later ones are, and the running product needs no test of its own: the
+    // weights from the stop on are masked afterwards
     float ev[8];
-    const bool open0 = !done;
-    int ustop = 8;
+    const float T0 = T;
+    unsigned n_ok = 0u;  // Gaussians in front of the stop
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      const float test = T * (1.0f - al[u]);
-      const bool act = !done && al[u] > 0.0f;
-      const bool stop = act && test < 1e-4f;
-      const bool tk = act && !stop;
-      ev[u] = tk ? al[u] * T : 0.0f;
-      T = tk ? test : T;
-      if (tk) last = wbase + j0 + g * 8 + u + 1;
-      n_contrib += tk ? 1u : 0u;
-      if (stop) ustop = u;
-      done = done || stop;
+      const float test = __fmul_rn(T, om[u]);
+      const bool ok = test >= 1e-4f;
+      ev[u] = ok ? al[u] * T : 0.0f;
+      n_ok += ok ? 1u : 0u;
+      T = test;
     }
-    // examined: the group's Gaussians in the warp's box while the pixel was open, up to the stop
-    if (open0) n_eval += __popc(rel8 & ((2u << ustop) - 1u));
+    if (T0 >= 1e-4f) {  // the pixel was open
+      pass &= (1u << n_ok) - 1u;
+      n_contrib += __popc(pass);
+      if (pass) last = wbase + j0 + g * 8 + 32 - __clz(pass);
+      // examined: the group's Gaussians in the warp's box up to the stop
+      n_eval += __popc(rel8 & ((2u << n_ok) - 1u));
+      Tout = T;
+      if (n_ok < 8u) {
+        Tout = T0;  // the transmittance in front of the stop
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (u < (int)n_ok) Tout = __fmul_rn(Tout, om[u]);
+      }
+    }
     uint4 hi, lo;
     split_bf16x2(ev[0], ev[1], hi.x, lo.x);
     split_bf16x2(ev[2], ev[3], hi.y, lo.y);
@@ -228,13 +251,14 @@ __device__ __forceinline__ bool walkers_or(bool p) {
 // One CTA per tile; one CTA per SM (the accumulator takes the SM's 512 TMEM
 // columns at C = 256, and the shared memory keeps a second CTA out).
 // second: the tiles recorded as open, each from the start of its whole list.
+template <int KT>
 __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
     const __grid_constant__ ViewJob view, int second, const int32_t* __restrict__ topk_idx,
     const float* __restrict__ topk_val, int K, int C, void* __restrict__ out, int out_bf16,
     float* __restrict__ out_T, int32_t* __restrict__ out_last) {
   extern __shared__ __align__(128) unsigned char msm_raw[];
   unsigned char* base = msm_raw + ((128u - (ptx::smem_u32(msm_raw) & 127u)) & 127u);
-  RenderMmaSmem& sm = *reinterpret_cast<RenderMmaSmem*>(base);
+  RenderMmaSmem<KT>& sm = *reinterpret_cast<RenderMmaSmem<KT>*>(base);
   const CamArgs& cam = view.cam;
   WsHeader* __restrict__ const hdr = view.hdr;
   const ProjRec* __restrict__ const proj = view.proj;
@@ -313,9 +337,20 @@ __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
   const int px = tx * kTile + (tid & (kTile - 1)), py = ty * kTile + (tid >> 4);
   const bool inside = px < cam.width && py < cam.height;
   const int half = tid >> 7, row = tid & 127;  // E row and TMEM lane of this pixel
-  float T = 1.0f;
+  float T = inside ? 1.0f : 0.0f, Tout = T;
   int last = 0;
-  bool done = !inside;
+  // W starts cleared; each thread clears what it wrote before the buffer's next use
+  for (int b = 0; b < 2; ++b)
+    for (int i = tid; i < 2 * kWBytes / 16; i += kMThreads)
+      reinterpret_cast<uint4*>(sm.buf[b].w[0])[i] = make_uint4(0u, 0u, 0u, 0u);
+  constexpr int kPer = (kChunk * KT + kMThreads - 1) / kMThreads;  // W entries of a thread per chunk
+  constexpr int kNone = 0xffff;
+  int wrote[kPer], wrote2[kPer];  // offsets written for the last chunk and the one before it
+#pragma unroll
+  for (int q = 0; q < kPer; ++q) wrote[q] = wrote2[q] = kNone;
+  // code rows by 16-byte loads (K = 4, 8, ..; the arrays may start anywhere)
+  const bool vec =
+      (K & 3) == 0 && ((reinterpret_cast<uintptr_t>(topk_idx) | reinterpret_cast<uintptr_t>(topk_val)) & 15) == 0;
   const OrderBuckets bk = order_buckets<MOrder>(hdr, cut);
   order_init<MOrder, 16>(sm.ord, list, bk);
 
@@ -331,26 +366,23 @@ __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
   while (!all_done && !aborted) {
     const int m = n > 0 ? order_next_window<MOrder, 16>(sm.ord, list, bk, ost, hdr) : 0;
     if (m <= 0) break;  // list exhausted, or an inconsistency (status already set)
-    // records of the window; the positions up to the next chunk boundary get
-    // a record no pixel accepts (tau = +inf)
+    // the window's records, which warps' blocks they may reach, and their code
+    // rows (one thread per Gaussian, all loads in flight together); the
+    // positions up to the next chunk boundary get a record no pixel accepts
+    // (tau = +inf)
     for (int j = tid; j < ((m + kChunk - 1) & ~(kChunk - 1)); j += kMThreads) {
-      if (j < m) {
-        const ProjRec pr = proj[(int)(sm.ord.win[j] & 0xffffffffull)];
-        sm.rec_a[j] = pr.a;
-        sm.rec_b[j] = pr.b;
-      } else {
+      if (j >= m) {
         sm.rec_a[j] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         sm.rec_b[j] = make_float4(0.0f, 0.0f, INFINITY, 0.0f);
+        continue;
       }
-    }
-    // one thread per Gaussian stages its whole code row (all loads in flight together)
-    for (int j = tid; j < m; j += kMThreads) {
       const int64_t g = (int64_t)(sm.ord.win[j] & 0xffffffffull);
-      int32_t ai[kMaxK];
-      float av[kMaxK];
-      if ((K & 3) == 0) {
+      const ProjRec pr = proj[g];
+      int32_t ai[KT];
+      float av[KT];
+      if (vec) {
 #pragma unroll
-        for (int k4 = 0; k4 < kMaxK / 4; ++k4)
+        for (int k4 = 0; k4 < KT / 4; ++k4)
           if (4 * k4 < K) {
             const int4 a = reinterpret_cast<const int4*>(topk_idx + g * K)[k4];
             const float4 v = reinterpret_cast<const float4*>(topk_val + g * K)[k4];
@@ -359,18 +391,32 @@ __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
           }
       } else {
 #pragma unroll
-        for (int k = 0; k < kMaxK; ++k)
+        for (int k = 0; k < KT; ++k)
           if (k < K) {
             ai[k] = topk_idx[g * K + k];
             av[k] = topk_val[g * K + k];
           }
       }
+      sm.rec_a[j] = pr.a;
+      sm.rec_b[j] = pr.b;
+      sm.rows[j] = (uint8_t)box_grid_mask<1, kMWarps>(pr, (float)(tx * kTile), (float)(ty * kTile), (float)kTile, 2.0f);
+      // repeated atoms of one code add up in the first of them
 #pragma unroll
-      for (int k = 0; k < kMaxK; ++k)
+      for (int k = 0; k < KT; ++k) {
+        int atom = -1;
         if (k < K) {
-          sm.code_idx[k * MOrder::kWin + j] = (short)(ai[k] >= 0 && ai[k] < C ? ai[k] : -1);
-          sm.code_val[k * MOrder::kWin + j] = av[k];
+          if (!(ai[k] >= 0 && ai[k] < C)) ai[k] = -1;
+#pragma unroll
+          for (int k2 = k + 1; k2 < KT; ++k2)
+            if (k2 < K && ai[k] >= 0 && ai[k2] == ai[k]) { av[k] += av[k2]; ai[k2] = -1; }
+          atom = ai[k];
+          const __nv_bfloat16 h = __float2bfloat16_rn(av[k]);
+          const __nv_bfloat16 l = __float2bfloat16_rn(av[k] - __bfloat162float(h));
+          sm.code_val[k * MOrder::kWin + j] =
+              (uint32_t)__bfloat16_as_ushort(h) | ((uint32_t)__bfloat16_as_ushort(l) << 16);
         }
+        sm.code_idx[k * MOrder::kWin + j] = (short)atom;
+      }
     }
     walkers_sync();
     for (int j0 = 0; j0 < m; j0 += kChunk, ++chunk) {
@@ -388,44 +434,39 @@ __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
         aborted = true;
         break;
       }
-      {
-        const int n16 = Np * kChunk * 2 / 16;  // uint4 per W tile in use
-        for (int i = tid; i < 2 * n16; i += kMThreads) {
-          const int t = i >= n16 ? 1 : 0;
-          reinterpret_cast<uint4*>(cb.w[t])[i - t * n16] = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+      for (int q = 0; q < kPer; ++q) {
+        if (wrote2[q] != kNone) {
+          *reinterpret_cast<uint16_t*>(cb.w[0] + wrote2[q]) = 0;
+          *reinterpret_cast<uint16_t*>(cb.w[1] + wrote2[q]) = 0;
         }
+        wrote2[q] = wrote[q];
+        wrote[q] = kNone;
       }
-      const bool any = walk_chunk(sm, j0, m, wbase, (float)px, (float)py, (float)(tx * kTile),
-                                  (float)(ty * kTile + 2 * warp), T, last, done, n_eval, n_contrib, cb.e[0][half],
-                                  cb.e[1][half], row);
+      const bool any = walk_chunk<KT>(sm, j0, m, wbase, (float)px, (float)py, T, Tout, last, n_eval, n_contrib,
+                                      cb.e[0][half], cb.e[1][half], row);
       const unsigned wany = __ballot_sync(0xffffffffu, any);
       if (lane == 0) sm.any_e[warp] = wany != 0u;
       walkers_sync();
       const bool any0 = (sm.any_e[0] | sm.any_e[1] | sm.any_e[2] | sm.any_e[3]) != 0;
       const bool any1 = (sm.any_e[4] | sm.any_e[5] | sm.any_e[6] | sm.any_e[7]) != 0;
       if (any0 || any1) {
-        // W (hi, lo): entry (atom, Gaussian); repeated atoms of one code add up
-        for (int t = tid; t < kChunk * K; t += kMThreads) {
-          const int jc = t & (kChunk - 1), k = t >> 5;
-          const int j = j0 + jc;
-          if (j >= m) continue;
+        // W (hi, lo): entry (atom, Gaussian)
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) {
+          const int t = tid + q * kMThreads, jc = t & (kChunk - 1), k = t / kChunk, j = j0 + jc;
+          if (k >= K || j >= m) continue;
           const int atom = sm.code_idx[k * MOrder::kWin + j];
           if (atom < 0) continue;
-          bool first = true;
-          for (int k2 = 0; k2 < k; ++k2) first = first && sm.code_idx[k2 * MOrder::kWin + j] != atom;
-          if (!first) continue;
-          float v = sm.code_val[k * MOrder::kWin + j];
-          for (int k2 = k + 1; k2 < K; ++k2)
-            if (sm.code_idx[k2 * MOrder::kWin + j] == atom) v += sm.code_val[k2 * MOrder::kWin + j];
-          const __nv_bfloat16 h = __float2bfloat16_rn(v);
-          const __nv_bfloat16 l = __float2bfloat16_rn(v - __bfloat162float(h));
+          const uint32_t v = sm.code_val[k * MOrder::kWin + j];
           const int o = core_off(atom, jc);
-          *reinterpret_cast<__nv_bfloat16*>(cb.w[0] + o) = h;
-          *reinterpret_cast<__nv_bfloat16*>(cb.w[1] + o) = l;
+          *reinterpret_cast<uint16_t*>(cb.w[0] + o) = (uint16_t)v;
+          *reinterpret_cast<uint16_t*>(cb.w[1] + o) = (uint16_t)(v >> 16);
+          wrote[q] = o;
         }
       }
       ptx::fence_async_shared();  // E and W are read by the tensor core (async proxy)
-      const bool open = walkers_or(!done);
+      const bool open = walkers_or(T >= 1e-4f);
       // hand the chunk to the MMA warp (thread 0's control words are
       // published by its own arrival)
       if (tid == 0) {
@@ -487,7 +528,6 @@ __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
   const int piece_cols = 512 / esz;
   if (!bad && C == Np && C % piece_cols == 0 && ((uintptr_t)out & 15u) == 0) {
     unsigned char* stg = reinterpret_cast<unsigned char*>(&sm.buf[0]) + warp * 16384;
-    unsigned char* orow = reinterpret_cast<unsigned char*>(out) + pix * (int64_t)C * esz;
     for (int p0 = 0; p0 < Np; p0 += piece_cols) {
       for (int c0 = p0; c0 < p0 + piece_cols; c0 += 32) {
         float v[32];
@@ -512,11 +552,14 @@ __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
         }
       }
       __syncwarp();
+      const int qx = tx * kTile, qy = ty * kTile + 2 * warp;  // the warp's 16 x 2 pixels
+#pragma unroll 8
       for (int r = 0; r < 32; ++r) {
         const uint4 val = *reinterpret_cast<const uint4*>(stg + r * 512 + ((lane ^ r) & 31) * 16);
-        const unsigned long long ra = __shfl_sync(0xffffffffu, (unsigned long long)(uintptr_t)orow, r);
-        if (__shfl_sync(0xffffffffu, inside, r))
-          *reinterpret_cast<uint4*>(reinterpret_cast<unsigned char*>((uintptr_t)ra) + p0 * esz + lane * 16) = val;
+        const int rx = qx + (r & 15), ry = qy + (r >> 4);
+        if (rx < cam.width && ry < cam.height)
+          *reinterpret_cast<uint4*>(reinterpret_cast<unsigned char*>(out) +
+                                    ((int64_t)ry * cam.width + rx) * (int64_t)C * esz + p0 * esz + lane * 16) = val;
       }
       __syncwarp();
     }
@@ -533,7 +576,7 @@ __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
     }
   }
   if (inside && !again) {
-    if (out_T) out_T[pix] = T;
+    if (out_T) out_T[pix] = Tout;
     if (out_last) out_last[pix] = last;
   }
   const unsigned we = __reduce_add_sync(0xffffffffu, n_eval);
@@ -556,18 +599,21 @@ __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
 
 bool render_mma_supported(int C, int K) { return C >= 1 && C <= kMaxN && K >= 1 && K <= kMaxK; }
 
-size_t render_mma_smem_bytes() { return sizeof(RenderMmaSmem) + 128; }
+size_t render_mma_smem_bytes(int K) {
+  return (K <= 4 ? sizeof(RenderMmaSmem<4>) : K <= 8 ? sizeof(RenderMmaSmem<8>) : sizeof(RenderMmaSmem<16>)) + 128;
+}
 
 cudaError_t launch_render_mma(const ViewJob& v, bool second, const int32_t* topk_idx,
                               const float* topk_val, int K, int C, void* out, int out_bf16, float* out_T,
                               int32_t* out_last, cudaStream_t st) {
   const int ntiles = v.cam.gx * v.cam.gy;
   if (ntiles <= 0) return cudaSuccess;
-  const size_t smem = render_mma_smem_bytes();
-  cudaError_t err = cudaFuncSetAttribute(render_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const size_t smem = render_mma_smem_bytes(K);
+  const auto kernel = K <= 4 ? render_mma_kernel<4> : K <= 8 ? render_mma_kernel<8> : render_mma_kernel<16>;
+  cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
-  render_mma_kernel<<<ntiles, kCtaThreads, smem, st>>>(v, second ? 1 : 0, topk_idx, topk_val, K, C, out, out_bf16, out_T,
-                                                      out_last);
+  kernel<<<ntiles, kCtaThreads, smem, st>>>(v, second ? 1 : 0, topk_idx, topk_val, K, C, out, out_bf16, out_T,
+                                            out_last);
   g_launches += 1;
   return cudaGetLastError();
 }

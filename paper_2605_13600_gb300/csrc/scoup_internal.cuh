@@ -412,7 +412,7 @@ cudaError_t launch_uplift_drain(const TileJob* jobs, int njobs, bool second, uin
 size_t render_smem_bytes(int C, int K);
 bool render_uses_mma(int C, int K);
 bool render_mma_supported(int C, int K);
-size_t render_mma_smem_bytes();
+size_t render_mma_smem_bytes(int K);
 cudaError_t launch_render_mma(const ViewJob& v, bool second, const int32_t* topk_idx,
                               const float* topk_val, int K, int C, void* out, int out_bf16, float* out_T,
                               int32_t* out_last, cudaStream_t st);
