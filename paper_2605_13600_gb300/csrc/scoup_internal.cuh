@@ -282,7 +282,7 @@ struct UpliftWs {
   uint32_t* run_base;       // [groups x box blocks] offset of each binning CTA's run in a list
   uint32_t* tile_start;     // [max_tiles + 1] first key of each list (TileList)
   uint32_t* tile_fill;      // [max_tiles]
-  float* pix_state;         // [max_tiles * 256] per pixel of an open tile: T, or < 0 = stopped; holds
+  float* pix_state;         // [max_tiles * 256] per pixel of an open tile: T (< 1e-4: stopped); holds
                             //     the depth cut's histogram while the view is projected
   uint32_t* zcut;           // [blocks] depth cut per block of 2 x 2 tiles (null: the part has no room)
   uint32_t* open_bits;      // [blocks high x open_words(gx)] bit per block with a tile recorded as open
