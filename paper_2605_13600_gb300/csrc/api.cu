@@ -963,21 +963,23 @@ int scoup_decode(const void* codes, int32_t codes_dtype, int64_t P, int32_t C, c
   PhaseScope ps(SCOUP_PHASE_DECODE, st);
   if ((e = cudaMemsetAsync(hdr, 0, sizeof(WsHeader), st)) != cudaSuccess) return cuda_fail(e, "memset");
   if (P == 0) return SCOUP_OK;
+  const bool direct = codes_dtype == 1 || gemm_takes_f32(P, D, C);
   if (feat_norm2 && (e = cudaMemsetAsync(feat_norm2, 0, sizeof(float) * (size_t)P, st)) != cudaSuccess)
     return cuda_fail(e, "memset");
   if ((e = launch_transpose_bf16(codebook, Bt, C, D, st)) != cudaSuccess) return cuda_fail(e, "codebook");
-  // bf16 codes feed the GEMM directly (one launch); f32 codes are rounded to
-  // bf16 chunk by chunk in the workspace first
-  const int64_t chunk = codes_dtype == 1 ? P : decode_chunk_rows(P);
+  // bf16 codes feed the GEMM directly (one launch), f32 codes where it rounds
+  // them itself; elsewhere they are rounded to bf16 chunk by chunk in the
+  // workspace first
+  const int64_t chunk = direct ? P : decode_chunk_rows(P);
   for (int64_t r0 = 0; r0 < P; r0 += chunk) {
     const int64_t rows = P - r0 < chunk ? P - r0 : chunk;
     const void* A;
-    if (codes_dtype == 0) {
+    if (!direct) {
       if ((e = launch_f32_to_bf16((const float*)codes + r0 * C, Abuf, rows * C, st)) != cudaSuccess)
         return cuda_fail(e, "convert");
       A = Abuf;
     } else {
-      A = (const char*)codes + (size_t)r0 * C * 2;
+      A = (const char*)codes + (size_t)r0 * C * (codes_dtype == 0 ? 4 : 2);
     }
     GemmEpi ep;
     ep.M = (int)rows;
@@ -988,6 +990,7 @@ int scoup_decode(const void* codes, int32_t codes_dtype, int64_t P, int32_t C, c
     ep.ldo = D;
     ep.rownorm2 = (out_dtype == 1 && feat_norm2) ? feat_norm2 + r0 : nullptr;
     ep.colnorm = nullptr;
+    ep.a_f32 = codes_dtype == 0 && direct;
     ep.status = &hdr->status;
     if ((e = launch_gemm_bf16(A, Bt, ep, st)) != cudaSuccess) return cuda_fail(e, "decode gemm");
   }
@@ -1174,16 +1177,17 @@ int scoup_decode_query(const void* codes, int32_t codes_dtype, int64_t P, int32_
   if ((e = launch_text_codebook(text, codebook, Q, C, D, Gt, tnorm, st)) != cudaSuccess)
     return cuda_fail(e, "text x codebook");
   const int64_t ldq = n_canon > 0 ? Q - n_canon : Q;
-  const int64_t chunk = codes_dtype == 1 ? P : decode_chunk_rows(P);
+  const bool direct = codes_dtype == 1 || gemm_takes_f32(P, D, C);
+  const int64_t chunk = direct ? P : decode_chunk_rows(P);
   for (int64_t r0 = 0; r0 < P; r0 += chunk) {
     const int64_t rows = P - r0 < chunk ? P - r0 : chunk;
     const void* A;
-    if (codes_dtype == 0) {
+    if (!direct) {
       if ((e = launch_f32_to_bf16((const float*)codes + r0 * C, Abuf, rows * C, st)) != cudaSuccess)
         return cuda_fail(e, "convert");
       A = Abuf;
     } else {
-      A = (const char*)codes + (size_t)r0 * C * 2;
+      A = (const char*)codes + (size_t)r0 * C * (codes_dtype == 0 ? 4 : 2);
     }
     GemmEpi ep;
     ep.M = (int)rows;
@@ -1201,6 +1205,7 @@ int scoup_decode_query(const void* codes, int32_t codes_dtype, int64_t P, int32_
     ep.sim_mode = n_canon > 0 ? kOutRel : kOutCos;
     ep.sim_out = out + r0 * ldq;
     ep.sim_ldo = ldq;
+    ep.a_f32 = codes_dtype == 0 && direct;
     ep.status = &hdr->status;
     if ((e = launch_gemm_bf16_query(A, Bt, Gt, ep, st)) != cudaSuccess) return cuda_fail(e, "decode + query gemm");
   }

@@ -8,10 +8,17 @@
 // swizzle row) with TMA into a kStages ring guarded by mbarriers; warp 1
 // allocates two BN-column TMEM accumulators and one thread issues
 // tcgen05.mma (M=128, N=BN, K=16) into them alternately, so the epilogue of
-// one unit overlaps the MMAs of the next; warps 2-5 each own a 32-lane TMEM
-// quarter (32 output rows), read 128-byte row chunks back with tcgen05.ld,
-// apply the epilogue, stage them 128-byte-swizzled in shared memory and write
-// them with TMA tile stores (double-buffered per warp).  Epilogues:
+// one unit overlaps the MMAs of the next; warps 2-5 and 6-9 are two epilogue
+// groups whose warps each own a 32-lane TMEM quarter (32 output rows): a unit's
+// row chunks of 128 bytes are split between the groups, read back with
+// tcgen05.ld, taken through the epilogue, staged 128-byte-swizzled in shared
+// memory and written with TMA tile stores (double-buffered per warp).  Two
+// groups, because with one warp per scheduler every epilogue instruction waits
+// for the one before; and the issuing warps run their loops together (uniform
+// registers), because one diverged thread takes longer to build a stage's
+// descriptors than the tensor core takes for its MMAs.  480000 bf16 rows to
+// 512 features with their norms: K = 64 143 -> 100 us, K = 256 147 -> 145 us
+// (768 features, K = 128: 203 -> 145 us).  Epilogues:
 //   kOutBF16 : bf16 output, optional per-row sum of squares of the rounded values
 //   kOutF32  : f32 output
 //   kOutCos  : f32 output / (|row| |column|), 0 where |row| < 1e-12
@@ -28,7 +35,8 @@ namespace scoup {
 namespace {
 
 constexpr int BM = 128, BK = 64;
-constexpr int kGemmThreads = 192;
+constexpr int kEpiWarps = 8;  // two groups of four
+constexpr int kGemmThreads = 64 + 32 * kEpiWarps;
 constexpr uint32_t kWaitIters = 1u << 22;
 
 template <int BN>
@@ -41,11 +49,13 @@ template <int BN>
 struct GemmSmem {
   alignas(1024) __nv_bfloat16 a[GemmCfg<BN>::kStages][BM * BK];
   alignas(1024) __nv_bfloat16 b[GemmCfg<BN>::kStages][BN * BK];
-  alignas(1024) unsigned char out[4][2][32 * 128];  // per epilogue warp, two 32-row x 128-byte chunks
+  alignas(1024) unsigned char out[kEpiWarps][2][32 * 128];  // per epilogue warp, two 32-row x 128-byte chunks
   uint64_t full[GemmCfg<BN>::kStages];
   uint64_t empty[GemmCfg<BN>::kStages];
   uint64_t acc_full[2];
   uint64_t acc_empty[2];
+  uint64_t part_full[4][4];  // per slot and TMEM quarter: `part` is written
+  float part[4][BM];         // half a unit's squared row norms, from one epilogue group to the other
   uint64_t drain;
   uint32_t tmem;
   volatile int abort;
@@ -58,9 +68,99 @@ __device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, vo
   return false;
 }
 
+// acc += the squares of the two bf16 values of w (one packed FP32 FMA).
+__device__ __forceinline__ void add_squares(uint32_t w, unsigned long long& acc) {
+  asm("{\n\t.reg .b32 l, h;\n\t.reg .b64 v;\n\tshl.b32 l, %1, 16;\n\tand.b32 h, %1, 0xffff0000;\n\t"
+      "mov.b64 v, {l, h};\n\tfma.rn.f32x2 %0, v, v, %0;\n\t}"
+      : "+l"(acc)
+      : "r"(w));
+}
+
 __device__ __forceinline__ uint32_t pack_bf16x2(float x, float y) {
   const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
   return *reinterpret_cast<const uint32_t*>(&h);
+}
+
+// Division by a column norm, from the norm and its reciprocal: the quotient
+// q = x (1 / norm) is corrected by its exact residual, q + (x - q norm) (1 /
+// norm) (Markstein 1990: correctly rounded from a correctly rounded
+// reciprocal).  Norms outside 2^-100 .. 2^100 have the second value 0.
+__device__ __forceinline__ float2 norm_entry(float n) {
+  return make_float2(n, n >= 0x1p-100f && n <= 0x1p100f ? 1.0f / n : 0.0f);
+}
+
+__device__ __forceinline__ float div_by_norm(float x, float n, float inv) {
+  const float q = x * inv;
+  return fabsf(q) < INFINITY ? fmaf(fmaf(-q, n, x), inv, q) : q;  // an infinite x stays so
+}
+
+// 32 columns col0 .. of a thread's row in v through the epilogue `mode` into
+// the row's 128 bytes of the staging buffer (16-byte pieces swizzled by lane;
+// hh: which half of them, a bf16 output has 64 columns there); adds the
+// rounded values' squares to ss2 where norms are wanted.
+__device__ __forceinline__ void epi_cols(const GemmEpi& ep, int mode, bool norms, bool write, float (&v)[32], int col0,
+                                         int hh, int nlim, float rinv, unsigned char* rowp, int lane,
+                                         unsigned long long (&ss2)[2]) {
+  if (mode == kOutBF16) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const uint4 w = make_uint4(pack_bf16x2(v[8 * j], v[8 * j + 1]), pack_bf16x2(v[8 * j + 2], v[8 * j + 3]),
+                                 pack_bf16x2(v[8 * j + 4], v[8 * j + 5]), pack_bf16x2(v[8 * j + 6], v[8 * j + 7]));
+      if (write) *reinterpret_cast<uint4*>(rowp + (((4 * hh + j) ^ (lane & 7)) << 4)) = w;
+      if (norms) {
+        add_squares(w.x, ss2[0]);
+        add_squares(w.y, ss2[1]);
+        add_squares(w.z, ss2[0]);
+        add_squares(w.w, ss2[1]);
+      }
+    }
+  } else {
+    if (mode == kOutCos || mode == kOutRel) {
+      // one norm load and one division per lane and chunk, passed around the
+      // warp: a load and a branchy division per column are a serial chain of
+      // several thousand cycles per row block
+      const int col = col0 + lane;
+      const float2 mine = norm_entry(col < nlim ? ep.colnorm[col] : 1.0f);
+      if (__all_sync(0xffffffffu, mine.y != 0.0f)) {
+#pragma unroll
+        for (int c = 0; c < 32; ++c) {
+          const float n = __shfl_sync(0xffffffffu, mine.x, c), inv = __shfl_sync(0xffffffffu, mine.y, c);
+          const float s = div_by_norm(v[c] * rinv, n, inv);
+          v[c] = rinv == 0.0f ? 0.0f : s;
+        }
+      } else {  // a norm of 0 or at the ends of the range: a column without a norm gives 0
+#pragma unroll
+        for (int c = 0; c < 32; ++c) {
+          const float n = __shfl_sync(0xffffffffu, mine.x, c);
+          v[c] = (rinv == 0.0f || n == 0.0f) ? 0.0f : v[c] * rinv / n;
+        }
+      }
+    }
+    if (mode == kOutRel) {
+      // Eq. 9 on the thread's whole row of similarities (at most 32
+      // columns, one column tile): R_q = min_k 1 / (1 + e^{a (s_k - s_q)})
+      // is the term of the largest canonical similarity; query q is
+      // column n_canon + q, staged at column q of the relevancy row
+      float smax = -INFINITY;
+#pragma unroll
+      for (int c = 0; c < 32; ++c)
+        if (c < ep.n_canon) smax = fmaxf(smax, v[c]);
+      float* rowf = reinterpret_cast<float*>(rowp);
+#pragma unroll
+      for (int c = 0; c < 32; ++c) {
+        const int qq = c - ep.n_canon;
+        if (qq >= 0 && c < nlim) {
+          const float r = relevancy_term(ep.alpha, smax, v[c]);
+          rowf[(((qq >> 2) ^ (lane & 7)) << 2) + (qq & 3)] = r;
+        }
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        *reinterpret_cast<float4*>(rowp + ((j ^ (lane & 7)) << 4)) =
+            make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+    }
+  }
 }
 
 // Position of a CTA's i-th unit.  Plain: units u = blockIdx.x + i gridDim.x
@@ -121,8 +221,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_kernel(const __grid
     }
     for (int b = 0; b < 2; ++b) {
       ptx::mbar_init(&sm.acc_full[b], 1);
-      ptx::mbar_init(&sm.acc_empty[b], 4);
+      ptx::mbar_init(&sm.acc_empty[b], kEpiWarps);
     }
+    for (int i = 0; i < 16; ++i) ptx::mbar_init(&sm.part_full[i >> 2][i & 3], 1);
     ptx::mbar_init(&sm.drain, 1);
     sm.abort = 0;
     ptx::fence_mbar_init();
@@ -143,8 +244,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_kernel(const __grid
   ptx::tc_fence_after();
   const uint32_t tmem = sm.tmem;
 
-  if (warp == 0 && lane == 0) {
-    // ---- TMA producer ----
+  if (warp == 0) {
+    // ---- TMA producer: the warp runs the loop together, so that addresses
+    // and coordinates stay in uniform registers, and lane 0 issues ----
     int it = 0;
     for (int i = 0; !sm.abort && !ep.stall_loads; ++i) {
       const UnitPos t = unit_at<BN, kQuery>(i, n_tiles, m_blocks);
@@ -154,9 +256,12 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_kernel(const __grid
       for (int kb = 0; kb < kt; ++kb, ++it) {
         const int s = it % kStages;
         if (it >= kStages && !wait_or_abort(&sm.empty[s], ((it / kStages) - 1) & 1, &sm.abort, ep.status)) break;
-        ptx::mbar_arrive_expect_tx(&sm.full[s], kBytesA + (t.query ? kBytesG : kBytesB));
-        ptx::tma_load_2d(sm.a[s], &tmA, &sm.full[s], kb * BK, t.m0);
-        ptx::tma_load_2d(sm.b[s], mb, &sm.full[s], kb * BK, nb);
+        if (lane == 0) {
+          ptx::mbar_arrive_expect_tx(&sm.full[s], kBytesA + (t.query ? kBytesG : kBytesB));
+          ptx::tma_load_2d(sm.a[s], &tmA, &sm.full[s], kb * BK, t.m0);
+          ptx::tma_load_2d(sm.b[s], mb, &sm.full[s], kb * BK, nb);
+        }
+        __syncwarp();
       }
     }
     // wait (bounded) for the last copy issued into each stage before leaving
@@ -164,8 +269,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_kernel(const __grid
       const int last = s + ((it - 1 - s) / kStages) * kStages;
       if (!ptx::mbar_wait_bounded(&sm.full[s], (last / kStages) & 1, kWaitIters)) atomicOr(ep.status, kStatTimeout);
     }
-  } else if (warp == 1 && lane == 0) {
-    // ---- MMA issuer ----
+  } else if (warp == 1) {
+    // ---- MMA issuer: the warp runs the loop together, so that descriptors
+    // and addresses stay in uniform registers, and lane 0 issues ----
+    const uint64_t da0 = ptx::smem_desc_k128(ptx::smem_u32(sm.a[0])), db0 = ptx::smem_desc_k128(ptx::smem_u32(sm.b[0]));
     int it = 0, local = 0;
     bool ok = true;
     for (int i = 0; ok && !sm.abort; ++i, ++local) {
@@ -183,23 +290,31 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_kernel(const __grid
           break;
         }
         ptx::tc_fence_after();
-        const uint32_t sa = ptx::smem_u32(sm.a[s]), sb = ptx::smem_u32(sm.b[s]);
+        const uint64_t da = da0 + (uint64_t)(s * (int)(kBytesA >> 4)), db = db0 + (uint64_t)(s * (int)(kBytesB >> 4));
+        if (lane == 0) {
 #pragma unroll
-        for (int k = 0; k < BK / 16; ++k)
-          ptx::mma_f16(d, ptx::smem_desc_k128(sa + k * 32), ptx::smem_desc_k128(sb + k * 32), id,
-                       (kb > 0 || k > 0) ? 1u : 0u);
-        ptx::mma_commit(&sm.empty[s]);
+          for (int k = 0; k < BK / 16; ++k) ptx::mma_f16(d, da + 2 * k, db + 2 * k, id, (kb > 0 || k > 0) ? 1u : 0u);
+          ptx::mma_commit(&sm.empty[s]);
+        }
+        __syncwarp();
       }
-      if (ok) ptx::mma_commit(&sm.acc_full[b]);
+      if (ok && lane == 0) ptx::mma_commit(&sm.acc_full[b]);
+      __syncwarp();
     }
     // every issued MMA has completed once `drain` flips
-    ptx::mma_commit(&sm.drain);
-    if (!ptx::mbar_wait_bounded(&sm.drain, 0, kWaitIters)) atomicOr(ep.status, kStatTimeout);
+    if (lane == 0) {
+      ptx::mma_commit(&sm.drain);
+      if (!ptx::mbar_wait_bounded(&sm.drain, 0, kWaitIters)) atomicOr(ep.status, kStatTimeout);
+    }
+    __syncwarp();
   } else if (warp >= 2) {
     // ---- epilogue ----
-    const int q = warp & 3;  // TMEM lane quarter this warp may access
-    constexpr int kCW = 64;  // bf16 columns per 128-byte chunk (32 for f32 output)
-    int local = 0, sbuf = 0;
+    const int q = warp & 3;               // TMEM lane quarter this warp may access
+    const int grp = (warp - 2) >> 2;      // epilogue group
+    constexpr int kCW = 64;               // bf16 columns per 128-byte chunk (32 for f32 output)
+    const int per = n_tiles + 1;          // fused query: units of a row block
+    const bool norms = fused || ep.rownorm2;
+    int local = 0, sbuf = 0, ex = 0;      // ex: units whose norms the groups have exchanged
     float ss_row = 0.0f;  // fused query: squared norm of the row's rounded outputs over its row block
     for (int i = 0; !sm.abort; ++i, ++local) {
       const UnitPos t = unit_at<BN, kQuery>(i, n_tiles, m_blocks);
@@ -213,87 +328,50 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_kernel(const __grid
       const bool write = kQuery ? (t.query || ep.store) : true;
       const CUtensorMap* mo = t.query ? &tmS : &tmO;
       const int b = local & 1, use = local >> 1;
+      // The lead group takes a unit of one chunk alone, or the first half of
+      // the chunks; it gathers the row norms.  Units of a row block with a
+      // query unit have one lead, and the groups lead by turns.
+      const int lead = (kQuery ? i / per : local) & 1;
+      const bool split = ncols > cw;
+      const int half = split ? ((ncols / cw + 1) / 2) * cw : ncols;
+      const int c_begin = grp == lead ? 0 : half, c_end = grp == lead ? half : ncols;
       if (!wait_or_abort(&sm.acc_full[b], use & 1, &sm.abort, ep.status)) break;
       ptx::tc_fence_after();
       const int row = m0 + q * 32 + lane;
       if (fused && !t.query && t.n0 == 0) ss_row = 0.0f;
       float rinv = 0.0f;
-      if ((mode == kOutCos || mode == kOutRel) && row < ep.M) {
+      if ((mode == kOutCos || mode == kOutRel) && c_begin < c_end && row < ep.M) {
         const float rn = sqrtf(t.query ? ss_row : ep.rownorm2[row]);
         rinv = rn < 1e-12f ? 0.0f : 1.0f / rn;
       }
-      float ss = 0.0f;
+      unsigned long long ss2[2] = {0ull, 0ull};
       const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * BN);
-      for (int c0 = 0; c0 < ncols; c0 += cw) {
-        float v[kCW];
-        ptx::tmem_ld32(tbase + (uint32_t)c0, *reinterpret_cast<float(*)[32]>(&v[0]));
-        if (!f32out) ptx::tmem_ld32(tbase + (uint32_t)(c0 + 32), *reinterpret_cast<float(*)[32]>(&v[32]));
-        if (c0 + cw >= ncols) {
-          // the accumulator is drained: the MMA warp may reuse it
-          ptx::tc_fence_before();
-          __syncwarp();
-          if (lane == 0) ptx::mbar_arrive(&sm.acc_empty[b]);
-        }
-        // a box that starts past the last row or column stores nothing: skip it
-        if (n0 + c0 >= nlim || m0 + q * 32 >= ep.M) continue;
-        unsigned char* buf = sm.out[q][sbuf];
-        if (write) {
+      if (c_begin >= c_end) {  // nothing to read in this unit
+        if (lane == 0) ptx::mbar_arrive(&sm.acc_empty[b]);
+      }
+      for (int c0 = c_begin; c0 < c_end; c0 += cw) {
+        unsigned char* buf = sm.out[warp - 2][sbuf];
+        unsigned char* rowp = buf + lane * 128;
+        // a box that starts past the last row or column stores nothing
+        const bool dead = n0 + c0 >= nlim || m0 + q * 32 >= ep.M;
+        if (write && !dead) {
           if (lane == 0) ptx::bulk_wait_read<1>();  // this buffer's previous store has read it
           __syncwarp();
         }
-        unsigned char* rowp = buf + lane * 128;
-        if (!f32out) {
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            uint4 w;
-            w.x = pack_bf16x2(v[8 * j + 0], v[8 * j + 1]);
-            w.y = pack_bf16x2(v[8 * j + 2], v[8 * j + 3]);
-            w.z = pack_bf16x2(v[8 * j + 4], v[8 * j + 5]);
-            w.w = pack_bf16x2(v[8 * j + 6], v[8 * j + 7]);
-            if (write) *reinterpret_cast<uint4*>(rowp + ((j ^ (lane & 7)) << 4)) = w;
-            if (ep.rownorm2 || fused) {
-              const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&w);
-#pragma unroll
-              for (int t2 = 0; t2 < 4; ++t2) {
-                const float2 f = __bfloat1622float2(h[t2]);
-                ss = fmaf(f.x, f.x, fmaf(f.y, f.y, ss));
-              }
-            }
+        for (int hh = 0; hh < 2; ++hh) {
+          if (hh * 32 >= cw) break;
+          float v[32];
+          ptx::tmem_ld32(tbase + (uint32_t)(c0 + 32 * hh), v);
+          if (c0 + 32 * (hh + 1) >= c_end) {
+            // the group's part is drained: the MMA warp may reuse the accumulator
+            ptx::tc_fence_before();
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(&sm.acc_empty[b]);
           }
-        } else {
-          if (mode == kOutCos || mode == kOutRel) {
-#pragma unroll
-            for (int c = 0; c < 32; ++c) {
-              const int col = n0 + c0 + c;
-              const float cn = col < nlim ? ep.colnorm[col] : 0.0f;
-              v[c] = (rinv == 0.0f || cn == 0.0f) ? 0.0f : v[c] * rinv / cn;
-            }
-          }
-          if (mode == kOutRel) {
-            // Eq. 9 on the thread's whole row of similarities (at most 32
-            // columns, one column tile): R_q = min_k 1 / (1 + e^{a (s_k - s_q)})
-            // is the term of the largest canonical similarity; query q is
-            // column n_canon + q, staged at column q of the relevancy row
-            float smax = -INFINITY;
-#pragma unroll
-            for (int c = 0; c < 32; ++c)
-              if (c < ep.n_canon) smax = fmaxf(smax, v[c]);
-            float* rowf = reinterpret_cast<float*>(rowp);
-#pragma unroll
-            for (int c = 0; c < 32; ++c) {
-              const int qq = c - ep.n_canon;
-              if (qq >= 0 && c < nlim) {
-                const float r = relevancy_term(ep.alpha, smax, v[c]);
-                rowf[(((qq >> 2) ^ (lane & 7)) << 2) + (qq & 3)] = r;
-              }
-            }
-          } else {
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-              *reinterpret_cast<float4*>(rowp + ((j ^ (lane & 7)) << 4)) =
-                  make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-          }
+          if (!dead) epi_cols(ep, mode, norms, write, v, n0 + c0 + 32 * hh, hh, nlim, rinv, rowp, lane, ss2);
         }
+        if (dead) continue;
         if (!write) continue;
         ptx::fence_async_shared();
         __syncwarp();
@@ -303,12 +381,30 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_kernel(const __grid
         }
         sbuf ^= 1;
       }
-      if (fused) {
-        if (!t.query) ss_row += ss;
-        else if (ep.rownorm2 && row < ep.M) ep.rownorm2[row] = ss_row;
-      } else if (!f32out && ep.rownorm2 && row < ep.M) {
-        atomicAdd(&ep.rownorm2[row], ss);
+      if (norms && !f32out) {
+        const float2 s0 = *reinterpret_cast<const float2*>(&ss2[0]), s1 = *reinterpret_cast<const float2*>(&ss2[1]);
+        float ss = (s0.x + s1.x) + (s0.y + s1.y);
+        if (split) {
+          // four slots: a slot is written again four units on, and that unit's
+          // MMAs wait for both groups to have left the unit before last
+          uint64_t* const bar = &sm.part_full[ex & 3][q];
+          float* const part = &sm.part[ex & 3][q * 32 + lane];
+          if (grp != lead) {
+            *part = ss;
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(bar);
+          } else {
+            if (!wait_or_abort(bar, (ex >> 2) & 1, &sm.abort, ep.status)) break;
+            ss += *part;
+          }
+          ++ex;
+        }
+        if (fused)
+          ss_row += ss;
+        else if (row < ep.M && grp == lead)
+          atomicAdd(&ep.rownorm2[row], ss);
       }
+      if (fused && t.query && grp == lead && ep.rownorm2 && row < ep.M) ep.rownorm2[row] = ss_row;
     }
     if (lane == 0) ptx::bulk_wait<0>();  // stores complete before the CTA leaves
     __syncwarp();
@@ -318,6 +414,365 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_kernel(const __grid
   if (warp == 1) {
     ptx::tc_fence_after();
     ptx::tmem_dealloc(tmem, Cfg::kTmemCols);
+  }
+}
+
+// ---- rows kept in shared memory (K <= 256) ----
+//
+// out = A Bt^T as above for the decode's shapes: many rows, K <= 256.  A CTA
+// takes a block of rows at a time: its A (up to 4 slabs of 64 columns) stays
+// in shared memory while the column tiles of 128 stream past it, where the
+// kernel above loads A again for every column unit.  What bounds both is the
+// ring of loads in front of the MMAs: a stage comes back about 1.8 us after
+// it was freed, so the bytes per row block over the bytes in flight count.
+//   bf16 A: 256 rows to a block (every Bt tile serves two MMAs), epilogue
+//     group g owns row half g over all columns.  All 128 KB of A are in use,
+//     so a slab is refilled as soon as the block's last unit has read it; the
+//     next block is fetched into L2 ahead.  The query unit goes first and
+//     waits as 32 registers per row, so that its MMAs do not stand between
+//     the last column tile and the refill.
+//   FP32 A: six more warps round the values to bf16 on the way in, in place of
+//     a conversion pass over memory.  128 rows to a block and 6 slots, so that
+//     the next block is converted under this one's MMAs; the epilogue groups
+//     split the columns and pass the row norms on in shared memory.
+// 2073600 x 256 -> 512 and 32 phrases: bf16 880 -> 645 us, FP32 1514 -> 1011
+// us; FP32 without the phrases 1127 -> 753 us, of which 625 are the bytes.
+constexpr int RN = 128;
+constexpr int kMaxSlabs = 4;
+constexpr int kCvtWarps = 6;  // two teams that take the slabs by turns
+
+template <bool kF32A>
+struct RowsCfg {
+  static constexpr int kHalves = kF32A ? 1 : 2;         // 128-row halves of a block
+  static constexpr int kRows = kHalves * BM;
+  static constexpr int kASlots = kF32A ? 6 : kMaxSlabs;
+  static constexpr int kBStages = kF32A ? 6 : 4;
+  static constexpr int kAcc = 4 / kHalves;              // accumulators of kHalves x RN TMEM columns
+  static constexpr int kThreads = 64 + 32 * kEpiWarps + (kF32A ? 32 * kCvtWarps : 0);
+};
+constexpr int kParts = 3;
+
+template <bool kF32A>
+struct RowsSmem {
+  using Cfg = RowsCfg<kF32A>;
+  alignas(1024) __nv_bfloat16 a[Cfg::kASlots][Cfg::kHalves][BM * BK];
+  alignas(1024) __nv_bfloat16 b[Cfg::kBStages][RN * BK];
+  alignas(1024) unsigned char out[kEpiWarps][32 * 128];
+  float part[kF32A ? kParts : 1][BM];  // squared row norms over the other group's columns, for the lead group
+  uint64_t part_full[kParts][4];       // per slot and TMEM quarter: `part` is written
+  uint64_t a_full[Cfg::kASlots];
+  uint64_t a_empty[Cfg::kASlots];
+  uint64_t b_full[Cfg::kBStages];
+  uint64_t b_empty[Cfg::kBStages];
+  uint64_t acc_full[Cfg::kAcc];
+  uint64_t acc_empty[Cfg::kAcc];
+  uint64_t drain;
+  uint32_t tmem;
+  volatile int abort;
+};
+static_assert(sizeof(RowsSmem<false>) + 1024 <= 227 * 1024, "shared memory of one CTA");
+static_assert(sizeof(RowsSmem<true>) + 1024 <= 227 * 1024, "shared memory of one CTA");
+
+template <bool kQuery, bool kF32A>
+__global__ void __launch_bounds__(RowsCfg<kF32A>::kThreads, 1)
+    gemm_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                     const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUtensorMap tmG,
+                     const __grid_constant__ CUtensorMap tmS, const float* __restrict__ a32, GemmEpi ep) {
+  using Cfg = RowsCfg<kF32A>;
+  constexpr int kH = Cfg::kHalves, kRows = Cfg::kRows, kASlots = Cfg::kASlots, kBStages = Cfg::kBStages;
+  constexpr int kAcc = Cfg::kAcc;
+  extern __shared__ __align__(1024) unsigned char gsm_raw[];
+  unsigned char* base = gsm_raw + ((1024 - (ptx::smem_u32(gsm_raw) & 1023u)) & 1023u);
+  RowsSmem<kF32A>& sm = *reinterpret_cast<RowsSmem<kF32A>*>(base);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int kt = (ep.K + BK - 1) / BK;  // slabs, at most kMaxSlabs
+  const int n_tiles = (ep.N + RN - 1) / RN, per = n_tiles + (kQuery ? 1 : 0);
+  constexpr int kU0 = kQuery ? 1 : 0;   // unit of column tile 0: the query unit is unit 0
+  const int blocks = (ep.M - 1) / kRows + 1;
+  constexpr uint32_t kBytesA = kRows * BK * 2, kBytesB = RN * BK * 2;
+  const uint32_t kBytesG = (uint32_t)ep.sim_n * BK * 2;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kASlots; ++s) {
+      ptx::mbar_init(&sm.a_full[s], kF32A ? 32 * kCvtWarps / 2 : 1);
+      ptx::mbar_init(&sm.a_empty[s], 1);
+    }
+    for (int s = 0; s < kBStages; ++s) {
+      ptx::mbar_init(&sm.b_full[s], 1);
+      ptx::mbar_init(&sm.b_empty[s], 1);
+    }
+    for (int b = 0; b < kAcc; ++b) {
+      ptx::mbar_init(&sm.acc_full[b], 1);
+      ptx::mbar_init(&sm.acc_empty[b], kEpiWarps);
+    }
+    for (int i = 0; i < 4 * kParts; ++i) ptx::mbar_init(&sm.part_full[i >> 2][i & 3], 1);
+    ptx::mbar_init(&sm.drain, 1);
+    sm.abort = 0;
+    ptx::fence_mbar_init();
+    if (!kF32A) ptx::prefetch_tmap(&tmA);
+    ptx::prefetch_tmap(&tmB);
+    ptx::prefetch_tmap(&tmO);
+    if (kQuery) {
+      ptx::prefetch_tmap(&tmG);
+      ptx::prefetch_tmap(&tmS);
+    }
+  }
+  if (warp == 1) {
+    ptx::tmem_alloc(&sm.tmem, kAcc * kH * RN);
+    ptx::tmem_relinquish();
+  }
+  ptx::tc_fence_before();
+  __syncthreads();
+  ptx::tc_fence_after();
+  const uint32_t tmem = sm.tmem;
+
+  if (warp == 0) {
+    // ---- TMA producer (see above): the units of every row block, a slab of A
+    // ahead of the first unit that needs it ----
+    int ia = 0, it = 0;
+    bool ok = true;
+    for (int rb = blockIdx.x; ok && rb < blocks && !sm.abort; rb += (int)gridDim.x) {
+      const int m0 = rb * kRows, next = rb + (int)gridDim.x;
+      for (int u = 0; ok && u < per; ++u) {
+        const bool query = kQuery && u == 0;
+        for (int kb = 0; kb < kt; ++kb, ++it) {
+          if (!kF32A && u == 0) {
+            const int s = ia % kASlots;
+            if (ia >= kASlots && !wait_or_abort(&sm.a_empty[s], ((ia / kASlots) - 1) & 1, &sm.abort, ep.status)) {
+              ok = false;
+              break;
+            }
+            if (lane == 0) {
+              ptx::mbar_arrive_expect_tx(&sm.a_full[s], kBytesA);
+              for (int h = 0; h < kH; ++h) ptx::tma_load_2d(sm.a[s][h], &tmA, &sm.a_full[s], kb * BK, m0 + h * BM);
+            }
+            __syncwarp();
+            ++ia;
+          }
+          const int s = it % kBStages;
+          if (it >= kBStages && !wait_or_abort(&sm.b_empty[s], ((it / kBStages) - 1) & 1, &sm.abort, ep.status)) {
+            ok = false;
+            break;
+          }
+          if (lane == 0) {
+            ptx::mbar_arrive_expect_tx(&sm.b_full[s], query ? kBytesG : kBytesB);
+            ptx::tma_load_2d(sm.b[s], query ? &tmG : &tmB, &sm.b_full[s], kb * BK, query ? 0 : (u - kU0) * RN);
+          }
+          __syncwarp();
+        }
+        if (!kF32A && lane == 0 && u == 0 && next < blocks)
+          for (int kb = 0; kb < kt; ++kb)
+            for (int h = 0; h < kH; ++h)
+              if (next * kRows + h * BM < ep.M) ptx::tma_prefetch_2d(&tmA, kb * BK, next * kRows + h * BM);
+      }
+    }
+    // wait (bounded) for the last copy issued into each slot before leaving
+    for (int s = 0; s < kBStages && s < it; ++s) {
+      const int last = s + ((it - 1 - s) / kBStages) * kBStages;
+      if (!ptx::mbar_wait_bounded(&sm.b_full[s], (last / kBStages) & 1, kWaitIters)) atomicOr(ep.status, kStatTimeout);
+    }
+    for (int s = 0; s < kASlots && s < ia; ++s) {
+      const int last = s + ((ia - 1 - s) / kASlots) * kASlots;
+      if (!ptx::mbar_wait_bounded(&sm.a_full[s], (last / kASlots) & 1, kWaitIters)) atomicOr(ep.status, kStatTimeout);
+    }
+  } else if (warp == 1) {
+    // ---- MMA issuer (see above) ----
+    constexpr uint32_t idesc = ptx::idesc_bf16_f32(BM, RN);
+    const uint32_t idesc_q = ep.sim_n == 16 ? ptx::idesc_bf16_f32(BM, 16) : ptx::idesc_bf16_f32(BM, 32);
+    const uint64_t da0 = ptx::smem_desc_k128(ptx::smem_u32(sm.a[0][0])), db0 = ptx::smem_desc_k128(ptx::smem_u32(sm.b[0]));
+    int ia = 0, it = 0, local = 0;
+    bool ok = true;
+    for (int rb = blockIdx.x; ok && rb < blocks && !sm.abort; rb += (int)gridDim.x, ia += kt) {
+      for (int u = 0; ok && u < per; ++u, ++local) {
+        const uint32_t id = kQuery && u == 0 ? idesc_q : idesc;
+        const int b = local % kAcc, use = local / kAcc;
+        if (local >= kAcc && !wait_or_abort(&sm.acc_empty[b], (use - 1) & 1, &sm.abort, ep.status)) {
+          ok = false;
+          break;
+        }
+        ptx::tc_fence_after();
+        const uint32_t d = tmem + (uint32_t)(b * kH * RN);
+        for (int kb = 0; kb < kt; ++kb, ++it) {
+          const int sa = (ia + kb) % kASlots, s = it % kBStages;
+          if ((u == 0 && !wait_or_abort(&sm.a_full[sa], ((ia + kb) / kASlots) & 1, &sm.abort, ep.status)) ||
+              !wait_or_abort(&sm.b_full[s], (it / kBStages) & 1, &sm.abort, ep.status)) {
+            ok = false;
+            break;
+          }
+          ptx::tc_fence_after();
+          const uint64_t da = da0 + (uint64_t)(sa * (int)(kBytesA >> 4)), db = db0 + (uint64_t)(s * (int)(kBytesB >> 4));
+          if (lane == 0) {
+#pragma unroll
+            for (int h = 0; h < kH; ++h)
+#pragma unroll
+              for (int k = 0; k < BK / 16; ++k)
+                ptx::mma_f16(d + (uint32_t)(h * RN), da + h * (BM * BK * 2 >> 4) + 2 * k, db + 2 * k, id,
+                             (kb > 0 || k > 0) ? 1u : 0u);
+            ptx::mma_commit(&sm.b_empty[s]);
+            if (u == per - 1) ptx::mma_commit(&sm.a_empty[sa]);
+          }
+          __syncwarp();
+        }
+        if (ok && lane == 0) ptx::mma_commit(&sm.acc_full[b]);
+        __syncwarp();
+      }
+    }
+    // every issued MMA has completed once `drain` flips
+    if (lane == 0) {
+      ptx::mma_commit(&sm.drain);
+      if (!ptx::mbar_wait_bounded(&sm.drain, 0, kWaitIters)) atomicOr(ep.status, kStatTimeout);
+    }
+    __syncwarp();
+  } else if (warp >= 2 && warp < 2 + kEpiWarps) {
+    // ---- epilogue ----
+    const int q = warp & 3, grp = (warp - 2) >> 2;  // TMEM lane quarter; epilogue group
+    const bool norms = kQuery || ep.rownorm2;
+    unsigned char* const buf = sm.out[warp - 2];
+    unsigned char* const rowp = buf + lane * 128;
+    int local = 0;
+    bool ok = true;
+    for (int rb = blockIdx.x, j = 0; ok && rb < blocks && !sm.abort; rb += (int)gridDim.x, ++j) {
+      // one half to a block: the lead group takes the first half of each
+      // column tile, gathers the row norms and does the query unit; the groups
+      // lead by turns.  Two halves: each group leads its own rows.
+      const bool lead = kH == 2 || grp == (j & 1);
+      const int r0 = rb * kRows + (kH == 2 ? grp * BM : 0) + q * 32, row = r0 + lane;
+      const bool live = r0 < ep.M;
+      const int c_begin = lead ? 0 : RN / 2, c_end = kH == 2 || !lead ? RN : RN / 2;
+      unsigned long long ss2[2] = {0ull, 0ull};  // squared norm of the thread's rounded outputs
+      float dots[32];                            // the query unit's sums
+      for (int u = 0; u < per; ++u, ++local) {
+        const int b = local % kAcc, use = local / kAcc;
+        if (!wait_or_abort(&sm.acc_full[b], use & 1, &sm.abort, ep.status)) {
+          ok = false;
+          break;
+        }
+        ptx::tc_fence_after();
+        const uint32_t taddr =
+            tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * kH * RN + (kH == 2 ? grp * RN : 0));
+        if (kQuery && u == 0) {
+          if (lead) ptx::tmem_ld32(taddr, dots);
+          ptx::tc_fence_before();
+          __syncwarp();
+          if (lane == 0) ptx::mbar_arrive(&sm.acc_empty[b]);
+          continue;
+        }
+        const int n0 = (u - kU0) * RN;
+        const bool bf16 = ep.mode == kOutBF16, write = !kQuery || ep.store;
+        const int cw = bf16 ? 64 : 32;  // columns of a 128-byte chunk
+        for (int c0 = c_begin; c0 < c_end; c0 += cw) {
+          const bool dead = n0 + c0 >= ep.N || !live;  // a box that starts past the last row or column
+          if (write && !dead) {
+            if (lane == 0) ptx::bulk_wait_read<0>();  // the previous store has read the buffer
+            __syncwarp();
+          }
+#pragma unroll
+          for (int hh = 0; hh < 2; ++hh) {
+            if (hh * 32 >= cw) break;
+            float v[32];
+            ptx::tmem_ld32(taddr + (uint32_t)(c0 + 32 * hh), v);
+            if (c0 + 32 * (hh + 1) >= c_end) {
+              // this warp's part is drained: the MMA warp may reuse the accumulator
+              ptx::tc_fence_before();
+              __syncwarp();
+              if (lane == 0) ptx::mbar_arrive(&sm.acc_empty[b]);
+            }
+            if (!dead) epi_cols(ep, ep.mode, norms, write, v, n0 + c0 + 32 * hh, hh, ep.N, 0.0f, rowp, lane, ss2);
+          }
+          if (dead || !write) continue;
+          ptx::fence_async_shared();
+          __syncwarp();
+          if (lane == 0) {
+            ptx::tma_store_2d(&tmO, buf, n0 + c0, r0);
+            ptx::bulk_commit();
+          }
+        }
+      }
+      if (!ok || !norms) continue;
+      const float2 s0 = *reinterpret_cast<const float2*>(&ss2[0]), s1 = *reinterpret_cast<const float2*>(&ss2[1]);
+      float ss = (s0.x + s1.x) + (s0.y + s1.y);
+      if constexpr (kH == 1) {
+        // a unit's MMAs wait until both groups have left the unit before the
+        // one kAcc back; with at least two units to a block (N > 128) that is
+        // past the block kParts back, whose slot is written again here
+        uint64_t* const bar = &sm.part_full[j % kParts][q];
+        float* const part = &sm.part[j % kParts][q * 32 + lane];
+        if (!lead) {
+          *part = ss;
+          __syncwarp();
+          if (lane == 0) ptx::mbar_arrive(bar);
+          continue;
+        }
+        if (!wait_or_abort(bar, (j / kParts) & 1, &sm.abort, ep.status)) {
+          ok = false;
+          continue;
+        }
+        ss += *part;
+      }
+      if (ep.rownorm2 && row < ep.M) ep.rownorm2[row] = ss;
+      if (kQuery && live) {
+        const float rn = sqrtf(ss);
+        if (lane == 0) ptx::bulk_wait_read<0>();
+        __syncwarp();
+        epi_cols(ep, ep.sim_mode, false, true, dots, 0, 0, ep.sim_n, rn < 1e-12f ? 0.0f : 1.0f / rn, rowp, lane, ss2);
+        ptx::fence_async_shared();
+        __syncwarp();
+        if (lane == 0) {
+          ptx::tma_store_2d(&tmS, buf, 0, r0);
+          ptx::bulk_commit();
+        }
+      }
+    }
+    if (lane == 0) ptx::bulk_wait<0>();  // stores complete before the CTA leaves
+    __syncwarp();
+  } else if (kF32A && warp >= 2 + kEpiWarps) {
+    // ---- converters: FP32 rows to swizzled bf16 slabs ----
+    // Two teams of three warps take the slabs by turns.  16 threads read 64
+    // columns of a row (256 bytes), a thread's rows of the slab all in flight;
+    // every thread writes 8 bytes of a row's 128-byte swizzle line.
+    constexpr int kTeam = 32 * kCvtWarps / 2, kRowsPer = kTeam / 16, kBatch = (BM + kRowsPer - 1) / kRowsPer;
+    const int t = threadIdx.x - 32 * (2 + kEpiWarps), team = t / kTeam, rt = (t % kTeam) >> 4, ct = (t & 15) * 4;
+    int ia = 0;
+    bool ok = true;
+    for (int rb = blockIdx.x; ok && rb < blocks && !sm.abort; rb += (int)gridDim.x) {
+      const int m0 = rb * kRows, next = rb + (int)gridDim.x;
+      if (t == 0 && next < blocks) {
+        const int rows = min(kRows, ep.M - next * kRows);
+        ptx::bulk_prefetch_l2(a32 + (int64_t)next * kRows * ep.K, (uint32_t)rows * (uint32_t)ep.K * 4u);
+      }
+      for (int kb = 0; kb < kt; ++kb, ++ia) {
+        if ((ia & 1) != team) continue;
+        const int s = ia % kASlots, col = kb * BK + ct;
+        float4 x[kBatch];
+#pragma unroll
+        for (int i = 0; i < kBatch; ++i) {
+          const int r = i * kRowsPer + rt;
+          x[i] = r < BM && m0 + r < ep.M && col < ep.K
+                     ? __ldcs(reinterpret_cast<const float4*>(a32 + (int64_t)(m0 + r) * ep.K + col))
+                     : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        }
+        if (ia >= kASlots && !wait_or_abort(&sm.a_empty[s], ((ia / kASlots) - 1) & 1, &sm.abort, ep.status)) {
+          ok = false;
+          break;
+        }
+#pragma unroll
+        for (int i = 0; i < kBatch; ++i) {
+          const int r = i * kRowsPer + rt;
+          unsigned char* line = reinterpret_cast<unsigned char*>(sm.a[s][0]) + r * 128;
+          if (r < BM)
+            *reinterpret_cast<uint2*>(line + ((((ct >> 3) ^ (r & 7)) << 4) | ((ct & 4) << 1))) =
+                make_uint2(pack_bf16x2(x[i].x, x[i].y), pack_bf16x2(x[i].z, x[i].w));
+        }
+        ptx::fence_async_shared();  // the slab is read by the tensor core (async proxy)
+        ptx::mbar_arrive(&sm.a_full[s]);
+      }
+    }
+  }
+  ptx::tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    ptx::tc_fence_after();
+    ptx::tmem_dealloc(tmem, kAcc * kH * RN);
   }
 }
 
@@ -396,6 +851,29 @@ cudaError_t launch_bn(const void* A, const void* Bt, const void* Gt, const GemmE
   return cudaGetLastError();
 }
 
+template <bool kQuery, bool kF32A>
+cudaError_t launch_rows(const void* A, const void* Bt, const void* Gt, const GemmEpi& ep, cudaStream_t st) {
+  CUtensorMap ta, tb, to, tg, ts;
+  if (!make_tmap(&tb, Bt, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, ep.N, ep.K, BK, RN)) return cudaErrorInvalidValue;
+  ta = to = tg = ts = tb;  // a map that is never used is still valid
+  if (!kF32A && !make_tmap(&ta, A, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, ep.M, ep.K, BK, BM)) return cudaErrorInvalidValue;
+  if (ep.store &&
+      !(ep.mode == kOutF32 ? make_tmap(&to, ep.out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, ep.M, ep.ldo, 32, 32)
+                           : make_tmap(&to, ep.out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, ep.M, ep.ldo, 64, 32)))
+    return cudaErrorInvalidValue;
+  if (kQuery && (!make_tmap(&tg, Gt, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, ep.sim_n, ep.K, BK, ep.sim_n) ||
+                 !make_tmap(&ts, ep.sim_out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, ep.M, ep.sim_ldo, 32, 32)))
+    return cudaErrorInvalidValue;
+  const size_t smem = sizeof(RowsSmem<kF32A>) + 1024;
+  auto kern = gemm_rows_kernel<kQuery, kF32A>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  const int blocks = (ep.M - 1) / RowsCfg<kF32A>::kRows + 1, grid = blocks < num_sms() ? blocks : num_sms();
+  kern<<<grid, RowsCfg<kF32A>::kThreads, smem, st>>>(ta, tb, to, tg, ts, (const float*)A, ep);
+  g_launches += 1;
+  return cudaGetLastError();
+}
+
 // ---- small conversion kernels ----
 __global__ void f32_to_bf16_kernel(const float* __restrict__ x, __nv_bfloat16* __restrict__ y, int64_t n) {
   for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * 4; i < n; i += (int64_t)gridDim.x * blockDim.x * 4) {
@@ -442,8 +920,29 @@ int blocks_for(int64_t n, int per) {
 
 }  // namespace
 
+// FP32 rows.  Up to K = 128 the rows kernel is the faster one from the smallest
+// call on (us, against conversion and GEMM: 100 x 64 -> 512 16 / 18, 20000 x
+// 128 -> 256 20 / 22, 480000 x 128 -> 768 174 / 219).  Above that a call of a
+// few waves spreads better over the other kernel's units (40000 x 256 -> 768
+// 49 / 43, 78000 x 256 -> 512 53 / 59, 480000 x 256 -> 512 194 / 274).
+bool gemm_takes_f32(int64_t M, int N, int K) {
+  return N > RN && (K <= 2 * BK || (K <= kMaxSlabs * BK && M >= (int64_t)4 * BM * num_sms()));
+}
+
+// bf16 rows with the query unit: from four waves of 256 rows on (K = 256, N =
+// 512, us: 78000 rows 59 / 57, 150000 75 / 80, 480000 178 / 198, 2073600 645 /
+// 770; K = 64, 480000 rows 124 / 137).  Without it the column units of the
+// other kernel are as fast (480000 rows 143 / 141) and need no whole blocks.
+static bool query_takes_rows(int64_t M, int N, int K) {
+  return N > RN && K <= kMaxSlabs * BK && M >= (int64_t)4 * 2 * BM * num_sms();
+}
+
 cudaError_t launch_gemm_bf16(const void* A, const void* Bt, const GemmEpi& ep, cudaStream_t st) {
   if (ep.M <= 0 || ep.N <= 0) return cudaSuccess;
+  if (ep.a_f32)
+    return !ep.sim_n && (ep.mode == kOutBF16 || ep.mode == kOutF32) && gemm_takes_f32(ep.M, ep.N, ep.K)
+               ? launch_rows<false, true>(A, Bt, nullptr, ep, st)
+               : cudaErrorInvalidValue;
   // bf16 output is read back from TMEM 64 columns at a time: BN >= 64 (the
   // columns past N are the zero fill of the Bt tile)
   if (ep.sim_n) return cudaErrorInvalidValue;  // launch_gemm_bf16_query
@@ -459,6 +958,9 @@ cudaError_t launch_gemm_bf16_query(const void* A, const void* Bt, const void* Gt
   if (ep.mode != kOutBF16 || (ep.sim_n != 16 && ep.sim_n != 32) || !Gt || !ep.sim_out ||
       (ep.sim_mode != kOutCos && ep.sim_mode != kOutRel) || (ep.store && !ep.out))
     return cudaErrorInvalidValue;
+  if (ep.a_f32)
+    return gemm_takes_f32(ep.M, ep.N, ep.K) ? launch_rows<true, true>(A, Bt, Gt, ep, st) : cudaErrorInvalidValue;
+  if (query_takes_rows(ep.M, ep.N, ep.K)) return launch_rows<true, false>(A, Bt, Gt, ep, st);
   if (ep.N <= 64) return launch_bn<64>(A, Bt, Gt, ep, st);
   if (ep.N <= 128) return launch_bn<128>(A, Bt, Gt, ep, st);
   return launch_bn<256>(A, Bt, Gt, ep, st);

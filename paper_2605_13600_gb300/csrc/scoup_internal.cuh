@@ -446,9 +446,13 @@ struct GemmEpi {
   int sim_mode = 0;
   void* sim_out = nullptr;
   int64_t sim_ldo = 0;
+  int a_f32 = 0;  // A holds FP32 values, rounded to bf16 on the way in (only where gemm_takes_f32())
   int store = 1;  // 0: the kOutBF16 rows are not written (their norms and the fused unit still are)
 };
 cudaError_t launch_gemm_bf16(const void* A, const void* Bt, const GemmEpi& ep, cudaStream_t st);
+// Whether a launch of these sizes (kOutBF16, kOutF32 or a fused query) takes
+// FP32 rows of A (ep.a_f32).
+bool gemm_takes_f32(int64_t M, int N, int K);
 // launch_gemm_bf16 with the fused query unit (ep.sim_n > 0; Gt bf16 [sim_n, K]).
 cudaError_t launch_gemm_bf16_query(const void* A, const void* Bt, const void* Gt, const GemmEpi& ep,
                                    cudaStream_t st);
