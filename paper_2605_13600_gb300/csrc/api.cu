@@ -177,10 +177,16 @@ size_t carve_view_part(void* base, int64_t n, int max_tiles, UpliftWs* w) {
   return off;
 }
 
-// From 64k Gaussians on the shorter lists pay for the cut's four small launches
-// (figures at launch_depth_cut); a cut belongs to a block's list.
-bool use_depth_cut(int64_t n, const CamArgs& cam, const UpliftWs& ws) {
-  return ws.zcut && n > 63488 && list_shift(n, cam.gx, cam.gy) == 1;
+// The cut's launches (three before the projection, five for the tiles still
+// open) pay where a chunk of views shares them and the lists are long (uplift
+// of 24 views in chunks of 8, 988x731, ms without / with: 70k Gaussians 3.17 /
+// 3.27, 300k 4.11 / 4.01 in blobs and 3.85 / 3.87 uniform, 1M 5.83 / 5.06 and
+// 6.29 / 5.71).  One view at a time they do not (uplift of 1M, 800x600: 517 /
+// 559 us), and a render, which cannot resume a tile, would start it again
+// (1M Gaussians, 1080p 1923 / 1949 us, 800x600 745 / 809).  A cut belongs to
+// a block's list.
+bool use_depth_cut(int64_t n, const CamArgs& cam, const UpliftWs& ws, int views) {
+  return ws.zcut && views > 1 && n >= (1 << 18) && list_shift(n, cam.gx, cam.gy) == 1;
 }
 
 ViewJob view_job(const scoup_scene& sc, const CamArgs& cam, const UpliftWs& ws, WsHeader* hdr, bool cut) {
@@ -422,7 +428,7 @@ static int uplift_views(const UpliftCall& c, const scoup_level* lv, int L, const
       const int v = v0 + k;
       const UpliftWs& w = parts[lane * chunk + k];
       const CamArgs cam = cam_args(c.cams[v]);
-      views[k] = view_job(*c.scene, cam, w, w.vhdr, use_depth_cut(c.scene->n, cam, w));
+      views[k] = view_job(*c.scene, cam, w, w.vhdr, use_depth_cut(c.scene->n, cam, w, nv));
       LevelCodes lc = LevelCodes();
       lc.L = L;
       for (int l = 0; l < L; ++l) {
@@ -653,7 +659,7 @@ int run_chunk(const ViewJob* views, const TileJob* jobs, int nv, uint32_t* ctr, 
     // the tiles still open behind their cut (all of these leave at once when there is none)
     {
       PhaseScope ps(SCOUP_PHASE_BINNING, cs.ls);
-      if ((e = launch_recover(views, nv, false, cs.ls)) != cudaSuccess ||
+      if ((e = launch_recover(views, nv, cs.ls)) != cudaSuccess ||
           (e = launch_binning(views, nv, true, ctr + 1, cs.ls)) != cudaSuccess)
         return cuda_fail(e, "second binning");
     }
@@ -831,21 +837,10 @@ static int bin_view(const scoup_scene& scene, const ViewJob& view, const UpliftW
   }
   if (view.n > 0) {
     PhaseScope ps(SCOUP_PHASE_PREPROCESS, st);
-    if ((e = launch_depth_cut(&view, 1, st)) != cudaSuccess || (e = launch_project(&view, 1, st)) != cudaSuccess)
-      return cuda_fail(e, "projection");
+    if ((e = launch_project(&view, 1, st)) != cudaSuccess) return cuda_fail(e, "projection");
   }
   PhaseScope ps(SCOUP_PHASE_BINNING, st);
   if ((e = launch_binning(&view, 1, false, nullptr, st)) != cudaSuccess) return cuda_fail(e, "binning");
-  return SCOUP_OK;
-}
-
-// The whole lists of the tiles that the first pass recorded as open.
-static int rebin_view(const ViewJob& view, cudaStream_t st) {
-  PhaseScope ps(SCOUP_PHASE_BINNING, st);
-  cudaError_t e;
-  if ((e = launch_recover(&view, 1, true, st)) != cudaSuccess ||
-      (e = launch_binning(&view, 1, true, nullptr, st)) != cudaSuccess)
-    return cuda_fail(e, "second binning");
   return SCOUP_OK;
 }
 
@@ -875,12 +870,11 @@ int scoup_render(const scoup_scene* scene, const int32_t* topk_idx, const float*
   const CamArgs ca = cam_args(*cam);
   cudaError_t e;
   if ((e = launch_begin(ws, true, max_tiles, st)) != cudaSuccess) return cuda_fail(e, "begin");
-  const ViewJob view = view_job(*scene, ca, ws, ws.hdr, use_depth_cut(n, ca, ws));
+  const ViewJob view = view_job(*scene, ca, ws, ws.hdr, false);
   if ((rc = bin_view(*scene, view, ws, st)) != SCOUP_OK) return rc;
-  for (int pass = 0; pass < (view.hist ? 2 : 1); ++pass) {
-    if (pass > 0 && (rc = rebin_view(view, st)) != SCOUP_OK) return rc;
+  {
     PhaseScope ps(SCOUP_PHASE_RENDER, st);
-    if ((e = launch_render_tiles(view, pass > 0, topk_idx, topk_val, K, C, out_codes, out_dtype, out_T, out_last, st)) !=
+    if ((e = launch_render_tiles(view, topk_idx, topk_val, K, C, out_codes, out_dtype, out_T, out_last, st)) !=
         cudaSuccess)
       return cuda_fail(e, "render tiles");
   }
@@ -915,12 +909,11 @@ int scoup_render_backward(const scoup_scene* scene, const int32_t* topk_idx, con
   const CamArgs ca = cam_args(*cam);
   cudaError_t e;
   if ((e = launch_begin(ws, true, max_tiles, st)) != cudaSuccess) return cuda_fail(e, "begin");
-  const ViewJob view = view_job(*scene, ca, ws, ws.hdr, use_depth_cut(n, ca, ws));
+  const ViewJob view = view_job(*scene, ca, ws, ws.hdr, false);
   if ((rc = bin_view(*scene, view, ws, st)) != SCOUP_OK) return rc;
-  for (int pass = 0; pass < (view.hist ? 2 : 1); ++pass) {
-    if (pass > 0 && (rc = rebin_view(view, st)) != SCOUP_OK) return rc;
+  {
     PhaseScope ps(SCOUP_PHASE_RENDER_BWD, st);
-    if ((e = launch_render_bwd(view, pass > 0, topk_idx, topk_val, K, C, dL_dcodes, d_topk_val, d_opacity, st)) !=
+    if ((e = launch_render_bwd(view, topk_idx, topk_val, K, C, dL_dcodes, d_topk_val, d_opacity, st)) !=
         cudaSuccess)
       return cuda_fail(e, "render backward");
   }

@@ -220,7 +220,7 @@ int drain_prepare(DrainLayout* d, const std::vector<scoup_batch_item>& items, co
       UpliftWs w = d->view[(c % lanes) * chunk + (j - c * chunk)];
       w.sp = d->scene[b].sp;
       const CamArgs cam = camera_args(it.cams[v]);
-      d->views[j] = view_job(it.scene, cam, w, w.vhdr, use_depth_cut(it.scene.n, cam, w));
+      d->views[j] = view_job(it.scene, cam, w, w.vhdr, use_depth_cut(it.scene.n, cam, w, std::min(chunk, njobs - c * chunk)));
       d->views[j].group = bin_group(n_max);  // the part's run offsets are laid out for this group size
       const bool filtered = d->fci[b] != nullptr;
       LevelCodes lc = LevelCodes();

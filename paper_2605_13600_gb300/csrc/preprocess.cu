@@ -299,12 +299,12 @@ __global__ void __launch_bounds__(256) cut_depth_kernel(const __grid_constant__ 
 }
 
 // Second pass: the kept bit of every Gaussian that reaches a block with a tile
-// recorded as open, behind its cut (restart: at any depth), and its record, which
-// the first pass stored only for the Gaussians it kept.  A CTA tests 1024
+// recorded as open, behind its cut, and its record, which the first pass stored
+// only for the Gaussians it kept.  A CTA tests 1024
 // Gaussians (four per thread, their loads in flight together), lists the few
 // that pass and projects the list, so that the projection runs in full warps.
 constexpr int kRecover = 1024;
-template <int N, bool kRestart>
+template <int N>
 __global__ void __launch_bounds__(256) recover_kernel(const __grid_constant__ ViewArgs<N> args) {
   const ViewJob& v = args.v[N == 1 ? 0 : blockIdx.y];
   if (v.hdr->open_tiles == 0u) return;
@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(256) recover_kernel(const __grid_constant__ Vi
             const int lo = max(x0 - 32 * w, 0), hi = min(x1 - 32 * w, 32);
             uint32_t m = __ldg(v.open_bits + by * ow + w) & (0xffffffffu << lo) & (0xffffffffu >> (32 - hi));
             for (; m != 0u && !keep; m &= m - 1u)
-              keep = kRestart || d[q] > __ldg(v.zcut + by * bw + 32 * w + __ffs(m) - 1);
+              keep = d[q] > __ldg(v.zcut + by * bw + 32 * w + __ffs(m) - 1);
           }
       }
       const unsigned word = __ballot_sync(0xffffffffu, keep);
@@ -417,12 +417,11 @@ cudaError_t launch_project(const ViewJob* v, int nv, cudaStream_t st) {
   });
 }
 
-cudaError_t launch_recover(const ViewJob* v, int nv, bool restart, cudaStream_t st) {
+cudaError_t launch_recover(const ViewJob* v, int nv, cudaStream_t st) {
   return with_views(v, nv, [&](const auto& a) {
     constexpr int N = sizeof(a.v) / sizeof(a.v[0]);
     const dim3 grid(view_grid((largest_n(v, nv) + kRecover - 1) / kRecover, nv, 8), nv);
-    if (restart) recover_kernel<N, true><<<grid, 256, 0, st>>>(a);
-    else recover_kernel<N, false><<<grid, 256, 0, st>>>(a);
+    recover_kernel<N><<<grid, 256, 0, st>>>(a);
     g_launches += 1;
     return cudaGetLastError();
   });

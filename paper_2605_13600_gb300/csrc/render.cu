@@ -149,7 +149,7 @@ __device__ __forceinline__ void write_row(void* __restrict__ out, int64_t pix, b
 // (measured 9.1 -> 5.5 ms per 1920x1080 view against 2 CTAs per SM; 5 spills more)
 template <bool kStaged>
 __global__ void __launch_bounds__(kRThreads, 4) render_tile_kernel(
-    const __grid_constant__ ViewJob view, int second, const int32_t* __restrict__ topk_idx,
+    const __grid_constant__ ViewJob view, const int32_t* __restrict__ topk_idx,
     const float* __restrict__ topk_val, int K, int C, void* __restrict__ out, int out_bf16, float* __restrict__ out_T,
     int32_t* __restrict__ out_last) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -157,11 +157,8 @@ __global__ void __launch_bounds__(kRThreads, 4) render_tile_kernel(
   const CamArgs& cam = view.cam;
   WsHeader* __restrict__ const hdr = view.hdr;
   const ProjRec* __restrict__ const proj = view.proj;
-  if (second && blockIdx.x >= hdr->open_tiles) return;
-  const int tile = second ? (int)view.open_list[blockIdx.x] : (int)blockIdx.x;
-  const TileList list = tile_list(view.keys, view.tile_start, second || !view.hist ? nullptr : view.zcut, view.shift,
-                                  cam.gx, tile);
-  const uint32_t cut = list.cut;
+  const int tile = (int)blockIdx.x;
+  const TileList list = tile_list(view.keys, view.tile_start, nullptr, view.shift, cam.gx, tile);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int tx = tile % cam.gx, ty = tile / cam.gx;
   const int n = list.n;
@@ -176,7 +173,7 @@ __global__ void __launch_bounds__(kRThreads, 4) render_tile_kernel(
     sm.done[p] = !(px < cam.width && py < cam.height);
   }
   if (tid < 2) sm.cnt[tid] = 0ull;
-  const OrderBuckets bk = order_buckets<ROrder>(hdr, cut);
+  const OrderBuckets bk = order_buckets<ROrder>(hdr);
   order_init(sm.ord, list, bk);  // ends with a barrier
   unsigned n_eval = 0, n_contrib = 0;
 
@@ -246,12 +243,7 @@ __global__ void __launch_bounds__(kRThreads, 4) render_tile_kernel(
     for (int p = tid; p < kTilePixels; p += kRThreads) open |= !sm.done[p];
     if (!__syncthreads_or(open)) break;
   }
-  // a tile still open at its depth cut is recorded and rendered again, from its whole list
-  int left = 0;
-  for (int p = tid; p < kTilePixels; p += kRThreads) left |= !sm.done[p];
-  const bool again = cut != kNoCut && __syncthreads_or(left);
-  if (again && tid == 0) record_open(hdr, view.open_bits, view.open_list, cam.gx, tile);
-  if (lane == 0 && !again) {
+  if (lane == 0) {
     atomicAdd(&sm.cnt[0], (unsigned long long)n_eval);
     atomicAdd(&sm.cnt[1], (unsigned long long)n_contrib);
   }
@@ -281,18 +273,18 @@ size_t render_smem_bytes(int C, int K) {
          (render_stages(K) ? staged_bytes(K) : 0);
 }
 
-cudaError_t launch_render_tiles(const ViewJob& v, bool second, const int32_t* topk_idx,
+cudaError_t launch_render_tiles(const ViewJob& v, const int32_t* topk_idx,
                                 const float* topk_val, int K, int C, void* out, int out_bf16, float* out_T,
                                 int32_t* out_last, cudaStream_t st) {
   if (render_uses_mma(C, K))
-    return launch_render_mma(v, second, topk_idx, topk_val, K, C, out, out_bf16, out_T, out_last, st);
+    return launch_render_mma(v, topk_idx, topk_val, K, C, out, out_bf16, out_T, out_last, st);
   const int ntiles = v.cam.gx * v.cam.gy;
   if (ntiles <= 0) return cudaSuccess;
   const size_t smem = render_smem_bytes(C, K);
   auto kern = render_stages(K) ? render_tile_kernel<true> : render_tile_kernel<false>;
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
-  kern<<<ntiles, kRThreads, smem, st>>>(v, second ? 1 : 0, topk_idx, topk_val, K, C, out, out_bf16, out_T, out_last);
+  kern<<<ntiles, kRThreads, smem, st>>>(v, topk_idx, topk_val, K, C, out, out_bf16, out_T, out_last);
   g_launches += 1;
   return cudaGetLastError();
 }

@@ -158,7 +158,7 @@ __device__ __forceinline__ bool walk_bwd(BwdSmem& sm, const BwdDyn& dy, const fl
 // sums, measured 4.9 -> 2.1 ms per 800x600 view (2 or 3 CTAs per SM: 2.4 ms)
 template <bool kStaged>
 __global__ void __launch_bounds__(kBThreads, 4) render_bwd_kernel(
-    const __grid_constant__ ViewJob view, int second, const int32_t* __restrict__ topk_idx,
+    const __grid_constant__ ViewJob view, const int32_t* __restrict__ topk_idx,
     const float* __restrict__ topk_val, int K, int C, const float* __restrict__ dL_dcodes,
     float* __restrict__ d_val, float* __restrict__ d_opacity) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -166,19 +166,16 @@ __global__ void __launch_bounds__(kBThreads, 4) render_bwd_kernel(
   const CamArgs& cam = view.cam;
   WsHeader* __restrict__ const hdr = view.hdr;
   const ProjRec* __restrict__ const proj = view.proj;
-  if (second && blockIdx.x >= hdr->open_tiles) return;
-  const int tile = second ? (int)view.open_list[blockIdx.x] : (int)blockIdx.x;
-  const TileList list = tile_list(view.keys, view.tile_start, second || !view.hist ? nullptr : view.zcut, view.shift,
-                                  cam.gx, tile);
-  const uint32_t cut = list.cut;
+  const int tile = (int)blockIdx.x;
+  const TileList list = tile_list(view.keys, view.tile_start, nullptr, view.shift, cam.gx, tile);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int tx = tile % cam.gx, ty = tile / cam.gx;
   const int n = list.n;
-  if (n == 0 && cut == kNoCut) return;
+  if (n == 0) return;
   if (hdr->status & kStatCapacity) return;
   const BwdDyn dy = bwd_dyn(sm, C, K);
   float* grow = dy.g + warp * C;
-  const OrderBuckets bk = order_buckets<BOrder>(hdr, cut);
+  const OrderBuckets bk = order_buckets<BOrder>(hdr);
   order_init(sm.ord, list, bk);
 
   for (int pass = 1; pass <= 2; ++pass) {
@@ -256,16 +253,6 @@ __global__ void __launch_bounds__(kBThreads, 4) render_bwd_kernel(
       if (!__syncthreads_or(open)) break;
     }
     __syncthreads();
-    if (pass == 1 && cut != kNoCut) {
-      // a tile still open at its depth cut is recorded and walked again, from
-      // its whole list: no gradient of it has been added yet
-      int left = 0;
-      for (int p = tid; p < kTilePixels; p += kBThreads) left |= !sm.done[p];
-      if (__syncthreads_or(left)) {
-        if (tid == 0) record_open(hdr, view.open_bits, view.open_list, cam.gx, tile);
-        return;
-      }
-    }
   }
 }
 
@@ -402,18 +389,16 @@ __device__ __forceinline__ void walk_pixels(const float4& a, const float4& b, bo
 // the latency of the scans (49% of the issue rate, 4 warps per scheduler).
 template <int KR, int kNP, bool kVec>
 __global__ void __launch_bounds__(kBThreads, 2) render_bwd_block_kernel(
-    const __grid_constant__ ViewJob view, int second, const int32_t* __restrict__ topk_idx,
+    const __grid_constant__ ViewJob view, const int32_t* __restrict__ topk_idx,
     const float* __restrict__ topk_val, int K, int C, const float* __restrict__ dL_dcodes,
     float* __restrict__ d_val, float* __restrict__ d_opacity) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   BwdBlockSmem& sm = *reinterpret_cast<BwdBlockSmem*>(smem_raw);
   const CamArgs& cam = view.cam;
   WsHeader* __restrict__ const hdr = view.hdr;
-  if (second && blockIdx.x >= hdr->open_tiles) return;
-  const int tile = second ? (int)view.open_list[blockIdx.x] : (int)blockIdx.x;
-  const TileList list = tile_list(view.keys, view.tile_start, second || !view.hist ? nullptr : view.zcut, view.shift,
-                                  cam.gx, tile);
-  if (list.n == 0 && list.cut == kNoCut) return;
+  const int tile = (int)blockIdx.x;
+  const TileList list = tile_list(view.keys, view.tile_start, nullptr, view.shift, cam.gx, tile);
+  if (list.n == 0) return;
   if (hdr->status & kStatCapacity) return;
   constexpr int kW = BOrder::kWin;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -426,7 +411,7 @@ __global__ void __launch_bounds__(kBThreads, 2) render_bwd_block_kernel(
   float* const dop_sum = dval + K * kW;
   const float* const gblock = dL_dcodes + ((int64_t)by * cam.width + bx) * C;
   if (lane < 2 * kNP) rows[lane * rw + C] = 0.0f;
-  const OrderBuckets bk = order_buckets<BOrder>(hdr, list.cut);
+  const OrderBuckets bk = order_buckets<BOrder>(hdr);
   order_init(sm.ord, list, bk);
 
   float S = 0.0f;  // lane p: sum of e gw of the block's pixel p (pass 1)
@@ -542,12 +527,6 @@ __global__ void __launch_bounds__(kBThreads, 2) render_bwd_block_kernel(
       }
       if (!__syncthreads_or(open)) break;
     }
-    // a tile still open at its depth cut is recorded and walked again, from
-    // its whole list: no gradient of it has been added yet
-    if (pass == 1 && list.cut != kNoCut && __syncthreads_or(open)) {
-      if (tid == 0) record_open(hdr, view.open_bits, view.open_list, cam.gx, tile);
-      return;
-    }
     __syncthreads();
   }
 }
@@ -569,7 +548,7 @@ size_t render_bwd_smem_bytes(int C, int K) {
          (bwd_stages(K) ? (size_t)K * BOrder::kWin * (sizeof(float) + sizeof(short)) : 0);
 }
 
-cudaError_t launch_render_bwd(const ViewJob& v, bool second, const int32_t* topk_idx,
+cudaError_t launch_render_bwd(const ViewJob& v, const int32_t* topk_idx,
                               const float* topk_val, int K, int C, const float* dL_dcodes, float* d_val,
                               float* d_opacity, cudaStream_t st) {
   const int ntiles = v.cam.gx * v.cam.gy;
@@ -585,7 +564,7 @@ cudaError_t launch_render_bwd(const ViewJob& v, bool second, const int32_t* topk
     const size_t bytes = bwd_block_smem(C, K);
     cudaError_t be = cudaFuncSetAttribute(bk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (be != cudaSuccess) return be;
-    bk<<<ntiles, kBThreads, bytes, st>>>(v, second ? 1 : 0, topk_idx, topk_val, K, C, dL_dcodes, d_val, d_opacity);
+    bk<<<ntiles, kBThreads, bytes, st>>>(v, topk_idx, topk_val, K, C, dL_dcodes, d_val, d_opacity);
     g_launches += 1;
     return cudaGetLastError();
   }
@@ -593,7 +572,7 @@ cudaError_t launch_render_bwd(const ViewJob& v, bool second, const int32_t* topk
   auto kern = bwd_stages(K) ? render_bwd_kernel<true> : render_bwd_kernel<false>;
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
-  kern<<<ntiles, kBThreads, smem, st>>>(v, second ? 1 : 0, topk_idx, topk_val, K, C, dL_dcodes, d_val, d_opacity);
+  kern<<<ntiles, kBThreads, smem, st>>>(v, topk_idx, topk_val, K, C, dL_dcodes, d_val, d_opacity);
   g_launches += 1;
   return cudaGetLastError();
 }

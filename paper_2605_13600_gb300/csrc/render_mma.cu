@@ -250,10 +250,9 @@ __device__ __forceinline__ bool walkers_or(bool p) {
 
 // One CTA per tile; one CTA per SM (the accumulator takes the SM's 512 TMEM
 // columns at C = 256, and the shared memory keeps a second CTA out).
-// second: the tiles recorded as open, each from the start of its whole list.
 template <int KT>
 __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
-    const __grid_constant__ ViewJob view, int second, const int32_t* __restrict__ topk_idx,
+    const __grid_constant__ ViewJob view, const int32_t* __restrict__ topk_idx,
     const float* __restrict__ topk_val, int K, int C, void* __restrict__ out, int out_bf16,
     float* __restrict__ out_T, int32_t* __restrict__ out_last) {
   extern __shared__ __align__(128) unsigned char msm_raw[];
@@ -263,11 +262,8 @@ __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
   WsHeader* __restrict__ const hdr = view.hdr;
   const ProjRec* __restrict__ const proj = view.proj;
   if (hdr->status & kStatCapacity) return;  // set by the binning before this launch: uniform
-  if (second && blockIdx.x >= hdr->open_tiles) return;
-  const int tile = second ? (int)view.open_list[blockIdx.x] : (int)blockIdx.x;
-  const TileList list = tile_list(view.keys, view.tile_start, second || !view.hist ? nullptr : view.zcut, view.shift,
-                                  cam.gx, tile);
-  const uint32_t cut = list.cut;
+  const int tile = (int)blockIdx.x;
+  const TileList list = tile_list(view.keys, view.tile_start, nullptr, view.shift, cam.gx, tile);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int tx = tile % cam.gx, ty = tile / cam.gx;
   const int n = list.n;
@@ -351,7 +347,7 @@ __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
   // code rows by 16-byte loads (K = 4, 8, ..; the arrays may start anywhere)
   const bool vec =
       (K & 3) == 0 && ((reinterpret_cast<uintptr_t>(topk_idx) | reinterpret_cast<uintptr_t>(topk_val)) & 15) == 0;
-  const OrderBuckets bk = order_buckets<MOrder>(hdr, cut);
+  const OrderBuckets bk = order_buckets<MOrder>(hdr);
   order_init<MOrder, 16>(sm.ord, list, bk);
 
   unsigned n_eval = 0, n_contrib = 0;
@@ -506,11 +502,7 @@ __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
     fin_ok = ptx::mbar_wait_bounded(&sm.fin, 0u, kWaitIters) && fin_ok;
     if (!fin_ok) atomicOr(&hdr->status, kStatTimeout);
   }
-  // a tile still open at its depth cut is recorded and rendered again, from
-  // its whole list: nothing of it is written or counted now
-  const bool again = cut != kNoCut && !all_done && !aborted;
-  if (again && tid == 0) record_open(hdr, view.open_bits, view.open_list, cam.gx, tile);
-  const bool bad = walkers_or(!fin_ok) || aborted || again;
+  const bool bad = walkers_or(!fin_ok) || aborted;
   ptx::tc_fence_after();
 
   // epilogue: each thread reads its own pixel's row (TMEM lane)
@@ -575,13 +567,13 @@ __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
       if (inside && !bad) store_cols(out, pix, C, c0, out_bf16 != 0, v);
     }
   }
-  if (inside && !again) {
+  if (inside) {
     if (out_T) out_T[pix] = Tout;
     if (out_last) out_last[pix] = last;
   }
   const unsigned we = __reduce_add_sync(0xffffffffu, n_eval);
   const unsigned wc = __reduce_add_sync(0xffffffffu, n_contrib);
-  if (lane == 0 && !again) {
+  if (lane == 0) {
     atomicAdd(&sm.cnt[0], (unsigned long long)we);
     atomicAdd(&sm.cnt[1], (unsigned long long)wc);
   }
@@ -603,7 +595,7 @@ size_t render_mma_smem_bytes(int K) {
   return (K <= 4 ? sizeof(RenderMmaSmem<4>) : K <= 8 ? sizeof(RenderMmaSmem<8>) : sizeof(RenderMmaSmem<16>)) + 128;
 }
 
-cudaError_t launch_render_mma(const ViewJob& v, bool second, const int32_t* topk_idx,
+cudaError_t launch_render_mma(const ViewJob& v, const int32_t* topk_idx,
                               const float* topk_val, int K, int C, void* out, int out_bf16, float* out_T,
                               int32_t* out_last, cudaStream_t st) {
   const int ntiles = v.cam.gx * v.cam.gy;
@@ -612,7 +604,7 @@ cudaError_t launch_render_mma(const ViewJob& v, bool second, const int32_t* topk
   const auto kernel = K <= 4 ? render_mma_kernel<4> : K <= 8 ? render_mma_kernel<8> : render_mma_kernel<16>;
   cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
-  kernel<<<ntiles, kCtaThreads, smem, st>>>(v, second ? 1 : 0, topk_idx, topk_val, K, C, out, out_bf16, out_T,
+  kernel<<<ntiles, kCtaThreads, smem, st>>>(v, topk_idx, topk_val, K, C, out, out_bf16, out_T,
                                             out_last);
   g_launches += 1;
   return cudaGetLastError();

@@ -240,8 +240,17 @@ struct TileList {
     return (k & 0xffffffff00000000ull) | ((uint32_t)k >> id_shift);
   }
 };
+//
+// A block's list serves the binning (a quarter of the lists to count and fill)
+// and costs every tile the keys of its three neighbours, read once per window.
+// With many Gaussians to a tile the windows' passes decide: uplift of 12 views
+// (ms, blocks / tiles; Gaussians per tile of the image): 526 2.66 / 2.86, 631
+// 0.90 / 0.87, 2105 1.99 / 1.79, 2560 0.79 / 0.71, 8550 3.68 / 2.49; one
+// render the same way around (526 0.745 / 0.754, 2105 0.73 / 0.68, 8550 1.69 /
+// 1.61).
+constexpr int64_t kDensePerTile = 560;
 __host__ __device__ inline int list_shift(int64_t n, int gx, int gy) {
-  return n < (1ll << 28) && gx >= 4 && gy >= 4 ? 1 : 0;
+  return n < (1ll << 28) && gx >= 4 && gy >= 4 && n <= kDensePerTile * gx * gy ? 1 : 0;
 }
 __host__ __device__ inline int list_dim(int g, int shift) { return (g + shift) >> shift; }
 
@@ -329,7 +338,8 @@ struct ViewArgs {
 static_assert(sizeof(ViewArgs<kMaxDrainJobs>) <= 32000, "kernel parameter space");
 ViewJob view_job(const scoup_scene& sc, const CamArgs& cam, const UpliftWs& ws, WsHeader* hdr, bool cut);
 // Whether views of this size get a depth cut (given room in the view part).
-bool use_depth_cut(int64_t n, const CamArgs& cam, const UpliftWs& ws);
+// views: how many views a launch of the view's chunk takes.
+bool use_depth_cut(int64_t n, const CamArgs& cam, const UpliftWs& ws, int views);
 // Gaussians per binning CTA; larger groups from 64k Gaussians on, of which the
 // depth cut leaves a fraction.
 inline int bin_group(int64_t n) { return n <= 63488 ? 512 : 1024; }
@@ -399,7 +409,7 @@ cudaError_t launch_depth_cut(const ViewJob* v, int nv, cudaStream_t st);
 cudaError_t launch_project(const ViewJob* v, int nv, cudaStream_t st);
 // Second pass, for the tiles recorded as open: keeps the Gaussians that reach
 // one of them behind its cut (restart: at any depth), with their records.
-cudaError_t launch_recover(const ViewJob* v, int nv, bool restart, cudaStream_t st);
+cudaError_t launch_recover(const ViewJob* v, int nv, cudaStream_t st);
 // Tile lists of the kept Gaussians; second: only of the open tiles.  The lane's
 // drain counter of the pass (ctr, may be null) is cleared on the way.
 cudaError_t launch_binning(const ViewJob* v, int nv, bool second, uint32_t* ctr, cudaStream_t st);
@@ -413,15 +423,14 @@ size_t render_smem_bytes(int C, int K);
 bool render_uses_mma(int C, int K);
 bool render_mma_supported(int C, int K);
 size_t render_mma_smem_bytes(int K);
-cudaError_t launch_render_mma(const ViewJob& v, bool second, const int32_t* topk_idx,
+cudaError_t launch_render_mma(const ViewJob& v, const int32_t* topk_idx,
                               const float* topk_val, int K, int C, void* out, int out_bf16, float* out_T,
                               int32_t* out_last, cudaStream_t st);
-// second: the open tiles only, from the start of their (then whole) lists.
-cudaError_t launch_render_tiles(const ViewJob& v, bool second, const int32_t* topk_idx,
+cudaError_t launch_render_tiles(const ViewJob& v, const int32_t* topk_idx,
                                 const float* topk_val, int K, int C, void* out, int out_bf16, float* out_T,
                                 int32_t* out_last, cudaStream_t st);
 size_t render_bwd_smem_bytes(int C, int K);
-cudaError_t launch_render_bwd(const ViewJob& v, bool second, const int32_t* topk_idx,
+cudaError_t launch_render_bwd(const ViewJob& v, const int32_t* topk_idx,
                               const float* topk_val, int K, int C, const float* dL_dcodes, float* d_val,
                               float* d_opacity, cudaStream_t st);
 constexpr int kOutBF16 = 0, kOutF32 = 1, kOutCos = 2, kOutRel = 3;

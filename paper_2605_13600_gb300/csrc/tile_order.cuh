@@ -65,12 +65,12 @@ struct OrderState {
   int consumed = 0;
 };
 
-// Buckets over the view's visible depths up to `cut`.
+// Buckets over the view's visible depths.
 template <class S>
-__device__ OrderBuckets order_buckets(const WsHeader* hdr, uint32_t cut) {
+__device__ OrderBuckets order_buckets(const WsHeader* hdr) {
   OrderBuckets bk;
-  const uint32_t dmin = hdr->drange[0], dmax = min(hdr->drange[1], cut);
-  bk.lo = dmax >= dmin ? dmin : 0u;  // nothing in front of the cut: no key has depth bits 0
+  const uint32_t dmin = hdr->drange[0], dmax = hdr->drange[1];
+  bk.lo = dmin;
   bk.span = dmax >= dmin ? dmax - dmin : 0u;
   const int nb = bk.span ? 32 - __clz((int)bk.span) : 0;
   bk.shift = nb > S::kLogNB ? nb - S::kLogNB : 0;

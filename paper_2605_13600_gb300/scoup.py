@@ -644,8 +644,10 @@ class Uplift:
     """
 
     # Largest workspace of the chunked form that run() takes by itself (see
-    # __init__): eight views of 300k Gaussians at 640x480 on each of two lanes.
-    CHUNK_BYTES = 1 << 30
+    # __init__): at 1M Gaussians and 1080p eight views on each of two lanes take
+    # about 4 GB.  24 views of 1M at 988x731, one view at a time / in chunks:
+    # 6.1 / 5.1 ms; of 300k 4.5 / 4.0 ms.
+    CHUNK_BYTES = 1 << 33
 
     def __init__(self, wl, device: str = "cuda", dup_capacity: Optional[int] = None,
                  headroom: float = 1.0, compensated: bool = False, topk: bool = True, chunked: bool = False):
