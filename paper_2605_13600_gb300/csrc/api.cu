@@ -954,12 +954,20 @@ int scoup_decode(const void* codes, int32_t codes_dtype, int64_t P, int32_t C, c
   void* Abuf = (char*)Bt + align_up((size_t)D * C * 2);
   cudaError_t e;
   PhaseScope ps(SCOUP_PHASE_DECODE, st);
-  if ((e = cudaMemsetAsync(hdr, 0, sizeof(WsHeader), st)) != cudaSuccess) return cuda_fail(e, "memset");
-  if (P == 0) return SCOUP_OK;
+  if (P == 0) {
+    e = cudaMemsetAsync(hdr, 0, sizeof(WsHeader), st);
+    return e == cudaSuccess ? SCOUP_OK : cuda_fail(e, "memset");
+  }
   const bool direct = codes_dtype == 1 || gemm_takes_f32(P, D, C);
-  if (feat_norm2 && (e = cudaMemsetAsync(feat_norm2, 0, sizeof(float) * (size_t)P, st)) != cudaSuccess)
-    return cuda_fail(e, "memset");
-  if ((e = launch_transpose_bf16(codebook, Bt, C, D, st)) != cudaSuccess) return cuda_fail(e, "codebook");
+  GemmPrep prep;
+  prep.hdr = hdr;
+  prep.codebook = codebook;
+  prep.Bt = Bt;
+  prep.C = C;
+  prep.D = D;
+  prep.rownorm2 = feat_norm2;
+  prep.rows = P;
+  if ((e = launch_decode_prep(prep, st)) != cudaSuccess) return cuda_fail(e, "codebook");
   // bf16 codes feed the GEMM directly (one launch), f32 codes where it rounds
   // them itself; elsewhere they are rounded to bf16 chunk by chunk in the
   // workspace first
@@ -1060,10 +1068,11 @@ int scoup_similarity(const void* features, int64_t P, int32_t D, const float* fe
   float* fnorm2 = (float*)((char*)tnorm + align_up((size_t)Q * 4));
   cudaError_t e;
   PhaseScope ps(SCOUP_PHASE_SIMILARITY, st);
-  if ((e = cudaMemsetAsync(hdr, 0, sizeof(WsHeader), st)) != cudaSuccess) return cuda_fail(e, "memset");
-  if (P == 0) return SCOUP_OK;
-  if ((e = launch_f32_to_bf16(text, tb, (int64_t)Q * D, st)) != cudaSuccess) return cuda_fail(e, "text");
-  if ((e = launch_row_norm_bf16(tb, Q, D, tnorm, 0, st)) != cudaSuccess) return cuda_fail(e, "text norms");
+  if (P == 0) {
+    e = cudaMemsetAsync(hdr, 0, sizeof(WsHeader), st);
+    return e == cudaSuccess ? SCOUP_OK : cuda_fail(e, "memset");
+  }
+  if ((e = launch_text_prep(hdr, text, Q, D, tb, tnorm, st)) != cudaSuccess) return cuda_fail(e, "text");
   const float* rn2 = feat_norm2;
   if (!rn2) {
     if ((e = launch_row_norm_bf16(features, P, D, fnorm2, 1, st)) != cudaSuccess) return cuda_fail(e, "norms");
@@ -1106,10 +1115,11 @@ int scoup_similarity_relevancy(const void* features, int64_t P, int32_t D, const
   float* fnorm2 = (float*)((char*)tnorm + align_up((size_t)Q * 4));
   cudaError_t e;
   PhaseScope ps(SCOUP_PHASE_SIMILARITY, st);
-  if ((e = cudaMemsetAsync(hdr, 0, sizeof(WsHeader), st)) != cudaSuccess) return cuda_fail(e, "memset");
-  if (P == 0) return SCOUP_OK;
-  if ((e = launch_f32_to_bf16(text, tb, (int64_t)Q * D, st)) != cudaSuccess) return cuda_fail(e, "text");
-  if ((e = launch_row_norm_bf16(tb, Q, D, tnorm, 0, st)) != cudaSuccess) return cuda_fail(e, "text norms");
+  if (P == 0) {
+    e = cudaMemsetAsync(hdr, 0, sizeof(WsHeader), st);
+    return e == cudaSuccess ? SCOUP_OK : cuda_fail(e, "memset");
+  }
+  if ((e = launch_text_prep(hdr, text, Q, D, tb, tnorm, st)) != cudaSuccess) return cuda_fail(e, "text");
   const float* rn2 = feat_norm2;
   if (!rn2) {
     if ((e = launch_row_norm_bf16(features, P, D, fnorm2, 1, st)) != cudaSuccess) return cuda_fail(e, "norms");
@@ -1164,11 +1174,21 @@ int scoup_decode_query(const void* codes, int32_t codes_dtype, int64_t P, int32_
   float* tnorm = (float*)((char*)Gt + align_up((size_t)Q * C * 2));
   cudaError_t e;
   PhaseScope ps(SCOUP_PHASE_DECODE, st);
-  if ((e = cudaMemsetAsync(hdr, 0, sizeof(WsHeader), st)) != cudaSuccess) return cuda_fail(e, "memset");
-  if (P == 0) return SCOUP_OK;
-  if ((e = launch_transpose_bf16(codebook, Bt, C, D, st)) != cudaSuccess) return cuda_fail(e, "codebook");
-  if ((e = launch_text_codebook(text, codebook, Q, C, D, Gt, tnorm, st)) != cudaSuccess)
-    return cuda_fail(e, "text x codebook");
+  if (P == 0) {
+    e = cudaMemsetAsync(hdr, 0, sizeof(WsHeader), st);
+    return e == cudaSuccess ? SCOUP_OK : cuda_fail(e, "memset");
+  }
+  GemmPrep prep;
+  prep.hdr = hdr;
+  prep.codebook = codebook;
+  prep.Bt = Bt;
+  prep.C = C;
+  prep.D = D;
+  prep.text = text;
+  prep.Q = Q;
+  prep.Gt = Gt;
+  prep.tnorm = tnorm;
+  if ((e = launch_decode_prep(prep, st)) != cudaSuccess) return cuda_fail(e, "codebook");
   const int64_t ldq = n_canon > 0 ? Q - n_canon : Q;
   const bool direct = codes_dtype == 1 || gemm_takes_f32(P, D, C);
   const int64_t chunk = direct ? P : decode_chunk_rows(P);
@@ -1229,9 +1249,11 @@ int scoup_decode_backward(const void* dF, int32_t dF_dtype, int64_t P, int32_t D
   void* Abuf = (char*)Bt + align_up((size_t)C * D * 2);
   cudaError_t e;
   PhaseScope ps(SCOUP_PHASE_DECODE, st);
-  if ((e = cudaMemsetAsync(hdr, 0, sizeof(WsHeader), st)) != cudaSuccess) return cuda_fail(e, "memset");
-  if (P == 0) return SCOUP_OK;
-  if ((e = launch_f32_to_bf16(codebook, Bt, (int64_t)C * D, st)) != cudaSuccess) return cuda_fail(e, "codebook");
+  if (P == 0) {
+    e = cudaMemsetAsync(hdr, 0, sizeof(WsHeader), st);
+    return e == cudaSuccess ? SCOUP_OK : cuda_fail(e, "memset");
+  }
+  if ((e = launch_f32_to_bf16(codebook, Bt, (int64_t)C * D, st, hdr)) != cudaSuccess) return cuda_fail(e, "codebook");
   const int64_t chunk = dF_dtype == 1 ? P : decode_chunk_rows(P);
   for (int64_t r0 = 0; r0 < P; r0 += chunk) {
     const int64_t rows = P - r0 < chunk ? P - r0 : chunk;

@@ -875,7 +875,9 @@ cudaError_t launch_rows(const void* A, const void* Bt, const void* Gt, const Gem
 }
 
 // ---- small conversion kernels ----
-__global__ void f32_to_bf16_kernel(const float* __restrict__ x, __nv_bfloat16* __restrict__ y, int64_t n) {
+__global__ void f32_to_bf16_kernel(const float* __restrict__ x, __nv_bfloat16* __restrict__ y, int64_t n, WsHeader* hdr) {
+  if (hdr && blockIdx.x == 0)  // a call's first launch clears its header
+    for (int i = threadIdx.x; i < (int)(sizeof(WsHeader) / 4); i += blockDim.x) ((uint32_t*)hdr)[i] = 0u;
   for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * 4; i < n; i += (int64_t)gridDim.x * blockDim.x * 4) {
     if (i + 3 < n) {
       const float4 v = *reinterpret_cast<const float4*>(x + i);
@@ -887,12 +889,89 @@ __global__ void f32_to_bf16_kernel(const float* __restrict__ x, __nv_bfloat16* _
   }
 }
 
-// Bt[d][c] = bf16(B[c][d])  (B is [Cdim, D] row-major)
-__global__ void transpose_bf16_kernel(const float* __restrict__ B, __nv_bfloat16* __restrict__ Bt, int Cdim, int D) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < (int64_t)Cdim * D;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int d = (int)(i / Cdim), c = (int)(i % Cdim);
-    Bt[i] = __float2bfloat16_rn(B[(int64_t)c * D + d]);
+// The work in front of a GEMM call in one launch (a memset or a small kernel
+// of its own is about 2 us of a call of 30): the call's header cleared, and
+// part by part of the grid what the operands want.
+constexpr int kPrepThreads = 256;
+
+__device__ __forceinline__ void clear_words(uint32_t* p, int64_t n, int block, int blocks) {
+  for (int64_t i = (int64_t)block * kPrepThreads + threadIdx.x; i < n; i += (int64_t)blocks * kPrepThreads) p[i] = 0u;
+}
+
+// Bt[d][c] = bf16(B[c][d]) (B is [C, D] row-major), 32 x 32 at a time through
+// shared memory so that both sides are coalesced
+__device__ void transpose_tiles(const float* __restrict__ B, __nv_bfloat16* __restrict__ Bt, int C, int D, int block,
+                                int blocks) {
+  __shared__ float t[32][33];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int ct = (C + 31) / 32;
+  const int64_t tiles = (int64_t)ct * ((D + 31) / 32);
+  for (int64_t k = block; k < tiles; k += blocks) {
+    const int c0 = (int)(k % ct) * 32, d0 = (int)(k / ct) * 32;
+    __syncthreads();
+    for (int r = w; r < 32; r += kPrepThreads / 32)
+      if (c0 + r < C && d0 + lane < D) t[r][lane] = B[(int64_t)(c0 + r) * D + d0 + lane];
+    __syncthreads();
+    for (int r = w; r < 32; r += kPrepThreads / 32)
+      if (d0 + r < D && c0 + lane < C) Bt[(int64_t)(d0 + r) * C + c0 + lane] = __float2bfloat16_rn(t[lane][r]);
+  }
+}
+
+// One warp per (q, c): Gt[q][c] = bf16(sum_d text[q][d] codebook[c][d]) with
+// FP32 sums; the warps of c = 0 also write |text_q|.
+__device__ void text_codebook(const float* __restrict__ text, const float* __restrict__ codebook, int Q, int C, int D,
+                              __nv_bfloat16* __restrict__ Gt, float* __restrict__ tnorm, int block, int blocks) {
+  const int lane = threadIdx.x & 31;
+  for (int64_t w = ((int64_t)block * kPrepThreads + threadIdx.x) / 32; w < (int64_t)Q * C;
+       w += (int64_t)blocks * kPrepThreads / 32) {
+    const int qi = (int)(w / C), c = (int)(w - (int64_t)qi * C);
+    float dot = 0.0f, sq = 0.0f;
+    for (int d = lane; d < D; d += 32) {
+      const float t = text[(int64_t)qi * D + d];
+      dot = fmaf(t, codebook[(int64_t)c * D + d], dot);
+      sq = fmaf(t, t, sq);
+    }
+    for (int off = 16; off > 0; off >>= 1) {
+      dot += __shfl_xor_sync(0xffffffffu, dot, off);
+      sq += __shfl_xor_sync(0xffffffffu, sq, off);
+    }
+    if (lane == 0) {
+      Gt[w] = __float2bfloat16_rn(dot);
+      if (c == 0) tnorm[qi] = sqrtf(sq);
+    }
+  }
+}
+
+// Blocks 0 .. tblocks - 1: the header and the transpose; the rest: the text
+// product (Q > 0) or the cleared row norms.
+__global__ void __launch_bounds__(kPrepThreads) decode_prep_kernel(GemmPrep p, int tblocks) {
+  const int b = blockIdx.x;
+  if (b < tblocks) {
+    if (b == 0) clear_words((uint32_t*)p.hdr, sizeof(WsHeader) / 4, 0, 1);
+    transpose_tiles(p.codebook, (__nv_bfloat16*)p.Bt, p.C, p.D, b, tblocks);
+  } else if (p.Q > 0) {
+    text_codebook(p.text, p.codebook, p.Q, p.C, p.D, (__nv_bfloat16*)p.Gt, p.tnorm, b - tblocks, gridDim.x - tblocks);
+  } else {
+    clear_words((uint32_t*)p.rownorm2, p.rows, b - tblocks, gridDim.x - tblocks);
+  }
+}
+
+// One warp per text vector: its bf16 row and the row's norm; block 0 clears the header.
+__global__ void __launch_bounds__(kPrepThreads) text_prep_kernel(WsHeader* hdr, const float* __restrict__ text, int Q,
+                                                                 int D, __nv_bfloat16* __restrict__ tb,
+                                                                 float* __restrict__ tnorm) {
+  if (blockIdx.x == 0) clear_words((uint32_t*)hdr, sizeof(WsHeader) / 4, 0, 1);
+  const int lane = threadIdx.x & 31;
+  for (int64_t r = (blockIdx.x * (int64_t)kPrepThreads + threadIdx.x) / 32; r < Q; r += (int64_t)gridDim.x * kPrepThreads / 32) {
+    float s = 0.0f;
+    for (int d = lane; d < D; d += 32) {
+      const __nv_bfloat16 h = __float2bfloat16_rn(text[r * D + d]);
+      const float v = __bfloat162float(h);
+      tb[r * D + d] = h;
+      s += v * v;
+    }
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (lane == 0) tnorm[r] = sqrtf(s);
   }
 }
 
@@ -966,49 +1045,25 @@ cudaError_t launch_gemm_bf16_query(const void* A, const void* Bt, const void* Gt
   return launch_bn<256>(A, Bt, Gt, ep, st);
 }
 
-// One warp per (q, c): Gt[q][c] = bf16(sum_d text[q][d] codebook[c][d]) with
-// FP32 sums; the warps of c = 0 also write |text_q|.
-__global__ void text_codebook_kernel(const float* __restrict__ text, const float* __restrict__ codebook, int Q,
-                                     int C, int D, __nv_bfloat16* __restrict__ Gt, float* __restrict__ tnorm) {
-  const int lane = threadIdx.x & 31;
-  for (int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32; w < (int64_t)Q * C;
-       w += (int64_t)gridDim.x * blockDim.x / 32) {
-    const int qi = (int)(w / C), c = (int)(w - (int64_t)qi * C);
-    float dot = 0.0f, sq = 0.0f;
-    for (int d = lane; d < D; d += 32) {
-      const float t = text[(int64_t)qi * D + d];
-      dot = fmaf(t, codebook[(int64_t)c * D + d], dot);
-      sq = fmaf(t, t, sq);
-    }
-    for (int off = 16; off > 0; off >>= 1) {
-      dot += __shfl_xor_sync(0xffffffffu, dot, off);
-      sq += __shfl_xor_sync(0xffffffffu, sq, off);
-    }
-    if (lane == 0) {
-      Gt[w] = __float2bfloat16_rn(dot);
-      if (c == 0) tnorm[qi] = sqrtf(sq);
-    }
-  }
-}
-
-cudaError_t launch_f32_to_bf16(const float* x, void* y, int64_t n, cudaStream_t st) {
+cudaError_t launch_f32_to_bf16(const float* x, void* y, int64_t n, cudaStream_t st, WsHeader* hdr) {
   if (n <= 0) return cudaSuccess;
-  f32_to_bf16_kernel<<<blocks_for(n / 4 + 1, 256), 256, 0, st>>>(x, (__nv_bfloat16*)y, n);
+  f32_to_bf16_kernel<<<blocks_for(n / 4 + 1, 256), 256, 0, st>>>(x, (__nv_bfloat16*)y, n, hdr);
   g_launches += 1;
   return cudaGetLastError();
 }
 
-cudaError_t launch_transpose_bf16(const float* B, void* Bt, int Cdim, int D, cudaStream_t st) {
-  transpose_bf16_kernel<<<blocks_for((int64_t)Cdim * D, 256), 256, 0, st>>>(B, (__nv_bfloat16*)Bt, Cdim, D);
+cudaError_t launch_decode_prep(const GemmPrep& p, cudaStream_t st) {
+  const int64_t tiles = (int64_t)((p.C + 31) / 32) * ((p.D + 31) / 32);
+  const int tblocks = blocks_for(tiles, 1);
+  const int more = p.Q > 0 ? blocks_for((int64_t)p.Q * p.C, kPrepThreads / 32)
+                           : p.rownorm2 ? blocks_for(p.rows, 4 * kPrepThreads) : 0;
+  decode_prep_kernel<<<tblocks + more, kPrepThreads, 0, st>>>(p, tblocks);
   g_launches += 1;
   return cudaGetLastError();
 }
 
-cudaError_t launch_text_codebook(const float* text, const float* codebook, int Q, int C, int D, void* Gt,
-                                 float* tnorm, cudaStream_t st) {
-  if (Q <= 0 || C <= 0) return cudaSuccess;
-  text_codebook_kernel<<<blocks_for((int64_t)Q * C * 32, 256), 256, 0, st>>>(text, codebook, Q, C, D,
-                                                                             (__nv_bfloat16*)Gt, tnorm);
+cudaError_t launch_text_prep(WsHeader* hdr, const float* text, int Q, int D, void* tb, float* tnorm, cudaStream_t st) {
+  text_prep_kernel<<<blocks_for(Q, kPrepThreads / 32), kPrepThreads, 0, st>>>(hdr, text, Q, D, (__nv_bfloat16*)tb, tnorm);
   g_launches += 1;
   return cudaGetLastError();
 }

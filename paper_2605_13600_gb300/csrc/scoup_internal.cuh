@@ -465,11 +465,27 @@ bool gemm_takes_f32(int64_t M, int N, int K);
 // launch_gemm_bf16 with the fused query unit (ep.sim_n > 0; Gt bf16 [sim_n, K]).
 cudaError_t launch_gemm_bf16_query(const void* A, const void* Bt, const void* Gt, const GemmEpi& ep,
                                    cudaStream_t st);
-// Gt[q][c] = bf16(sum_d text[q][d] codebook[c][d]) (FP32 sums) and tnorm[q] = |text_q| (FP32).
-cudaError_t launch_text_codebook(const float* text, const float* codebook, int Q, int C, int D, void* Gt,
-                                 float* tnorm, cudaStream_t st);
-cudaError_t launch_f32_to_bf16(const float* x, void* y, int64_t n, cudaStream_t st);
-cudaError_t launch_transpose_bf16(const float* B, void* Bt, int Cdim, int D, cudaStream_t st);
+// Before a decode's GEMM: *hdr cleared, Bt [D, C] = bf16 of the transposed
+// codebook [C, D], and either (Q > 0) Gt[q][c] = bf16(sum_d text[q][d]
+// codebook[c][d]) (FP32 sums) with tnorm[q] = |text_q| (FP32), or (rownorm2)
+// rows cleared row norms.
+struct GemmPrep {
+  WsHeader* hdr;
+  const float* codebook;
+  void* Bt;
+  int C, D;
+  const float* text = nullptr;
+  int Q = 0;
+  void* Gt = nullptr;
+  float* tnorm = nullptr;
+  float* rownorm2 = nullptr;
+  int64_t rows = 0;
+};
+cudaError_t launch_decode_prep(const GemmPrep& p, cudaStream_t st);
+// Before a similarity's GEMM: *hdr cleared, tb = bf16 of text [Q, D], tnorm = the norms of its rows.
+cudaError_t launch_text_prep(WsHeader* hdr, const float* text, int Q, int D, void* tb, float* tnorm, cudaStream_t st);
+// hdr: cleared by the same launch (null: none).
+cudaError_t launch_f32_to_bf16(const float* x, void* y, int64_t n, cudaStream_t st, WsHeader* hdr = nullptr);
 cudaError_t launch_row_norm_bf16(const void* X, int64_t R, int D, float* out, int squared, cudaStream_t st);
 bool gemm_tma_available();
 int gemm_timeout_selftest(void* workspace, size_t ws_bytes, cudaStream_t st);
