@@ -24,23 +24,33 @@ def _ptr(t) -> Optional[int]:
 
 
 def _stream(stream) -> Optional[int]:
+    # the raw handle: torch.cuda.current_stream() builds a Stream object first,
+    # 3 us of the 20 that a small call spends on the host
     import torch
     if stream is None:
+        if torch.cuda.is_initialized():
+            return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
         stream = torch.cuda.current_stream()
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
+_Tensor = None  # torch.Tensor, once torch is in use
+
+
 def _need(t, dtype, name):
-    import torch
+    global _Tensor
     if t is None:
         return
-    if not isinstance(t, torch.Tensor):
+    if _Tensor is None:
+        import torch
+        _Tensor = torch.Tensor
+    if not isinstance(t, _Tensor):
         raise TypeError(f"{name} must be a torch.Tensor")
     if t.dtype != dtype:
         raise TypeError(f"{name} must be {dtype}, got {t.dtype}")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
-    if t.numel() and not t.is_cuda:
+    if not t.is_cuda and t.numel():
         raise ValueError(f"{name} must be a CUDA tensor")
 
 
