@@ -29,14 +29,15 @@
 //
 // The bound is the walkers' instruction issue with nine warps to an SM (the
 // pipes are below 40 % busy, DRAM below 10 %), so the work per chunk is kept
-// down: codes are merged and split into their bf16 parts once per window and
-// not per chunk, the warps a Gaussian may reach are a byte staged with it, the
-// walk multiplies the transmittance down without a test per step and masks the
-// weights behind the stop, and W is cleared by undoing the entries that were
-// written (32 KB of zeros per chunk at C = 256 otherwise).  With these, 1M
-// Gaussians at 1080p, C = 256, K = 8 (reorder to similarity in one call) went
-// from 2.87 to 2.83 ms, forward and backward of an 800 x 600 view from 2.04 to
-// 2.02 ms and a 161 x 119 view of 10k Gaussians at C = 64 from 155 to 146 us.
+// down: a warp walks only the Gaussians that may reach its 8 x 4 block and
+// scatters their weights into E (all 32 of a chunk in 16 x 2 blocks before:
+// 161 x 119, 10k Gaussians, C = 64 146 -> 129 us, forward and backward at 800
+// x 600 1.96 -> 1.93 ms, 1080p with query 2.59 -> 2.56 ms); codes are merged
+// and split into their bf16 parts once per window and not per chunk, the warps
+// a Gaussian may reach are a byte staged with it, the walk multiplies the
+// transmittance down without a test per step and masks the weights behind the
+// stop, and E and W are cleared only where they were written (155 -> 146 us,
+// 2.04 -> 2.02 ms and 2.87 -> 2.83 ms for the same three).
 // Half-tile CTAs, two to an SM, take 1.84 ms where this kernel takes 1.61 ms
 // (1080p): every half orders and stages the tile's list again.
 //
@@ -85,11 +86,11 @@ template <int KT>
 struct RenderMmaSmem {
   ChunkBuf buf[2];
   MOrder ord;
-  float4 rec_a[MOrder::kWin];
-  float4 rec_b[MOrder::kWin];
+  float4 rec_a[MOrder::kWin + 1];  // one more: a record that no pixel accepts
+  float4 rec_b[MOrder::kWin + 1];
   uint32_t code_val[KT * MOrder::kWin];  // [k][window position]: the value's bf16 parts, hi | lo << 16
   short code_idx[KT * MOrder::kWin];     // atom; -1: no entry, or added to an earlier entry of the atom
-  uint8_t rows[MOrder::kWin];            // bit w: the Gaussian may reach warp w's 16 x 2 block
+  uint8_t rows[MOrder::kWin];            // bit w: the Gaussian may reach warp w's 8 x 4 block
   uint64_t mma_done[2];  // per chunk buffer: the MMAs that read it have completed
   uint64_t ready[2];     // per chunk buffer: the walkers have written E and W (and ctl)
   uint64_t fin;
@@ -121,35 +122,41 @@ __device__ __forceinline__ void split_bf16x2(float x, float y, uint32_t& hi, uin
 // row of E (hi and lo parts, zero where a Gaussian does not contribute);
 // returns whether any weight of the row is nonzero.  T below the cutoff: the
 // pixel has stopped, and Tout holds its transmittance.
-// Gaussians that cannot pass the alpha test at any pixel of the warp's 16 x 2
-// block (sm.rows) are skipped, 8 at a time when none of 8 can.
+// Only the Gaussians that may pass the alpha test at some pixel of the warp's
+// 8 x 4 block (sm.rows) are walked, eight at a time in list order, and their
+// weights scattered to their columns.  `held`: the columns of the buffer's row
+// groups that may hold weights of an earlier chunk (bit per column, uniform
+// over the warp), cleared here eight columns at a time.
 template <int KT>
 __device__ __forceinline__ bool walk_chunk(const RenderMmaSmem<KT>& sm, int j0, int m, int wbase, float fpx, float fpy,
                                            float& T, float& Tout, int& last, unsigned& n_eval, unsigned& n_contrib,
-                                           unsigned char* e_hi, unsigned char* e_lo, int row) {
+                                           unsigned& held, unsigned char* e_hi, unsigned char* e_lo) {
   unsigned rel = 0u;
   if (!__all_sync(0xffffffffu, T < 1e-4f)) {
     const int jl = j0 + (int)(threadIdx.x & 31);
     rel = __ballot_sync(0xffffffffu, jl < m && ((sm.rows[jl] >> (threadIdx.x >> 5)) & 1u));
   }
-  bool any = false;
 #pragma unroll
-  for (int g = 0; g < kChunk / 8; ++g) {
-    const unsigned rel8 = (rel >> (8 * g)) & 0xffu;
-    if (rel8 == 0u) {  // warp-uniform
-      *reinterpret_cast<uint4*>(e_hi + core_off(row, g * 8)) = make_uint4(0u, 0u, 0u, 0u);
-      *reinterpret_cast<uint4*>(e_lo + core_off(row, g * 8)) = make_uint4(0u, 0u, 0u, 0u);
-      continue;
+  for (int g = 0; g < kChunk / 8; ++g)
+    if (((held | rel) >> (8 * g)) & 0xffu) {  // warp-uniform
+      *reinterpret_cast<uint4*>(e_hi + g * (int)kLBO) = make_uint4(0u, 0u, 0u, 0u);
+      *reinterpret_cast<uint4*>(e_lo + g * (int)kLBO) = make_uint4(0u, 0u, 0u, 0u);
     }
-    // independent per Gaussian: exponent, alpha test and alpha (8 chains in
-    // flight).  Positions past the window hold records that never pass (tau =
-    // +inf), and a Gaussian outside the warp's box cannot pass either, so
-    // alpha > 0 exactly when the Gaussian passes the alpha test here.
+  held = rel;
+  uint32_t any = 0u;
+  while (rel != 0u && !__all_sync(0xffffffffu, T < 1e-4f)) {
+    // the next eight (past the last: a record that never passes, tau = +inf).
+    // Independent per Gaussian: exponent, alpha test and alpha (8 chains in
+    // flight).
+    int jj[8];
     float al[8], om[8];
     unsigned pass = 0u;
+    const int cnt = min(8, __popc(rel));
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      const int j = j0 + g * 8 + u;
+      jj[u] = __ffs(rel) - 1;  // -1: none
+      rel &= rel - 1u;
+      const int j = jj[u] >= 0 ? j0 + jj[u] : MOrder::kWin;
       const float4 a = sm.rec_a[j];
       const float4 b = sm.rec_b[j];
       const float dx = a.x - fpx, dy = a.y - fpy;
@@ -176,9 +183,8 @@ __device__ __forceinline__ bool walk_chunk(const RenderMmaSmem<KT>& sm, int j0, 
     if (T0 >= 1e-4f) {  // the pixel was open
       pass &= (1u << n_ok) - 1u;
       n_contrib += __popc(pass);
-      if (pass) last = wbase + j0 + g * 8 + 32 - __clz(pass);
-      // examined: the group's Gaussians in the warp's box up to the stop
-      n_eval += __popc(rel8 & ((2u << n_ok) - 1u));
+      // examined: up to and including the stop
+      n_eval += min(cnt, (int)n_ok + 1);
       Tout = T;
       if (n_ok < 8u) {
         Tout = T0;  // the transmittance in front of the stop
@@ -186,17 +192,28 @@ __device__ __forceinline__ bool walk_chunk(const RenderMmaSmem<KT>& sm, int j0, 
         for (int u = 0; u < 8; ++u)
           if (u < (int)n_ok) Tout = __fmul_rn(Tout, om[u]);
       }
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if ((pass >> u) & 1u) last = wbase + j0 + jj[u] + 1;
     }
-    uint4 hi, lo;
-    split_bf16x2(ev[0], ev[1], hi.x, lo.x);
-    split_bf16x2(ev[2], ev[3], hi.y, lo.y);
-    split_bf16x2(ev[4], ev[5], hi.z, lo.z);
-    split_bf16x2(ev[6], ev[7], hi.w, lo.w);
-    any = any || ((hi.x | hi.y | hi.z | hi.w) != 0u);
-    *reinterpret_cast<uint4*>(e_hi + core_off(row, g * 8)) = hi;
-    *reinterpret_cast<uint4*>(e_lo + core_off(row, g * 8)) = lo;
+#pragma unroll
+    for (int u = 0; u < 8; u += 2) {
+      uint32_t hi, lo;
+      split_bf16x2(ev[u], ev[u + 1], hi, lo);
+      any |= hi;
+      if (jj[u] >= 0) {  // uniform
+        const int o = (jj[u] >> 3) * (int)kLBO + (jj[u] & 7) * 2;
+        *reinterpret_cast<uint16_t*>(e_hi + o) = (uint16_t)hi;
+        *reinterpret_cast<uint16_t*>(e_lo + o) = (uint16_t)lo;
+      }
+      if (jj[u + 1] >= 0) {
+        const int o = (jj[u + 1] >> 3) * (int)kLBO + (jj[u + 1] & 7) * 2;
+        *reinterpret_cast<uint16_t*>(e_hi + o) = (uint16_t)(hi >> 16);
+        *reinterpret_cast<uint16_t*>(e_lo + o) = (uint16_t)(lo >> 16);
+      }
+    }
   }
-  return any;
+  return any != 0u;
 }
 
 __device__ __forceinline__ uint32_t pack2_bf16(float x, float y) {
@@ -330,7 +347,9 @@ __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
     __syncwarp();
   } else {
   // ---- walkers ----
-  const int px = tx * kTile + (tid & (kTile - 1)), py = ty * kTile + (tid >> 4);
+  // a warp's pixels are an 8 x 4 block, its rows of E in that order
+  const int wx = tx * kTile + (warp & 1) * 8, wy = ty * kTile + (warp >> 1) * 4;
+  const int px = wx + (lane & 7), py = wy + (lane >> 3);
   const bool inside = px < cam.width && py < cam.height;
   const int half = tid >> 7, row = tid & 127;  // E row and TMEM lane of this pixel
   float T = inside ? 1.0f : 0.0f, Tout = T;
@@ -344,6 +363,11 @@ __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
   int wrote[kPer], wrote2[kPer];  // offsets written for the last chunk and the one before it
 #pragma unroll
   for (int q = 0; q < kPer; ++q) wrote[q] = wrote2[q] = kNone;
+  unsigned held[2] = {0xffffffffu, 0xffffffffu};
+  if (tid == 0) {
+    sm.rec_a[MOrder::kWin] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    sm.rec_b[MOrder::kWin] = make_float4(0.0f, 0.0f, INFINITY, 0.0f);
+  }
   // code rows by 16-byte loads (K = 4, 8, ..; the arrays may start anywhere)
   const bool vec =
       (K & 3) == 0 && ((reinterpret_cast<uintptr_t>(topk_idx) | reinterpret_cast<uintptr_t>(topk_val)) & 15) == 0;
@@ -363,15 +387,8 @@ __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
     const int m = n > 0 ? order_next_window<MOrder, 16>(sm.ord, list, bk, ost, hdr) : 0;
     if (m <= 0) break;  // list exhausted, or an inconsistency (status already set)
     // the window's records, which warps' blocks they may reach, and their code
-    // rows (one thread per Gaussian, all loads in flight together); the
-    // positions up to the next chunk boundary get a record no pixel accepts
-    // (tau = +inf)
-    for (int j = tid; j < ((m + kChunk - 1) & ~(kChunk - 1)); j += kMThreads) {
-      if (j >= m) {
-        sm.rec_a[j] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        sm.rec_b[j] = make_float4(0.0f, 0.0f, INFINITY, 0.0f);
-        continue;
-      }
+    // rows (one thread per Gaussian, all loads in flight together)
+    for (int j = tid; j < m; j += kMThreads) {
       const int64_t g = (int64_t)(sm.ord.win[j] & 0xffffffffull);
       const ProjRec pr = proj[g];
       int32_t ai[KT];
@@ -395,7 +412,7 @@ __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
       }
       sm.rec_a[j] = pr.a;
       sm.rec_b[j] = pr.b;
-      sm.rows[j] = (uint8_t)box_grid_mask<1, kMWarps>(pr, (float)(tx * kTile), (float)(ty * kTile), (float)kTile, 2.0f);
+      sm.rows[j] = (uint8_t)box_grid_mask<2, 4>(pr, (float)(tx * kTile), (float)(ty * kTile), 8.0f, 4.0f);
       // repeated atoms of one code add up in the first of them
 #pragma unroll
       for (int k = 0; k < KT; ++k) {
@@ -439,8 +456,11 @@ __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
         wrote2[q] = wrote[q];
         wrote[q] = kNone;
       }
-      const bool any = walk_chunk<KT>(sm, j0, m, wbase, (float)px, (float)py, T, Tout, last, n_eval, n_contrib,
-                                      cb.e[0][half], cb.e[1][half], row);
+      const bool any = walk_chunk<KT>(sm, j0, m, wbase, (float)px, (float)py, T, Tout, last, n_eval, n_contrib, held[0],
+                                      cb.e[0][half] + core_off(row, 0), cb.e[1][half] + core_off(row, 0));
+      const unsigned swap = held[0];  // of this buffer; the next chunk takes the other one
+      held[0] = held[1];
+      held[1] = swap;
       const unsigned wany = __ballot_sync(0xffffffffu, any);
       if (lane == 0) sm.any_e[warp] = wany != 0u;
       walkers_sync();
@@ -544,11 +564,10 @@ __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
         }
       }
       __syncwarp();
-      const int qx = tx * kTile, qy = ty * kTile + 2 * warp;  // the warp's 16 x 2 pixels
 #pragma unroll 8
       for (int r = 0; r < 32; ++r) {
         const uint4 val = *reinterpret_cast<const uint4*>(stg + r * 512 + ((lane ^ r) & 31) * 16);
-        const int rx = qx + (r & 15), ry = qy + (r >> 4);
+        const int rx = wx + (r & 7), ry = wy + (r >> 3);
         if (rx < cam.width && ry < cam.height)
           *reinterpret_cast<uint4*>(reinterpret_cast<unsigned char*>(out) +
                                     ((int64_t)ry * cam.width + rx) * (int64_t)C * esz + p0 * esz + lane * 16) = val;
