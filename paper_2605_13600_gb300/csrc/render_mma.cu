@@ -9,43 +9,49 @@
 // (two 128-pixel halves x C FP32 columns) and adds every chunk with
 // tcgen05.mma; the rows leave the SM once, at the end of the tile.
 //
-// One CTA per tile: 256 walkers (one thread per pixel) and a ninth warp that
-// issues the MMAs.  The walkers order the list window by window as in the
-// uplift (tile_order.cuh, on a named barrier of their own).  Per chunk every
-// walker walks its pixel front to back over the chunk's Gaussians (the
-// binary32 exponent, alpha test and T-stop rule of the uplift) and writes its
-// row of E, the walkers expand the chunk's codes into W and arrive on the
-// chunk buffer's mbarrier; the MMA warp waits on it, issues the chunk's MMAs
-// and commits them to the buffer's completion barrier (every chunk, also one
-// without MMAs, so the walkers are never two chunks ahead on a buffer).  The bf16 operands are split, e = e_hi +
+// One CTA of 256 threads per tile, two CTAs per SM.  A CTA orders its list
+// window by window as in the uplift (tile_order.cuh).  Per chunk every thread
+// walks its pixel front to back over the chunk's Gaussians (the binary32
+// exponent, alpha test and T-stop rule of the uplift) and writes its row of E,
+// the threads expand the chunk's codes into W, and warp 0 issues the chunk's
+// MMAs and commits them to the completion barrier, on which the next chunk's
+// writes wait.  The bf16 operands are split, e = e_hi +
 // e_lo and w = w_hi + w_lo (each part rounded to bf16), and three MMAs add
 // E_hi W_hi + E_hi W_lo + E_lo W_hi.  With u = 2^-8 (bf16 unit roundoff)
 // each split leaves u^2 of its value and the dropped E_lo W_lo is below u^2
 // of the product: at most about 3 u^2 = 3 * 2^-16 (4.6e-5) relative per
-// product before FP32 accumulation.
-// Chunk buffers are double-buffered, so the walk of one chunk overlaps the
-// MMAs of the previous one.  A chunk in which a pixel half has no weight
-// issues no MMA for that half.
+// product before FP32 accumulation.  A chunk in which a pixel half has no
+// weight issues no MMA for that half.
 //
-// The bound is the walkers' instruction issue with nine warps to an SM (the
-// pipes are below 40 % busy, DRAM below 10 %), so the work per chunk is kept
-// down: a warp walks only the Gaussians that may reach its 8 x 4 block and
-// scatters their weights into E (all 32 of a chunk in 16 x 2 blocks before:
-// 161 x 119, 10k Gaussians, C = 64 146 -> 129 us, forward and backward at 800
-// x 600 1.96 -> 1.93 ms, 1080p with query 2.59 -> 2.56 ms); codes are merged
-// and split into their bf16 parts once per window and not per chunk, the warps
-// a Gaussian may reach are a byte staged with it, the walk multiplies the
-// transmittance down without a test per step and masks the weights behind the
-// stop, and E and W are cleared only where they were written (155 -> 146 us,
-// 2.04 -> 2.02 ms and 2.87 -> 2.83 ms for the same three).
-// Half-tile CTAs, two to an SM, take 1.84 ms where this kernel takes 1.61 ms
-// (1080p): every half orders and stages the tile's list again.
+// What bounds it is latency: ordering, staging, walk and epilogue of a tile
+// follow each other (at 1080p, 1M Gaussians, C = 256, cycles: order 12k, stage
+// 7k, walk 24k, expansion and barriers 7k, epilogue 11k of 63k), and with one
+// CTA per SM the issue slots are 35 % used.  At C = 256 a tile takes all 512
+// TMEM columns, so two CTAs cannot both hold an accumulator: it is allocated
+// only in front of the first MMA, and the SM's other CTA orders, stages and
+// walks its first chunk until this one frees it.  One chunk buffer in place of
+// two and the MMAs issued by a walker warp make room for the second CTA (64 KB
+// less shared memory, 128 registers a thread).  1080p with query, 1M
+// Gaussians, C = 256: 2.56 -> 2.13 ms; forward and backward at 800 x 600 1.93
+// -> 1.87 ms; a grid that does not fill the SMs once (161 x 119, C = 64) waits
+// for its single buffer, 129 -> 134 us.
 //
-// Every wait (the MMA warp's on a chunk, the walkers' on a completion) is
-// bounded; a wait that gives up sets the timeout status, the walkers stop,
-// a stop still reaches the MMA warp, and TMEM is freed on every path.  The
-// tile's rows are written at the end through the free chunk buffers, in
-// coalesced 512-byte pieces.
+// The work per chunk is kept down: a warp walks only the Gaussians that may
+// reach its 8 x 4 block and scatters their weights into E (all 32 of a chunk
+// in 16 x 2 blocks before: 161 x 119 146 -> 129 us, 800 x 600 1.96 -> 1.93 ms,
+// 1080p 2.59 -> 2.56 ms); codes are merged and split into their bf16 parts
+// once per window and not per chunk, the warps a Gaussian may reach are a byte
+// staged with it, the walk multiplies the transmittance down without a test
+// per step and masks the weights behind the stop, and E and W are cleared only
+// where they were written (155 -> 146 us, 2.04 -> 2.02 ms and 2.87 -> 2.83 ms
+// for the same three).  Half-tile CTAs (128 pixels) take 1.84 ms where whole
+// tiles with one CTA per SM take 1.61 ms (1080p): every half orders and stages
+// the tile's list again.
+//
+// Every wait on a completion is bounded; a wait that gives up sets the timeout
+// status and the tile ends; TMEM is freed on every path (the allocation itself
+// waits for the SM's other CTA, which never waits for this one).  The rows are
+// written at the end through the chunk buffer, in coalesced 256-byte pieces.
 #include <cuda_bf16.h>
 #include <math.h>
 
@@ -55,15 +61,13 @@
 namespace scoup {
 namespace {
 
-constexpr int kMThreads = 256;  // walkers: one thread per pixel of the 16 x 16 tile
+constexpr int kMThreads = 256;  // one thread per pixel of the 16 x 16 tile
 constexpr int kMWarps = kMThreads / 32;
-constexpr int kMmaWarp = kMWarps;               // a ninth warp issues the tensor-core MMAs
-constexpr int kCtaThreads = kMThreads + 32;
 constexpr int kChunk = 32;      // Gaussians per chunk (contraction depth of one round of MMAs)
 constexpr int kMaxN = 256;      // widest code row: two 128-lane halves of N FP32 TMEM columns
 constexpr int kMaxK = 16;       // largest Top-K staged per window
 constexpr uint32_t kWaitIters = 1u << 22;
-using MOrder = OrderSmem<256, 10, kMThreads>;  // the walkers order alone (named barrier 1)
+using MOrder = OrderSmem<256, 10>;
 
 // Operand tiles are K-major without swizzle, built from 8-row x 16-byte core
 // matrices: the 4 core matrices of an 8-row group (32 bf16 along K) are
@@ -84,23 +88,23 @@ struct alignas(128) ChunkBuf {
 
 template <int KT>
 struct RenderMmaSmem {
-  ChunkBuf buf[2];
+  ChunkBuf buf;
   MOrder ord;
   float4 rec_a[MOrder::kWin + 1];  // one more: a record that no pixel accepts
   float4 rec_b[MOrder::kWin + 1];
   uint32_t code_val[KT * MOrder::kWin];  // [k][window position]: the value's bf16 parts, hi | lo << 16
   short code_idx[KT * MOrder::kWin];     // atom; -1: no entry, or added to an earlier entry of the atom
   uint8_t rows[MOrder::kWin];            // bit w: the Gaussian may reach warp w's 8 x 4 block
-  uint64_t mma_done[2];  // per chunk buffer: the MMAs that read it have completed
-  uint64_t ready[2];     // per chunk buffer: the walkers have written E and W (and ctl)
-  uint64_t fin;
+  uint64_t mma_done;  // the MMAs that read the chunk buffer have completed
   uint32_t tmem;
   int any_e[kMWarps];
-  int ctl[2][3];  // per chunk buffer: MMAs for pixel half 0, half 1; stop
+  int abort;  // a wait gave up
   unsigned long long cnt[2];
 };
 
-static_assert(sizeof(ChunkBuf) * 2 >= kMWarps * 16384, "the epilogue stages 16 KB per warp in the chunk buffers");
+constexpr int kPieceBytes = 256;  // of a row, per epilogue store
+static_assert(sizeof(ChunkBuf) >= kMWarps * 32 * kPieceBytes, "the epilogue stages a piece per row in the buffer");
+static_assert(sizeof(RenderMmaSmem<kMaxK>) + 128 <= 113 * 1024, "two CTAs per SM");
 
 // TMEM columns: a power of two holding two halves of Np columns, each half a
 // multiple of 32 columns (the width of one tcgen05.ld).
@@ -252,23 +256,9 @@ __device__ __forceinline__ void store_cols(void* __restrict__ out, int64_t pix, 
   }
 }
 
-// Barriers of the 256 walkers (named barrier 1; the MMA warp is not in it).
-__device__ __forceinline__ void walkers_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
-__device__ __forceinline__ bool walkers_or(bool p) {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred pi, po;\n\tsetp.ne.u32 pi, %1, 0;\n\tbar.red.or.pred po, 1, 256, pi;\n\t"
-      "selp.u32 %0, 1, 0, po;\n\t}"
-      : "=r"(r)
-      : "r"((uint32_t)p)
-      : "memory");
-  return r != 0u;
-}
-
-// One CTA per tile; one CTA per SM (the accumulator takes the SM's 512 TMEM
-// columns at C = 256, and the shared memory keeps a second CTA out).
+// One CTA per tile, two CTAs per SM.
 template <int KT>
-__global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
+__global__ void __launch_bounds__(kMThreads, 2) render_mma_kernel(
     const __grid_constant__ ViewJob view, const int32_t* __restrict__ topk_idx,
     const float* __restrict__ topk_val, int K, int C, void* __restrict__ out, int out_bf16,
     float* __restrict__ out_T, int32_t* __restrict__ out_last) {
@@ -288,65 +278,11 @@ __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
   const uint32_t cols = mma_tmem_cols(Np), half_cols = cols / 2;
 
   if (tid == 0) {
-    ptx::mbar_init(&sm.mma_done[0], 1);
-    ptx::mbar_init(&sm.mma_done[1], 1);
-    ptx::mbar_init(&sm.ready[0], kMThreads);
-    ptx::mbar_init(&sm.ready[1], kMThreads);
-    ptx::mbar_init(&sm.fin, 1);
+    ptx::mbar_init(&sm.mma_done, 1);
     ptx::fence_mbar_init();
     sm.cnt[0] = sm.cnt[1] = 0ull;
+    sm.abort = 0;
   }
-  if (warp == 0) {
-    ptx::tmem_alloc(&sm.tmem, cols);
-    ptx::tmem_relinquish();
-  }
-  ptx::tc_fence_before();
-  __syncthreads();  // the whole CTA: TMEM address and mbarriers are visible
-  ptx::tc_fence_after();
-  const uint32_t tmem = sm.tmem;
-
-  if (warp == kMmaWarp) {
-    // ---- MMA warp: one thread issues each chunk's MMAs once the walkers
-    // have written it, and commits every chunk (also one without MMAs) to its
-    // buffer's mma_done, so the walkers never run two chunks ahead of it ----
-    if (lane == 0) {
-      const uint32_t idesc = ptx::idesc_bf16_f32(128, Np);
-      unsigned acc_init = 0u;  // bit h: pixel half h has received an MMA
-      for (int chunk = 0;; ++chunk) {
-        const int b = chunk & 1;
-        if (!ptx::mbar_wait_bounded(&sm.ready[b], (uint32_t)(chunk >> 1) & 1u, kWaitIters)) {
-          atomicOr(&hdr->status, kStatTimeout);
-          break;
-        }
-        const int any0 = *(volatile int*)&sm.ctl[b][0], any1 = *(volatile int*)&sm.ctl[b][1];
-        const int stop = *(volatile int*)&sm.ctl[b][2];
-        if (stop) break;
-        ptx::tc_fence_after();
-        const ChunkBuf& cb = sm.buf[b];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          if (!(h ? any1 : any0)) continue;
-          const uint32_t d = tmem + (uint32_t)h * half_cols;
-#pragma unroll
-          for (int pass = 0; pass < 3; ++pass) {
-            const uint32_t ea = ptx::smem_u32(cb.e[pass == 2 ? 1 : 0][h]);
-            const uint32_t wb = ptx::smem_u32(cb.w[pass == 1 ? 1 : 0]);
-#pragma unroll
-            for (int ks = 0; ks < kChunk / 16; ++ks)
-              ptx::mma_f16(d, ptx::smem_desc_kmajor_none(ea + ks * 2 * kLBO, kLBO, kSBO),
-                           ptx::smem_desc_kmajor_none(wb + ks * 2 * kLBO, kLBO, kSBO), idesc,
-                           (((acc_init >> h) & 1u) || pass > 0 || ks > 0) ? 1u : 0u);
-          }
-        }
-        acc_init |= (any0 ? 1u : 0u) | (any1 ? 2u : 0u);
-        ptx::mma_commit(&sm.mma_done[b]);
-      }
-      // arrives once every MMA issued above has completed
-      ptx::mma_commit(&sm.fin);
-    }
-    __syncwarp();
-  } else {
-  // ---- walkers ----
   // a warp's pixels are an 8 x 4 block, its rows of E in that order
   const int wx = tx * kTile + (warp & 1) * 8, wy = ty * kTile + (warp >> 1) * 4;
   const int px = wx + (lane & 7), py = wy + (lane >> 3);
@@ -354,16 +290,15 @@ __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
   const int half = tid >> 7, row = tid & 127;  // E row and TMEM lane of this pixel
   float T = inside ? 1.0f : 0.0f, Tout = T;
   int last = 0;
-  // W starts cleared; each thread clears what it wrote before the buffer's next use
-  for (int b = 0; b < 2; ++b)
-    for (int i = tid; i < 2 * kWBytes / 16; i += kMThreads)
-      reinterpret_cast<uint4*>(sm.buf[b].w[0])[i] = make_uint4(0u, 0u, 0u, 0u);
+  // W starts cleared; each thread clears what it wrote for the last chunk
+  for (int i = tid; i < 2 * kWBytes / 16; i += kMThreads)
+    reinterpret_cast<uint4*>(sm.buf.w[0])[i] = make_uint4(0u, 0u, 0u, 0u);
   constexpr int kPer = (kChunk * KT + kMThreads - 1) / kMThreads;  // W entries of a thread per chunk
   constexpr int kNone = 0xffff;
-  int wrote[kPer], wrote2[kPer];  // offsets written for the last chunk and the one before it
+  int wrote[kPer];  // offsets written for the last chunk
 #pragma unroll
-  for (int q = 0; q < kPer; ++q) wrote[q] = wrote2[q] = kNone;
-  unsigned held[2] = {0xffffffffu, 0xffffffffu};
+  for (int q = 0; q < kPer; ++q) wrote[q] = kNone;
+  unsigned held = 0xffffffffu;
   if (tid == 0) {
     sm.rec_a[MOrder::kWin] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     sm.rec_b[MOrder::kWin] = make_float4(0.0f, 0.0f, INFINITY, 0.0f);
@@ -376,12 +311,8 @@ __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
 
   unsigned n_eval = 0, n_contrib = 0;
   unsigned acc_init = 0u;  // bit h: pixel half h has received an MMA
-  // thread 0: per chunk buffer b, bit b of `pending` = a chunk handed to the
-  // MMA warp whose commit has not been waited for, bit b of `phase` = parity
-  // of that commit's completion
-  unsigned pending = 0u, phase = 0u;
   bool aborted = false, all_done = false;
-  int chunk = 0, wbase = 0;
+  int wbase = 0, issued = 0;  // list positions in front of the window; chunks with MMAs
   OrderState ost;
   while (!all_done && !aborted) {
     const int m = n > 0 ? order_next_window<MOrder, 16>(sm.ord, list, bk, ost, hdr) : 0;
@@ -431,42 +362,41 @@ __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
         sm.code_idx[k * MOrder::kWin + j] = (short)atom;
       }
     }
-    walkers_sync();
-    for (int j0 = 0; j0 < m; j0 += kChunk, ++chunk) {
-      const int b = chunk & 1;
-      ChunkBuf& cb = sm.buf[b];
-      // the MMAs that last read this buffer have completed
-      bool timed_out = false;
-      if (tid == 0 && ((pending >> b) & 1u)) {
-        timed_out = !ptx::mbar_wait_bounded(&sm.mma_done[b], (phase >> b) & 1u, kWaitIters);
-        pending &= ~(1u << b);
-        phase ^= 1u << b;
-        if (timed_out) atomicOr(&hdr->status, kStatTimeout);
-      }
-      if (walkers_or(timed_out)) {
-        aborted = true;
-        break;
+    __syncthreads();
+    for (int j0 = 0; j0 < m; j0 += kChunk) {
+      ChunkBuf& cb = sm.buf;
+      // the MMAs that last read the buffer have completed (every thread waits)
+      if (issued > 0 && !ptx::mbar_wait_bounded(&sm.mma_done, (uint32_t)(issued - 1) & 1u, kWaitIters)) {
+        atomicOr(&hdr->status, kStatTimeout);
+        *(volatile int*)&sm.abort = 1;
       }
 #pragma unroll
       for (int q = 0; q < kPer; ++q) {
-        if (wrote2[q] != kNone) {
-          *reinterpret_cast<uint16_t*>(cb.w[0] + wrote2[q]) = 0;
-          *reinterpret_cast<uint16_t*>(cb.w[1] + wrote2[q]) = 0;
+        if (wrote[q] != kNone) {
+          *reinterpret_cast<uint16_t*>(cb.w[0] + wrote[q]) = 0;
+          *reinterpret_cast<uint16_t*>(cb.w[1] + wrote[q]) = 0;
         }
-        wrote2[q] = wrote[q];
         wrote[q] = kNone;
       }
-      const bool any = walk_chunk<KT>(sm, j0, m, wbase, (float)px, (float)py, T, Tout, last, n_eval, n_contrib, held[0],
+      const bool any = walk_chunk<KT>(sm, j0, m, wbase, (float)px, (float)py, T, Tout, last, n_eval, n_contrib, held,
                                       cb.e[0][half] + core_off(row, 0), cb.e[1][half] + core_off(row, 0));
-      const unsigned swap = held[0];  // of this buffer; the next chunk takes the other one
-      held[0] = held[1];
-      held[1] = swap;
       const unsigned wany = __ballot_sync(0xffffffffu, any);
       if (lane == 0) sm.any_e[warp] = wany != 0u;
-      walkers_sync();
+      __syncthreads();
+      if (*(volatile int*)&sm.abort) {  // set before the barrier
+        aborted = true;
+        break;
+      }
       const bool any0 = (sm.any_e[0] | sm.any_e[1] | sm.any_e[2] | sm.any_e[3]) != 0;
       const bool any1 = (sm.any_e[4] | sm.any_e[5] | sm.any_e[6] | sm.any_e[7]) != 0;
       if (any0 || any1) {
+        // the accumulator: allocated late, so that the SM's other CTA orders,
+        // stages and walks while this one holds all of tensor memory
+        if (acc_init == 0u && warp == 0) {
+          ptx::tmem_alloc(&sm.tmem, cols);
+          ptx::tmem_relinquish();
+          ptx::tc_fence_before();
+        }
         // W (hi, lo): entry (atom, Gaussian)
 #pragma unroll
         for (int q = 0; q < kPer; ++q) {
@@ -482,47 +412,50 @@ __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
         }
       }
       ptx::fence_async_shared();  // E and W are read by the tensor core (async proxy)
-      const bool open = walkers_or(T >= 1e-4f);
-      // hand the chunk to the MMA warp (thread 0's control words are
-      // published by its own arrival)
-      if (tid == 0) {
-        sm.ctl[b][0] = any0 ? 1 : 0;
-        sm.ctl[b][1] = any1 ? 1 : 0;
-        sm.ctl[b][2] = 0;
-        pending |= 1u << b;
+      const bool open = __syncthreads_or(T >= 1e-4f);
+      if (any0 || any1) {
+        if (warp == 0) {
+          // the warp builds the descriptors together (uniform registers), lane 0 issues
+          ptx::tc_fence_after();
+          const uint32_t idesc = ptx::idesc_bf16_f32(128, Np), tmem = *(volatile uint32_t*)&sm.tmem;
+          const uint64_t eb = ptx::smem_desc_kmajor_none(ptx::smem_u32(cb.e[0][0]), kLBO, kSBO);
+          const uint64_t wb = ptx::smem_desc_kmajor_none(ptx::smem_u32(cb.w[0]), kLBO, kSBO);
+          if (lane == 0) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              if (!(h ? any1 : any0)) continue;
+              const uint32_t d = tmem + (uint32_t)h * half_cols;
+#pragma unroll
+              for (int pass = 0; pass < 3; ++pass)
+#pragma unroll
+                for (int ks = 0; ks < kChunk / 16; ++ks)
+                  ptx::mma_f16(d, eb + ((((pass == 2 ? 2 : 0) + h) * kEBytes + ks * 2 * (int)kLBO) >> 4),
+                               wb + (((pass == 1 ? kWBytes : 0) + ks * 2 * (int)kLBO) >> 4), idesc,
+                               (((acc_init >> h) & 1u) || pass > 0 || ks > 0) ? 1u : 0u);
+            }
+            ptx::mma_commit(&sm.mma_done);
+          }
+          __syncwarp();
+        }
+        acc_init |= (any0 ? 1u : 0u) | (any1 ? 2u : 0u);
+        ++issued;
       }
-      ptx::mbar_arrive(&sm.ready[b]);
-      acc_init |= (any0 ? 1u : 0u) | (any1 ? 2u : 0u);
       if (!open) {
         all_done = true;
-        ++chunk;  // the stop goes to the next chunk
         break;
       }
     }
     wbase += m;
   }
 
-  // stop the MMA warp: the stop travels on the next chunk's buffer, once the
-  // MMA warp has taken that buffer's previous chunk; then every MMA has
-  // completed before the accumulator is read and TMEM freed
+  // every MMA has completed before the accumulator is read and TMEM freed
   bool fin_ok = true;
-  {
-    const int b = chunk & 1;
-    if (tid == 0) {
-      if ((pending >> b) & 1u) {
-        fin_ok = ptx::mbar_wait_bounded(&sm.mma_done[b], (phase >> b) & 1u, kWaitIters);
-        pending &= ~(1u << b);
-        phase ^= 1u << b;
-      }
-      sm.ctl[b][2] = 1;
-    }
-    ptx::mbar_arrive(&sm.ready[b]);
-  }
-  if (tid == 0) {
-    fin_ok = ptx::mbar_wait_bounded(&sm.fin, 0u, kWaitIters) && fin_ok;
+  if (tid == 0 && issued > 0) {
+    fin_ok = ptx::mbar_wait_bounded(&sm.mma_done, (uint32_t)(issued - 1) & 1u, kWaitIters);
     if (!fin_ok) atomicOr(&hdr->status, kStatTimeout);
   }
-  const bool bad = walkers_or(!fin_ok) || aborted;
+  const bool bad = __syncthreads_or(!fin_ok) || aborted;
+  const uint32_t tmem = *(volatile uint32_t*)&sm.tmem;  // with acc_init only
   ptx::tc_fence_after();
 
   // epilogue: each thread reads its own pixel's row (TMEM lane)
@@ -530,16 +463,16 @@ __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
   const uint32_t tb = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)half * half_cols;
   const int64_t pix = (int64_t)py * cam.width + px;
   const bool have = ((acc_init >> half) & 1u) && !bad;  // uniform over the warp
-  // Rows that split into 512-byte pieces (bf16 with C a multiple of 256, FP32
-  // with C a multiple of 128) go through shared memory: the warp stages one
+  // Rows that split into 256-byte pieces (bf16 with C a multiple of 128, FP32
+  // with C a multiple of 64) go through shared memory: the warp stages one
   // piece of each of its 32 pixel rows (16-byte chunks XOR-swizzled by row,
   // so neither the staging stores nor the reads conflict) in the chunk
-  // buffers, free once the last MMA has completed, and writes every row's
-  // piece with one coalesced warp store; other rows are stored per thread.
+  // buffer, free once the last MMA has completed, and writes two rows'
+  // pieces with each coalesced warp store; other rows are stored per thread.
   const int esz = out_bf16 ? 2 : 4;
-  const int piece_cols = 512 / esz;
+  const int piece_cols = kPieceBytes / esz;
   if (!bad && C == Np && C % piece_cols == 0 && ((uintptr_t)out & 15u) == 0) {
-    unsigned char* stg = reinterpret_cast<unsigned char*>(&sm.buf[0]) + warp * 16384;
+    unsigned char* stg = reinterpret_cast<unsigned char*>(&sm.buf) + warp * 32 * kPieceBytes;
     for (int p0 = 0; p0 < Np; p0 += piece_cols) {
       for (int c0 = p0; c0 < p0 + piece_cols; c0 += 32) {
         float v[32];
@@ -553,24 +486,25 @@ __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
         if (out_bf16) {
 #pragma unroll
           for (int j = 0; j < 4; ++j)
-            *reinterpret_cast<uint4*>(stg + lane * 512 + (((k0 + j) ^ lane) & 31) * 16) =
+            *reinterpret_cast<uint4*>(stg + lane * kPieceBytes + (((k0 + j) ^ lane) & 15) * 16) =
                 make_uint4(pack2_bf16(v[8 * j], v[8 * j + 1]), pack2_bf16(v[8 * j + 2], v[8 * j + 3]),
                            pack2_bf16(v[8 * j + 4], v[8 * j + 5]), pack2_bf16(v[8 * j + 6], v[8 * j + 7]));
         } else {
 #pragma unroll
           for (int j = 0; j < 8; ++j)
-            *reinterpret_cast<float4*>(stg + lane * 512 + (((k0 + j) ^ lane) & 31) * 16) =
+            *reinterpret_cast<float4*>(stg + lane * kPieceBytes + (((k0 + j) ^ lane) & 15) * 16) =
                 make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
         }
       }
       __syncwarp();
-#pragma unroll 8
-      for (int r = 0; r < 32; ++r) {
-        const uint4 val = *reinterpret_cast<const uint4*>(stg + r * 512 + ((lane ^ r) & 31) * 16);
+#pragma unroll 4
+      for (int r0 = 0; r0 < 32; r0 += 2) {
+        const int r = r0 + (lane >> 4), ch = lane & 15;
+        const uint4 val = *reinterpret_cast<const uint4*>(stg + r * kPieceBytes + ((ch ^ r) & 15) * 16);
         const int rx = wx + (r & 7), ry = wy + (r >> 3);
         if (rx < cam.width && ry < cam.height)
           *reinterpret_cast<uint4*>(reinterpret_cast<unsigned char*>(out) +
-                                    ((int64_t)ry * cam.width + rx) * (int64_t)C * esz + p0 * esz + lane * 16) = val;
+                                    ((int64_t)ry * cam.width + rx) * (int64_t)C * esz + p0 * esz + ch * 16) = val;
       }
       __syncwarp();
     }
@@ -596,10 +530,9 @@ __global__ void __launch_bounds__(kCtaThreads, 1) render_mma_kernel(
     atomicAdd(&sm.cnt[0], (unsigned long long)we);
     atomicAdd(&sm.cnt[1], (unsigned long long)wc);
   }
-  }  // walkers
   ptx::tc_fence_before();
   __syncthreads();
-  if (warp == 0) ptx::tmem_dealloc(tmem, cols);
+  if (warp == 0 && acc_init != 0u) ptx::tmem_dealloc(tmem, cols);
   if (tid == 0) {
     atomicAdd(&hdr->evaluated, sm.cnt[0]);
     atomicAdd(&hdr->contributions, sm.cnt[1]);
@@ -623,7 +556,7 @@ cudaError_t launch_render_mma(const ViewJob& v, const int32_t* topk_idx,
   const auto kernel = K <= 4 ? render_mma_kernel<4> : K <= 8 ? render_mma_kernel<8> : render_mma_kernel<16>;
   cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
-  kernel<<<ntiles, kCtaThreads, smem, st>>>(v, topk_idx, topk_val, K, C, out, out_bf16, out_T,
+  kernel<<<ntiles, kMThreads, smem, st>>>(v, topk_idx, topk_val, K, C, out, out_bf16, out_T,
                                             out_last);
   g_launches += 1;
   return cudaGetLastError();
