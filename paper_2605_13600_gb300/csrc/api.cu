@@ -186,7 +186,7 @@ size_t carve_view_part(void* base, int64_t n, int max_tiles, UpliftWs* w) {
 // (1M Gaussians, 1080p 1923 / 1949 us, 800x600 745 / 809).  A cut belongs to
 // a block's list.
 bool use_depth_cut(int64_t n, const CamArgs& cam, const UpliftWs& ws, int views) {
-  return ws.zcut && views > 1 && n >= (1 << 18) && list_shift(n, cam.gx, cam.gy) == 1;
+  return ws.zcut && views > 1 && n >= (1 << 18) && list_shift(n, cam.gx, cam.gy, dense_limit(n, true)) == 1;
 }
 
 ViewJob view_job(const scoup_scene& sc, const CamArgs& cam, const UpliftWs& ws, WsHeader* hdr, bool cut) {
@@ -216,7 +216,7 @@ ViewJob view_job(const scoup_scene& sc, const CamArgs& cam, const UpliftWs& ws, 
   v.pix_state = ws.pix_state;
   v.n = (int)sc.n;
   v.group = bin_group(sc.n);
-  v.shift = list_shift(sc.n, cam.gx, cam.gy);
+  v.shift = list_shift(sc.n, cam.gx, cam.gy, dense_limit(sc.n, cut));
   return v;
 }
 

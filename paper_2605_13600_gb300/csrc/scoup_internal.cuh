@@ -247,10 +247,15 @@ struct TileList {
 // (ms, blocks / tiles; Gaussians per tile of the image): 526 2.66 / 2.86, 631
 // 0.90 / 0.87, 2105 1.99 / 1.79, 2560 0.79 / 0.71, 8550 3.68 / 2.49; one
 // render the same way around (526 0.745 / 0.754, 2105 0.73 / 0.68, 8550 1.69 /
-// 1.61).
-constexpr int64_t kDensePerTile = 560;
-__host__ __device__ inline int list_shift(int64_t n, int gx, int gy) {
-  return n < (1ll << 28) && gx >= 4 && gy >= 4 && n <= kDensePerTile * gx * gy ? 1 : 0;
+// 1.61).  Behind the depth cut of a large scene a block's list is short up to
+// a later point (24 views in chunks, cut block lists / tile lists: 1M Gaussians
+// 833 3.15 / 3.85 in blobs and 4.25 / 4.33 uniform, 2105 2.52 / 2.83 and 4.08 /
+// 3.54; 300k Gaussians 631 1.67 / 1.58 and 1.88 / 1.61).
+constexpr int64_t kDensePerTile = 560, kDenseCut = 1400;
+constexpr int64_t kDenseCutFrom = 1 << 19;  // Gaussians
+inline int64_t dense_limit(int64_t n, bool cut) { return cut && n >= kDenseCutFrom ? kDenseCut : kDensePerTile; }
+inline int list_shift(int64_t n, int gx, int gy, int64_t dense) {
+  return n < (1ll << 28) && gx >= 4 && gy >= 4 && n <= dense * gx * gy ? 1 : 0;
 }
 __host__ __device__ inline int list_dim(int g, int shift) { return (g + shift) >> shift; }
 

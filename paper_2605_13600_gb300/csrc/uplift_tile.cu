@@ -140,10 +140,12 @@ struct Buckets {
 
 // f(key) for every key of the list, kLoads loads of a thread in flight at a
 // time: the passes over a list are a thread's serial chain of loads otherwise.
-// One load at a time against 8: 1877 -> 1033 us per 200 x 140 view of 1M
-// Gaussians (about 100k keys to a tile's list, one view at a time), 41.7 ->
-// 40.6 ms for 200 views of 988 x 731 (2k keys).
-constexpr int kLoads = 8;
+// Loads at a time 1 / 4 / 8: 200 views of 988 x 731, 1M Gaussians (2k keys to
+// a tile's list) 41.7 / 40.1 / 40.7 ms, 24 views of 640 x 480, 300k 2.38 / 2.29
+// / 2.32 ms; 24 views of 200 x 140, 1M (100k keys) - / 2.86 / 2.64 ms, and one
+// such view at a time 1877 us with 1, 1033 with 8.  Eight cost registers that
+// the walk then spills.
+constexpr int kLoads = 4;
 template <typename F>
 __device__ __forceinline__ void for_keys(const TileList& l, F f) {
   const unsigned long long* __restrict__ const keys = l.keys;
