@@ -163,6 +163,13 @@ def peaks():
     return {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "sm_max_mhz": 2070.0, "source": "fallback"}
 
 
+def make_uplift(gb, wl, dev, per_view: bool, **kw):
+    """An Uplift in the chunked form, or one that composites one view at a time
+    (run() takes chunks by itself where their workspace is at most CHUNK_BYTES)."""
+    cls = type("PerViewUplift", (gb.Uplift,), {"CHUNK_BYTES": 0}) if per_view else gb.Uplift
+    return cls(wl, device=str(dev), chunked=not per_view, **kw)
+
+
 def profiled_traffic(kernel: str, source: str):
     """DRAM bytes per launch of `kernel` from its committed ncu summary, or None
     when the summary is missing or was taken on a different source file."""
@@ -275,7 +282,7 @@ def run_gb300(args, dist):
     wl = synth.uplift_cfg2(device=str(dev), V=args.views)
     # the chunked form (SCOUP_UPLIFT_CHUNKED): chunks of 8 views on two lanes,
     # one persistent tile launch per chunk
-    up = gb.Uplift(wl, device=str(dev), chunked=not args.per_view)
+    up = make_uplift(gb, wl, dev, args.per_view)
     st0 = up.run(stats=True)
     if st0["status"] != 0:
         raise RuntimeError(f"uplift status {st0['status']}")
@@ -368,14 +375,15 @@ def run_gb300(args, dist):
     prof = gb.scoup_profile_read()
     gb.scoup_profile_enable(False)
     step_ms = {k: v[0] / 2 for k, v in prof.items()}
-    tiles_ms, tiles_n = prof.get("uplift_tiles", (0.0, 1))
-    per_launch_s = tiles_ms / tiles_n / 1e3
-
     # roofline of the dominant kernel (per-tile composite + scatter: one drain
-    # launch per chunk of views, or one launch per view in the per-view form)
+    # launch per chunk of 8 views, with the drain of its tiles still open behind
+    # the depth cut counted to it, or one launch per view in the per-view form)
     pk = peaks()
     V = len(up.cams)
-    views_per_launch = V / (tiles_n / 2)
+    tiles_ms = prof.get("uplift_tiles", (0.0, 1))[0]
+    chunks = V if args.per_view else (V + 7) // 8
+    per_launch_s = tiles_ms / 2 / chunks / 1e3
+    views_per_launch = V / chunks
     evaluated_per_launch = st0["evaluated_pairs"] / V * views_per_launch
     # FP32-pipe work of Eq. 2 for every evaluated Gaussian-pixel pair, accepted
     # or not (a lower bound for any implementation; the exp runs on the SFU and
@@ -391,8 +399,8 @@ def run_gb300(args, dist):
     # algorithmic HBM bytes of one view: region map + one FP32 read-modify-write per
     # accumulator update issued + one 32-byte record per visible Gaussian
     bytes_launch = (4.0 * npx + 8.0 * st0["atomics"] / V + 32.0 * st0["visible"] / V) * views_per_launch
-    kname = "uplift_tile_kernel" if args.per_view else "uplift_drain_kernel"
-    traffic = profiled_traffic(kname, "uplift_tile.cu")
+    kname = "uplift_drain_kernel"
+    traffic = None if args.per_view else profiled_traffic(kname, "uplift_tile.cu")
     roofline = {"kernel": kname, "views_per_launch": views_per_launch, "bound": "alu", "achieved": achieved / 1e12,
                 "peak": alu_peak / 1e12, "unit": "Tops/s (FP32 lane ops)",
                 "frac": achieved / alu_peak, "traffic": traffic,
@@ -408,7 +416,7 @@ def run_gb300(args, dist):
     # the other form on the same workload, for comparison (not the headline)
     other = None
     if not args.no_form_compare:
-        upo = gb.Uplift(wl, device=str(dev), dup_capacity=up.dup_capacity, chunked=args.per_view)
+        upo = make_uplift(gb, wl, dev, not args.per_view, dup_capacity=up.dup_capacity)
         so = upo.run(stats=True)
         if so["status"] != 0 or so["contributions"] != contrib:
             raise RuntimeError("the two uplift forms disagree on the contributions")
