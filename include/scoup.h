@@ -134,11 +134,12 @@ int scoup_uplift_plan(const scoup_scene* scene, const scoup_camera* cams, int32_
  *               as does the product code value x weight; Top-K ranks
  *               sum + term.  Slower (one more atomic per update).
  *               SCOUP_UPLIFT_CHUNKED (the fast form; single level): the
- *               views are cut into chunks of 8 on two lanes (streams); each
- *               view of a chunk is projected and binned into a view part of
- *               its own, then ONE persistent tile launch composites every
- *               (view, tile) item of the chunk, its CTAs taking items from
- *               an atomic counter.  Same results up to the order of FP32
+ *               views are cut into chunks of 8 on two lanes (streams); the
+ *               views of a chunk are projected and binned into view parts of
+ *               their own, one launch per stage, then a persistent tile
+ *               launch composites every (view, tile) item of the chunk, its
+ *               CTAs taking items from an atomic counter (large scenes: a
+ *               second one resumes the tiles still open behind a depth cut).  Same results up to the order of FP32
  *               atomic additions; same counters.  The workspace must then be
  *               sized by scoup_uplift_chunked_workspace_size (16 view parts).
  *  topk_idx     int32 [n, K] or NULL (accumulate only); topk_val float32 [n, K].

@@ -211,6 +211,7 @@ struct SceneP {
 // is still open at its cut is recorded, with its pixels' state, and a second
 // pass lists what lies behind the cut for the recorded tiles alone.  The
 // estimate decides speed only: every tile sees its whole list, in order.
+// Taken by the uplift's chunks of views of large scenes (use_depth_cut).
 constexpr int kCutBins = 512;                // 64 per octave of depth, from 0.2 up
 constexpr uint32_t kCutBase = 0x3E4CCCCDu;   // bits of 0.2f
 constexpr int kCutShift = 17;
@@ -227,7 +228,7 @@ __host__ __device__ inline int open_words(int gx) { return (cut_blocks(gx) + 31)
 // rectangle meets (bit (ty & 1) * 2 + (tx & 1)).  Views less than 4 tiles wide
 // or high, where blocks save nothing, and scenes of 2^28 Gaussians, whose
 // index leaves no room for the bits, have one list per tile and no bits
-// (shift 0).
+// (shift 0), and so have images dense in Gaussians (list_shift).
 struct TileList {
   const unsigned long long* keys;
   int n;             // keys of the list; those of the tile are among them

@@ -42,8 +42,8 @@ struct OrderSmem {
   int sel_digit, sel_rank, win_b1;
 };
 
-// Depths [lo, lo + span] over nb buckets, monotone in the key; keys behind the
-// tile's depth cut go to nb, which no window takes.
+// Depths [lo, lo + span] over nb buckets, monotone in the key; other tiles'
+// keys go to nb, which no window takes.
 struct OrderBuckets {
   uint32_t lo, span;
   int shift;
