@@ -211,10 +211,12 @@ __global__ void __launch_bounds__(256) project_kernel(const __grid_constant__ Vi
 // of that.  1M blob Gaussians, 988x731 (4249 listed per tile without a cut):
 // 739 listed per tile and 0.9% of the tiles open at 24, 826 and 0.1% at 28, 912
 // and none at 32, 1066 at 40 (1920x1080: 3.5, 1.8, 0.8, 0.1% open).  With
-// half the sample (1 << 17, of 1M) 5.3% were open at 24 and 1.4% at 32.
+// half the sample (1 << 17, of 1M) 5.3% were open at 24 and 1.4% at 32.  Few
+// open tiles already cost a chunk its second pass (the 8 views of a chunk share
+// it): 200 views 40.3 ms at 32, 39.0 at 42, 39.6 at 56.
 constexpr int kCutSample = 1 << 18;      // Gaussians sampled per view, about
 constexpr float kMassUnit = 4.0f;        // histogram units per pixel of optical depth 1
-constexpr float kCutOptical = 32.0f;     // mean optical depth of a block at its cut
+constexpr float kCutOptical = 42.0f;     // mean optical depth of a block at its cut
 constexpr float kBlockPixels = 4.0f * kTilePixels;
 
 template <int N>
