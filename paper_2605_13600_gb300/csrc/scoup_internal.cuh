@@ -59,39 +59,6 @@ struct __align__(16) ProjRec {
   float4 b;
 };
 
-// Conservative test: can any pixel centre of the box [x0, x0+w-1] x
-// [y0, y0+h-1] reach power >= tau for this record?  The maximum of the concave
-// exponent over the box is at the clamped centre or on one of the four edges
-// (each a 1D concave quadratic with its vertex clamped to the edge); the box
-// is rejected only if that maximum is below tau by a margin far above the
-// binary32 rounding of either evaluation, so a rejected box holds no pixel
-// that passes the per-pixel alpha test.
-__device__ __forceinline__ bool box_may_hit(const ProjRec& r, float x0, float y0, float w, float h) {
-  const float mx = r.a.x, my = r.a.y, qa = r.a.z, qb = r.a.w, qc = r.b.x, tau = r.b.z;
-  if (!(qa < 0.0f && qc < 0.0f)) return true;
-  const float x1 = x0 + (w - 1.0f), y1 = y0 + (h - 1.0f);
-  if (mx >= x0 && mx <= x1 && my >= y0 && my <= y1) return true;
-  // argmax over dy along an edge x = const (dy = kx * dx) and over dx along an
-  // edge y = const (dx = ky * dy); an approximate quotient only moves the
-  // evaluation point slightly on a flat maximum, far inside the margin below
-  const float kx = __fdividef(-qb, 2.0f * qc);
-  const float ky = __fdividef(-qb, 2.0f * qa);
-  float best = -INFINITY;
-#pragma unroll
-  for (int e = 0; e < 2; ++e) {
-    const float dx = mx - (e ? x1 : x0);
-    const float dy = my - fminf(y1, fmaxf(y0, my - kx * dx));
-    best = fmaxf(best, qa * dx * dx + qb * dx * dy + qc * dy * dy);
-  }
-#pragma unroll
-  for (int e = 0; e < 2; ++e) {
-    const float dy = my - (e ? y1 : y0);
-    const float dx = mx - fminf(x1, fmaxf(x0, mx - ky * dy));
-    best = fmaxf(best, qa * dx * dx + qb * dx * dy + qc * dy * dy);
-  }
-  return best >= tau - (0.01f + 1e-3f * fabsf(best));
-}
-
 // Conservative test of a whole grid of boxes at once: bit r * kCols + c is
 // set when box (c, r) -- pixels x0 + c w .. x0 + c w + w - 1 by
 // y0 + r h .. y0 + r h + h - 1 -- may hold a pixel centre with power >= tau.
