@@ -84,8 +84,8 @@ __device__ __forceinline__ void store8(float* p, const float (&x)[8]) {
   reinterpret_cast<float4*>(p)[1] = make_float4(x[4], x[5], x[6], x[7]);
 }
 
-// Rows of D features, D a multiple of 8 and both matrices 16-byte aligned: a
-// warp takes a row, eight features per lane and step, so that a 512-feature
+// Rows of D features, D a multiple of 8, both matrices and the targets 16-byte
+// aligned: a warp takes a row, eight features per lane and step, so that a 512-feature
 // bf16 row is two 16-byte loads and stores per lane.  Bound by HBM: read and
 // write once (480k x 512 bf16, 983 MB: 200 us with a feature per lane and
 // step, 174 now).
@@ -176,7 +176,8 @@ cudaError_t launch_l2_grad(const void* F, int F_bf16, int64_t P, int D, const in
                            const float* target, void* dF, int dF_bf16, double* loss, int* status, cudaStream_t st) {
   if (P <= 0) return cudaSuccess;
   const int b = blocks_for_warps(P);
-  if (D % 8 == 0 && (((uintptr_t)F | (uintptr_t)dF) & 15u) == 0) {  // target is the workspace's, aligned
+  // the targets lie in the caller's workspace, which may start at any 4-byte boundary
+  if (D % 8 == 0 && (((uintptr_t)F | (uintptr_t)dF | (uintptr_t)target) & 15u) == 0) {
     auto run = [&](auto* f, auto* d) {
       l2_grad_vec_kernel<<<b, 256, 0, st>>>(f, P, D, rmap, R, target, d, loss, status);
     };
