@@ -24,7 +24,9 @@
 //   kOutCos  : f32 output / (|row| |column|), 0 where |row| < 1e-12
 // Every mbarrier wait is bounded; a wait that gives up records an error in
 // *status, raises the CTA's abort flag, and every role leaves after draining
-// its own copies in flight; TMEM is freed on every path.
+// its own copies in flight; TMEM is freed on every path.  A role's loop is left
+// by whole warps: the lanes vote on each wait and on the flag, so that no lane
+// stays behind at a warp barrier that another one has skipped.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -61,12 +63,17 @@ struct GemmSmem {
   volatile int abort;
 };
 
+// Both are called by whole warps and give every lane the same answer: lanes
+// poll the barrier and read the flag on their own, and one of them may see what
+// the next one has just missed.
 __device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abort, int* status) {
-  if (ptx::mbar_wait_bounded(bar, parity, kWaitIters)) return true;
+  if (__all_sync(0xffffffffu, ptx::mbar_wait_bounded(bar, parity, kWaitIters))) return true;
   atomicOr(status, kStatTimeout);
   *abort = 1;
   return false;
 }
+
+__device__ __forceinline__ bool gave_up(const volatile int* abort) { return __any_sync(0xffffffffu, *abort != 0); }
 
 // acc += the squares of the two bf16 values of w (one packed FP32 FMA).
 __device__ __forceinline__ void add_squares(uint32_t w, unsigned long long& acc) {
@@ -248,7 +255,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_kernel(const __grid
     // ---- TMA producer: the warp runs the loop together, so that addresses
     // and coordinates stay in uniform registers, and lane 0 issues ----
     int it = 0;
-    for (int i = 0; !sm.abort && !ep.stall_loads; ++i) {
+    for (int i = 0; !ep.stall_loads && !gave_up(&sm.abort); ++i) {
       const UnitPos t = unit_at<BN, kQuery>(i, n_tiles, m_blocks);
       if (!t.valid) break;
       const CUtensorMap* mb = t.query ? &tmG : &tmB;
@@ -275,7 +282,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_kernel(const __grid
     const uint64_t da0 = ptx::smem_desc_k128(ptx::smem_u32(sm.a[0])), db0 = ptx::smem_desc_k128(ptx::smem_u32(sm.b[0]));
     int it = 0, local = 0;
     bool ok = true;
-    for (int i = 0; ok && !sm.abort; ++i, ++local) {
+    for (int i = 0; ok && !gave_up(&sm.abort); ++i, ++local) {
       const UnitPos t = unit_at<BN, kQuery>(i, n_tiles, m_blocks);
       if (!t.valid) break;
       const uint32_t id = t.query ? idesc_q : idesc;
@@ -316,7 +323,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_kernel(const __grid
     const bool norms = fused || ep.rownorm2;
     int local = 0, sbuf = 0, ex = 0;      // ex: units whose norms the groups have exchanged
     float ss_row = 0.0f;  // fused query: squared norm of the row's rounded outputs over its row block
-    for (int i = 0; !sm.abort; ++i, ++local) {
+    for (int i = 0; !gave_up(&sm.abort); ++i, ++local) {
       const UnitPos t = unit_at<BN, kQuery>(i, n_tiles, m_blocks);
       if (!t.valid) break;
       const int m0 = t.m0, n0 = t.query ? 0 : t.n0;
@@ -530,8 +537,8 @@ __global__ void __launch_bounds__(RowsCfg<kF32A>::kThreads, 1)
     // ---- TMA producer (see above): the units of every row block, a slab of A
     // ahead of the first unit that needs it ----
     int ia = 0, it = 0;
-    bool ok = true;
-    for (int rb = blockIdx.x; ok && rb < blocks && !sm.abort; rb += (int)gridDim.x) {
+    bool ok = !ep.stall_loads;
+    for (int rb = blockIdx.x; ok && rb < blocks && !gave_up(&sm.abort); rb += (int)gridDim.x) {
       const int m0 = rb * kRows, next = rb + (int)gridDim.x;
       for (int u = 0; ok && u < per; ++u) {
         const bool query = kQuery && u == 0;
@@ -582,7 +589,7 @@ __global__ void __launch_bounds__(RowsCfg<kF32A>::kThreads, 1)
     const uint64_t da0 = ptx::smem_desc_k128(ptx::smem_u32(sm.a[0][0])), db0 = ptx::smem_desc_k128(ptx::smem_u32(sm.b[0]));
     int ia = 0, it = 0, local = 0;
     bool ok = true;
-    for (int rb = blockIdx.x; ok && rb < blocks && !sm.abort; rb += (int)gridDim.x, ia += kt) {
+    for (int rb = blockIdx.x; ok && rb < blocks && !gave_up(&sm.abort); rb += (int)gridDim.x, ia += kt) {
       for (int u = 0; ok && u < per; ++u, ++local) {
         const uint32_t id = kQuery && u == 0 ? idesc_q : idesc;
         const int b = local % kAcc, use = local / kAcc;
@@ -631,7 +638,7 @@ __global__ void __launch_bounds__(RowsCfg<kF32A>::kThreads, 1)
     unsigned char* const rowp = buf + lane * 128;
     int local = 0;
     bool ok = true;
-    for (int rb = blockIdx.x, j = 0; ok && rb < blocks && !sm.abort; rb += (int)gridDim.x, ++j) {
+    for (int rb = blockIdx.x, j = 0; ok && rb < blocks && !gave_up(&sm.abort); rb += (int)gridDim.x, ++j) {
       // one half to a block: the lead group takes the first half of each
       // column tile, gathers the row norms and does the query unit; the groups
       // lead by turns.  Two halves: each group leads its own rows.
@@ -734,7 +741,7 @@ __global__ void __launch_bounds__(RowsCfg<kF32A>::kThreads, 1)
     const int t = threadIdx.x - 32 * (2 + kEpiWarps), team = t / kTeam, rt = (t % kTeam) >> 4, ct = (t & 15) * 4;
     int ia = 0;
     bool ok = true;
-    for (int rb = blockIdx.x; ok && rb < blocks && !sm.abort; rb += (int)gridDim.x) {
+    for (int rb = blockIdx.x; ok && rb < blocks && !gave_up(&sm.abort); rb += (int)gridDim.x) {
       const int m0 = rb * kRows, next = rb + (int)gridDim.x;
       if (t == 0 && next < blocks) {
         const int rows = min(kRows, ep.M - next * kRows);
@@ -1077,35 +1084,48 @@ cudaError_t launch_row_norm_bf16(const void* X, int64_t R, int D, float* out, in
 
 bool gemm_tma_available() { return encode_fn() != nullptr; }
 
-// Runs a 128 x 64 x 64 GEMM whose producer issues no loads: the MMA and
+// Runs small GEMMs whose producer issues no loads, one in each form of the two
+// kernels (plain and with the query unit, bf16 and FP32 rows): the MMA and
 // epilogue warps' bounded waits run out, the kernel records kStatTimeout and
-// frees its TMEM, and the context stays usable.  Returns the device status.
+// frees its TMEM, and the context stays usable.
 int gemm_timeout_selftest(void* workspace, size_t ws_bytes, cudaStream_t st) {
-  const size_t need = 256 + 3 * (size_t)128 * 64 * 2;
-  if (!workspace || ws_bytes < need || ((uintptr_t)workspace & 255u)) return SCOUP_ERR_INVALID_ARG;
+  constexpr int M = 16, N = 144, K = 64, Q = 16;
+  constexpr size_t kA = 256, kB = kA + (size_t)M * K * 4, kG = kB + (size_t)N * K * 2, kNorm = kG + (size_t)Q * K * 2,
+                   kSim = kNorm + 256, kOut = kSim + (size_t)M * Q * 4, need = kOut + (size_t)M * N * 2;
+  static_assert(need <= 49408, "the documented workspace");
+  if (!workspace || ws_bytes < 49408 || ((uintptr_t)workspace & 255u)) return SCOUP_ERR_INVALID_ARG;
   char* w = (char*)workspace;
-  int* status = (int*)w;
-  void* A = w + 256;
-  void* B = (char*)A + 128 * 64 * 2;
-  void* out = (char*)B + 128 * 64 * 2;
-  if (cudaMemsetAsync(w, 0, need, st) != cudaSuccess) return SCOUP_ERR_CUDA;
   GemmEpi ep;
-  ep.M = 128;
-  ep.N = 64;
-  ep.K = 64;
+  ep.M = M;
+  ep.N = N;
+  ep.K = K;
   ep.mode = kOutBF16;
-  ep.out = out;
-  ep.ldo = 64;
+  ep.out = w + kOut;
+  ep.ldo = N;
   ep.rownorm2 = nullptr;
-  ep.colnorm = nullptr;
-  ep.status = status;
+  ep.colnorm = (const float*)(w + kNorm);
+  ep.status = (int*)w;
   ep.stall_loads = 1;
-  if (launch_gemm_bf16(A, B, ep, st) != cudaSuccess) return SCOUP_ERR_CUDA;
-  int h = 0;
-  if (cudaMemcpyAsync(&h, status, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-      cudaStreamSynchronize(st) != cudaSuccess)
-    return SCOUP_ERR_CUDA;
-  return (h & kStatTimeout) ? SCOUP_ERR_TIMEOUT : SCOUP_OK;
+  GemmEpi eq = ep;
+  eq.sim_n = Q;
+  eq.sim_mode = kOutCos;
+  eq.sim_out = w + kSim;
+  eq.sim_ldo = Q;
+  const void *A = w + kA, *B = w + kB, *G = w + kG;
+  for (int form = 0; form < 5; ++form) {
+    if (cudaMemsetAsync(w, 0, need, st) != cudaSuccess) return SCOUP_ERR_CUDA;
+    const cudaError_t e = form == 0   ? launch_bn<256>(A, B, nullptr, ep, st)
+                          : form == 1 ? launch_bn<256>(A, B, G, eq, st)
+                          : form == 2 ? launch_rows<true, false>(A, B, G, eq, st)
+                          : form == 3 ? launch_rows<false, true>(A, B, nullptr, ep, st)
+                                      : launch_rows<true, true>(A, B, G, eq, st);
+    int h = 0;
+    if (e != cudaSuccess || cudaMemcpyAsync(&h, w, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaStreamSynchronize(st) != cudaSuccess)
+      return SCOUP_ERR_CUDA;
+    if (!(h & kStatTimeout)) return SCOUP_OK;
+  }
+  return SCOUP_ERR_TIMEOUT;
 }
 
 }  // namespace scoup
