@@ -693,8 +693,10 @@ class Uplift:
             del probe
         self.dup_capacity = dup_capacity
         self.chunked = bool(chunked)
+        # a view part of the chunked form holds keys or is refused: no capacity, no chunks
         self._chunk_views = self.chunked or (
-            len(self.cams) > 1 and scoup_uplift_chunked_workspace_size(n, maxw, maxh, dup_capacity) <= self.CHUNK_BYTES)
+            len(self.cams) > 1 and dup_capacity > 0 and
+            scoup_uplift_chunked_workspace_size(n, maxw, maxh, dup_capacity) <= self.CHUNK_BYTES)
         size = scoup_uplift_chunked_workspace_size if self._chunk_views else scoup_uplift_workspace_size
         self.workspace = torch.empty(size(n, maxw, maxh, dup_capacity) + extra, dtype=torch.uint8, device=dev)
         self.maxw, self.maxh, self.extra, self.device = maxw, maxh, extra, dev
