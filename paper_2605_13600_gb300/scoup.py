@@ -658,6 +658,7 @@ class Uplift:
     # about 4 GB.  24 views of 1M at 988x731, one view at a time / in chunks:
     # 6.1 / 5.1 ms; of 300k 4.5 / 4.0 ms.
     CHUNK_BYTES = 1 << 33
+    _chunk_alone = True  # False: run() takes the chunked form only when asked for
 
     def __init__(self, wl, device: str = "cuda", dup_capacity: Optional[int] = None,
                  headroom: float = 1.0, compensated: bool = False, topk: bool = True, chunked: bool = False):
@@ -695,7 +696,7 @@ class Uplift:
         self.chunked = bool(chunked)
         # a view part of the chunked form holds keys or is refused: no capacity, no chunks
         self._chunk_views = self.chunked or (
-            len(self.cams) > 1 and dup_capacity > 0 and
+            self._chunk_alone and len(self.cams) > 1 and dup_capacity > 0 and
             scoup_uplift_chunked_workspace_size(n, maxw, maxh, dup_capacity) <= self.CHUNK_BYTES)
         size = scoup_uplift_chunked_workspace_size if self._chunk_views else scoup_uplift_workspace_size
         self.workspace = torch.empty(size(n, maxw, maxh, dup_capacity) + extra, dtype=torch.uint8, device=dev)
@@ -753,6 +754,12 @@ class Uplift:
         return self.accum
 
 
+class _LevelBase(Uplift):
+    """The scene, views and workspace of a LevelUplift: scoup_uplift_levels runs one
+    view at a time on two streams and has no use for the chunked form's view parts."""
+    _chunk_alone = False
+
+
 class LevelUplift:
     """L semantic levels (workloads sharing scene, cameras and map offsets) uplifted
     in one pass through scoup_uplift_levels.  accum is [n, L*C] (level l in
@@ -764,7 +771,7 @@ class LevelUplift:
         self.wls = list(wls)
         self.L = len(self.wls)
         base = self.wls[0]
-        self.base = Uplift(base, device=device, dup_capacity=dup_capacity, topk=False)
+        self.base = _LevelBase(base, device=device, dup_capacity=dup_capacity, topk=False)
         self.C, self.K = int(base.C), int(base.K)
         n = base.scene.n
         self.compensated = bool(compensated)

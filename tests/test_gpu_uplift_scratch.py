@@ -21,3 +21,12 @@ def test_no_capacity_for_views_that_list_nothing(gb):  # noqa: F811
         st = up.run()
         assert st["status"] == 0 and st["visible"] == 0 and st["contributions"] == 0
         assert not up.accum.any() and (up.topk_idx == -1).all()
+
+
+def test_levels_hold_no_view_parts_of_chunks(gb):  # noqa: F811
+    """scoup_uplift_levels runs one view at a time: its workspace is that form's."""
+    base = synth.tiny_workload(3, n=2000, V=4)
+    up = gb.LevelUplift(synth.level_workloads(base, (2, 4, 8)))
+    b = up.base
+    assert b.workspace.numel() == gb.scoup_uplift_workspace_size(b.n, b.maxw, b.maxh, b.dup_capacity)
+    assert up.run()["status"] == 0
