@@ -656,17 +656,21 @@ class Uplift:
     # Largest workspace of the chunked form that run() takes by itself (see
     # __init__): at 1M Gaussians and 1080p eight views on each of two lanes take
     # about 4 GB.  24 views of 1M at 988x731, one view at a time / in chunks:
-    # 6.1 / 5.1 ms; of 300k 4.5 / 4.0 ms.
+    # 6.1 / 5.1 ms; of 300k 4.5 / 4.0 ms.  It is seven times the other form's,
+    # so it is taken only out of plenty: a program that fits beside the small
+    # one keeps the rest of the memory.
     CHUNK_BYTES = 1 << 33
+    CHUNK_SHARE = 0.125  # of the free memory, the Uplift's own arrays allocated
     _chunk_alone = True  # False: run() takes the chunked form only when asked for
 
     def __init__(self, wl, device: str = "cuda", dup_capacity: Optional[int] = None,
                  headroom: float = 1.0, compensated: bool = False, topk: bool = True, chunked: bool = False):
         """chunked=True: run() uses the chunked form (SCOUP_UPLIFT_CHUNKED) and
         the workspace is sized for it.  Otherwise run() still takes that form
-        (same results and counters) where its workspace is at most
-        CHUNK_BYTES and there is more than one view: views of such scenes
-        leave most of the chip idle when composited one at a time."""
+        (same results and counters) where there is more than one view and its
+        workspace is at most CHUNK_BYTES and CHUNK_SHARE of the free memory:
+        views of such scenes leave most of the chip idle when composited one
+        at a time."""
         import torch
         dev = torch.device(device)
         sc = wl.scene
@@ -693,20 +697,36 @@ class Uplift:
             dup_capacity = int(scoup_uplift_plan(self.scene, self.cams, probe) * headroom) + 1
             del probe
         self.dup_capacity = dup_capacity
-        self.chunked = bool(chunked)
-        # a view part of the chunked form holds keys or is refused: no capacity, no chunks
-        self._chunk_views = self.chunked or (
-            self._chunk_alone and len(self.cams) > 1 and dup_capacity > 0 and
-            scoup_uplift_chunked_workspace_size(n, maxw, maxh, dup_capacity) <= self.CHUNK_BYTES)
-        size = scoup_uplift_chunked_workspace_size if self._chunk_views else scoup_uplift_workspace_size
-        self.workspace = torch.empty(size(n, maxw, maxh, dup_capacity) + extra, dtype=torch.uint8, device=dev)
-        self.maxw, self.maxh, self.extra, self.device = maxw, maxh, extra, dev
-        self._host_ws = None
         self.compensated = bool(compensated)
         self.accum = torch.empty(((2, n, self.C) if compensated else (n, self.C)), dtype=torch.float32,
                                  device=dev)
         self.topk_idx = torch.empty((n, self.K), dtype=torch.int32, device=dev) if topk else None
         self.topk_val = torch.empty((n, self.K), dtype=torch.float32, device=dev) if topk else None
+        self.maxw, self.maxh, self.extra, self.device = maxw, maxh, extra, dev
+        self._host_ws = None
+        self.chunked = bool(chunked)
+        need = scoup_uplift_chunked_workspace_size(n, maxw, maxh, dup_capacity) + extra
+        # a view part of the chunked form holds keys or is refused: no capacity, no chunks
+        self._chunk_views = self.chunked or (self._chunk_alone and len(self.cams) > 1 and dup_capacity > 0 and
+                                             need <= self.CHUNK_BYTES and self._has_room(need))
+        if self._chunk_views:
+            try:
+                self.workspace = torch.empty(need, dtype=torch.uint8, device=dev)
+            except torch.cuda.OutOfMemoryError:  # free memory in too many pieces
+                if self.chunked:
+                    raise
+                self._chunk_views = False
+        if not self._chunk_views:
+            self.workspace = torch.empty(scoup_uplift_workspace_size(n, maxw, maxh, dup_capacity) + extra,
+                                         dtype=torch.uint8, device=dev)
+
+    def _has_room(self, need: int) -> bool:
+        """Whether `need` bytes are at most CHUNK_SHARE of the device's free memory
+        (what the caching allocator holds in reserve included)."""
+        import torch
+        free = (torch.cuda.mem_get_info(self.device)[0] + torch.cuda.memory_reserved(self.device)
+                - torch.cuda.memory_allocated(self.device))
+        return need <= self.CHUNK_SHARE * free
 
     def run(self, stats: bool = True, accum_mode: int = 0, views=None, stream=None, topk: bool = True):
         """One uplift; topk=False (or an Uplift built with topk=False) accumulates only."""
