@@ -34,6 +34,7 @@ struct scoup_plan {
   bool tuned = false;
   std::vector<int64_t> max_dups;  // per scene
   std::vector<double> cost;       // per scene
+  int lane_views = 1;             // view parts of a lane workspace
   size_t lane_bytes = 0;          // bytes of one lane workspace
   std::vector<void*> lane_ws;
   std::vector<cudaStream_t> lane_st;
@@ -53,8 +54,12 @@ namespace {
 constexpr int kMaxLanes = 8;
 // Views that a lane composites together (its workspace holds as many view
 // parts): the tiles of one view of a mid-sized scene are two or three waves of
-// the chip.
+// the chip.  Five scenes of 80k to 900k Gaussians, 8 to 12 views of 648 x 484:
+// 6.5 to 7.0 ms with one view at a time, 5.7 with four, for 2.5 GB of lane
+// workspaces in place of 0.8.  One view at a time where the larger ones are
+// more than an eighth of the free memory, or cannot be allocated.
 constexpr int kLaneViews = 4;
+constexpr size_t kLaneShare = 8;
 
 int err(int code, const char* msg) { return set_error(code, msg); }
 
@@ -70,12 +75,32 @@ void drop_graph(scoup_plan* p) {
   p->graph_kernels = 0;
 }
 
+// Sizes the lane workspaces for `views` view parts each.
+void size_lanes(scoup_plan* p, int views) {
+  p->lane_views = views;
+  p->lane_bytes = 0;
+  for (size_t b = 0; b < p->items.size(); ++b) {
+    const scoup_batch_item& it = p->items[b];
+    p->lane_bytes = std::max(p->lane_bytes, uplift_required_bytes(it.scene.n, it.cams, it.V, it.s, p->K, it.R_total,
+                                                                  p->max_dups[b] + 1, views));
+  }
+}
+
 // Lane workspaces, streams and events for `lanes` lanes (grows or shrinks).
 int ensure_lanes(scoup_plan* p, int lanes) {
   cudaError_t e;
   while ((int)p->lane_ws.size() < lanes) {
     void* w = nullptr;
-    if ((e = cudaMalloc(&w, p->lane_bytes)) != cudaSuccess) return cuda_err(e, "lane workspace");
+    if ((e = cudaMalloc(&w, p->lane_bytes)) != cudaSuccess) {
+      if (e != cudaErrorMemoryAllocation || p->lane_views == 1) return cuda_err(e, "lane workspace");
+      // no room for these: all lanes again, one view part each
+      cudaGetLastError();
+      drop_graph(p);
+      const int rc = ensure_lanes(p, 0);
+      if (rc != SCOUP_OK) return rc;
+      size_lanes(p, 1);
+      continue;
+    }
     cudaStream_t s = nullptr;
     if ((e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking)) != cudaSuccess) {
       cudaFree(w);
@@ -144,6 +169,8 @@ ItemView sample_views(const scoup_batch_item& it, int max_views) {
 int enqueue_batch(scoup_plan* p, int lanes, int warp_w, int sample, bool copy_stats, cudaStream_t st,
                   int chunk = 0) {
   cudaError_t e;
+  if (lanes > (int)p->lane_ws.size())
+    return err(SCOUP_ERR_OOM, "the plan's lane workspaces could not be allocated again (scoup_plan_set tries anew)");
   if (chunk > 0) {
     const DrainLayout& d = p->drain;
     if (!d.mem || d.chunk != chunk || d.lanes != lanes || d.sample != sample)
@@ -171,7 +198,7 @@ int enqueue_batch(scoup_plan* p, int lanes, int warp_w, int sample, bool copy_st
       const UpliftCall c{&it.scene, cams, V, it.region_maps, offs, it.R_total, it.code_idx, it.code_val, it.s,
                          p->C, p->K, it.accum, p->accum_mode, it.topk_idx, it.topk_val};
       const WsHeader* hdr = nullptr;
-      const int rc = uplift_call(c, p->lane_ws[l], p->lane_bytes, warp_w, &hdr, ls, 1, kLaneViews);
+      const int rc = uplift_call(c, p->lane_ws[l], p->lane_bytes, warp_w, &hdr, ls, 1, p->lane_views);
       if (rc != SCOUP_OK) return rc;
       if (copy_stats &&
           (e = cudaMemcpyAsync(p->stats_dev + b, hdr, sizeof(WsHeader), cudaMemcpyDeviceToDevice, ls)) !=
@@ -275,11 +302,6 @@ int scoup_plan_create(const scoup_batch_item* items, int32_t B, int32_t C, int32
     delete p;
     return rc;
   }
-  for (int b = 0; b < B; ++b) {
-    const scoup_batch_item& it = p->items[b];
-    p->lane_bytes = std::max(p->lane_bytes, uplift_required_bytes(it.scene.n, it.cams, it.V, it.s, K, it.R_total,
-                                                                  p->max_dups[b] + 1, kLaneViews));
-  }
   if ((e = cudaEventCreateWithFlags(&p->fork_ev, cudaEventDisableTiming)) != cudaSuccess ||
       (e = cudaStreamCreateWithFlags(&p->cap_st, cudaStreamNonBlocking)) != cudaSuccess ||
       (B > 0 && (e = cudaMalloc(&p->stats_dev, sizeof(WsHeader) * (size_t)B)) != cudaSuccess)) {
@@ -291,6 +313,13 @@ int scoup_plan_create(const scoup_batch_item* items, int32_t B, int32_t C, int32
     return cuda_err(e, "memset");
   }
   p->lanes = std::max(1, std::min(4, B));
+  size_t free_bytes = 0, total_bytes = 0;
+  if ((e = cudaMemGetInfo(&free_bytes, &total_bytes)) != cudaSuccess) {
+    scoup_plan_destroy(p);
+    return cuda_err(e, "free memory");
+  }
+  size_lanes(p, kLaneViews);
+  if (p->lane_bytes * (size_t)p->lanes > free_bytes / kLaneShare) size_lanes(p, 1);
   if ((rc = ensure_lanes(p, p->lanes)) != SCOUP_OK) {
     scoup_plan_destroy(p);
     return rc;
