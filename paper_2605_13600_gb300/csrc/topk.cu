@@ -5,16 +5,20 @@
 // registers; the row is read once from HBM (coalesced).  The pass is bound by
 // instruction issue, not by HBM (86% of the issue rate at 27% of the bandwidth
 // before the 32-row spans).
-//  - K <= 16: the K-th largest of the 32 lane maxima
+//  - 3 <= K <= 16: the K-th largest of the 32 lane maxima
 //    (K warp max-reductions of one word) is a lower bound of the row's K-th
 //    entry, so only entries at or above it can be kept, about K + 2 of them;
 //    they are compacted in atom order and each finds its place by counting the
 //    candidates in front of it.  (K rounds of a full arg-max, each a scan of
 //    the lane's entries and two reductions, took 740 us on a 30%-dense 1M x 256
 //    accumulator with the entropy, K = 8; 390 us so.)
-//  - Otherwise, and for a row with more than 32 candidates (many equal
-//    entries): each of the K rounds picks the largest remaining positive entry,
-//    ties to the lower atom index.
+//  - K <= 2, K > 16 (topk_rounds_kernel), and a row with more than 32 candidates
+//    (many equal entries): each of the K rounds picks the largest remaining
+//    positive entry, ties to the lower atom index.  One or two rounds are less
+//    work than the bound and the compaction (us, rounds / candidates: K = 1,
+//    400k x 96 74 / 109, 400k x 256 103 / 122, 60k x 1024 57 / 66; K = 2, 400k x
+//    96 83 / 99, 60k x 384 28 / 33).  Above 16 a warp per row keeps twice the
+//    warps in flight that spans of rows do (60k x 256, K = 24: 128 / 151).
 // With a compensation array (the compensated uplift) each entry is the FP32
 // sum of the running sum and its compensation.  Optionally the same pass
 // writes the entropy of the row's coefficient distribution,
@@ -30,6 +34,23 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 
 constexpr int kFastK = 16;  // largest K of the candidate form
+
+// sum w and sum w log w over the positive entries of the row.
+template <int VPL>
+__device__ __forceinline__ void entropy_sums(const float (&v)[VPL], float& S, float& WL) {
+  S = 0.0f;
+  WL = 0.0f;
+#pragma unroll
+  for (int k = 0; k < VPL; ++k)
+    if (v[k] > 0.0f) {
+      S += v[k];
+      WL = fmaf(v[k], __logf(v[k]), WL);
+    }
+  for (int off = 16; off > 0; off >>= 1) {
+    S += __shfl_xor_sync(kFull, S, off);
+    WL += __shfl_xor_sync(kFull, WL, off);
+  }
+}
 
 // K rounds of arg-max over the row's entries v (in registers).
 template <int VPL>
@@ -54,6 +75,44 @@ __device__ __forceinline__ int topk_rounds(const float (&v)[VPL], int K, int32_t
     sum += bv;
   }
   return r;
+}
+
+// One warp per row, K rounds.
+template <int VPL>
+__global__ void __launch_bounds__(256) topk_rounds_kernel(const float* __restrict__ acc, const float* __restrict__ comp,
+                                                          int64_t n, int C, int64_t ld, int K,
+                                                          int32_t* __restrict__ idx, float* __restrict__ val,
+                                                          float* __restrict__ entropy) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = (int64_t)gridDim.x * 8;
+  for (int64_t row = blockIdx.x * (int64_t)8 + (threadIdx.x >> 5); row < n; row += warps) {
+    const float* a = acc + row * ld;
+    float v[VPL];
+#pragma unroll
+    for (int k = 0; k < VPL; ++k) {
+      const int j = lane + 32 * k;
+      v[k] = j < C ? (comp ? __fadd_rn(a[j], comp[row * ld + j]) : a[j]) : 0.0f;
+    }
+    if (entropy) {
+      float S, WL;
+      entropy_sums<VPL>(v, S, WL);
+      if (lane == 0) entropy[row] = S > 0.0f ? fmaxf(0.0f, logf(S) - WL / S) : 0.0f;
+    }
+    int32_t* orow_i = idx + row * K;
+    float* orow_v = val + row * K;
+    float sum = 0.0f;
+    const int r = topk_rounds<VPL>(v, K, orow_i, orow_v, sum);
+    __syncwarp();
+    for (int k = lane; k < K; k += 32) {
+      if (k < r) {
+        orow_v[k] = orow_v[k] / sum;
+      } else {
+        orow_i[k] = -1;
+        orow_v[k] = 0.0f;
+      }
+    }
+    __syncwarp();
+  }
 }
 
 // A warp takes `span` (<= 32) consecutive rows at a time; the lane of a row in
@@ -88,23 +147,14 @@ __global__ void __launch_bounds__(256) topk_kernel(const float* __restrict__ acc
         else v[k] = lane + 32 * k < C ? (ac ? __fadd_rn(a[32 * k], ac[it * ld + 32 * k]) : a[32 * k]) : 0.0f;
       }
       if constexpr (kEntropy) {
-        float S = 0.0f, WL = 0.0f;
-#pragma unroll
-        for (int k = 0; k < VPL; ++k)
-          if (v[k] > 0.0f) {
-            S += v[k];
-            WL = fmaf(v[k], __logf(v[k]), WL);
-          }
-        for (int off = 16; off > 0; off >>= 1) {
-          S += __shfl_xor_sync(kFull, S, off);
-          WL += __shfl_xor_sync(kFull, WL, off);
-        }
+        float S, WL;
+        entropy_sums<VPL>(v, S, WL);
         if (lane == it) { keep_s = S; keep_wl = WL; }
       }
       float sum = 0.0f;
       int r = 0;
       bool fast = false;
-      if (K <= kFastK) {
+      {
         float m = 0.0f;
 #pragma unroll
         for (int k = 0; k < VPL; ++k) m = fmaxf(m, v[k]);
@@ -113,6 +163,7 @@ __global__ void __launch_bounds__(256) topk_kernel(const float* __restrict__ acc
         for (int q = 0; q < K; ++q) {
           t = __reduce_max_sync(kFull, __float_as_uint(m));  // 0 once fewer than K lanes hold a positive entry
           if (__float_as_uint(m) == t) m = 0.0f;
+          if (!KT && t == 0u) break;
         }
         const float bound = t ? __uint_as_float(t) : 1e-45f;
         int cnt = 0;
@@ -199,8 +250,15 @@ __global__ void code_topk_kernel(const int32_t* __restrict__ ci, const float* __
 template <int VPL, bool kEntropy>
 cudaError_t launch_vpl(const float* acc, const float* comp, int64_t n, int C, int64_t ld, int K, int32_t* idx,
                        float* val, float* entropy, cudaStream_t st) {
-  // 32-row spans once there are enough rows for 32 warps per SM
-  int64_t span = n / (num_sms() * 32);
+  if (K <= 2 || K > kFastK) {
+    const int64_t blocks = (n + 7) / 8 < num_sms() * 16 ? (n + 7) / 8 : num_sms() * 16;
+    topk_rounds_kernel<VPL><<<(int)blocks, 256, 0, st>>>(acc, comp, n, C, ld, K, idx, val, entropy);
+    g_launches += 1;
+    return cudaGetLastError();
+  }
+  // 32-row spans once there are enough rows for 64 warps per SM (32 warps: 60k x
+  // 16, K = 16, few positive entries 28 us against 25)
+  int64_t span = n / (num_sms() * 64);
   span = span < 1 ? 1 : span > 32 ? 32 : span;
   int64_t blocks = (n + 8 * span - 1) / (8 * span);
   if (blocks > num_sms() * 16) blocks = num_sms() * 16;
