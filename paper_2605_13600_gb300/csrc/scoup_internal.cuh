@@ -207,6 +207,10 @@ struct TileList {
   __device__ __forceinline__ unsigned long long plain(unsigned long long k) const {
     return (k & 0xffffffff00000000ull) | ((uint32_t)k >> id_shift);
   }
+  // the largest key of a list that stands for the plain key k
+  __device__ __forceinline__ unsigned long long last_as_listed(unsigned long long k) const {
+    return (k & 0xffffffff00000000ull) | ((uint32_t)k << id_shift) | ((1u << id_shift) - 1u);
+  }
 };
 //
 // A block's list serves the binning (a quarter of the lists to count and fill)

@@ -56,6 +56,11 @@ struct OrderBuckets {
   __device__ __forceinline__ int operator()(const TileList& l, unsigned long long key) const {
     return l.mine(key) ? (*this)(key) : nb;
   }
+  // the depths of buckets [b0, b1): d - lo <= span (unsigned)
+  __device__ __forceinline__ uint2 depths(int b0, int b1) const {
+    const uint32_t first = (uint32_t)b0 << shift;
+    return make_uint2(lo + first, (uint32_t)min(((unsigned long long)b1 << shift) - 1ull, (unsigned long long)span) - first);
+  }
 };
 
 struct OrderState {
@@ -122,17 +127,18 @@ __device__ void order_init(S& sm, const TileList& l, const OrderBuckets& bk) {
   S::sync();
 }
 
-// The rank-th smallest (0-based) key in bucket b with (first || key > last).
+// The rank-th smallest (0-based) of the tile's keys in [from, to], as they
+// stand in the list (unique, in the order of depth and index).
 template <class S>
-__device__ unsigned long long order_select(S& sm, const TileList& l, const OrderBuckets& bk, int b,
-                                           unsigned long long last, bool first, int rank) {
+__device__ unsigned long long order_select(S& sm, const TileList& l, unsigned long long from, unsigned long long to,
+                                           int rank) {
   const int n = l.n, tid = threadIdx.x, nt = S::nthreads();
   if (tid == 0) { sm.red_min = ~0ull; sm.red_max = 0ull; }
   S::sync();
   unsigned long long lmin = ~0ull, lmax = 0ull;
   for (int i = tid; i < n; i += nt) {
-    const unsigned long long raw = l.keys[i], k = l.plain(raw);
-    if (bk(l, raw) == b && (first || k > last)) { lmin = min(lmin, k); lmax = max(lmax, k); }
+    const unsigned long long k = l.keys[i];
+    if (k >= from && k <= to && l.mine(k)) { lmin = min(lmin, k); lmax = max(lmax, k); }
   }
   for (int off = 16; off > 0; off >>= 1) {
     lmin = min(lmin, __shfl_xor_sync(0xffffffffu, lmin, off));
@@ -147,8 +153,8 @@ __device__ unsigned long long order_select(S& sm, const TileList& l, const Order
     for (int d = tid; d < 256; d += nt) sm.hist[d] = 0u;
     S::sync();
     for (int i = tid; i < n; i += nt) {
-      const unsigned long long raw = l.keys[i], k = l.plain(raw);
-      if (bk(l, raw) == b && (first || k > last)) {
+      const unsigned long long k = l.keys[i];
+      if (k >= from && k <= to && l.mine(k)) {
         const unsigned long long x = k - base;
         if ((x & pmask) == prefix) atomicAdd(&sm.hist[(x >> shift) & 255u], 1u);
       }
@@ -231,6 +237,7 @@ __device__ int order_next_window(S& sm, const TileList& l, const OrderBuckets& b
     m = (int)(sm.bstart[b1] - base);
     for (int b = st.b0 + tid; b < b1; b += nt) sm.bcur[b] = sm.bstart[b] - base;
     S::sync();
+    const uint2 in = bk.depths(st.b0, b1);
     for (int i0 = tid; i0 < n; i0 += kLB * nt) {
       unsigned long long kk[kLB];
 #pragma unroll
@@ -240,9 +247,8 @@ __device__ int order_next_window(S& sm, const TileList& l, const OrderBuckets& b
       }
 #pragma unroll
       for (int u = 0; u < kLB; ++u) {
-        const int b = bk(l, kk[u]);
-        if (i0 + u * nt < n && b >= st.b0 && b < b1) {
-          const uint32_t pos = atomicAdd(&sm.bcur[b], 1u);
+        if (i0 + u * nt < n && (uint32_t)(kk[u] >> 32) - in.x <= in.y && l.mine(kk[u])) {
+          const uint32_t pos = atomicAdd(&sm.bcur[bk(kk[u])], 1u);
           if (pos < (uint32_t)kWin) sm.win[pos] = l.plain(kk[u]);
         }
       }
@@ -276,15 +282,18 @@ __device__ int order_next_window(S& sm, const TileList& l, const OrderBuckets& b
     if (!st.in_split) { st.in_split = true; st.split_first = true; st.consumed = 0; }
     if (tid == 0) atomicAdd(&hdr->split_windows, 1ull);
     const int left = total_b0 - st.consumed;
-    unsigned long long hi_key = ~0ull;
-    if (left > kWin) hi_key = order_select(sm, l, bk, st.b0, st.split_last, st.split_first, kWin - 1);
+    const uint2 in = bk.depths(st.b0, st.b0 + 1);
+    const unsigned long long from =
+        st.split_first ? (unsigned long long)in.x << 32 : l.last_as_listed(st.split_last) + 1ull;
+    unsigned long long to = ((unsigned long long)(in.x + in.y) << 32) | 0xffffffffull;
+    if (left > kWin) to = order_select(sm, l, from, to, kWin - 1);
     if (tid == 0) sm.cursor = 0u;
     S::sync();
     for (int i = tid; i < n; i += nt) {
-      const unsigned long long raw = l.keys[i], k = l.plain(raw);
-      if (bk(l, raw) == st.b0 && (st.split_first || k > st.split_last) && k <= hi_key) {
+      const unsigned long long k = l.keys[i];
+      if (k >= from && k <= to && l.mine(k)) {
         const unsigned pos = atomicAdd(&sm.cursor, 1u);
-        if (pos < (unsigned)kWin) sm.win[pos] = k;
+        if (pos < (unsigned)kWin) sm.win[pos] = l.plain(k);
       }
     }
     S::sync();

@@ -136,6 +136,11 @@ struct Buckets {
   __device__ __forceinline__ int operator()(const TileList& l, unsigned long long key) const {
     return l.mine(key) ? (*this)(key) : kNB;
   }
+  // the depths of buckets [b0, b1): d - lo <= span (unsigned)
+  __device__ __forceinline__ uint2 depths(int b0, int b1) const {
+    const uint32_t first = (uint32_t)b0 << shift;
+    return make_uint2(lo + first, (uint32_t)min(((unsigned long long)b1 << shift) - 1ull, (unsigned long long)span) - first);
+  }
 };
 
 // f(key) for every key of the list, kLoads loads of a thread in flight at a
@@ -144,38 +149,39 @@ struct Buckets {
 // a tile's list) 41.7 / 40.1 / 40.7 ms, 24 views of 640 x 480, 300k 2.38 / 2.29
 // / 2.32 ms; 24 views of 200 x 140, 1M (100k keys) - / 2.86 / 2.64 ms, and one
 // such view at a time 1877 us with 1, 1033 with 8.  Eight cost registers that
-// the walk then spills.
-constexpr int kLoads = 4;
-template <typename F>
+// the walk then spills; the select, a function of its own, takes eight (one
+// view of 32 x 24, 200k: 132 ms with four, 110 with eight).
+constexpr int kLoads = 4, kSelectLoads = 8;
+template <int kL = kLoads, typename F>
 __device__ __forceinline__ void for_keys(const TileList& l, F f) {
   const unsigned long long* __restrict__ const keys = l.keys;
   const int n = l.n;
-  for (int i0 = threadIdx.x; i0 < n; i0 += kLoads * kThreads) {
-    unsigned long long k[kLoads];
+  for (int i0 = threadIdx.x; i0 < n; i0 += kL * kThreads) {
+    unsigned long long k[kL];
 #pragma unroll
-    for (int u = 0; u < kLoads; ++u) {
+    for (int u = 0; u < kL; ++u) {
       const int i = i0 + u * kThreads;
       k[u] = i < n ? keys[i] : 0ull;
     }
 #pragma unroll
-    for (int u = 0; u < kLoads; ++u)
+    for (int u = 0; u < kL; ++u)
       if (i0 + u * kThreads < n) f(k[u]);
   }
 }
 
-// Block-wide: the rank-th smallest (0-based) key among those in bucket b
-// with (first || key > last).  Keys are unique; requires rank < their count.
+// Block-wide: the rank-th smallest (0-based) of the tile's keys in [from, to],
+// as they stand in the list (a list's keys are unique, tile bits and all, and
+// in the order of depth and index); requires rank < their count.
 template <class Smem>
-__device__ __noinline__ unsigned long long select_in_bucket(Smem& sm, const TileList& list, const Buckets& bk, int b,
-                                                            unsigned long long last, bool first, int rank) {
+__device__ __noinline__ unsigned long long select_in_range(Smem& sm, const TileList& list, unsigned long long from,
+                                                           unsigned long long to, int rank) {
   const int tid = threadIdx.x;
   const TileList l = list;
   if (tid == 0) { sm.red_min = ~0ull; sm.red_max = 0ull; }
   __syncthreads();
   unsigned long long lmin = ~0ull, lmax = 0ull;
-  for_keys(l, [&](unsigned long long raw) {
-    const unsigned long long k = l.plain(raw);
-    if (bk(l, raw) == b && (first || k > last)) { lmin = min(lmin, k); lmax = max(lmax, k); }
+  for_keys<kSelectLoads>(l, [&](unsigned long long k) {
+    if (k >= from && k <= to && l.mine(k)) { lmin = min(lmin, k); lmax = max(lmax, k); }
   });
   for (int off = 16; off > 0; off >>= 1) {
     lmin = min(lmin, __shfl_xor_sync(kFull, lmin, off));
@@ -189,9 +195,8 @@ __device__ __noinline__ unsigned long long select_in_bucket(Smem& sm, const Tile
   for (int shift = ((nbits - 1) / 8) * 8; shift >= 0; shift -= 8) {
     sm.hist[tid] = 0u;
     __syncthreads();
-    for_keys(l, [&](unsigned long long raw) {
-      const unsigned long long k = l.plain(raw);
-      if (bk(l, raw) == b && (first || k > last)) {
+    for_keys<kSelectLoads>(l, [&](unsigned long long k) {
+      if (k >= from && k <= to && l.mine(k)) {
         const unsigned long long x = k - base;
         if ((x & pmask) == prefix) atomicAdd(&sm.hist[(x >> shift) & 255u], 1u);
       }
@@ -499,10 +504,10 @@ __device__ __forceinline__ void tile_pass(TileSmem<kComp, kL>& sm, const int til
       for (int b = b0 + tid; b < b1; b += kThreads) sm.bcur[b] = sm.bstart[b] - base;
       __syncthreads();
       const TileList l = sm.list;
+      const uint2 in = bk.depths(b0, b1);
       for_keys(l, [&](unsigned long long k) {
-        const int b = bk(l, k);
-        if (b >= b0 && b < b1) {
-          const uint32_t pos = atomicAdd(&sm.bcur[b], 1u);
+        if ((uint32_t)(k >> 32) - in.x <= in.y && l.mine(k)) {
+          const uint32_t pos = atomicAdd(&sm.bcur[bk(k)], 1u);
           if (pos < (uint32_t)kWin) sm.win[pos] = l.plain(k);
         }
       });
@@ -533,17 +538,17 @@ __device__ __forceinline__ void tile_pass(TileSmem<kComp, kL>& sm, const int til
       if (!in_split) { in_split = true; split_first = true; consumed = 0; }
       if (tid == 0) atomicAdd(&hdr->split_windows, 1ull);
       const int left = total_b0 - consumed;
-      unsigned long long hi_key = ~0ull;
-      const TileList& list = sm.list;
-      if (left > kWin) hi_key = select_in_bucket(sm, list, bk, b0, split_last, split_first, kWin - 1);
+      const TileList l = sm.list;
+      const uint2 in = bk.depths(b0, b0 + 1);
+      const unsigned long long from = split_first ? (unsigned long long)in.x << 32 : l.last_as_listed(split_last) + 1ull;
+      unsigned long long to = ((unsigned long long)(in.x + in.y) << 32) | 0xffffffffull;
+      if (left > kWin) to = select_in_range(sm, sm.list, from, to, kWin - 1);
       if (tid == 0) sm.cursor = 0u;
       __syncthreads();
-      const TileList l = list;
-      for_keys(l, [&](unsigned long long raw) {
-        const unsigned long long k = l.plain(raw);
-        if (bk(l, raw) == b0 && (split_first || k > split_last) && k <= hi_key) {
+      for_keys(l, [&](unsigned long long k) {
+        if (k >= from && k <= to && l.mine(k)) {
           const unsigned pos = atomicAdd(&sm.cursor, 1u);
-          if (pos < (unsigned)kWin) sm.win[pos] = k;
+          if (pos < (unsigned)kWin) sm.win[pos] = l.plain(k);
         }
       });
       __syncthreads();
