@@ -23,7 +23,11 @@
 // in the lane's registers: a (pixel, Gaussian) pair costs the exponent, its
 // share of two warp scans and one gather of K words of the pixel's gradient
 // row, without a shared atomic.  Longer codes take render_bwd_kernel (a warp
-// per pixel, every window entry).
+// per pixel, every window entry).  Up to 16 entries the block kernel is the
+// faster one at every width, though its gradient rows leave one CTA per SM at C =
+// 1024 (its time over the other's, K = 4 / 8 / 16, 500k Gaussians, 800 x 600: C =
+// 256 0.62 / 0.54 / 0.48, 512 0.61 / 0.50 / 0.40, 1024 0.73 / 0.56 / 0.57; 10k,
+// 160 x 120: 0.27 / 0.23 / 0.22, 0.27 / 0.24 / 0.23, 0.26 / 0.25 / 0.24).
 #include <math.h>
 
 #include "tile_order.cuh"
@@ -154,10 +158,14 @@ __device__ __forceinline__ bool walk_bwd(BwdSmem& sm, const BwdDyn& dy, const fl
   return false;
 }
 
-// 4 CTAs per SM: with 256-key windows, staged codes and entry-major gradient
-// sums, measured 4.9 -> 2.1 ms per 800x600 view (2 or 3 CTAs per SM: 2.4 ms)
+// Codes of more than 16 entries: their gradient sums and staged codes take the
+// shared memory of two or three CTAs per SM, so the launch bound is two, which
+// leaves the walk's registers alone (at four, 64 registers, the walk is 3 to 6 %
+// slower and spills; 500k Gaussians, 800x600, ms at four / two: C = 64, K = 17
+// 3.9 / 3.7, C = 256, K = 24 6.3 / 5.8, C = 512, K = 32 13.7 / 12.3; C = 256,
+// K = 33, codes not staged, 17.3 / 11.6).
 template <bool kStaged>
-__global__ void __launch_bounds__(kBThreads, 4) render_bwd_kernel(
+__global__ void __launch_bounds__(kBThreads, 2) render_bwd_kernel(
     const __grid_constant__ ViewJob view, const int32_t* __restrict__ topk_idx,
     const float* __restrict__ topk_val, int K, int C, const float* __restrict__ dL_dcodes,
     float* __restrict__ d_val, float* __restrict__ d_opacity) {
