@@ -1,10 +1,11 @@
 /*
  * scoup_selftest.h -- self-tests and measurement helpers of libscoup.so.
- * The paper has no counterpart to either: the first checks the library's own
+ * The paper has no counterpart to them: the first checks the library's own
  * guard that a tensor-core pipeline wait which never completes gives up,
  * reports an error and leaves the GPU usable, without faulting anything; the
  * second measures the GPU's atomic-update ceiling that bounds the uplift's
- * scatter (Eq. 5), for the roofline of the uplift step.
+ * scatter (Eq. 5), for the roofline of the uplift step; the third counts what
+ * an uplift did again behind its depth cut.
  */
 #ifndef SCOUP_SELFTEST_H
 #define SCOUP_SELFTEST_H
@@ -40,6 +41,14 @@ int scoup_selftest_gemm_timeout(void* workspace, size_t ws_bytes, void* stream);
  * stream.  Returns SCOUP_ERR_INVALID_ARG on a bad argument, SCOUP_ERR_CUDA on a
  * launch error. */
 int scoup_selftest_red_throughput(float* buf, int32_t log2_n, int64_t count, uint32_t seed, void* stream);
+
+/* Tiles that the last uplift on this workspace left open at their depth cut
+ * and took up again in a second pass over the lists behind it (large scenes in
+ * chunks of views; 0 where no view has a cut).  The results do not depend on it:
+ * the counter says whether a test reaches the second pass.
+ *  workspace  DEVICE, that of a finished scoup_uplift (header first).
+ * Synchronises `stream`. */
+int scoup_selftest_resumed_tiles(const void* workspace, size_t ws_bytes, int64_t* tiles, void* stream);
 
 #ifdef __cplusplus
 }

@@ -1411,6 +1411,17 @@ int scoup_selftest_gemm_timeout(void* workspace, size_t ws_bytes, void* stream) 
   return fail(SCOUP_ERR_DEVICE_CHECK, "self-test: the stalled pipeline did not report a timeout");
 }
 
+int scoup_selftest_resumed_tiles(const void* workspace, size_t ws_bytes, int64_t* tiles, void* stream) {
+  if (!workspace || ws_bytes < sizeof(WsHeader)) return fail(SCOUP_ERR_INVALID_ARG, "bad workspace");
+  if (!tiles) return fail(SCOUP_ERR_INVALID_ARG, "tiles is NULL");
+  WsHeader h;
+  cudaError_t e = cudaMemcpyAsync(&h, workspace, sizeof(h), cudaMemcpyDeviceToHost, (cudaStream_t)stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize((cudaStream_t)stream);
+  if (e != cudaSuccess) return cuda_fail(e, "read header");
+  *tiles = (int64_t)h.resumed_tiles;
+  return SCOUP_OK;
+}
+
 int scoup_read_stats(const void* workspace, size_t ws_bytes, scoup_stats* stats, void* stream) {
   if (!workspace || ws_bytes < sizeof(WsHeader)) return fail(SCOUP_ERR_INVALID_ARG, "bad workspace");
   if (!stats) return fail(SCOUP_ERR_INVALID_ARG, "stats is NULL");

@@ -73,6 +73,7 @@ __global__ void view_merge_kernel(const __grid_constant__ MergeArgs a) {
   atomicAdd(&s->atomics, v->atomics);
   atomicAdd(&s->listed, v->listed);
   atomicAdd(&s->split_windows, v->split_windows);
+  atomicAdd(&s->resumed_tiles, (unsigned long long)v->open_tiles);
   atomicMax(&s->max_dups_view, v->max_dups_view);
   if (v->status) atomicOr(&s->status, v->status);
   v->visible = v->duplicates = v->evaluated = v->contributions = 0ull;

@@ -43,9 +43,10 @@ struct WsHeader {
   unsigned long long atomics;
   unsigned long long listed;
   unsigned long long split_windows;  // windows cut out of a depth bucket holding more than a window
+  unsigned long long resumed_tiles;  // scene header: tiles that a second pass took up behind the depth cut
   uint32_t open_tiles;               // tiles still open behind the depth cut (length of open_list)
   uint32_t drain_ctr[2][2];          // scene header: item counters of each chunk lane's two drains
-  uint32_t reserved[33];
+  uint32_t reserved[31];
 };
 static_assert(sizeof(WsHeader) == 256, "header size");
 

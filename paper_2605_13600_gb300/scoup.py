@@ -622,6 +622,13 @@ def scoup_selftest_gemm_timeout(stream=None) -> tuple:
     return int(rc), (msg.decode() if msg else "")
 
 
+def scoup_selftest_resumed_tiles(workspace, stream=None) -> int:
+    """Tiles that the last uplift on this workspace took up again behind their depth cut."""
+    out = ct.c_int64(0)
+    check(load().scoup_selftest_resumed_tiles(_ptr(workspace), workspace.numel(), ct.byref(out), _stream(stream)))
+    return int(out.value)
+
+
 def scoup_read_stats(workspace, stream=None) -> dict:
     st = Stats()
     check(load().scoup_read_stats(_ptr(workspace), workspace.numel(), ct.byref(st), _stream(stream)))
@@ -938,7 +945,7 @@ __all__ = ["ScoupError", "SCOUP_ACCUM_CONTINUE", "SCOUP_ACCUM_COMPENSATED", "SCO
            "scoup_render", "scoup_render_backward", "Render", "Uplift",
            "scoup_decode_workspace_size", "scoup_decode", "scoup_similarity_workspace_size",
            "scoup_similarity", "scoup_decode_fp32", "scoup_similarity_fp32", "BatchedUplift",
-           "SCOUP_BATCH_EAGER", "LevelUplift", "scoup_selftest_gemm_timeout", "scoup_selftest_red_throughput", "scoup_topk_entropy", "scoup_entropy_filter", "scoup_entropy_filter_workspace_size", "scoup_relevancy",
+           "SCOUP_BATCH_EAGER", "LevelUplift", "scoup_selftest_gemm_timeout", "scoup_selftest_red_throughput", "scoup_selftest_resumed_tiles", "scoup_topk_entropy", "scoup_entropy_filter", "scoup_entropy_filter_workspace_size", "scoup_relevancy",
            "scoup_render_decode_workspace_size", "scoup_render_decode_fused",
            "scoup_uplift_host_maps_workspace_size", "scoup_uplift_host_maps",
            "scoup_similarity_relevancy", "scoup_decode_query", "scoup_decode_query_workspace_size", "scoup_decode_backward", "scoup_decode_backward_fp32",
