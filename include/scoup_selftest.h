@@ -4,8 +4,8 @@
  * guard that a tensor-core pipeline wait which never completes gives up,
  * reports an error and leaves the GPU usable, without faulting anything; the
  * second measures the GPU's atomic-update ceiling that bounds the uplift's
- * scatter (Eq. 5), for the roofline of the uplift step; the third counts what
- * an uplift did again behind its depth cut.
+ * scatter (Eq. 5), for the roofline of the uplift step; the others show what an
+ * uplift did again behind its depth cut and the thresholds of the alpha test.
  */
 #ifndef SCOUP_SELFTEST_H
 #define SCOUP_SELFTEST_H
@@ -49,6 +49,13 @@ int scoup_selftest_red_throughput(float* buf, int32_t log2_n, int64_t count, uin
  *  workspace  DEVICE, that of a finished scoup_uplift (header first).
  * Synchronises `stream`. */
 int scoup_selftest_resumed_tiles(const void* workspace, size_t ws_bytes, int64_t* tiles, void* stream);
+
+/* The alpha-threshold exponent of each opacity, as the projection uses it: the
+ * smallest binary32 tau with opacity * exp(tau) >= 1/255, i.e. -log(255 opacity)
+ * rounded up (+inf for an opacity that is not positive).  Every alpha test rests
+ * on it.
+ *  opacity, tau  DEVICE float32 [n].  Asynchronous on `stream`. */
+int scoup_selftest_alpha_threshold(const float* opacity, int64_t n, float* tau, void* stream);
 
 #ifdef __cplusplus
 }

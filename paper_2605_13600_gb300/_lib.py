@@ -145,6 +145,7 @@ PROTOS = {
                                         P, ct.c_int32, P, ct.c_int32, P, P, SZ, P]),
     "scoup_selftest_red_throughput": (ct.c_int, [P, ct.c_int32, ct.c_int64, ct.c_uint32, P]),
     "scoup_selftest_resumed_tiles": (ct.c_int, [P, SZ, ct.POINTER(I64), P]),
+    "scoup_selftest_alpha_threshold": (ct.c_int, [P, I64, P, P]),
     "scoup_profile_enable": (ct.c_int, [I32]),
     "scoup_profile_read": (ct.c_int, [P, P, I32]),
     "scoup_launch_count": (I64, []),

@@ -1422,6 +1422,13 @@ int scoup_selftest_resumed_tiles(const void* workspace, size_t ws_bytes, int64_t
   return SCOUP_OK;
 }
 
+int scoup_selftest_alpha_threshold(const float* opacity, int64_t n, float* tau, void* stream) {
+  if (n < 0) return fail(SCOUP_ERR_INVALID_ARG, "n < 0");
+  if (n > 0 && (!opacity || !tau)) return fail(SCOUP_ERR_INVALID_ARG, "NULL array");
+  const cudaError_t e = launch_alpha_thresholds(opacity, n, tau, (cudaStream_t)stream);
+  return e == cudaSuccess ? SCOUP_OK : cuda_fail(e, "alpha thresholds");
+}
+
 int scoup_read_stats(const void* workspace, size_t ws_bytes, scoup_stats* stats, void* stream) {
   if (!workspace || ws_bytes < sizeof(WsHeader)) return fail(SCOUP_ERR_INVALID_ARG, "bad workspace");
   if (!stats) return fail(SCOUP_ERR_INVALID_ARG, "stats is NULL");

@@ -219,6 +219,11 @@ __global__ void __launch_bounds__(256) gather_kernel(const float* __restrict__ m
   }
 }
 
+__global__ void __launch_bounds__(256) threshold_kernel(const float* __restrict__ o, int64_t n, float* __restrict__ tau) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    tau[i] = alpha_threshold(o[i]);
+}
+
 // Everything a call starts from, in one launch: the header (zero but for the
 // empty depth range and bounding box), the cell counts, and the binning
 // counters of a render's view.
@@ -250,6 +255,13 @@ int grid_for(int64_t n, int per_sm) {
 }  // namespace
 
 size_t reorder_scratch_bytes() { return sizeof(uint32_t) * (size_t)(3 * kCells); }
+
+cudaError_t launch_alpha_thresholds(const float* opacity, int64_t n, float* tau, cudaStream_t st) {
+  if (n <= 0) return cudaSuccess;
+  threshold_kernel<<<grid_for(n, 8), 256, 0, st>>>(opacity, n, tau);
+  g_launches += 1;
+  return cudaGetLastError();
+}
 
 cudaError_t launch_begin(const UpliftWs& ws, bool view, int max_tiles, cudaStream_t st) {
   BeginArgs a = {};

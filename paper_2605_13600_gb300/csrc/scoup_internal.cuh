@@ -376,6 +376,8 @@ int check_scene_views(const scoup_scene* scene, const scoup_camera* cams, int32_
 void header_stats(const struct WsHeader& h, scoup_stats* stats);
 
 // Launchers (each defined in its own translation unit).
+// Self-test: the alpha-threshold exponents that the reorder gives n opacities.
+cudaError_t launch_alpha_thresholds(const float* opacity, int64_t n, float* tau, cudaStream_t st);
 size_t reorder_scratch_bytes();
 // First launch of a call: sets up the scene header, the reorder's cell counts
 // and (view: a render, whose view uses the scene's header) the binning counters.

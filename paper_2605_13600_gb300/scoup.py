@@ -629,6 +629,16 @@ def scoup_selftest_resumed_tiles(workspace, stream=None) -> int:
     return int(out.value)
 
 
+def scoup_selftest_alpha_threshold(opacity, tau, stream=None) -> None:
+    """tau [n] = the alpha-threshold exponents of the opacities [n] (float32)."""
+    import torch
+    _need(opacity, torch.float32, "opacity")
+    _need(tau, torch.float32, "tau")
+    if tau.numel() < opacity.numel():
+        raise ValueError("tau is too short")
+    check(load().scoup_selftest_alpha_threshold(_ptr(opacity), opacity.numel(), _ptr(tau), _stream(stream)))
+
+
 def scoup_read_stats(workspace, stream=None) -> dict:
     st = Stats()
     check(load().scoup_read_stats(_ptr(workspace), workspace.numel(), ct.byref(st), _stream(stream)))
@@ -945,7 +955,7 @@ __all__ = ["ScoupError", "SCOUP_ACCUM_CONTINUE", "SCOUP_ACCUM_COMPENSATED", "SCO
            "scoup_render", "scoup_render_backward", "Render", "Uplift",
            "scoup_decode_workspace_size", "scoup_decode", "scoup_similarity_workspace_size",
            "scoup_similarity", "scoup_decode_fp32", "scoup_similarity_fp32", "BatchedUplift",
-           "SCOUP_BATCH_EAGER", "LevelUplift", "scoup_selftest_gemm_timeout", "scoup_selftest_red_throughput", "scoup_selftest_resumed_tiles", "scoup_topk_entropy", "scoup_entropy_filter", "scoup_entropy_filter_workspace_size", "scoup_relevancy",
+           "SCOUP_BATCH_EAGER", "LevelUplift", "scoup_selftest_gemm_timeout", "scoup_selftest_red_throughput", "scoup_selftest_resumed_tiles", "scoup_selftest_alpha_threshold", "scoup_topk_entropy", "scoup_entropy_filter", "scoup_entropy_filter_workspace_size", "scoup_relevancy",
            "scoup_render_decode_workspace_size", "scoup_render_decode_fused",
            "scoup_uplift_host_maps_workspace_size", "scoup_uplift_host_maps",
            "scoup_similarity_relevancy", "scoup_decode_query", "scoup_decode_query_workspace_size", "scoup_decode_backward", "scoup_decode_backward_fp32",
