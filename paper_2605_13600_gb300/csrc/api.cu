@@ -99,9 +99,8 @@ size_t shared_bytes(int64_t n, int64_t code_rows_k) {
 // Regions of a view part whose use the sizes of the view decide (carve_view_part):
 // run_bytes: the binning groups' reserved-run offsets (16 KB per group of
 // bin_group(n) Gaussians, at least 512), and behind them, with the larger
-// groups from 64k Gaussians on, the kept bits and the depth cut's arrays;
+// groups of scenes above kSmallScene, the kept bits and the depth cut's arrays;
 // aux: the part's header and the kept bits of a smaller scene.
-constexpr size_t kAuxBytes = 8192;
 constexpr size_t kRunBytes = 16384;
 size_t run_bytes(int64_t n) { return kRunBytes * (size_t)((n + 511) / 512); }
 
@@ -113,7 +112,6 @@ size_t lane_bytes(int64_t n, int max_tiles) {
   b += 4 * align_up(sizeof(uint32_t) * ((size_t)max_tiles + 1));
   b += align_up(run_bytes(n));                            // binning runs, kept bits, depth cut
   b += align_up(sizeof(float) * kTilePixels * (size_t)max_tiles);  // pixels of open tiles / depth-cut histogram
-  b += align_up((size_t)max_tiles);
   b += kAuxBytes;
   return b;
 }
@@ -156,7 +154,6 @@ size_t carve_view_part(void* base, int64_t n, int max_tiles, UpliftWs* w) {
   w->tile_start = (uint32_t*)take(sizeof(uint32_t) * ((size_t)max_tiles + 1));
   w->tile_fill = (uint32_t*)take(sizeof(uint32_t) * ((size_t)max_tiles + 1));
   w->pix_state = (float*)take(sizeof(float) * kTilePixels * (size_t)max_tiles);
-  take((size_t)max_tiles);
   char* aux = (char*)take(kAuxBytes);
   w->vhdr = (WsHeader*)aux;
   w->run_base = (uint32_t*)runs;
@@ -440,7 +437,7 @@ static int uplift_views(const UpliftCall& c, const scoup_level* lv, int L, const
         lc.R[l] = lv[l].R_total;
         lc.s_tot += lv[l].s;
       }
-      jobs[k] = tile_job(views[k], lc, c.accum, comp, sw.hdr, c.C, L * c.C, 0);
+      jobs[k] = tile_job(views[k], lc, c.accum, comp, sw.hdr, c.C, L * c.C);
     }
     ChunkStreams cs{lane_st[lane]};
     if (c.maps_on_host) {
@@ -607,8 +604,7 @@ size_t uplift_required_bytes(int64_t n, const scoup_camera* cams, int32_t V, int
          (size_t)parts * sizeof(unsigned long long) * (size_t)dup_capacity;
 }
 
-TileJob tile_job(const ViewJob& v, const LevelCodes& lc, float* accum, float* comp, WsHeader* scene_hdr, int C, int Crow,
-                 int scene) {
+TileJob tile_job(const ViewJob& v, const LevelCodes& lc, float* accum, float* comp, WsHeader* scene_hdr, int C, int Crow) {
   TileJob J = TileJob();
   J.cam = v.cam;
   J.lc = lc;
@@ -627,7 +623,6 @@ TileJob tile_job(const ViewJob& v, const LevelCodes& lc, float* accum, float* co
   J.Crow = Crow;
   J.shift = v.shift;
   J.tiles = v.cam.gx * v.cam.gy;
-  J.scene = scene;
   return J;
 }
 

@@ -232,7 +232,7 @@ int drain_prepare(DrainLayout* d, const std::vector<scoup_batch_item>& items, co
       lc.cv[0] = filtered ? d->fcv[b] : it.code_val;
       lc.R[0] = it.R_total;
       float* comp = compensated ? it.accum + (size_t)it.scene.n * (size_t)C : nullptr;
-      d->jobs[j] = tile_job(d->views[j], lc, it.accum, comp, d->scene[b].hdr, C, C, b);
+      d->jobs[j] = tile_job(d->views[j], lc, it.accum, comp, d->scene[b].hdr, C, C);
     }
   }
   d->chunk = chunk;

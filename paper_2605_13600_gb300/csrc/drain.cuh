@@ -23,8 +23,7 @@ struct ChunkStreams {
 };
 
 // The drain's side of a view.
-TileJob tile_job(const ViewJob& v, const LevelCodes& lc, float* accum, float* comp, WsHeader* scene_hdr, int C, int Crow,
-                 int scene);
+TileJob tile_job(const ViewJob& v, const LevelCodes& lc, float* accum, float* comp, WsHeader* scene_hdr, int C, int Crow);
 
 // One chunk of nv <= kMaxDrainJobs views (HOST arrays, each view with a view
 // part of its own): depth cut, projection and binning, one drain launch over

@@ -154,7 +154,6 @@ struct TileJob {
   int C, Crow;          // accumulator rows hold Crow = levels x C floats
   int shift;            // of the view's tile lists (TileList)
   int tiles;
-  int scene;
 };
 
 // Scene copy in spatial (Morton) order: one 48-byte record per Gaussian, with
@@ -186,7 +185,6 @@ constexpr int kCutShift = 17;
 constexpr uint32_t kNoCut = 0xffffffffu;
 __host__ __device__ inline int cut_blocks(int g) { return (g + 1) >> 1; }
 __host__ __device__ inline int open_words(int gx) { return (cut_blocks(gx) + 31) >> 5; }  // per row of blocks
-
 
 // Tile lists.  A list belongs to a block of 2 x 2 tiles: a Gaussian meets
 // several neighbouring tiles, so a view has less than half as many (Gaussian,
@@ -318,9 +316,13 @@ ViewJob view_job(const scoup_scene& sc, const CamArgs& cam, const UpliftWs& ws, 
 // Whether views of this size get a depth cut (given room in the view part).
 // views: how many views a launch of the view's chunk takes.
 bool use_depth_cut(int64_t n, const CamArgs& cam, const UpliftWs& ws, int views);
-// Gaussians per binning CTA; larger groups from 64k Gaussians on, of which the
-// depth cut leaves a fraction.
-inline int bin_group(int64_t n) { return n <= 63488 ? 512 : 1024; }
+// Gaussians per binning CTA; larger groups for scenes above kSmallScene, of which
+// the depth cut leaves a fraction, and whose kept bits have room beside the runs.
+// The kept bits of a smaller scene lie behind the view part's header (kAuxBytes).
+constexpr int64_t kSmallScene = 63488;
+constexpr size_t kAuxBytes = 8192;
+static_assert(sizeof(WsHeader) + (kSmallScene + 31) / 32 * 4 <= kAuxBytes, "kept bits of the largest small scene");
+inline int bin_group(int64_t n) { return n <= kSmallScene ? 512 : 1024; }
 
 // Records msg as the calling thread's last error and returns code.
 int set_error(int code, const char* msg);
@@ -388,7 +390,7 @@ cudaError_t launch_reorder(const scoup_scene& sc, const UpliftWs& ws, cudaStream
 cudaError_t launch_depth_cut(const ViewJob* v, int nv, cudaStream_t st);
 cudaError_t launch_project(const ViewJob* v, int nv, cudaStream_t st);
 // Second pass, for the tiles recorded as open: keeps the Gaussians that reach
-// one of them behind its cut (restart: at any depth), with their records.
+// one of them behind its cut, with their records.
 cudaError_t launch_recover(const ViewJob* v, int nv, cudaStream_t st);
 // Tile lists of the kept Gaussians; second: only of the open tiles.  The lane's
 // drain counter of the pass (ctr, may be null) is cleared on the way.

@@ -18,21 +18,11 @@ namespace scoup {
 // registers allow.
 constexpr int kLoadBatch = 4;
 
-// kSync_: 0 when the whole CTA orders (the functions below synchronise with
-// __syncthreads and stride by blockDim.x); otherwise the number of threads,
-// the CTA's first kSync_, that order on named barrier 1 while the rest of the
-// CTA does other work.
-template <int kWin_, int kLogNB_, int kSync_ = 0>
+template <int kWin_, int kLogNB_>
 struct OrderSmem {
   static constexpr int kWin = kWin_;
   static constexpr int kNB = 1 << kLogNB_;
   static constexpr int kLogNB = kLogNB_;
-  static constexpr int kSync = kSync_;
-  __device__ static __forceinline__ int nthreads() { return kSync ? kSync : (int)blockDim.x; }
-  __device__ static __forceinline__ void sync() {
-    if constexpr (kSync > 0) asm volatile("bar.sync 1, %0;" ::"n"(kSync) : "memory");
-    else __syncthreads();
-  }
   uint32_t bstart[kNB + 1];
   uint32_t bcur[kNB];
   unsigned long long win[kWin];
@@ -83,13 +73,13 @@ __device__ OrderBuckets order_buckets(const WsHeader* hdr) {
   return bk;
 }
 
-// Histogram + exclusive scan into sm.bstart (S::nthreads() threads, a
+// Histogram + exclusive scan into sm.bstart (blockDim.x threads, a
 // multiple of 32 dividing kNB).
 template <class S, int kLB = kLoadBatch>
 __device__ void order_init(S& sm, const TileList& l, const OrderBuckets& bk) {
-  const int n = l.n, tid = threadIdx.x, nt = S::nthreads(), lane = tid & 31, warp = tid >> 5;
+  const int n = l.n, tid = threadIdx.x, nt = (int)blockDim.x, lane = tid & 31, warp = tid >> 5;
   for (int b = tid; b < S::kNB; b += nt) sm.bcur[b] = 0u;
-  S::sync();
+  __syncthreads();
   // kLB keys per thread are loaded before their atomics, so each
   // thread has that many global loads in flight at once
   for (int i0 = tid; i0 < n; i0 += kLB * nt) {
@@ -105,7 +95,7 @@ __device__ void order_init(S& sm, const TileList& l, const OrderBuckets& bk) {
       if (i0 + u * nt < n && b < S::kNB) atomicAdd(&sm.bcur[b], 1u);
     }
   }
-  S::sync();
+  __syncthreads();
   const int per = S::kNB / nt;
   uint32_t sum = 0;
   for (int q = 0; q < per; ++q) sum += sm.bcur[tid * per + q];
@@ -115,7 +105,7 @@ __device__ void order_init(S& sm, const TileList& l, const OrderBuckets& bk) {
     if (lane >= off) incl += y;
   }
   if (lane == 31) sm.hist[warp] = incl;
-  S::sync();
+  __syncthreads();
   uint32_t run = incl - sum;
   for (int w = 0; w < warp; ++w) run += sm.hist[w];
   for (int q = 0; q < per; ++q) {
@@ -124,7 +114,7 @@ __device__ void order_init(S& sm, const TileList& l, const OrderBuckets& bk) {
     run += c;
   }
   if (tid == nt - 1) sm.bstart[S::kNB] = run;
-  S::sync();
+  __syncthreads();
 }
 
 // The rank-th smallest (0-based) of the tile's keys in [from, to], as they
@@ -132,9 +122,9 @@ __device__ void order_init(S& sm, const TileList& l, const OrderBuckets& bk) {
 template <class S>
 __device__ unsigned long long order_select(S& sm, const TileList& l, unsigned long long from, unsigned long long to,
                                            int rank) {
-  const int n = l.n, tid = threadIdx.x, nt = S::nthreads();
+  const int n = l.n, tid = threadIdx.x, nt = (int)blockDim.x;
   if (tid == 0) { sm.red_min = ~0ull; sm.red_max = 0ull; }
-  S::sync();
+  __syncthreads();
   unsigned long long lmin = ~0ull, lmax = 0ull;
   for (int i = tid; i < n; i += nt) {
     const unsigned long long k = l.keys[i];
@@ -145,13 +135,13 @@ __device__ unsigned long long order_select(S& sm, const TileList& l, unsigned lo
     lmax = max(lmax, __shfl_xor_sync(0xffffffffu, lmax, off));
   }
   if ((tid & 31) == 0) { atomicMin(&sm.red_min, lmin); atomicMax(&sm.red_max, lmax); }
-  S::sync();
+  __syncthreads();
   const unsigned long long base = sm.red_min, span = sm.red_max - sm.red_min;
   const int nbits = span ? 64 - __clzll((long long)span) : 1;
   unsigned long long prefix = 0ull, pmask = 0ull;
   for (int shift = ((nbits - 1) / 8) * 8; shift >= 0; shift -= 8) {
     for (int d = tid; d < 256; d += nt) sm.hist[d] = 0u;
-    S::sync();
+    __syncthreads();
     for (int i = tid; i < n; i += nt) {
       const unsigned long long k = l.keys[i];
       if (k >= from && k <= to && l.mine(k)) {
@@ -159,7 +149,7 @@ __device__ unsigned long long order_select(S& sm, const TileList& l, unsigned lo
         if ((x & pmask) == prefix) atomicAdd(&sm.hist[(x >> shift) & 255u], 1u);
       }
     }
-    S::sync();
+    __syncthreads();
     if (tid < 32) {
       uint32_t c[8], sum = 0;
       for (int d = 0; d < 8; ++d) { c[d] = sm.hist[tid * 8 + d]; sum += c[d]; }
@@ -177,11 +167,11 @@ __device__ unsigned long long order_select(S& sm, const TileList& l, unsigned lo
         }
       }
     }
-    S::sync();
+    __syncthreads();
     prefix |= (unsigned long long)sm.sel_digit << shift;
     pmask |= 0xffull << shift;
     rank = sm.sel_rank;
-    S::sync();
+    __syncthreads();
   }
   return base + prefix;
 }
@@ -191,7 +181,7 @@ __device__ unsigned long long order_select(S& sm, const TileList& l, unsigned lo
 // Block-uniform; every thread of the CTA must call it.
 template <class S, int kLB = kLoadBatch>
 __device__ int order_next_window(S& sm, const TileList& l, const OrderBuckets& bk, OrderState& st, WsHeader* hdr) {
-  const int n = l.n, tid = threadIdx.x, nt = S::nthreads();
+  const int n = l.n, tid = threadIdx.x, nt = (int)blockDim.x;
   constexpr int kWin = S::kWin, kNB = S::kNB;
   // the in-place permutation below reads a whole window before writing it
   if (kWin > 4 * nt) {
@@ -209,9 +199,9 @@ __device__ int order_next_window(S& sm, const TileList& l, const OrderBuckets& b
       }
       sm.win_b1 = lo;
     }
-    S::sync();
+    __syncthreads();
     st.b0 = sm.win_b1;
-    S::sync();
+    __syncthreads();
   }
   if (st.b0 >= kNB) return 0;
   const uint32_t base = sm.bstart[st.b0];
@@ -229,14 +219,14 @@ __device__ int order_next_window(S& sm, const TileList& l, const OrderBuckets& b
         sm.win_b1 = lo;
       }
     }
-    S::sync();
+    __syncthreads();
   }
   const int b1 = sm.win_b1;
   int m;
   if (!st.in_split && b1 > st.b0) {
     m = (int)(sm.bstart[b1] - base);
     for (int b = st.b0 + tid; b < b1; b += nt) sm.bcur[b] = sm.bstart[b] - base;
-    S::sync();
+    __syncthreads();
     const uint2 in = bk.depths(st.b0, b1);
     for (int i0 = tid; i0 < n; i0 += kLB * nt) {
       unsigned long long kk[kLB];
@@ -253,7 +243,7 @@ __device__ int order_next_window(S& sm, const TileList& l, const OrderBuckets& b
         }
       }
     }
-    S::sync();
+    __syncthreads();
     // rank inside the bucket, then permute in place (m <= kWin <= 4 nt: one pass)
     for (int p0 = 0; p0 < m; p0 += nt * 4) {
       unsigned long long kk[4];
@@ -272,11 +262,11 @@ __device__ int order_next_window(S& sm, const TileList& l, const OrderBuckets& b
           dst[u] = lo + r;
         }
       }
-      S::sync();
+      __syncthreads();
 #pragma unroll
       for (int u = 0; u < 4; ++u)
         if (dst[u] >= 0) sm.win[dst[u]] = kk[u];
-      S::sync();
+      __syncthreads();
     }
   } else {
     if (!st.in_split) { st.in_split = true; st.split_first = true; st.consumed = 0; }
@@ -288,7 +278,7 @@ __device__ int order_next_window(S& sm, const TileList& l, const OrderBuckets& b
     unsigned long long to = ((unsigned long long)(in.x + in.y) << 32) | 0xffffffffull;
     if (left > kWin) to = order_select(sm, l, from, to, kWin - 1);
     if (tid == 0) sm.cursor = 0u;
-    S::sync();
+    __syncthreads();
     for (int i = tid; i < n; i += nt) {
       const unsigned long long k = l.keys[i];
       if (k >= from && k <= to && l.mine(k)) {
@@ -296,7 +286,7 @@ __device__ int order_next_window(S& sm, const TileList& l, const OrderBuckets& b
         if (pos < (unsigned)kWin) sm.win[pos] = l.plain(k);
       }
     }
-    S::sync();
+    __syncthreads();
     m = (int)min(sm.cursor, (unsigned)kWin);
     for (int p0 = 0; p0 < m; p0 += nt * 4) {
       unsigned long long kk[4];
@@ -313,14 +303,14 @@ __device__ int order_next_window(S& sm, const TileList& l, const OrderBuckets& b
           dst[u] = r;
         }
       }
-      S::sync();
+      __syncthreads();
 #pragma unroll
       for (int u = 0; u < 4; ++u)
         if (dst[u] >= 0) sm.win[dst[u]] = kk[u];
-      S::sync();
+      __syncthreads();
     }
   }
-  S::sync();
+  __syncthreads();
   if (m <= 0) {
     if (tid == 0) atomicOr(&hdr->status, kStatDeviceCheck);
     return -1;

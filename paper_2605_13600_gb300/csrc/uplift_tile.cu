@@ -79,7 +79,9 @@ constexpr int kMaxS = 64;  // codes of up to kMaxS entries are staged in shared 
                            // ones (dense features, Eq. 3) are read from the code table in the flush
 constexpr int kGroup = 8;
 // Each warp compacts the window entries whose box mask has its bit (up to
-// kCompact at a time) and composites that list in full groups of kGroup.
+// kCompact at a time, here a whole window) and composites that list in full
+// groups of kGroup.  Written without the loop over batches the same walk compiles
+// to 1 to 2.5 % more time (200 views of 1M 38.7 / 39.1 ms, three levels 2.94 / 3.02).
 constexpr int kCompact = kWin;
 constexpr unsigned kFull = 0xffffffffu;
 constexpr float kLog2e = 1.4426950408889634f;
