@@ -449,7 +449,11 @@ typedef struct scoup_plan_info {
 /* Creates a plan for the batch: counts every view's (Gaussian, tile) pairs
  * exactly (synchronising `stream`), sizes one uplift workspace for the
  * largest scene and allocates it for each lane (default lanes: min(4, B),
- * warp block 8x4).  The plan keeps a copy of `items` (the arrays they point
+ * warp block 8x4).  A lane's workspace holds four views, which a lane projects,
+ * bins and composites together, if all lanes' are at most an eighth of the
+ * device's free memory at this call, and one view otherwise, or when an
+ * allocation fails later (scoup_plan_info.workspace_bytes tells; results and
+ * counters are the same).  The plan keeps a copy of `items` (the arrays they point
  * to must stay valid and unchanged in size while the plan lives).  The plan
  * owns its device memory until scoup_plan_destroy. */
 int scoup_plan_create(const scoup_batch_item* items, int32_t B, int32_t C, int32_t K, int32_t accum_mode,
@@ -460,10 +464,10 @@ int scoup_plan_create(const scoup_batch_item* items, int32_t B, int32_t C, int32
 int scoup_plan_set(scoup_plan* plan, int32_t lanes, int32_t warp_w);
 
 /* Selects the batch's execution form.  chunk_views = 0 (the default): each
- * lane runs whole scenes one after another, every view with its own
- * projection, binning and tile launch.  chunk_views in [1, 64]: the views of
- * all scenes are interleaved (view r of every scene, then view r + 1, ...)
- * and cut into chunks of chunk_views views; each view of a chunk is projected
+ * lane runs whole scenes one after another, up to four views (or one, see
+ * scoup_plan_create) to a projection, binning and tile launch.  chunk_views in
+ * [1, 64]: the views of all scenes are interleaved (view r of every scene, then
+ * view r + 1, ...) and cut into chunks of chunk_views views; each view of a chunk is projected
  * and binned into a view workspace of its own, then ONE persistent tile launch
  * composites every (scene, view, tile) item of the chunk, its CTAs taking
  * items from an atomic counter; `lanes` chunks are in flight on the lanes'
@@ -578,7 +582,7 @@ int scoup_decode_backward_fp32(const float* dF, int64_t P, int32_t D, const floa
  *  dF          DEVICE [P, D] float32 (dF_dtype 0) or bf16 (dF_dtype 1): overwritten.
  *  loss        DEVICE double: L is added to it (FP32 terms, FP64 sum), or NULL.
  *  workspace   DEVICE, >= scoup_region_l2_grad_workspace_size(R, D) bytes
- *              (the decoded region targets, FP32).
+ *              (the decoded region targets, FP32), any 4-byte aligned address.
  * A region id >= R or an atom >= C sets the device status read by
  * scoup_read_stats(workspace) (SCOUP_ERR_DEVICE_CHECK).  Asynchronous. */
 size_t scoup_region_l2_grad_workspace_size(int32_t R, int32_t D);

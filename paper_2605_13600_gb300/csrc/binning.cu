@@ -77,8 +77,9 @@ struct LocalBox {
 
 __device__ __forceinline__ bool big(const ushort4& r) { return (r.z - r.x) * (r.w - r.y) > kBigRect; }
 
-// Warp-cooperative expansion of the (Gaussian, tile) items of the 32
-// Gaussians held by the lanes (lane l holds rectangle r): the items are
+// Warp-cooperative expansion of the (Gaussian, list) items of the 32 Gaussians
+// held by the lanes (lane l holds rectangle r, in blocks of tiles where the
+// lists are blocks'): the items are
 // numbered by an exclusive scan of the rectangle areas and dealt out 32 at a
 // time, one per lane, so every lane works on one item per round whatever the
 // rectangle sizes.  f(src_lane, tx, ty) is called for each item.
