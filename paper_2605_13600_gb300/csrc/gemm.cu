@@ -24,9 +24,9 @@
 //   kOutCos  : f32 output / (|row| |column|), 0 where |row| < 1e-12
 // Every mbarrier wait is bounded; a wait that gives up records an error in
 // *status, raises the CTA's abort flag, and every role leaves after draining
-// its own copies in flight; TMEM is freed on every path.  A role's loop is left
-// by whole warps: the lanes vote on each wait and on the flag, so that no lane
-// stays behind at a warp barrier that another one has skipped.
+// its own copies in flight; TMEM is freed on every path.  No lane
+// is left behind at a warp barrier that another one has skipped (wait_or_abort,
+// issuer_wait).
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -61,14 +61,14 @@ struct GemmSmem {
   uint64_t drain;
   uint32_t tmem;
   volatile int abort;
+  int ignored;  // what the MMA warp's lanes beside lane 0 report (issuer_wait)
 };
 
-// Both are called by whole warps and give every lane the same answer: lanes
-// poll the barrier and read the flag on their own, and one of them may see what
-// the next one has just missed.  The vote keeps the warp together, so the
-// issuing loops have no other warp barrier.  Its price is 2 % of a decode, loss
-// and backward of 480000 rows (548 us if every lane may leave alone, 559 so);
-// one polling lane and a shuffle cost 6 %, a vote behind the issue 10 %.
+// The lanes of a warp poll a barrier and read the flag on their own, and one of
+// them may see what the next one has just missed.  A warp whose loop holds warp
+// barriers or warp-wide instructions therefore votes, and all its lanes leave
+// together (the vote also keeps an issuing warp converged: the producers' loops
+// have no other warp barrier).
 __device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abort, int* status) {
   if (__all_sync(0xffffffffu, ptx::mbar_wait_bounded(bar, parity, kWaitIters))) return true;
   atomicOr(status, kStatTimeout);
@@ -77,6 +77,19 @@ __device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, vo
 }
 
 __device__ __forceinline__ bool gave_up(const volatile int* abort) { return __any_sync(0xffffffffu, *abort != 0); }
+
+// The MMA issuer does not vote: in front of every stage's MMAs the vote costs 2 to
+// 8 % (2073600 FP32 rows of 256 to 512 features 802 us, 741 so).  Its loop holds
+// nothing warp-wide, so a lane may leave alone, and lane 0, which issues, alone
+// decides: the other lanes report into words that nobody reads, and one that
+// gives up only stops keeping lane 0 company.  (Words instead of a branch on the
+// lane, which costs as much as the vote.)
+__device__ __forceinline__ bool issuer_wait(uint64_t* bar, uint32_t parity, int* abort, int* status) {
+  if (ptx::mbar_wait_bounded(bar, parity, kWaitIters)) return true;
+  atomicOr(status, kStatTimeout);
+  *(volatile int*)abort = 1;
+  return false;
+}
 
 // acc += the squares of the two bf16 values of w (one packed FP32 FMA).
 __device__ __forceinline__ void add_squares(uint32_t w, unsigned long long& acc) {
@@ -284,17 +297,19 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_kernel(const __grid
     const uint64_t da0 = ptx::smem_desc_k128(ptx::smem_u32(sm.a[0])), db0 = ptx::smem_desc_k128(ptx::smem_u32(sm.b[0]));
     int it = 0, local = 0;
     bool ok = true;
-    for (int i = 0; ok && !gave_up(&sm.abort); ++i, ++local) {
+    int* const my_abort = lane == 0 ? const_cast<int*>(&sm.abort) : &sm.ignored;
+    int* const my_status = lane == 0 ? ep.status : &sm.ignored;
+    for (int i = 0; ok && !sm.abort; ++i, ++local) {
       const UnitPos t = unit_at<BN, kQuery>(i, n_tiles, m_blocks);
       if (!t.valid) break;
       const uint32_t id = t.query ? idesc_q : idesc;
       const int b = local & 1, use = local >> 1;
-      if (local >= 2 && !wait_or_abort(&sm.acc_empty[b], (use - 1) & 1, &sm.abort, ep.status)) break;
+      if (local >= 2 && !issuer_wait(&sm.acc_empty[b], (use - 1) & 1, my_abort, my_status)) break;
       ptx::tc_fence_after();
       const uint32_t d = tmem + (uint32_t)(b * BN);
       for (int kb = 0; kb < kt; ++kb, ++it) {
         const int s = it % kStages;
-        if (!wait_or_abort(&sm.full[s], (it / kStages) & 1, &sm.abort, ep.status)) {
+        if (!issuer_wait(&sm.full[s], (it / kStages) & 1, my_abort, my_status)) {
           ok = false;
           break;
         }
@@ -476,6 +491,7 @@ struct RowsSmem {
   uint64_t drain;
   uint32_t tmem;
   volatile int abort;
+  int ignored;  // what the MMA warp's lanes beside lane 0 report (issuer_wait)
 };
 static_assert(sizeof(RowsSmem<false>) + 1024 <= 227 * 1024, "shared memory of one CTA");
 static_assert(sizeof(RowsSmem<true>) + 1024 <= 227 * 1024, "shared memory of one CTA");
@@ -587,11 +603,13 @@ __global__ void __launch_bounds__(RowsCfg<kF32A>::kThreads, 1)
     const uint64_t da0 = ptx::smem_desc_k128(ptx::smem_u32(sm.a[0][0])), db0 = ptx::smem_desc_k128(ptx::smem_u32(sm.b[0]));
     int ia = 0, it = 0, local = 0;
     bool ok = true;
-    for (int rb = blockIdx.x; ok && rb < blocks && !gave_up(&sm.abort); rb += (int)gridDim.x, ia += kt) {
+    int* const my_abort = lane == 0 ? const_cast<int*>(&sm.abort) : &sm.ignored;
+    int* const my_status = lane == 0 ? ep.status : &sm.ignored;
+    for (int rb = blockIdx.x; ok && rb < blocks && !sm.abort; rb += (int)gridDim.x, ia += kt) {
       for (int u = 0; ok && u < per; ++u, ++local) {
         const uint32_t id = kQuery && u == 0 ? idesc_q : idesc;
         const int b = local % kAcc, use = local / kAcc;
-        if (local >= kAcc && !wait_or_abort(&sm.acc_empty[b], (use - 1) & 1, &sm.abort, ep.status)) {
+        if (local >= kAcc && !issuer_wait(&sm.acc_empty[b], (use - 1) & 1, my_abort, my_status)) {
           ok = false;
           break;
         }
@@ -599,8 +617,8 @@ __global__ void __launch_bounds__(RowsCfg<kF32A>::kThreads, 1)
         const uint32_t d = tmem + (uint32_t)(b * kH * RN);
         for (int kb = 0; kb < kt; ++kb, ++it) {
           const int sa = (ia + kb) % kASlots, s = it % kBStages;
-          if ((u == 0 && !wait_or_abort(&sm.a_full[sa], ((ia + kb) / kASlots) & 1, &sm.abort, ep.status)) ||
-              !wait_or_abort(&sm.b_full[s], (it / kBStages) & 1, &sm.abort, ep.status)) {
+          if ((u == 0 && !issuer_wait(&sm.a_full[sa], ((ia + kb) / kASlots) & 1, my_abort, my_status)) ||
+              !issuer_wait(&sm.b_full[s], (it / kBStages) & 1, my_abort, my_status)) {
             ok = false;
             break;
           }
