@@ -457,8 +457,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_bf16_kernel(const __grid
 //     a conversion pass over memory.  128 rows to a block and 6 slots, so that
 //     the next block is converted under this one's MMAs; the epilogue groups
 //     split the columns and pass the row norms on in shared memory.
-// 2073600 x 256 -> 512 and 32 phrases: bf16 880 -> 645 us, FP32 1514 -> 1011
-// us; FP32 without the phrases 1127 -> 753 us, of which 625 are the bytes.
+// 2073600 x 256 -> 512 and 32 phrases: bf16 880 -> 643 us, FP32 1514 -> 998
+// us; FP32 without the phrases 1127 -> 741 us, of which 625 are the bytes.
 constexpr int RN = 128;
 constexpr int kMaxSlabs = 4;
 constexpr int kCvtWarps = 6;  // two teams that take the slabs by turns
